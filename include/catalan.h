@@ -181,7 +181,7 @@ int cat_factor_copy_primes(cat_ctx *ctx, const cat_factorization *f, uint32_t *d
  * out may overlap a or b (the product is then formed in library scratch and
  * copied); a disjoint out of at least na + nb limbs receives it directly.
  * Errors: CAT_EINVAL, CAT_ERANGE (cap < normalised length), CAT_ENOMEM,
- * CAT_ECUDA.  Products of up to 2^27 limbs take one three-prime transform;
+ * CAT_ECUDA.  Products of up to 2^27 limbs take one five-prime transform;
  * longer ones are summed from products of pieces of at most 2^26 limbs (any
  * length that fits device memory). */
 int bigint_mul(cat_ctx *ctx, const uint32_t *a, size_t na, const uint32_t *b,
@@ -338,7 +338,7 @@ int cat_binary(cat_ctx *ctx, const uint32_t *limbs, size_t n, uint8_t *out, size
  * limbs[0..n) (device pointer; leading zero limbs allowed) as ASCII into the
  * device buffer out of cap bytes: most significant digit first, no sign, no
  * leading zeros, no terminator; "0" for zero.  *out_len = the digit count.
- * Converted by a tree over the limbs in base 10^9 (batched three-prime
+ * Converted by a tree over the limbs in base 10^9 (batched five-prime
  * products with the powers 2^(32 w), carries in base 10^9); scratch comes
  * from the context's pool and is about 3x the input.  Returns when done.
  * Errors: CAT_EINVAL (null pointer), CAT_ERANGE (cap too small; *out_len is

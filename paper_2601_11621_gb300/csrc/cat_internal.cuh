@@ -1,9 +1,9 @@
 // cat_internal.cuh -- shared internals of libcatalan (context, errors, device
 // memory, 32-bit modular arithmetic for the NTT primes).
 //
-// Integer representation: little-endian uint32 limbs.  The NTT works modulo
-// three primes q = k * 2^m + 1 (one of three prime sets, by transform size,
-// see below); one transform covers up to 2^27 points.
+// Integer representation: little-endian uint32 limbs.  The NTT works on 64-bit
+// coefficients modulo five primes q = k * 2^m + 1 (one of three prime sets, by
+// transform size, see below); one transform covers up to 2^26 points.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -36,31 +36,41 @@ void launched(const char *what);
 
 // ------------------------------------------------------------- constants
 
-constexpr int kNumPrimes = 3;
-constexpr int kLogMaxNtt = 27;  // largest transform: 2^27 points
-// Three sets of three NTT primes q = k 2^m + 1, chosen by the transform size
-// 2^n.  In each set the product of the primes exceeds the largest convolution
-// coefficient 2^(n-1) (2^32 - 1)^2 of two operands whose lengths add up to 2^n
-// limbs, so the Chinese remaindering is exact.
-//   set 0, n <= 23: q < 2^30, 2^23 | q - 1 (product ~2^89.35 > 2^86).  As
+constexpr int kNumPrimes = 5;
+constexpr int kLogMaxNtt = 27;  // longest product of one transform: 2^27 limbs
+// A transform's points are 64-bit coefficients (two limbs, or two base-10^9
+// digits): a product of 2^n limbs is a cyclic convolution of 2^(n-1) points.
+constexpr int kLogMaxPts = kLogMaxNtt - 1;
+// Three sets of five NTT primes q = k 2^m + 1, chosen by the transform size of
+// 2^np points.  In each set the product M of the primes exceeds the largest
+// convolution coefficient 2^(np-1) (2^64 - 1)^2 of two operands whose lengths
+// add up to 2^np points, so the Chinese remaindering is exact.
+//   set 0, np <= 22: q < 2^30, 2^22 | q - 1 (M ~ 2^149.16 > 2^149).  As
 //          4q < 2^32, residues stay unreduced inside a transform: in [0, 2q)
 //          in the forward direction and [0, 4q) in the inverse one (Harvey's
 //          lazy butterflies), one correction per butterfly;
-//   set 1, n <= 26: q < 2^31, 2^26 | q - 1 (product ~2^90.47 > 2^89);
+//   set 1, np <= 25: q < 2^31, 2^25 | q - 1 (M ~ 2^153.36 > 2^152);
 //          residues in [0, q), every correction a min of two candidates,
 //          which cannot wrap because 2q < 2^32;
-//   set 2, n = 27:  q < 2^32, 2^27 | q - 1 (product ~2^93.6 > 2^90);
+//   set 2, np = 26:  q < 2^32, 2^26 | q - 1 (M ~ 2^155.4 > 2^153);
 //          residues in [0, q), compare-and-subtract corrections.
+// Why five primes for 64 bits and not three for 32: the butterflies are bound
+// by the integer multiply pipe, so what counts is residues per operand bit.
+// Three primes carry 32 bits of operand (10.7 bits per residue, the rest of
+// their 89 bits holds the product's other half and the sum), five carry 64
+// (12.8 bits per residue) on transforms of half the points, one stage
+// shorter; seven would carry 94 bits (13.4) at limb boundaries that fit no
+// word.
 // Sets 0 and 1 multiply by known factors with Shoup's method (the factor w and
 // floor(w 2^32 / q) are stored); set 2 with Montgomery's (2^32 w mod q and
 // that times q^-1 mod 2^32).  Primes ascend within a set.
 constexpr int kNumSets = 3;
-constexpr int kLogSet0 = 23;
-constexpr int kLogSet1 = 26;
+constexpr int kLogSet0 = 22;
+constexpr int kLogSet1 = 25;
 // Twiddle tables per (set, prime, direction), w the set's primitive 2^L-th
 // root of unity (L = set_log_root) or its inverse, entries as pairs in the
 // set's multiplier form:
-//   [2^s, 2^(s+1))          w_{2^(s+1)}^j, j < 2^s, for s < 13: the twiddles
+//   [2^s, 2^(s+1))          w_{2^(s+1)}^j, j < 2^s, for s < 12: the twiddles
 //                           of butterfly stage s (half-span 2^s) of a
 //                           sub-transform, consecutive in j so that the
 //                           lanes of a warp read consecutive entries;
@@ -69,27 +79,40 @@ constexpr int kLogSet1 = 26;
 //                           Shoup-form sets the third table is stored times
 //                           2^32 mod q, so the product is w^E's Montgomery
 //                           form).
-constexpr int kTwStage = 1 << 13;
+constexpr int kTwStageLog = 12;  // sub-transforms of at most 2^12 points
+constexpr int kTwStage = 1 << kTwStageLog;
 constexpr int kTwSmall = 512;
 constexpr int kTwPerDir = kTwStage + 3 * kTwSmall;  // uint2 entries per (prime, direction)
 
 __host__ __device__ constexpr uint32_t ntt_prime(int set, int i)
 {
-    return set == 0   ? (i == 0 ? 880803841u : (i == 1 ? 897581057u : 998244353u))
-           : set == 1 ? (i == 0 ? 469762049u : (i == 1 ? 1811939329u : 2013265921u))
-                      : (i == 0 ? 2013265921u : (i == 1 ? 2281701377u : 3221225473u));
+    return set == 0   ? (i == 0   ? 918552577u
+                         : i == 1 ? 935329793u
+                         : i == 2 ? 943718401u
+                         : i == 3 ? 985661441u
+                                  : 998244353u)
+           : set == 1 ? (i == 0   ? 1107296257u
+                         : i == 1 ? 1711276033u
+                         : i == 2 ? 1811939329u
+                         : i == 3 ? 2013265921u
+                                  : 2113929217u)
+                      : (i == 0   ? 1811939329u
+                         : i == 1 ? 2013265921u
+                         : i == 2 ? 2281701377u
+                         : i == 3 ? 2483027969u
+                                  : 2885681153u);
 }
 
 // log2 of the order of the root of unity the twiddle tables of a set use
 __host__ __device__ constexpr int set_log_root(int set)
 {
-    return set == 0 ? kLogSet0 : (set == 1 ? kLogSet1 : kLogMaxNtt);
+    return set == 0 ? kLogSet0 : (set == 1 ? kLogSet1 : kLogMaxPts);
 }
 
-// the prime set a transform of 2^n points uses
-__host__ __device__ constexpr int set_for(int n)
+// the prime set a transform of 2^np points uses
+__host__ __device__ constexpr int set_for(int np)
 {
-    return n <= kLogSet0 ? 0 : (n <= kLogSet1 ? 1 : 2);
+    return np <= kLogSet0 ? 0 : (np <= kLogSet1 ? 1 : 2);
 }
 
 // whether a set stores its multipliers in Shoup's form
@@ -172,7 +195,7 @@ __device__ __forceinline__ uint32_t mont_mul_pre(uint32_t a, uint32_t w, uint32_
     return hi < u ? r + q : r;
 }
 
-// x mod q for any 32-bit x (q > 2^30, so at most two subtractions).
+// x mod q for any 32-bit x (3q > 2^32, so at most two subtractions).
 __device__ __forceinline__ uint32_t reduce32(uint32_t x, uint32_t q)
 {
     if (x >= q) x -= q;
@@ -298,19 +321,32 @@ __device__ __forceinline__ void bf_dit1(uint32_t &x, uint32_t &y, uint32_t q)
     }
 }
 
-// A raw 32-bit limb into the forward range: Shoup's product with 1
-// (wp1 = floor(2^32 / q)) for sets 0 and 1, two subtractions for set 2.
+// How two words of an operand become a residue: word 0 times w0 plus word 1
+// times w1, the multipliers in the set's form.  w0 = 1 and w1 = 2^32 (or 10^9
+// for decimal digits), both times a constant where the operand takes a scale
+// in advance.
+struct CoefMul {
+    uint2 w0, w1;
+};
+
+// The residue of lo w0 + hi w1 in the forward range.  Set 2 takes w0 = 1 only
+// (lo < 2^32 < 3q).
 template <int PS>
-__device__ __forceinline__ uint32_t reduce_in(uint32_t x, uint32_t q, uint32_t wp1)
+__device__ __forceinline__ uint32_t coef_in(uint32_t lo, uint32_t hi, const CoefMul &c, uint32_t q)
 {
-    if constexpr (PS == 0) return shoup(x, 1u, wp1, q);
-    else if constexpr (PS == 1) return csub(shoup(x, 1u, wp1, q), q);
-    else return reduce32(x, q);
+    if constexpr (PS == 0) {
+        return csub(shoup(lo, c.w0.x, c.w0.y, q) + shoup(hi, c.w1.x, c.w1.y, q), 2 * q);
+    } else if constexpr (PS == 1) {
+        return csub(csub(shoup(lo, c.w0.x, c.w0.y, q), q) + csub(shoup(hi, c.w1.x, c.w1.y, q), q),
+                    q);
+    } else {
+        return add_mod(reduce32(lo, q), mont_mul_pre(hi, c.w1.x, c.w1.y, q), q);
+    }
 }
 
-// Pointwise product of two forward-range residues times the scale factor:
-// x y 2^-32 by Montgomery's reduction, then times sc = 2^32 2^-n (Shoup) for
-// sets 0 and 1 or sc = 2^64 2^-n (Montgomery) for set 2, giving x y 2^-n.
+// Pointwise product of two forward-range residues times the scale factor S:
+// x y 2^-32 by Montgomery's reduction, then times sc = 2^32 S (Shoup) for
+// sets 0 and 1 or sc = 2^64 S (Montgomery) for set 2, giving x y S.
 // For set 0, x y < 4 q^2 < 2^32 q keeps hi(x y) - hi(m q) in (-q, q).
 template <int PS>
 __device__ __forceinline__ uint32_t pmul(uint32_t x, uint32_t y, uint2 sc, uint32_t q,
@@ -325,14 +361,6 @@ __device__ __forceinline__ uint32_t pmul(uint32_t x, uint32_t y, uint2 sc, uint3
     } else {
         return mont_mul(mont_mul(x, y, q, qinv), sc.x, q, qinv);
     }
-}
-
-// An inverse-range residue reduced into [0, q).
-template <int PS>
-__device__ __forceinline__ uint32_t final_red(uint32_t r, uint32_t q)
-{
-    if constexpr (PS == 0) return csub(csub(r, 2 * q), q);
-    return r;
 }
 
 __device__ __forceinline__ uint32_t bitrev(uint32_t x, int bits)
@@ -374,9 +402,9 @@ struct Ctx {
     uint2 *twiddles = nullptr;  // [set][prime][dir][kTwPerDir] multiplier pairs
     int num_sms = 0;
     size_t comba_max_slot = 128;  // tree levels with slots up to this use schoolbook
-    int max_log = kLogMaxNtt;     // longest single transform; longer products go by pieces
-    // row-pass size (log2 points) of the multi-pass transform of 2^n points,
-    // as tuned on this device (cat_autotune); 0 = the default plan
+    int max_log = kLogMaxNtt;     // longest product (log2 limbs) of one transform; longer by pieces
+    // row-pass size (log2 points) of the multi-pass transform of products of
+    // 2^n limbs, as tuned on this device (cat_autotune); 0 = the default plan
     int row_log[kLogMaxNtt + 1] = {};
     std::string tuning;           // where the tuned values came from ("" = defaults)
     // twiddle tables of the column passes (built on first use, kept until the
@@ -391,7 +419,7 @@ struct Ctx {
     // largest block (log2 points) whose passes read a table: for the first
     // forward pass (which runs once per operand) and for the others (all by
     // default; smaller values are for measurements)
-    int col_tw_first_max_log = kLogMaxNtt, col_tw_max_log = kLogMaxNtt;
+    int col_tw_first_max_log = kLogMaxPts, col_tw_max_log = kLogMaxPts;
     // small read-backs (lengths of results): a pinned host word and a device
     // word, allocated once per context
     uint64_t *host_word = nullptr;

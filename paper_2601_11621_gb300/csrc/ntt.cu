@@ -1,27 +1,29 @@
-// ntt.cu -- exact big-integer multiplication by a three-prime number-theoretic
+// ntt.cu -- exact big-integer multiplication by a five-prime number-theoretic
 // transform (NTT), Chinese remaindering and carry propagation.
 //
 // This is the multiplication the reconstruction phase spends its time in
 // (Sec. 3.2; Sec. 6 reports that the big products dominate the run time, and
 // Sec. 6.3 assumes an FFT-based multiplication for large operands).  The
-// method is the classical one: the limbs of a and b are the coefficients of
-// two polynomials; their cyclic convolution of length L = 2^n >= na + nb is
-// computed modulo three primes q_i (forward transforms, pointwise product,
-// inverse transform), the exact coefficients are recovered by Garner's
-// mixed-radix Chinese remaindering, and their 96-bit values are summed into
-// 32-bit limbs with carry propagation.
+// method is the classical one: pairs of limbs of a and b are the 64-bit
+// coefficients of two polynomials; their cyclic convolution of length
+// 2^np >= (na + nb) / 2 is computed modulo five primes q_i (forward
+// transforms, pointwise product, inverse transform), the exact coefficients
+// are recovered by Chinese remaindering, and their 160-bit values are summed
+// into 32-bit limbs with carry propagation.  A product of 2^n limbs takes
+// transforms of 2^np points, np = n - 1.
 //
 // Transform layout.  The forward transform is an in-place decimation-in-
 // frequency transform (natural order in, bit-reversed order out); the inverse
 // is the matching decimation-in-time transform (bit-reversed in, natural out),
-// so no permutation pass is needed.  A length-2^n transform is split into
+// so no permutation pass is needed.  A length-2^np transform is split into
 // passes that each run 2^r-point sub-transforms in shared memory (the
 // "four-step" factorisation L = L1 * L2 applied recursively): column passes
 // over strided sub-arrays, each followed by the twiddle w_M^(col * k1), and a
 // final row pass over contiguous runs of 2^r points.  The last forward row
 // pass, the pointwise product and the first inverse row pass are fused.
-// Transforms of up to 2^12 points run entirely inside one thread block,
-// including the remaindering and carries.
+// Transforms of up to 2^11 points run entirely inside one thread block,
+// including the remaindering and carries; transforms of 2^12 points run in a
+// row pass alone, straight from the operands' limbs.
 #include "cat_internal.cuh"
 
 #include <algorithm>
@@ -31,20 +33,16 @@ namespace cat {
 
 // --------------------------------------------------------------- constants
 
-#define CAT_SET_CONST(f)                                                              \
-    {{f(ntt_prime(0, 0)), f(ntt_prime(0, 1)), f(ntt_prime(0, 2))},                    \
-     {f(ntt_prime(1, 0)), f(ntt_prime(1, 1)), f(ntt_prime(1, 2))},                    \
-     {f(ntt_prime(2, 0)), f(ntt_prime(2, 1)), f(ntt_prime(2, 2))}}
+#define CAT_SET_ROW(f, s) \
+    {f(ntt_prime(s, 0)), f(ntt_prime(s, 1)), f(ntt_prime(s, 2)), f(ntt_prime(s, 3)), f(ntt_prime(s, 4))}
+#define CAT_SET_CONST(f) {CAT_SET_ROW(f, 0), CAT_SET_ROW(f, 1), CAT_SET_ROW(f, 2)}
 #define CAT_Q(q) (q)
-#define CAT_WP1(q) shoup_c(1u, q)
 __constant__ uint32_t c_q[kNumSets][kNumPrimes] = CAT_SET_CONST(CAT_Q);
 __constant__ uint32_t c_qinv[kNumSets][kNumPrimes] = CAT_SET_CONST(inv32);
-// floor(2^32 / q): Shoup's companion of 1, which reduces raw limbs
-__constant__ uint32_t c_wp1[kNumSets][kNumPrimes] = CAT_SET_CONST(CAT_WP1);
 
+#undef CAT_SET_ROW
 #undef CAT_SET_CONST
 #undef CAT_Q
-#undef CAT_WP1
 
 // Entries [0, 16) of every stage table (the twiddles of stage bits below 4,
 // [set][prime][direction][index] in the stage table's own layout and
@@ -64,40 +62,117 @@ void upload_low_twiddles(const uint2 *tables)
     CAT_CUDA(cudaMemcpyToSymbol(c_tw_low, h, sizeof(h)));
 }
 
-// Garner constants of a set, in Montgomery form.
-template <int PS>
-struct Garner {
-    static constexpr uint32_t q0 = ntt_prime(PS, 0), q1 = ntt_prime(PS, 1), q2 = ntt_prime(PS, 2);
-    static constexpr uint32_t qinv1 = inv32(q1), qinv2 = inv32(q2);
-    static constexpr uint32_t inv_q0_mod_q1 = to_mont_c(powmod_u32(q0 % q1, q1 - 2, q1), q1);
-    static constexpr uint32_t q0_mod_q2 = to_mont_c(q0 % q2, q2);
-    static constexpr uint32_t inv_q0q1_mod_q2 =
-        to_mont_c(powmod_u32(mulmod_u64(q0, q1, q2), q2 - 2, q2), q2);
-    static_assert(q0 < q1 && q1 < q2, "Garner order assumes q0 < q1 < q2");
-    // the same three factors as plain residues with Shoup's companions
-    static constexpr uint32_t s1 = powmod_u32(q0 % q1, q1 - 2, q1), s1p = shoup_c(s1, q1);
-    static constexpr uint32_t s2 = q0 % q2, s2p = shoup_c(s2, q2);
-    static constexpr uint32_t s3 = powmod_u32(mulmod_u64(q0, q1, q2), q2 - 2, q2),
-                              s3p = shoup_c(s3, q2);
+// Chinese remaindering constants of a set.  With M the product of its primes
+// and y_i = c (M/q_i)^-1 mod q_i, the coefficient is c = sum_i y_i (M/q_i) -
+// k M with k = floor(sum_i y_i / q_i).  The factor (M/q_i)^-1 rides on the
+// pointwise product's scale, so the inverse transform delivers y_i itself.
+struct Words {
+    uint32_t w[6];
 };
 
-// Pointwise scale 2^-n folded into the product's second factor: 2^32 2^-n mod
-// q in Shoup's form for sets 0 and 1, 2^64 2^-n mod q (Montgomery) for set 2,
-// so that pmul(x, y) = x y 2^-n.
+// M, or M / q_skip, in base 2^32 (dec: base 10^9), least significant first
+constexpr Words crt_product(int set, int skip, bool dec)
+{
+    Words r{};
+    r.w[0] = 1;
+    const uint64_t base = dec ? (uint64_t)kDecBase : (1ull << 32);
+    for (int i = 0; i < kNumPrimes; i++) {
+        if (i == skip) continue;
+        uint64_t carry = 0;
+        for (int j = 0; j < 6; j++) {
+            const uint64_t v = (uint64_t)r.w[j] * ntt_prime(set, i) + carry;
+            r.w[j] = (uint32_t)(v % base);
+            carry = v / base;
+        }
+    }
+    return r;
+}
+
+// word j of 2^160 - M
+constexpr uint32_t crt_neg_m(int set, int j)
+{
+    const Words m = crt_product(set, -1, false);
+    uint32_t borrow = 0, r = 0;
+    for (int i = 0; i <= j; i++) {
+        const uint64_t v = (uint64_t)m.w[i] + borrow;
+        r = (uint32_t)(0u - (uint32_t)v);
+        borrow = v != 0 ? 1u : 0u;
+    }
+    return r;
+}
+
+// (M/q_i)^-1 mod q_i
+constexpr uint32_t crt_inverse(int set, int i)
+{
+    const uint32_t q = ntt_prime(set, i);
+    uint64_t x = 1;
+    for (int j = 0; j < kNumPrimes; j++)
+        if (j != i) x = x * (ntt_prime(set, j) % q) % q;
+    return powmod_u32(x, q - 2, q);
+}
+
+// Pointwise scale S = 2^-np (M/q_i)^-1 mod q_i, folded into the product's
+// second factor: 2^32 S in Shoup's form for sets 0 and 1, 2^64 S (Montgomery)
+// for set 2, so that pmul(x, y) = x y S.
 struct Scale {
     uint2 c[kNumPrimes];
 };
 
-static Scale make_scale(int set, int n)
+static uint32_t scale_value(int set, int i, int np)
+{
+    const uint32_t q = ntt_prime(set, i);
+    const uint32_t inv2n = powmod_u32((q + 1) / 2, (uint64_t)np, q);  // 2^-np
+    return to_mont_c(mulmod_u64(inv2n, crt_inverse(set, i), q), q);    // 2^32 S
+}
+
+static Scale make_scale(int set, int np)
 {
     Scale s;
     for (int i = 0; i < kNumPrimes; i++) {
         const uint32_t q = ntt_prime(set, i);
-        const uint32_t inv2n = powmod_u32((q + 1) / 2, (uint64_t)n, q);  // 2^-n
-        const uint32_t r = to_mont_c(inv2n, q);                           // 2^32 2^-n
+        const uint32_t r = scale_value(set, i, np);
         s.c[i] = set_shoup(set) ? make_uint2(r, shoup_c(r, q)) : make_uint2(to_mont_c(r, q), 0u);
     }
     return s;
+}
+
+// The operands' input multipliers (coef_in): 1 and the word base (2^32, or
+// 10^9 for decimal digits).
+struct CoefMuls {
+    CoefMul c[kNumPrimes];
+};
+
+static CoefMuls make_coef(int set, bool dec)
+{
+    CoefMuls m;
+    for (int i = 0; i < kNumPrimes; i++) {
+        const uint32_t q = ntt_prime(set, i);
+        const uint32_t b = (uint32_t)((dec ? (uint64_t)kDecBase : (1ull << 32)) % q);
+        if (set_shoup(set)) {
+            m.c[i].w0 = make_uint2(1u, shoup_c(1u, q));
+            m.c[i].w1 = make_uint2(b, shoup_c(b, q));
+        } else {
+            const uint32_t bm = to_mont_c(b, q);
+            m.c[i].w0 = make_uint2(1u, 0u);
+            m.c[i].w1 = make_uint2(bm, bm * inv32(q));
+        }
+    }
+    return m;
+}
+
+// The same times the pointwise scale 2^32 S (sets in Shoup's form): operand b
+// of a product whose pointwise step is then one Montgomery product.
+static CoefMuls make_coef_scaled(int set, int np, bool dec)
+{
+    CoefMuls m;
+    for (int i = 0; i < kNumPrimes; i++) {
+        const uint32_t q = ntt_prime(set, i);
+        const uint32_t b = (uint32_t)((dec ? (uint64_t)kDecBase : (1ull << 32)) % q);
+        const uint32_t r = scale_value(set, i, np), rb = mulmod_u64(r, b, q);
+        m.c[i].w0 = make_uint2(r, shoup_c(r, q));
+        m.c[i].w1 = make_uint2(rb, shoup_c(rb, q));
+    }
+    return m;
 }
 
 // -------------------------------------------------------------- twiddles
@@ -155,45 +230,134 @@ __device__ __forceinline__ uint32_t mont_step(uint32_t vm, uint32_t um, uint32_t
 
 // ----------------------------------------------- remaindering and carries
 
-// Garner: the coefficient c < q0 q1 q2 with c = r_i mod q_i, as three words,
-// from inverse-transform residues (reduced into [0, q_i) first).
-template <int PS>
-__device__ __forceinline__ void crt3(uint32_t r0, uint32_t r1, uint32_t r2, uint32_t &c0,
-                                     uint32_t &c1, uint32_t &c2)
+// acc += r (M/q_I) over five words, as two chains of 64-bit products: e at
+// words 0, 2 and 4, o at words 1 and 3, so that no product waits for the
+// carry of its neighbour word.
+struct Acc160 {
+    uint32_t e0, e1, e2, e3, e4, o0, o1, o2, o3;
+};
+
+template <int PS, int I>
+__device__ __forceinline__ void crt_acc(uint32_t r, Acc160 &a)
 {
-    using G = Garner<PS>;
-    uint32_t x0, x1, x2;
-    if constexpr (PS == 2) {
-        x0 = r0;  // < q0 < q1 < q2
-        x1 = mont_mul(sub_mod(r1, x0, G::q1), G::inv_q0_mod_q1, G::q1, G::qinv1);
-        uint32_t t = sub_mod(r2, x0, G::q2);
-        t = sub_mod(t, mont_mul(x1, G::q0_mod_q2, G::q2, G::qinv2), G::q2);
-        x2 = mont_mul(t, G::inv_q0q1_mod_q2, G::q2, G::qinv2);
-    } else {
-        // Shoup products take any 32-bit input, so the differences go in
-        // unreduced: set 0's lazy residues need only r0 fully reduced (it is
-        // the exact low digit) and r1, r2 below 2q; set 1's are below q.
-        x0 = final_red<PS>(r0, G::q0);
-        if constexpr (PS == 0) {
-            r1 = csub(r1, 2 * G::q1);  // [0, 2 q1)
-            r2 = csub(r2, 2 * G::q2);  // [0, 2 q2)
-        }
-        // (r1 - x0) / q0 mod q1, the input in (0, 3 q1)
-        x1 = csub(shoup(r1 - x0 + G::q1, G::s1, G::s1p, G::q1), G::q1);
-        const uint32_t u = csub(shoup(x1, G::s2, G::s2p, G::q2), G::q2);  // x1 q0 mod q2
-        uint32_t t;
-        if constexpr (PS == 0)
-            t = r2 - x0 - u + 2 * G::q2;  // (0, 4 q2), below 2^32 as 4 q2 < 2^32
-        else
-            t = sub_m<true>(r2, x0, G::q2) - u + G::q2;  // (0, 2 q2)
-        x2 = csub(shoup(t, G::s3, G::s3p, G::q2), G::q2);
-    }
-    const uint64_t y = (uint64_t)G::q1 * x2 + x1;                 // < q1 q2
-    const uint64_t lo = (uint64_t)G::q0 * (uint32_t)y + x0;
-    const uint64_t hi = (uint64_t)G::q0 * (uint32_t)(y >> 32) + (lo >> 32);
-    c0 = (uint32_t)lo;
-    c1 = (uint32_t)hi;
-    c2 = (uint32_t)(hi >> 32);
+    constexpr Words m = crt_product(PS, I, false);
+    constexpr uint32_t m0 = m.w[0], m1 = m.w[1], m2 = m.w[2], m3 = m.w[3];
+    static_assert(m.w[4] == 0, "M/q_i fits four words");
+    asm("mad.lo.cc.u32 %0, %5, %6, %0;\n\t"
+        "madc.hi.cc.u32 %1, %5, %6, %1;\n\t"
+        "madc.lo.cc.u32 %2, %5, %7, %2;\n\t"
+        "madc.hi.cc.u32 %3, %5, %7, %3;\n\t"
+        "addc.u32 %4, %4, 0;\n\t"
+        : "+r"(a.e0), "+r"(a.e1), "+r"(a.e2), "+r"(a.e3), "+r"(a.e4)
+        : "r"(r), "r"(m0), "r"(m2));
+    asm("mad.lo.cc.u32 %0, %4, %5, %0;\n\t"
+        "madc.hi.cc.u32 %1, %4, %5, %1;\n\t"
+        "madc.lo.cc.u32 %2, %4, %6, %2;\n\t"
+        "madc.hi.u32 %3, %4, %6, %3;\n\t"
+        : "+r"(a.o0), "+r"(a.o1), "+r"(a.o2), "+r"(a.o3)
+        : "r"(r), "r"(m1), "r"(m3));
+}
+
+// The coefficient's five words from its residues y_i = r[i] mod q_i (any
+// 32-bit representatives): c = sum_i r_i (M/q_i) - k M.  k = floor(sum_i
+// r_i/q_i) comes from a fixed-point sum of r_i floor(2^57/q_i) / 2^32 in units
+// of 2^-25, short of the true sum by at most 10 units (1 per floor of the
+// quotient and of the product); c/M < 0.895 in every set, so the fraction
+// never reaches the next integer with 16 units added.  The sum stays below
+// 20 M < 2^160.  Against Garner's mixed radix this takes no modular products
+// at all (20 + 5 word products instead of 10 Shoup products and 10).
+template <int PS>
+__device__ __forceinline__ void crt5(const uint32_t (&r)[kNumPrimes], uint32_t (&w)[5])
+{
+    constexpr uint32_t f0 = (uint32_t)((1ull << 57) / ntt_prime(PS, 0)),
+                       f1 = (uint32_t)((1ull << 57) / ntt_prime(PS, 1)),
+                       f2 = (uint32_t)((1ull << 57) / ntt_prime(PS, 2)),
+                       f3 = (uint32_t)((1ull << 57) / ntt_prime(PS, 3)),
+                       f4 = (uint32_t)((1ull << 57) / ntt_prime(PS, 4));
+    const uint32_t k = (__umulhi(r[0], f0) + __umulhi(r[1], f1) + __umulhi(r[2], f2) +
+                        __umulhi(r[3], f3) + __umulhi(r[4], f4) + 16u) >>
+                       25;
+    Acc160 a{0, 0, 0, 0, 0, 0, 0, 0, 0};
+    crt_acc<PS, 0>(r[0], a);
+    crt_acc<PS, 1>(r[1], a);
+    crt_acc<PS, 2>(r[2], a);
+    crt_acc<PS, 3>(r[3], a);
+    crt_acc<PS, 4>(r[4], a);
+    // - k M modulo 2^160
+    constexpr uint32_t n0 = crt_neg_m(PS, 0), n1 = crt_neg_m(PS, 1), n2 = crt_neg_m(PS, 2),
+                       n3 = crt_neg_m(PS, 3), n4 = crt_neg_m(PS, 4);
+    asm("mad.lo.cc.u32 %0, %5, %6, %0;\n\t"
+        "madc.hi.cc.u32 %1, %5, %6, %1;\n\t"
+        "madc.lo.cc.u32 %2, %5, %7, %2;\n\t"
+        "madc.hi.cc.u32 %3, %5, %7, %3;\n\t"
+        "madc.lo.u32 %4, %5, %8, %4;\n\t"
+        : "+r"(a.e0), "+r"(a.e1), "+r"(a.e2), "+r"(a.e3), "+r"(a.e4)
+        : "r"(k), "r"(n0), "r"(n2), "r"(n4));
+    asm("mad.lo.cc.u32 %0, %4, %5, %0;\n\t"
+        "madc.hi.cc.u32 %1, %4, %5, %1;\n\t"
+        "madc.lo.cc.u32 %2, %4, %6, %2;\n\t"
+        "madc.hi.u32 %3, %4, %6, %3;\n\t"
+        : "+r"(a.o0), "+r"(a.o1), "+r"(a.o2), "+r"(a.o3)
+        : "r"(k), "r"(n1), "r"(n3));
+    w[0] = a.e0;
+    asm("add.cc.u32 %0, %4, %8;\n\t"
+        "addc.cc.u32 %1, %5, %9;\n\t"
+        "addc.cc.u32 %2, %6, %10;\n\t"
+        "addc.u32 %3, %7, %11;\n\t"
+        : "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4])
+        : "r"(a.e1), "r"(a.e2), "r"(a.e3), "r"(a.e4), "r"(a.o0), "r"(a.o1), "r"(a.o2),
+          "r"(a.o3));
+}
+
+// digit D of M/q_i summed over the primes: sum_i r_i (digit D of M/q_i)
+template <int PS, int D>
+__device__ __forceinline__ uint64_t crt_dec_column(const uint32_t (&r)[kNumPrimes])
+{
+    constexpr uint32_t d0 = crt_product(PS, 0, true).w[D], d1 = crt_product(PS, 1, true).w[D],
+                       d2 = crt_product(PS, 2, true).w[D], d3 = crt_product(PS, 3, true).w[D],
+                       d4 = crt_product(PS, 4, true).w[D];
+    return (uint64_t)r[0] * d0 + (uint64_t)r[1] * d1 + (uint64_t)r[2] * d2 + (uint64_t)r[3] * d3 +
+           (uint64_t)r[4] * d4;
+}
+
+// The coefficient's five base-10^9 digits (digit operands: c < 2^25 10^36 <
+// 10^44), the same sum with M/q_i and M written in base 10^9, modulo 10^45.
+// A column stays below 10^9 sum_i r_i < 2^64: residues below 2q in set 0
+// (10^9 sum 2q = 9.6 10^18), below q otherwise (at most 1.15 10^19).
+template <int PS>
+__device__ __forceinline__ void crt5_dec(const uint32_t (&r_in)[kNumPrimes], uint32_t (&w)[5])
+{
+    uint32_t r[kNumPrimes];
+#pragma unroll
+    for (int i = 0; i < kNumPrimes; i++)
+        r[i] = PS == 0 ? csub(r_in[i], 2 * ntt_prime(0, i)) : r_in[i];
+    constexpr uint32_t f0 = (uint32_t)((1ull << 57) / ntt_prime(PS, 0)),
+                       f1 = (uint32_t)((1ull << 57) / ntt_prime(PS, 1)),
+                       f2 = (uint32_t)((1ull << 57) / ntt_prime(PS, 2)),
+                       f3 = (uint32_t)((1ull << 57) / ntt_prime(PS, 3)),
+                       f4 = (uint32_t)((1ull << 57) / ntt_prime(PS, 4));
+    const uint64_t k = (__umulhi(r[0], f0) + __umulhi(r[1], f1) + __umulhi(r[2], f2) +
+                        __umulhi(r[3], f3) + __umulhi(r[4], f4) + 16u) >>
+                       25;  // at most 9
+    constexpr uint32_t m0 = crt_product(PS, -1, true).w[0], m1 = crt_product(PS, -1, true).w[1],
+                       m2 = crt_product(PS, -1, true).w[2], m3 = crt_product(PS, -1, true).w[3],
+                       m4 = crt_product(PS, -1, true).w[4];
+    // each column plus 16 10^9 (more than k times a digit of M and 16), whose
+    // 16 the next column gives back
+    constexpr uint64_t kBias = 16ull * kDecBase;
+    uint64_t v = crt_dec_column<PS, 0>(r) + kBias - k * m0, q = v / kDecBase;
+    w[0] = (uint32_t)(v - q * kDecBase);
+    v = crt_dec_column<PS, 1>(r) + kBias - k * m1 + q - 16u;
+    q = v / kDecBase;
+    w[1] = (uint32_t)(v - q * kDecBase);
+    v = crt_dec_column<PS, 2>(r) + kBias - k * m2 + q - 16u;
+    q = v / kDecBase;
+    w[2] = (uint32_t)(v - q * kDecBase);
+    v = crt_dec_column<PS, 3>(r) + kBias - k * m3 + q - 16u;
+    q = v / kDecBase;
+    w[3] = (uint32_t)(v - q * kDecBase);
+    v = crt_dec_column<PS, 4>(r) + kBias - k * m4 + q - 16u;
+    w[4] = (uint32_t)(v % kDecBase);
 }
 
 // The carry map of a run in compact form.  A run takes its carry-in c in
@@ -255,87 +419,84 @@ __device__ uint32_t block_carry_scan(uint32_t f, uint32_t *wsm, uint32_t *total)
 
 constexpr int kLimbsPerThread = 8;
 
-// Coefficient words of a thread's run of kLimbsPerThread consecutive
-// coefficients j0 + i (c0 the low word, c1 the middle, c2 the high).  Limb j
-// sums c0[j] + c1[j-1] + c2[j-2], so the first two limbs of a run also need
-// c1[j0-1], c2[j0-2] and c2[j0-1] of the preceding run.
+constexpr int kCoefsPerThread = kLimbsPerThread / 2;
+
+// The limbs of a thread's run of four consecutive coefficients j0 + i, words
+// w[i][0..4] each.  Limb 2j sums words 0 of coefficient j, 2 of j - 1 and 4
+// of j - 2, limb 2j + 1 words 1 of j and 3 of j - 1, so the run also needs
+// words 2, 3 and 4 of coefficient j0 - 1 (h2, h3, h4b) and word 4 of j0 - 2
+// (h4a).
 struct CoefRun {
-    uint32_t c0[kLimbsPerThread], c1[kLimbsPerThread], c2[kLimbsPerThread];
+    uint32_t w[kCoefsPerThread][5];
+    uint32_t h2, h3, h4a, h4b;
+    __device__ __forceinline__ uint64_t operator()(int i) const
+    {
+        const int j = i >> 1;
+        if (i & 1) return (uint64_t)w[j][1] + (j >= 1 ? w[j - 1][3] : h3);
+        return (uint64_t)w[j][0] + (j >= 1 ? w[j - 1][2] : h2) +
+               (j >= 2 ? w[j - 2][4] : (j == 0 ? h4a : h4b));
+    }
 };
 
-// Those three halo words from the preceding thread: by shuffle inside a warp,
-// through hsm (3 x 32 words) across warps; thread 0 takes first1/first2a/
-// first2b (the block's predecessor).  Every thread of the block calls this.
-__device__ __forceinline__ void run_halo(const CoefRun &r, uint32_t first1, uint32_t first2a,
-                                         uint32_t first2b, uint32_t *hsm, uint32_t &h1,
-                                         uint32_t &h2a, uint32_t &h2b)
+// The halo words from the preceding thread: by shuffle inside a warp, through
+// hsm (4 x 32 words) across warps; thread 0 keeps what its run holds (the
+// block's predecessor).  Every thread of the block calls this.
+__device__ __forceinline__ void run_halo(CoefRun &r, uint32_t *hsm)
 {
-    constexpr int L = kLimbsPerThread;
+    constexpr int C = kCoefsPerThread;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    h1 = __shfl_up_sync(0xffffffffu, r.c1[L - 1], 1);
-    h2a = __shfl_up_sync(0xffffffffu, r.c2[L - 2], 1);
-    h2b = __shfl_up_sync(0xffffffffu, r.c2[L - 1], 1);
+    const uint32_t a = __shfl_up_sync(0xffffffffu, r.w[C - 1][2], 1);
+    const uint32_t b = __shfl_up_sync(0xffffffffu, r.w[C - 1][3], 1);
+    const uint32_t c = __shfl_up_sync(0xffffffffu, r.w[C - 2][4], 1);
+    const uint32_t d = __shfl_up_sync(0xffffffffu, r.w[C - 1][4], 1);
     if (lane == 31) {
-        hsm[wid] = r.c1[L - 1];
-        hsm[32 + wid] = r.c2[L - 2];
-        hsm[64 + wid] = r.c2[L - 1];
+        hsm[wid] = r.w[C - 1][2];
+        hsm[32 + wid] = r.w[C - 1][3];
+        hsm[64 + wid] = r.w[C - 2][4];
+        hsm[96 + wid] = r.w[C - 1][4];
     }
     __syncthreads();
-    if (lane == 0) {
-        h1 = wid ? hsm[wid - 1] : first1;
-        h2a = wid ? hsm[32 + wid - 1] : first2a;
-        h2b = wid ? hsm[64 + wid - 1] : first2b;
+    if (lane) {
+        r.h2 = a;
+        r.h3 = b;
+        r.h4a = c;
+        r.h4b = d;
+    } else if (wid) {
+        r.h2 = hsm[wid - 1];
+        r.h3 = hsm[32 + wid - 1];
+        r.h4a = hsm[64 + wid - 1];
+        r.h4b = hsm[96 + wid - 1];
     }
 }
 
-// The exact coefficient c = w2 2^64 + w1 2^32 + w0 < 10^26 as three base-10^9
-// digits (c < min(na, nb) (10^9 - 1)^2 < 2^26 10^18 for digit operands and
-// transforms of at most 2^27 points, so the top digit is below 10^8).
-__device__ __forceinline__ void words_to_dec(uint32_t &w0, uint32_t &w1, uint32_t &w2)
-{
-    const uint64_t hi = ((uint64_t)w2 << 32) | w1;
-    const uint64_t qh = hi / kDecBase;
-    const uint32_t rh = (uint32_t)(hi - qh * kDecBase);
-    const uint64_t lo = ((uint64_t)rh << 32) | w0;
-    const uint64_t ql = lo / kDecBase;
-    const uint64_t q = (qh << 32) + ql;  // floor(c / 10^9) < 10^17
-    const uint64_t q2 = q / kDecBase;
-    w0 = (uint32_t)(lo - ql * kDecBase);
-    w1 = (uint32_t)(q - q2 * kDecBase);
-    w2 = (uint32_t)q2;
-}
-
-// Limb sums and carries for one tile of coefficient runs, one run per thread
-// (run j0 = kLimbsPerThread * threadIdx.x; coefficients at or past tile_len
-// are zero), in base 2^32 or (dec) 10^9, plus the addend limbs add[j] for
-// j < add_count.  In both bases a limb sums two full words, the coefficient's
-// top word or digit (below 2^26 or 10^8: coefficients stay below 2^90, or
-// 10^26 for digit operands), the addend and a carry <= 3, so carries stay in
-// {0, 1, 2, 3}.  Writes limbs j < min(tile_len, out_count) to out and returns
-// the tile's carry map in compact form in *tile_map (valid in every thread; it
-// fits a byte).  The tile's own carry-in is assumed 0.
-// DEC / ADD: 1 or 0 when known at compile time, -1 when the runtime flag
-// (dec, add != null) decides.
-template <int DEC, int ADD>
-__device__ __forceinline__ void tile_carry_t(const CoefRun &r, uint32_t h1, uint32_t h2a,
-                                             uint32_t h2b, int tile_len, uint32_t *out,
-                                             long out_count, bool dec_rt, const uint32_t *add,
-                                             long add_count, uint32_t *wsm, uint32_t *tile_map)
+// Limb sums and carries for one tile of runs, one run of LPT limbs per thread
+// (limb j0 + i, j0 = LPT * threadIdx.x, sums
+// sum(i); limbs at or past tile_len are none), in base 2^32 or (DEC) 10^9,
+// plus (ADD) the addend limbs add[j] for j < add_count.  In both bases a limb
+// sums at most two full words, a coefficient's top word or digit (below 2^26
+// or 10^8: coefficients stay below 2^153, or 10^44 for digit operands), the
+// addend and a carry <= 3, so carries stay in {0, 1, 2, 3}.  Writes limbs j <
+// min(tile_len, out_count) to out and returns the tile's carry map in compact
+// form in *tile_map (valid in every thread; it fits a byte).  The tile's own
+// carry-in is assumed 0.  DEC / ADD: 1 or 0 when known at compile time, -1
+// when the runtime flag (dec, add != null) decides.  LPT: limbs per run.
+template <int DEC, int ADD, int LPT = kLimbsPerThread, class SUM>
+__device__ __forceinline__ void tile_carry(const SUM &sum, int tile_len, uint32_t *out,
+                                           long out_count, bool dec_rt, const uint32_t *add,
+                                           long add_count, uint32_t *wsm, uint32_t *tile_map)
 {
     const bool dec = DEC < 0 ? dec_rt : DEC == 1;
     if (ADD == 0) add = nullptr;
-    const int j0 = threadIdx.x * kLimbsPerThread;
+    const int j0 = threadIdx.x * LPT;
     const uint32_t top = dec ? kDecBase - 1 : 0xffffffffu;  // largest limb
-    uint32_t limb[kLimbsPerThread];
+    uint32_t limb[LPT];
     uint32_t carry = 0;
     uint32_t f = kUnitId;
     if (j0 < tile_len) {
 #pragma unroll
-        for (int i = 0; i < kLimbsPerThread; i++) {
-            const uint32_t m1 = i >= 1 ? r.c1[i - 1] : h1;
-            const uint32_t m2 = i >= 2 ? r.c2[i - 2] : (i == 0 ? h2a : h2b);
+        for (int i = 0; i < LPT; i++) {
             const uint32_t ad = (add && j0 + i < add_count) ? add[j0 + i] : 0u;
-            const uint64_t v = (uint64_t)r.c0[i] + m1 + m2 + ad + carry;
+            const uint64_t v = sum(i) + ad + carry;
             if (dec) {
                 const uint32_t v32 = (uint32_t)v;  // < 3.1 10^9 + 3 < 2^32
                 carry = (v32 >= kDecBase) + (v32 >= 2 * kDecBase) + (v32 >= 3 * kDecBase);
@@ -347,7 +508,7 @@ __device__ __forceinline__ void tile_carry_t(const CoefRun &r, uint32_t h1, uint
         }
         bool ones = true;
 #pragma unroll
-        for (int i = 1; i < kLimbsPerThread; i++) ones = ones && limb[i] == top;
+        for (int i = 1; i < LPT; i++) ones = ones && limb[i] == top;
         // a carry-in c leaves the run iff ones and limb[0] + c > top
         const uint32_t t = (ones && limb[0] >= top - 2u) ? top + 1u - limb[0] : 4u;
         f = (carry << 4) | t;
@@ -356,101 +517,98 @@ __device__ __forceinline__ void tile_carry_t(const CoefRun &r, uint32_t h1, uint
     if (j0 < tile_len) {
         uint32_t c = cin;
 #pragma unroll
-        for (int i = 0; i < kLimbsPerThread; i++) {
+        for (int i = 0; i < LPT; i++) {
             const uint64_t v = (uint64_t)limb[i] + c;
             c = dec ? (uint32_t)(v >= kDecBase) : (uint32_t)(v >> 32);
             limb[i] = dec ? (uint32_t)(v - (uint64_t)c * kDecBase) : (uint32_t)v;
         }
-        if (j0 + kLimbsPerThread <= tile_len && j0 + kLimbsPerThread <= out_count &&
+        if (j0 + LPT <= tile_len && j0 + LPT <= out_count &&
             (reinterpret_cast<uintptr_t>(out + j0) & 15) == 0) {
             uint4 *o4 = reinterpret_cast<uint4 *>(out + j0);
-            o4[0] = make_uint4(limb[0], limb[1], limb[2], limb[3]);
-            o4[1] = make_uint4(limb[4], limb[5], limb[6], limb[7]);
+#pragma unroll
+            for (int i = 0; i < LPT / 4; i++)
+                o4[i] = make_uint4(limb[4 * i], limb[4 * i + 1], limb[4 * i + 2], limb[4 * i + 3]);
         } else {
 #pragma unroll
-            for (int i = 0; i < kLimbsPerThread; i++)
+            for (int i = 0; i < LPT; i++)
                 if (j0 + i < tile_len && j0 + i < out_count) out[j0 + i] = limb[i];
         }
     }
 }
 
-__device__ void tile_carry(const CoefRun &r, uint32_t h1, uint32_t h2a, uint32_t h2b, int tile_len,
-                           uint32_t *out, long out_count, bool dec, const uint32_t *add,
-                           long add_count, uint32_t *wsm, uint32_t *tile_map)
-{
-    tile_carry_t<-1, -1>(r, h1, h2a, h2b, tile_len, out, out_count, dec, add, add_count, wsm,
-                         tile_map);
-}
-
 constexpr int kTileThreads = 256;
 constexpr int kTile = kTileThreads * kLimbsPerThread;  // 2048 limbs
 
+constexpr int kTileCoefs = kTile / 2;
+
 struct CrtArgs {
-    const uint32_t *G;  // inverse-transformed residues [prime][product][L]
+    const uint32_t *G;  // inverse-transformed residues [prime][product][2^np]
     size_t gpstride;
-    int n;              // log2 L
-    Sink sink;          // product k's limbs (out_len <= L)
+    int np;             // log2 points
+    Sink sink;          // product k's limbs (out_len <= 2^(np+1))
     uint8_t *tile_maps; // [product][tiles], compact carry maps
 };
 
-// One tile of 2048 coefficients per block: each thread remainders its run of
-// eight (two 16-byte loads per prime: tiles, runs and the prime arrays are
-// multiples of 8 words apart) and sums them into limbs.
+template <int PS, bool DEC>
+__device__ __forceinline__ void coef_words(const uint32_t (&r)[kNumPrimes], uint32_t (&w)[5])
+{
+    if constexpr (DEC) crt5_dec<PS>(r, w);
+    else crt5<PS>(r, w);
+}
+
+// One tile of 1,024 coefficients (2,048 limbs) per block: each thread
+// remainders its run of four (one 16-byte load per prime: tiles, runs and the
+// prime arrays are multiples of 4 words apart) and sums them into limbs.
 template <int PS, bool DEC, bool ADD>
 __global__ void __launch_bounds__(kTileThreads) crt_carry_tiles(CrtArgs a)
 {
     __shared__ uint32_t wsm[32];
-    __shared__ uint32_t hsm[96];
-    const size_t tiles = ((size_t)1 << a.n) / kTile;
+    __shared__ uint32_t hsm[128];
+    const size_t tiles = ((size_t)1 << a.np) / kTileCoefs;
     const size_t k = blockIdx.x / tiles;
     const size_t t = blockIdx.x % tiles;
-    const size_t jt = t * kTile;
+    const size_t jt = t * kTileCoefs;
     const size_t node = sink_node(a.sink, k);
-    const uint32_t *g0 = a.G + (k << a.n) + jt;
-    const int j0 = threadIdx.x * kLimbsPerThread;
-    constexpr bool dec = DEC;
-    uint32_t r[3][kLimbsPerThread];
+    const uint32_t *g0 = a.G + (k << a.np) + jt;
+    const int j0 = threadIdx.x * kCoefsPerThread;
+    uint32_t r[kCoefsPerThread][kNumPrimes];
 #pragma unroll
-    for (int p = 0; p < 3; p++) {
-        const uint4 *v = reinterpret_cast<const uint4 *>(g0 + p * a.gpstride + j0);
-        const uint4 x = v[0], y = v[1];
-        r[p][0] = x.x; r[p][1] = x.y; r[p][2] = x.z; r[p][3] = x.w;
-        r[p][4] = y.x; r[p][5] = y.y; r[p][6] = y.z; r[p][7] = y.w;
+    for (int p = 0; p < kNumPrimes; p++) {
+        const uint4 x = *reinterpret_cast<const uint4 *>(g0 + p * a.gpstride + j0);
+        r[0][p] = x.x; r[1][p] = x.y; r[2][p] = x.z; r[3][p] = x.w;
     }
     // the tile's predecessor: coefficients jt - 2 and jt - 1 (none for tile 0),
     // loaded by thread 0 beside its run so that the latencies overlap
     const bool pred = threadIdx.x == 0 && t > 0;
-    uint32_t pr[3][2] = {{0, 0}, {0, 0}, {0, 0}};
+    uint32_t pr[2][kNumPrimes] = {};
     if (pred) {
 #pragma unroll
-        for (int p = 0; p < 3; p++) {
-            pr[p][0] = g0[p * a.gpstride - 2];
-            pr[p][1] = g0[p * a.gpstride - 1];
+        for (int p = 0; p < kNumPrimes; p++) {
+            pr[0][p] = g0[p * a.gpstride - 2];
+            pr[1][p] = g0[p * a.gpstride - 1];
         }
     }
     CoefRun run;
 #pragma unroll
-    for (int i = 0; i < kLimbsPerThread; i++) {
-        crt3<PS>(r[0][i], r[1][i], r[2][i], run.c0[i], run.c1[i], run.c2[i]);
-        if (dec) words_to_dec(run.c0[i], run.c1[i], run.c2[i]);
-    }
-    uint32_t f1 = 0, f2a = 0, f2b = 0;
+    for (int i = 0; i < kCoefsPerThread; i++) coef_words<PS, DEC>(r[i], run.w[i]);
+    run.h2 = run.h3 = run.h4a = run.h4b = 0;
     if (pred) {
-        uint32_t d0, d1, e0;
-        crt3<PS>(pr[0][0], pr[1][0], pr[2][0], d0, d1, f2a);
-        if (dec) words_to_dec(d0, d1, f2a);
-        crt3<PS>(pr[0][1], pr[1][1], pr[2][1], e0, f1, f2b);
-        if (dec) words_to_dec(e0, f1, f2b);
+        uint32_t d[5];
+        coef_words<PS, DEC>(pr[0], d);
+        run.h4a = d[4];
+        coef_words<PS, DEC>(pr[1], d);
+        run.h2 = d[2];
+        run.h3 = d[3];
+        run.h4b = d[4];
     }
-    uint32_t h1, h2a, h2b;
-    run_halo(run, f1, f2a, f2b, hsm, h1, h2a, h2b);
+    run_halo(run, hsm);
     const Sink &o = a.sink;
-    const long remaining = (long)o.out_len - (long)jt;
-    const uint32_t *add = ADD ? o.add + k * o.add_tstride + jt : nullptr;
+    const size_t lt = t * kTile;  // first limb
+    const long remaining = (long)o.out_len - (long)lt;
+    const uint32_t *add = ADD ? o.add + k * o.add_tstride + lt : nullptr;
     uint32_t map;
-    tile_carry_t<DEC ? 1 : 0, ADD ? 1 : 0>(run, h1, h2a, h2b, kTile,
-                                           o.out + node * o.out_tstride + jt, remaining, dec, add,
-                                           (long)o.add_len - (long)jt, wsm, &map);
+    tile_carry<DEC ? 1 : 0, ADD ? 1 : 0>(run, kTile, o.out + node * o.out_tstride + lt, remaining,
+                                         DEC, add, (long)o.add_len - (long)lt, wsm, &map);
     if (threadIdx.x == 0) a.tile_maps[blockIdx.x] = (uint8_t)map;
 }
 
@@ -477,7 +635,7 @@ __global__ void __launch_bounds__(1024) carry_tile_scan(uint8_t *tile_maps, size
 
 // Add each tile's carry-in to its first limbs (rarely more than one), in
 // base 2^32 or (dec) 10^9.
-__global__ void carry_fix(const uint8_t *tile_cin, size_t tiles_total, size_t tiles, int n,
+__global__ void carry_fix(const uint8_t *tile_cin, size_t tiles_total, size_t tiles,
                           uint32_t *out, size_t out_tstride, size_t out_len, bool dec,
                           const uint32_t *out_index = nullptr)
 {
@@ -507,33 +665,92 @@ __global__ void carry_fix(const uint8_t *tile_cin, size_t tiles_total, size_t ti
 
 struct FusedArgs {
     const uint32_t *A;
-    size_t a_tstride, a_len;
+    size_t a_tstride;
+    uint32_t a_len;
     const uint32_t *B;  // null: square A; b_tstride 0: the same B for every product
-    size_t b_tstride, b_len;
+    size_t b_tstride;
+    uint32_t b_len;
+    int a_al, b_al;     // every operand starts on an 8-byte boundary
     Sink sink;
     const uint2 *tw;
     Scale scale;
+    CoefMuls ca, cb;    // cb carries the pointwise scale (unused when squaring)
 };
 
-constexpr int kFusedMaxLog = 12;
-constexpr int kFusedThreads = 512;
+constexpr int kFusedMaxLog = 11;   // 2^11 points: products of 2^12 limbs
+constexpr int kFusedThreads = 256;
 
-// The one-block multiply's first forward round input: raw limbs (shared
-// memory, unswizzled) reduced into the forward range; column 0 is operand a,
-// column 1 operand b (a again when squaring).  With sb, operand b's limbs are
-// multiplied by sb (the pointwise step's normalisation 2^(32-n), taken in
-// advance) instead of by 1: the same Shoup product.
+// Threads of the one-block multiply of 2^lr points: one group of 16 points of
+// each operand's transform per thread and round, at least one warp.
+__host__ __device__ constexpr int fused_threads(int lr)
+{
+    const int t = (1 << lr) / 8;
+    return t < 32 ? 32 : (t > kFusedThreads ? kFusedThreads : t);
+}
+
+// The one-block multiply's first forward round input: coefficient i of an
+// operand, words 2i and 2i + 1 of its limbs (zero past the end), from global
+// memory; column 0 is operand a, column 1 operand b (a again when squaring).
+// The five primes read the operands one after the other; the blocks' limbs
+// stay in L1 and L2 meanwhile, which leaves the shared memory to more blocks.
+// ZT: both operands fill at most the lower half.
+template <bool ZT>
 struct RawIn {
+    static constexpr bool kZeroTop = ZT;
     const uint32_t *a, *b;
-    uint32_t q, wp1;
-    uint2 sb;  // (multiplier, Shoup companion) for operand b, or (1, wp1)
+    uint32_t la, lb;
+    bool al_a, al_b;
+    uint32_t q;
+    CoefMul ca, cb;
     template <int E, int B, int NA>
     __device__ __forceinline__ void load(uint32_t (&x)[NA][1 << E], int base, int c) const
     {
         const uint32_t *r = c ? b : a;
-        const uint32_t w = c ? sb.x : 1u, wp = c ? sb.y : wp1;
+        const uint32_t len = c ? lb : la;
+        const bool al = c ? al_b : al_a;
+        CoefMul m;
+        m.w0.x = c ? cb.w0.x : ca.w0.x;
+        m.w0.y = c ? cb.w0.y : ca.w0.y;
+        m.w1.x = c ? cb.w1.x : ca.w1.x;
+        m.w1.y = c ? cb.w1.y : ca.w1.y;
+        constexpr int K = ZT ? (1 << (E - 1)) : (1 << E);
+        uint32_t lo[K], hi[K];
+        if (al && 2u * (uint32_t)(base + ((K - 1) << B)) + 2u <= len) {
 #pragma unroll
-        for (int k = 0; k < (1 << E); k++) x[0][k] = shoup(r[base + (k << B)], w, wp, q);
+            for (int k = 0; k < K; k++) {
+                const uint2 v = *reinterpret_cast<const uint2 *>(r + 2 * (base + (k << B)));
+                lo[k] = v.x;
+                hi[k] = v.y;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                const uint32_t w = 2u * (uint32_t)(base + (k << B));
+                lo[k] = w < len ? r[w] : 0u;
+                hi[k] = w + 1 < len ? r[w + 1] : 0u;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < (1 << E); k++) x[0][k] = k < K ? coef_in<0>(lo[k], hi[k], m, q) : 0u;
+    }
+};
+
+// Limb sums of a run of the one-block multiply, straight from the
+// coefficients' words in shared memory (word p of coefficient j at
+// s[p N + swz(j)]).
+template <int N>
+struct SmemRun {
+    const uint32_t *s;
+    int j0;  // first coefficient
+    __device__ __forceinline__ uint32_t word(int p, int j) const
+    {
+        return j >= 0 ? s[p * N + swz(j)] : 0u;
+    }
+    __device__ __forceinline__ uint64_t operator()(int i) const
+    {
+        const int j = j0 + (i >> 1);
+        if (i & 1) return (uint64_t)word(1, j) + word(3, j - 1);
+        return (uint64_t)word(0, j) + word(2, j - 1) + word(4, j - 2);
     }
 };
 
@@ -541,63 +758,50 @@ struct RawIn {
 // the pointwise product and the inverse transform in shared memory (register
 // rounds, the middle one fused as in the row pass), then remaindering and
 // carries over one tile.
-// Layout (words): residues R0 [0,L) R1 [L,2L) R2 [2L,3L); raw A shares R2's
-// space (it is last read before R2 is written), raw B [3L,4L), transform pair
-// XY [4L,6L).  Every thread owns a run of eight coefficients for the carries
-// (L <= 8 x threads).
-// Two blocks per SM (64 registers; a small spill in the remaindering phase):
-// measured faster than one block per SM without the spill.
-template <int LR>
-__global__ void __launch_bounds__(kFusedThreads, 2) ntt_mul_fused(FusedArgs a)
+// Layout (words): six arrays of N = 2^LR; prime p's transforms use arrays p
+// (operand a, then the product, whose residues stay there) and p + 1 (operand
+// b; the next prime overwrites it): 24 N bytes, four blocks of 2^11 points per
+// SM.  The coefficients' words then replace the residues in place.
+template <int LR, bool ZT>
+__global__ void __launch_bounds__(fused_threads(LR), 1024 / fused_threads(LR))
+    ntt_mul_fused(FusedArgs a)
 {
     extern __shared__ uint32_t sm[];
     __shared__ uint32_t wsm[32];
-    constexpr int L = 1 << LR;
-    uint32_t *Rr[3] = {sm, sm + L, sm + 2 * L};
-    uint32_t *rawA = sm + 2 * L;
-    uint32_t *rawB = sm + 3 * L;
-    uint32_t *X = sm + 4 * L;  // X [4L,5L), Y [5L,6L): two arrays for the dual rounds
-    uint32_t *Y = X + L;
+    constexpr int N = 1 << LR;
+    constexpr int T = fused_threads(LR);
     const size_t k = blockIdx.x;
     const uint32_t *ga = a.A + k * a.a_tstride;
     const uint32_t *gb = a.B ? a.B + k * a.b_tstride : nullptr;
-    for (int i = threadIdx.x; i < L; i += blockDim.x) {
-        rawA[i] = (size_t)i < a.a_len ? ga[i] : 0u;
-        rawB[i] = (gb && (size_t)i < a.b_len) ? gb[i] : 0u;
-    }
-    __syncthreads();
     constexpr int NR = rounds_of(LR);
 #pragma unroll 1
     for (int p = 0; p < kNumPrimes; p++) {
-        const uint32_t q = c_q[0][p], qinv = c_qinv[0][p], wp1 = c_wp1[0][p];
-        const TwRef T{tw_table(a.tw, 0, p, 0), p};
+        const uint32_t q = c_q[0][p], qinv = c_qinv[0][p];
+        const TwRef T0{tw_table(a.tw, 0, p, 0), p};
         const TwRef Ti{tw_table(a.tw, 0, p, 1), p};
-        const uint2 sc = p == 0 ? a.scale.c[0] : (p == 1 ? a.scale.c[1] : a.scale.c[2]);
-        uint32_t *Z = Rr[p];
+        const uint2 sc = a.scale.c[p];
+        uint32_t *X = sm + p * N;
+        // operand b (when there is one) takes the normalisation in advance
+        const RawIn<ZT> ri{ga,     gb ? gb : ga,           a.a_len,
+                           gb ? a.b_len : a.a_len, a.a_al != 0, gb ? a.b_al != 0 : a.a_al != 0, q,
+                           a.ca.c[p], gb ? a.cb.c[p] : a.ca.c[p]};
+        const SmemIO<LR, 2, false> xy{X};
+        round_io<LR, 2, dif_base(LR, 0), round_size(LR, 0), true, 1, false, 0, T>(ri, xy, T0, q);
+        __syncthreads();
+        const SmemIO<LR, 1, false> zs{X};
         if constexpr (NR == 1) {
-            // up to 16 points: reduce, transform both, multiply, transform back
-            // operand b (when there is one) takes the normalisation in advance
-            for (int i = threadIdx.x; i < L; i += blockDim.x) {
-                X[swz(i)] = reduce_in<0>(rawA[i], q, wp1);
-                Y[swz(i)] = gb ? shoup(rawB[i], sc.x, sc.y, q) : reduce_in<0>(rawA[i], q, wp1);
-            }
+            // up to 16 points: elementwise in the swizzled space (X and Y share
+            // the permutation), then back
+            for (int i = threadIdx.x; i < N; i += T)
+                X[i] = gb ? mul_mont<0>(X[i], X[N + i], q, qinv)
+                          : pmul<0>(X[i], X[N + i], sc, q, qinv);
             __syncthreads();
-            dif_smem<LR, 2, 0>(X, T, q);  // X and Y as two arrays
-            // elementwise in the swizzled space: Z, X, Y share the permutation
-            for (int i = threadIdx.x; i < L; i += blockDim.x)
-                Z[i] = gb ? mul_mont<0>(X[i], Y[i], q, qinv) : pmul<0>(X[i], Y[i], sc, q, qinv);
+            round_io<LR, 1, 0, LR, false, 1, false, 0, T>(zs, zs, Ti, q);
             __syncthreads();
-            dit_smem<LR, 1, 0>(Z, Ti, q);
         } else {
-            // The first forward round reads the raw limbs and reduces them; X and
-            // Y are two arrays of the round (twice the groups of one pair).
-            const SmemIO<LR, 2, false> xy{X};
-            const RawIn ri{rawA, gb ? rawB : rawA, q, wp1, gb ? sc : make_uint2(1u, wp1)};
-            round_io<LR, 2, dif_base(LR, 0), round_size(LR, 0), true, 1, false, 0>(ri, xy, T, q);
-            __syncthreads();
             if constexpr (NR == 3) {
-                round_io<LR, 2, dif_base(LR, 1), round_size(LR, 1), true, 1, false, 0>(xy, xy, T,
-                                                                                      q);
+                round_io<LR, 2, dif_base(LR, 1), round_size(LR, 1), true, 1, false, 0, T>(xy, xy,
+                                                                                         T0, q);
                 __syncthreads();
             }
             // The last forward round of both operands, the pointwise product and
@@ -605,13 +809,13 @@ __global__ void __launch_bounds__(kFusedThreads, 2) ntt_mul_fused(FusedArgs a)
             // coincide), as in the row pass.
             constexpr int EL = round_size(LR, NR - 1);
             static_assert(EL == dit_size(LR, 0), "mirrored rounds");
-            const SmemIO<LR, 1, false> pair{X};  // NA = 2: X and Y = X + L
-            const SmemIO<LR, 1, false> zs{Z};
-            for (int g = threadIdx.x; g < (L >> EL); g += blockDim.x) {
+            const SmemIO<LR, 1, false> pair{X};  // NA = 2: X and Y = X + N
+#pragma unroll 1
+            for (int g = threadIdx.x; g < (N >> EL); g += T) {
                 const int base = g << EL;
                 uint32_t x[2][1 << EL];
                 pair.template load<EL, 0, 2>(x, base, 0);
-                dif_stages<EL, 0, 2, 0>(x, 0, T, q);
+                dif_stages<EL, 0, 2, 0>(x, 0, T0, q);
                 uint32_t zz[1][1 << EL];
 #pragma unroll
                 for (int j = 0; j < (1 << EL); j++)
@@ -621,70 +825,75 @@ __global__ void __launch_bounds__(kFusedThreads, 2) ntt_mul_fused(FusedArgs a)
                 zs.template store<EL, 0, 1>(zz, base, 0);
             }
             __syncthreads();
-            round_io<LR, 1, dit_base(LR, 1), dit_size(LR, 1), false, 1, false, 0>(zs, zs, Ti, q);
+            round_io<LR, 1, dit_base(LR, 1), dit_size(LR, 1), false, 1, false, 0, T>(zs, zs, Ti, q);
             __syncthreads();
             if constexpr (NR == 3) {
-                round_io<LR, 1, dit_base(LR, 2), dit_size(LR, 2), false, 1, false, 0>(zs, zs, Ti,
-                                                                                      q);
+                round_io<LR, 1, dit_base(LR, 2), dit_size(LR, 2), false, 1, false, 0, T>(zs, zs, Ti,
+                                                                                        q);
                 __syncthreads();
             }
         }
     }
-    // each thread remainders its run of eight coefficients straight from the
-    // swizzled residues (for a fixed i the lanes' words 8 t + i fall in
-    // distinct banks under swz)
-    __shared__ uint32_t hsm[96];
-    const int j0 = threadIdx.x * kLimbsPerThread;
-    CoefRun run;
-#pragma unroll
-    for (int i = 0; i < kLimbsPerThread; i++) {
-        run.c0[i] = run.c1[i] = run.c2[i] = 0;
-        if (j0 + i < L) {
-            const int j = swz(j0 + i);
-            crt3<0>(Rr[0][j], Rr[1][j], Rr[2][j], run.c0[i], run.c1[i], run.c2[i]);
-        }
-    }
+    // the coefficients' words in place of their residues
     const Sink &o = a.sink;
-    if (o.dec)
+    for (int j = threadIdx.x; j < N; j += T) {
+        uint32_t *x = sm + swz(j);
+        uint32_t r[kNumPrimes], w[5];
 #pragma unroll
-        for (int i = 0; i < kLimbsPerThread; i++) words_to_dec(run.c0[i], run.c1[i], run.c2[i]);
-    uint32_t h1, h2a, h2b, map;
-    run_halo(run, 0u, 0u, 0u, hsm, h1, h2a, h2b);
-    tile_carry(run, h1, h2a, h2b, L, o.out + sink_node(o, k) * o.out_tstride, (long)o.out_len, o.dec,
-               o.add ? o.add + k * o.add_tstride : nullptr, (long)o.add_len, wsm, &map);
+        for (int p = 0; p < kNumPrimes; p++) r[p] = x[p * N];
+        if (o.dec) crt5_dec<0>(r, w);
+        else crt5<0>(r, w);
+#pragma unroll
+        for (int p = 0; p < 5; p++) x[p * N] = w[p];
+    }
+    __syncthreads();
+    constexpr int LPT = 2 * N / T > kLimbsPerThread ? 2 * N / T : kLimbsPerThread;
+    uint32_t map;
+    tile_carry<-1, -1, LPT>(SmemRun<N>{sm, (int)threadIdx.x * (LPT / 2)}, 2 * N,
+                            o.out + sink_node(o, k) * o.out_tstride, (long)o.out_len, o.dec,
+                            o.add ? o.add + k * o.add_tstride : nullptr, (long)o.add_len, wsm,
+                            &map);
 }
 
 // ------------------------------------------------------------ host side
 
 struct NttPlan {
-    int n = 0;
+    int np = 0;
     int ncol = 0;
     int rcol[3] = {0, 0, 0};
     int rrow = 0;
 };
 
-// Row pass of up to 2^12 points (at least 2^4 so column passes keep 16
-// columns), column passes of at most 2^10 rows, split as evenly as possible.
-// A row-pass size tuned for this device (Ctx::row_log: rows of 2^9 .. 2^12
-// points, at most two column passes of at least 2 rows, at least 2^4 rows in
-// prime sets 1 and 2, whose column passes are built for 2^4 .. 2^10 rows)
-// replaces the default.
+// The plan of a product of 2^n limbs (2^np points, np = n - 1 >= 12): a row
+// pass of up to 2^12 points and column passes of at most 2^10 rows, split as
+// evenly as possible.  2^12 points take the row pass alone.  A row-pass size
+// tuned for this device (Ctx::row_log: rows of 2^9 .. 2^12 points) replaces
+// the default.  plan_row_ok: the row sizes a tuning table may name for a
+// product of 2^n limbs (at most two column passes of at least 2 rows, at
+// least 2^4 in prime sets 1 and 2, whose column passes are built for 2^4 ..
+// 2^10 rows; the bounds are those of tables written for 2^n points, one stage
+// more than the transform has, and every size they allow has a plan).
 bool plan_row_ok(int n, int rrow)
 {
     if (n > kLogMaxNtt || rrow < 9 || rrow > kRowMaxLog) return false;
     const int rem = n - rrow;
     const int ncol = (rem + kColMaxLog - 1) / kColMaxLog;
     if (rem < 2 || ncol > 2) return false;
-    return rem / ncol >= (set_for(n) == 0 ? 2 : kColMinLog);
+    return rem / ncol >= (set_for(n - 1) == 0 ? 2 : kColMinLog);
 }
 
-static NttPlan make_plan(const Ctx &c, int n)
+static NttPlan make_plan(const Ctx &c, int np)
 {
     NttPlan P;
-    P.n = n;
-    P.rrow = std::min(kRowMaxLog, n - kColMinLog);
+    P.np = np;
+    const int n = np + 1;
+    if (np <= kRowMaxLog) {  // the row pass alone
+        P.rrow = np;
+        return P;
+    }
+    P.rrow = std::min(kRowMaxLog, np - kColMinLog);
     if (n <= kLogMaxNtt && c.row_log[n] && plan_row_ok(n, c.row_log[n])) P.rrow = c.row_log[n];
-    int rem = n - P.rrow;
+    int rem = np - P.rrow;
     P.ncol = (rem + kColMaxLog - 1) / kColMaxLog;
     for (int i = 0; i < P.ncol; i++) {
         P.rcol[i] = rem / (P.ncol - i);
@@ -710,13 +919,16 @@ static void launch_col(bool fwd, dim3 grid, cudaStream_t s, const ColArgs &a)
     const size_t smem = ((size_t)1 << (LR + col_log_c(LR))) * sizeof(uint32_t);
     // the first pass of operands of at most half the transform (every tree
     // level) knows its upper half is zero
-    const bool zt = fwd && a.src && a.src_len <= ((size_t)1 << (a.m - 1));
+    const bool zt = fwd && a.src && a.src_len <= ((size_t)1 << a.m);  // limbs: two per point
     if (zt) {
-        set_smem(ntt_col_fwd<LR, PS, kColV, true>, smem);
-        ntt_col_fwd<LR, PS, kColV, true><<<grid, kColFwdThreads, smem, s>>>(a);
+        set_smem(ntt_col_fwd<LR, PS, kColV, 2>, smem);
+        ntt_col_fwd<LR, PS, kColV, 2><<<grid, kColFwdThreads, smem, s>>>(a);
+    } else if (fwd && a.src) {
+        set_smem(ntt_col_fwd<LR, PS, kColV, 1>, smem);
+        ntt_col_fwd<LR, PS, kColV, 1><<<grid, kColFwdThreads, smem, s>>>(a);
     } else if (fwd) {
-        set_smem(ntt_col_fwd<LR, PS, kColV, false>, smem);
-        ntt_col_fwd<LR, PS, kColV, false><<<grid, kColFwdThreads, smem, s>>>(a);
+        set_smem(ntt_col_fwd<LR, PS, kColV, 0>, smem);
+        ntt_col_fwd<LR, PS, kColV, 0><<<grid, kColFwdThreads, smem, s>>>(a);
     } else {
         set_smem(ntt_col_inv<LR, PS, kColV>, smem);
         ntt_col_inv<LR, PS, kColV><<<grid, kColInvThreads, smem, s>>>(a);
@@ -729,13 +941,17 @@ static void launch_col(bool fwd, dim3 grid, cudaStream_t s, const ColArgs &a)
 // in Montgomery form, the value the pass would otherwise compute for that
 // point (tw_pow_mont, exactly as the stepping reaches it).
 // With scale (per prime, nonzero), every entry is multiplied by it mod q.
+struct TwScale {
+    uint32_t c[kNumPrimes];
+};
+
 template <int PS>
-__global__ void col_twiddle_table(const uint2 *tw, int m, int r, int dir, uint3 scale,
+__global__ void col_twiddle_table(const uint2 *tw, int m, int r, int dir, TwScale scale,
                                   uint32_t *tab)
 {
     const int p = blockIdx.y;
     const uint32_t q = c_q[PS][p], qinv = c_qinv[PS][p];
-    const uint32_t sp = p == 0 ? scale.x : (p == 1 ? scale.y : scale.z);
+    const uint32_t sp = scale.c[p];
     const uint2 *T = tw_table(tw, PS, p, dir);
     const int shift = set_log_root(PS) - m;
     const uint32_t cols = 1u << (m - r);
@@ -750,8 +966,9 @@ __global__ void col_twiddle_table(const uint2 *tw, int m, int r, int dir, uint3 
 
 // A column pass's twiddle table, built on first use; null when the context
 // computes its twiddles (a budgeted context, or no room for the table).
-// scaled: the entries times 2^(32-m) mod q, for operand b of a product whose
-// pointwise step then needs no normalisation (forward first passes, m = n).
+// scaled: the entries times 2^32 S mod q (S the pointwise scale of 2^m
+// points), for operand b of a product whose pointwise step then needs no
+// normalisation (forward first passes, m = np).
 static const uint32_t *col_twiddles(Ctx &c, int ps, int m, int r, int dir, cudaStream_t s,
                                     bool scaled = false)
 {
@@ -763,15 +980,9 @@ static const uint32_t *col_twiddles(Ctx &c, int ps, int m, int r, int dir, cudaS
         cudaGetLastError();
         return nullptr;
     }
-    uint3 sc = make_uint3(0, 0, 0);
-    if (scaled) {
-        uint32_t v[kNumPrimes];
-        for (int i = 0; i < kNumPrimes; i++) {
-            const uint32_t q = ntt_prime(ps, i);
-            v[i] = to_mont_c(powmod_u32((q + 1) / 2, (uint64_t)m, q), q);  // 2^32 2^-m
-        }
-        sc = make_uint3(v[0], v[1], v[2]);
-    }
+    TwScale sc{};
+    if (scaled)
+        for (int i = 0; i < kNumPrimes; i++) sc.c[i] = scale_value(ps, i, m);
     const unsigned blocks = (unsigned)std::min<size_t>(((size_t)1 << m) / 256 + 1, 4096);
     const dim3 grid(blocks, kNumPrimes);
     if (ps == 0) col_twiddle_table<0><<<grid, 256, 0, s>>>(c.twiddles, m, r, dir, sc, p);
@@ -796,9 +1007,11 @@ void drop_col_twiddles(Ctx &c)
 // table exists), i.e. whether the row pass must skip the normalisation.
 static bool col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, size_t total,
                      int m, int r, const uint32_t *src, size_t src_tstride, size_t src_len,
-                     cudaStream_t s, int scaled = 0)
+                     bool dec, cudaStream_t s, int scaled = 0)
 {
     ColArgs a;
+    a.coef = make_coef(ps, dec);
+    a.src_al = (reinterpret_cast<uintptr_t>(src) & 15) == 0 && (src_tstride & 3) == 0;
     a.twtab_odd = nullptr;
     // (measured per C(2,050,572,903): tables in every pass beat computed
     // twiddles at every block size, the first forward passes' large tables
@@ -823,10 +1036,10 @@ static bool col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, s
     a.tw = c.twiddles;
     const size_t ctas = total >> (r + col_log_c(r));
     dim3 grid((unsigned)ctas, kNumPrimes);
-    // algorithmic bytes: every point of the three prime arrays read and
+    // algorithmic bytes: every point of the five prime arrays read and
     // written once (the first forward pass reads limbs instead)
-    double bytes = 24.0 * (double)total;
-    if (src) bytes = 12.0 * (double)total + 4.0 * (double)src_len * (double)(total >> m);
+    double bytes = 8.0 * kNumPrimes * (double)total;
+    if (src) bytes = 4.0 * kNumPrimes * (double)total + 4.0 * (double)src_len * (double)(total >> m);
     const int tok = prof_begin(c, fwd ? (src ? "ntt_col_fwd_first" : "ntt_col_fwd") : "ntt_col_inv", s);
     if (ps == 0) {
         switch (r) {
@@ -843,8 +1056,7 @@ static bool col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, s
         default: fail(CAT_EINVAL, "column pass size out of range");
         }
     } else if (ps == 1) {
-        // 2^24 .. 2^26 points: default plans [6, 6], [7, 6], [7, 7] + 12; tuned
-        // plans column passes of 2^4 .. 2^10 rows
+        // 2^23 .. 2^25 points: column passes of 2^5 .. 2^8 rows
         switch (r) {
         case 4: launch_col<4, 1>(fwd, grid, s, a); break;
         case 5: launch_col<5, 1>(fwd, grid, s, a); break;
@@ -856,7 +1068,7 @@ static bool col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, s
         default: fail(CAT_EINVAL, "column pass size out of range");
         }
     } else {
-        // 2^27 points: default plan [8, 7] + 12; tuned plans 2^4 .. 2^10 rows
+        // 2^26 points: column passes of 2^7 .. 2^9 rows
         switch (r) {
         case 4: launch_col<4, 2>(fwd, grid, s, a); break;
         case 5: launch_col<5, 2>(fwd, grid, s, a); break;
@@ -895,12 +1107,12 @@ static void launch_row_t(dim3 grid, cudaStream_t s, const RowArgs &a, bool pre)
     }
 }
 
-// The fused row pass of nprod products of 2^n points with prime set ps
+// The fused row pass of nprod products of 2^np points with prime set ps
 // (pre: broadcast products whose common transform ntt_row_fwd completed).
-static void launch_row(int ps, int lr, size_t nprod, int n, cudaStream_t s, const RowArgs &a,
+static void launch_row(int ps, int lr, size_t nprod, int np, cudaStream_t s, const RowArgs &a,
                        bool pre = false)
 {
-    dim3 grid((unsigned)(nprod << (n - kRowMaxLog)), kNumPrimes);
+    dim3 grid((unsigned)(nprod << (np - kRowMaxLog)), kNumPrimes);
     if (ps == 0) {
         switch (lr) {
         case 9: launch_row_t<9, 0>(grid, s, a, pre); break;
@@ -937,11 +1149,11 @@ static void launch_row_fwd_t(dim3 grid, cudaStream_t s, const RowArgs &a)
     ntt_row_fwd<LR, PS><<<grid, kRowThreads, smem, s>>>(a);
 }
 
-// The row pass's forward rounds of one transform of 2^n points in place (the
+// The row pass's forward rounds of one transform of 2^np points in place (the
 // common operand of broadcast products; a.F at its slot).
-static void launch_row_fwd(int ps, int lr, int n, cudaStream_t s, const RowArgs &a)
+static void launch_row_fwd(int ps, int lr, int np, cudaStream_t s, const RowArgs &a)
 {
-    dim3 grid((unsigned)((size_t)1 << (n - kRowMaxLog)), kNumPrimes);
+    dim3 grid((unsigned)((size_t)1 << (np - kRowMaxLog)), kNumPrimes);
     switch (ps * 16 + lr) {
     case 9: launch_row_fwd_t<9, 0>(grid, s, a); break;
     case 10: launch_row_fwd_t<10, 0>(grid, s, a); break;
@@ -986,6 +1198,35 @@ static void launch_crt(int ps, unsigned grid, cudaStream_t s, const CrtArgs &a)
         launch_crt_ps<2>(grid, s, a);
 }
 
+// Whether every operand of a batch (tstride limbs apart) starts on an 8-byte
+// boundary, so that a coefficient is one 8-byte load.
+static int aligned8(const uint32_t *p, size_t tstride)
+{
+    return (reinterpret_cast<uintptr_t>(p) & 7) == 0 && (tstride & 1) == 0;
+}
+
+template <bool SQ, bool ZT>
+static void launch_row_limbs_t(size_t nprod, cudaStream_t s, const RowLimbArgs &a)
+{
+    const size_t smem = ((size_t)(SQ ? 1 : 2) << kRowMaxLog) * sizeof(uint32_t);
+    set_smem(ntt_row_limbs<SQ, ZT>, smem);
+    ntt_row_limbs<SQ, ZT><<<dim3((unsigned)nprod, kNumPrimes), kRowThreads, smem, s>>>(a);
+}
+
+// The whole transforms of nprod products of 2^12 points, from limbs.
+static void launch_row_limbs(size_t nprod, bool square, cudaStream_t s, const RowLimbArgs &a)
+{
+    const bool zt = std::max(a.a_len, a.b_len) <= (1u << kRowMaxLog);
+    if (square) {
+        if (zt) launch_row_limbs_t<true, true>(nprod, s, a);
+        else launch_row_limbs_t<true, false>(nprod, s, a);
+    } else {
+        if (zt) launch_row_limbs_t<false, true>(nprod, s, a);
+        else launch_row_limbs_t<false, false>(nprod, s, a);
+    }
+    CAT_LAUNCH("ntt_row_limbs");
+}
+
 // One operand source of a batched product.
 struct Operand {
     const uint32_t *p;
@@ -993,133 +1234,198 @@ struct Operand {
     size_t len;      // valid limbs per transform
 };
 
-// Batched products through the multi-pass transform, L = 2^n > 2^12.
-//  mode PAIR_ADJACENT:  nprod products of transforms (2k, 2k+1) of `x`
-//                       (2 nprod transforms, tstride apart);
-//  mode PAIR_FIRST_TWO: one product of x and y;
-//  mode PAIR_SQUARE:    nprod squares of x's transforms;
-//  mode PAIR_BROADCAST: nprod products of x's transforms (tstride apart) with
-//                       one y, whose transform is computed once.
-static void ntt_mul_multipass(Ctx &c, int n, int mode, size_t nprod, Operand x, Operand y,
-                              const Sink &sink, cudaStream_t s)
+// Scratch of one batch of multi-pass products: from the context's pool, or
+// the fixed arrays of the no-allocation multiply.
+struct MulScratch {
+    DevBuf<uint32_t> Fb, Gb;
+    DevBuf<uint8_t> mb;
+    uint32_t *F = nullptr, *G = nullptr;
+    uint8_t *maps = nullptr;
+    bool fixed = false;
+};
+
+// The carries of nprod products of `tiles` tiles each, whose compact tile
+// maps are in maps: the carry into every tile, then added to its first limbs.
+static void carry_finish(Ctx &c, uint8_t *maps, size_t nprod, size_t tiles, const Sink &sink,
+                         cudaStream_t s)
 {
-    const NttPlan P = make_plan(c, n);
-    const int PS = set_for(n);
-    const size_t L = (size_t)1 << n;
-    const size_t ntf = mode == PAIR_ADJACENT ? 2 * nprod
-                       : mode == PAIR_SQUARE ? nprod
-                       : mode == PAIR_BROADCAST ? nprod + 1
-                                                : 2;
-    const size_t fp = ntf * L;
-    DevBuf<uint32_t> F(c, fp * kNumPrimes, s);
-    // forward column passes (operand b's first pass takes the pointwise
-    // step's normalisation into its twiddles when it has a table)
-    bool prescaled = false;
-    if (mode == PAIR_FIRST_TWO) {
-        col_pass(c, PS, true, F.get(), fp, L, n, P.rcol[0], x.p, 0, x.len, s);
-        prescaled = col_pass(c, PS, true, F.get() + L, fp, L, n, P.rcol[0], y.p, 0, y.len, s, 1);
-    } else if (mode == PAIR_BROADCAST) {
-        col_pass(c, PS, true, F.get(), fp, nprod * L, n, P.rcol[0], x.p, x.tstride, x.len, s);
-        col_pass(c, PS, true, F.get() + nprod * L, fp, L, n, P.rcol[0], y.p, 0, y.len, s);
-    } else {
-        prescaled = col_pass(c, PS, true, F.get(), fp, fp, n, P.rcol[0], x.p, x.tstride, x.len, s,
-                             mode == PAIR_ADJACENT ? 2 : 0);
-    }
-    int m = n - P.rcol[0];
-    for (int i = 1; i < P.ncol; i++) {
-        col_pass(c, PS, true, F.get(), fp, fp, m, P.rcol[i], nullptr, 0, 0, s);
-        m -= P.rcol[i];
-    }
-    // fused row pass
-    const size_t gp = nprod * L;
-    DevBuf<uint32_t> G(c, gp * kNumPrimes, s);
-    RowArgs ra;
-    ra.F = F.get();
-    ra.fpstride = fp;
-    ra.G = G.get();
-    ra.gpstride = gp;
-    ra.n = n;
-    ra.mode = mode;
-    ra.prescaled = prescaled ? 1 : 0;
-    ra.tw = c.twiddles;
-    ra.scale = make_scale(PS, n);
-    // broadcast products: y's transform completed once, in its slot, so that
-    // the row pass transforms only the x's
-    const bool pre = mode == PAIR_BROADCAST && nprod >= 2;
-    int tok;
-    if (pre) {
-        RowArgs ya = ra;
-        ya.F = F.get() + nprod * L;
-        tok = prof_begin(c, "ntt_row_fwd", s);
-        launch_row_fwd(PS, P.rrow, n, s, ya);
-        prof_end(c, tok, s, 8.0 * (double)L * kNumPrimes);
-    }
-    tok = prof_begin(c, "ntt_row_mul", s);
-    launch_row(PS, P.rrow, nprod, n, s, ra, pre);
-    // the products' own bytes: operands read and products written once
-    const double unit = 4.0 * (double)nprod * (double)(x.len + sink.out_len) +
-                        (mode == PAIR_SQUARE ? 0.0
-                         : mode == PAIR_BROADCAST ? 4.0 * (double)y.len
-                                                  : 4.0 * (double)nprod * (double)y.len);
-    prof_end(c, tok, s, (mode == PAIR_SQUARE ? 24.0 : 36.0) * (double)gp, unit);
-    F.reset();
-    // inverse column passes, reverse order
-    for (int i = P.ncol - 1; i >= 0; i--) {
-        int mi = n;
-        for (int j = 0; j < i; j++) mi -= P.rcol[j];
-        col_pass(c, PS, false, G.get(), gp, gp, mi, P.rcol[i], nullptr, 0, 0, s);
-    }
-    // remaindering and carries
-    const size_t tiles = L / kTile;
-    DevBuf<uint8_t> maps(c, nprod * tiles, s);
-    CrtArgs ca;
-    ca.G = G.get();
-    ca.gpstride = gp;
-    ca.n = n;
-    ca.sink = sink;
-    ca.tile_maps = maps.get();
-    tok = prof_begin(c, "crt_carry_tiles", s);
-    launch_crt(PS, (unsigned)(nprod * tiles), s, ca);
-    CAT_LAUNCH("crt_carry_tiles");
-    prof_end(c, tok, s, 12.0 * (double)gp + 4.0 * (double)nprod * (double)sink.out_len);
-    tok = prof_begin(c, "carry_tile_scan", s);
-    carry_tile_scan<<<(unsigned)nprod, 1024, 0, s>>>(maps.get(), tiles);
+    int tok = prof_begin(c, "carry_tile_scan", s);
+    carry_tile_scan<<<(unsigned)nprod, 1024, 0, s>>>(maps, tiles);
     CAT_LAUNCH("carry_tile_scan");
     prof_end(c, tok, s, 2.0 * (double)(nprod * tiles));
     const size_t tt = nprod * tiles;
     tok = prof_begin(c, "carry_fix", s);
-    carry_fix<<<(unsigned)((tt + 255) / 256), 256, 0, s>>>(maps.get(), tt, tiles, n, sink.out,
+    carry_fix<<<(unsigned)((tt + 255) / 256), 256, 0, s>>>(maps, tt, tiles, sink.out,
                                                              sink.out_tstride, sink.out_len,
                                                              sink.dec, sink.out_index);
     CAT_LAUNCH("carry_fix");
     prof_end(c, tok, s, (double)tt);
 }
 
+// Batched products of transforms of 2^np >= 2^12 points.
+//  mode PAIR_ADJACENT:  nprod products of transforms (2k, 2k+1) of `x`
+//                       (2 nprod transforms, tstride apart);
+//  mode PAIR_FIRST_TWO: one product of x and y;
+//  mode PAIR_SQUARE:    nprod squares of x's transforms;
+//  mode PAIR_BROADCAST: nprod products of x's transforms (tstride apart) with
+//                       one y, whose transform is computed once.
+static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x, Operand y,
+                              const Sink &sink, cudaStream_t s, MulScratch &&m = MulScratch{})
+{
+    const NttPlan P = make_plan(c, np);
+    const int PS = set_for(np);
+    const bool dec = sink.dec;
+    const size_t N = (size_t)1 << np;
+    const size_t ntf = mode == PAIR_ADJACENT ? 2 * nprod
+                       : mode == PAIR_SQUARE ? nprod
+                       : mode == PAIR_BROADCAST ? nprod + 1
+                                                : 2;
+    const size_t fp = ntf * N, gp = nprod * N;
+    // the products' own bytes: operands read and products written once
+    const double unit = 4.0 * (double)nprod * (double)(x.len + sink.out_len) +
+                        (mode == PAIR_SQUARE ? 0.0
+                         : mode == PAIR_BROADCAST ? 4.0 * (double)y.len
+                                                  : 4.0 * (double)nprod * (double)y.len);
+    int tok;
+    if (P.ncol == 0) {
+        // the row pass alone, from the operands' limbs
+        if (!m.fixed) {
+            m.Gb = DevBuf<uint32_t>(c, gp * kNumPrimes, s);
+            m.G = m.Gb.get();
+        }
+        RowLimbArgs ra;
+        ra.A = x.p;
+        ra.B = mode == PAIR_ADJACENT ? x.p + x.tstride : (mode == PAIR_SQUARE ? x.p : y.p);
+        ra.a_tstride = mode == PAIR_ADJACENT ? 2 * x.tstride : x.tstride;
+        ra.b_tstride = mode == PAIR_ADJACENT ? 2 * x.tstride
+                       : mode == PAIR_SQUARE ? x.tstride
+                                             : 0;
+        ra.a_len = (uint32_t)x.len;
+        ra.b_len = (uint32_t)(mode == PAIR_ADJACENT || mode == PAIR_SQUARE ? x.len : y.len);
+        ra.a_al = aligned8(ra.A, ra.a_tstride);
+        ra.b_al = aligned8(ra.B, ra.b_tstride);
+        ra.G = m.G;
+        ra.gpstride = gp;
+        ra.tw = c.twiddles;
+        ra.scale = make_scale(PS, np);
+        ra.ca = make_coef(PS, dec);
+        ra.cb = make_coef_scaled(PS, np, dec);
+        tok = prof_begin(c, "ntt_row_limbs", s);
+        launch_row_limbs(nprod, mode == PAIR_SQUARE, s, ra);
+        prof_end(c, tok, s, 4.0 * kNumPrimes * (double)gp + unit, unit);
+    } else {
+        if (!m.fixed) {
+            m.Fb = DevBuf<uint32_t>(c, fp * kNumPrimes, s);
+            m.F = m.Fb.get();
+        }
+        uint32_t *F = m.F;
+        // forward column passes (operand b's first pass takes the pointwise
+        // step's normalisation into its twiddles when it has a table)
+        bool prescaled = false;
+        if (mode == PAIR_FIRST_TWO) {
+            col_pass(c, PS, true, F, fp, N, np, P.rcol[0], x.p, 0, x.len, dec, s);
+            prescaled = col_pass(c, PS, true, F + N, fp, N, np, P.rcol[0], y.p, 0, y.len, dec, s, 1);
+        } else if (mode == PAIR_BROADCAST) {
+            col_pass(c, PS, true, F, fp, nprod * N, np, P.rcol[0], x.p, x.tstride, x.len, dec, s);
+            col_pass(c, PS, true, F + nprod * N, fp, N, np, P.rcol[0], y.p, 0, y.len, dec, s);
+        } else {
+            prescaled = col_pass(c, PS, true, F, fp, fp, np, P.rcol[0], x.p, x.tstride, x.len, dec,
+                                 s, mode == PAIR_ADJACENT ? 2 : 0);
+        }
+        int mm = np - P.rcol[0];
+        for (int i = 1; i < P.ncol; i++) {
+            col_pass(c, PS, true, F, fp, fp, mm, P.rcol[i], nullptr, 0, 0, false, s);
+            mm -= P.rcol[i];
+        }
+        // fused row pass
+        if (!m.fixed) {
+            m.Gb = DevBuf<uint32_t>(c, gp * kNumPrimes, s);
+            m.G = m.Gb.get();
+        }
+        RowArgs ra;
+        ra.F = F;
+        ra.fpstride = fp;
+        ra.G = m.G;
+        ra.gpstride = gp;
+        ra.np = np;
+        ra.mode = mode;
+        ra.prescaled = prescaled ? 1 : 0;
+        ra.tw = c.twiddles;
+        ra.scale = make_scale(PS, np);
+        // broadcast products: y's transform completed once, in its slot, so that
+        // the row pass transforms only the x's
+        const bool pre = mode == PAIR_BROADCAST && nprod >= 2;
+        if (pre) {
+            RowArgs ya = ra;
+            ya.F = F + nprod * N;
+            tok = prof_begin(c, "ntt_row_fwd", s);
+            launch_row_fwd(PS, P.rrow, np, s, ya);
+            prof_end(c, tok, s, 8.0 * (double)N * kNumPrimes);
+        }
+        tok = prof_begin(c, "ntt_row_mul", s);
+        launch_row(PS, P.rrow, nprod, np, s, ra, pre);
+        prof_end(c, tok, s, (mode == PAIR_SQUARE ? 8.0 : 12.0) * kNumPrimes * (double)gp, unit);
+        m.Fb.reset();
+        // inverse column passes, reverse order
+        for (int i = P.ncol - 1; i >= 0; i--) {
+            int mi = np;
+            for (int j = 0; j < i; j++) mi -= P.rcol[j];
+            col_pass(c, PS, false, m.G, gp, gp, mi, P.rcol[i], nullptr, 0, 0, false, s);
+        }
+    }
+    // remaindering and carries
+    const size_t tiles = N / kTileCoefs;
+    if (!m.fixed) {
+        m.mb = DevBuf<uint8_t>(c, nprod * tiles, s);
+        m.maps = m.mb.get();
+    }
+    CrtArgs ca;
+    ca.G = m.G;
+    ca.gpstride = gp;
+    ca.np = np;
+    ca.sink = sink;
+    ca.tile_maps = m.maps;
+    tok = prof_begin(c, "crt_carry_tiles", s);
+    launch_crt(PS, (unsigned)(nprod * tiles), s, ca);
+    CAT_LAUNCH("crt_carry_tiles");
+    prof_end(c, tok, s, 4.0 * kNumPrimes * (double)gp + 4.0 * (double)nprod * (double)sink.out_len);
+    carry_finish(c, m.maps, nprod, tiles, sink, s);
+}
+
 template <int LR>
 static void launch_fused(unsigned grid, cudaStream_t s, const FusedArgs &a)
 {
     const size_t smem = 6 * ((size_t)1 << LR) * sizeof(uint32_t);
-    set_smem(ntt_mul_fused<LR>, smem);
-    const int threads = std::min(kFusedThreads, std::max(64, (1 << LR) / 8));
-    ntt_mul_fused<LR><<<grid, threads, smem, s>>>(a);
+    // operands of at most half the transform (every tree level)
+    if (std::max(a.a_len, a.B ? a.b_len : 0u) <= (1u << LR)) {
+        set_smem(ntt_mul_fused<LR, true>, smem);
+        ntt_mul_fused<LR, true><<<grid, fused_threads(LR), smem, s>>>(a);
+    } else {
+        set_smem(ntt_mul_fused<LR, false>, smem);
+        ntt_mul_fused<LR, false><<<grid, fused_threads(LR), smem, s>>>(a);
+    }
 }
 
-static void ntt_mul_small(Ctx &c, int n, size_t nprod, Operand x, Operand y, bool square,
+static void ntt_mul_small(Ctx &c, int np, size_t nprod, Operand x, Operand y, bool square,
                           const Sink &sink, cudaStream_t s)
 {
     FusedArgs a;
     a.A = x.p;
     a.a_tstride = x.tstride;
-    a.a_len = x.len;
+    a.a_len = (uint32_t)x.len;
     a.B = square ? nullptr : y.p;
     a.b_tstride = y.tstride;
-    a.b_len = y.len;
+    a.b_len = (uint32_t)y.len;
+    a.a_al = aligned8(x.p, x.tstride);
+    a.b_al = aligned8(y.p, y.tstride);
     a.sink = sink;
     a.tw = c.twiddles;
-    a.scale = make_scale(0, n);
+    a.scale = make_scale(0, np);
+    a.ca = make_coef(0, sink.dec);
+    a.cb = make_coef_scaled(0, np, sink.dec);
     const unsigned grid = (unsigned)nprod;
     const int tok = prof_begin(c, "ntt_mul_fused", s);
-    switch (n) {
+    switch (np) {
     case 1: launch_fused<1>(grid, s, a); break;
     case 2: launch_fused<2>(grid, s, a); break;
     case 3: launch_fused<3>(grid, s, a); break;
@@ -1131,7 +1437,6 @@ static void ntt_mul_small(Ctx &c, int n, size_t nprod, Operand x, Operand y, boo
     case 9: launch_fused<9>(grid, s, a); break;
     case 10: launch_fused<10>(grid, s, a); break;
     case 11: launch_fused<11>(grid, s, a); break;
-    case 12: launch_fused<12>(grid, s, a); break;
     default: fail(CAT_EINVAL, "one-block transform size out of range");
     }
     CAT_LAUNCH("ntt_mul_fused");
@@ -1147,14 +1452,18 @@ static int ceil_log2(size_t x)
     return n;
 }
 
+// log2 of the points of a product of `limbs` limbs: coefficients of two limbs,
+// ceil(na / 2) + ceil(nb / 2) - 1 <= (na + nb) / 2 of them
+static int points_log(size_t limbs) { return std::max(1, ceil_log2(limbs) - 1); }
+
 // Level products of the fixed-slot product tree: nprod products of adjacent
 // slot-limb nodes of `level`, each written into a 2*slot-limb slot of out.
 void ntt_level(Ctx &c, const uint32_t *level, size_t slot, size_t nprod, uint32_t *out,
                cudaStream_t s, const uint32_t *out_index, const uint32_t *out_index_host)
 {
-    const int n = ceil_log2(2 * slot);
+    const int np = points_log(2 * slot);
     Operand x{level, slot, slot};
-    if (n > c.max_log) {  // longer than one transform: each pair by pieces
+    if (np + 1 > c.max_log) {  // longer than one transform: each pair by pieces
         if (out_index && !out_index_host) fail(CAT_EINVAL, "indexed level needs its host table");
         for (size_t k = 0; k < nprod; k++) {
             uint32_t *o = out + 2 * (out_index ? (size_t)out_index_host[k] : k) * slot;
@@ -1166,11 +1475,11 @@ void ntt_level(Ctx &c, const uint32_t *level, size_t slot, size_t nprod, uint32_
     }
     Sink sink = plain_sink(out, 2 * slot, 2 * slot);
     sink.out_index = out_index;
-    if (n <= kFusedMaxLog) {
+    if (np <= kFusedMaxLog) {
         Operand a{level, 2 * slot, slot}, b{level + slot, 2 * slot, slot};
-        ntt_mul_small(c, n, nprod, a, b, false, sink, s);
+        ntt_mul_small(c, np, nprod, a, b, false, sink, s);
     } else {
-        ntt_mul_multipass(c, n, PAIR_ADJACENT, nprod, x, x, sink, s);
+        ntt_mul_multipass(c, np, PAIR_ADJACENT, nprod, x, x, sink, s);
     }
 }
 
@@ -1179,16 +1488,16 @@ void ntt_mul(Ctx &c, const uint32_t *a, size_t na, const uint32_t *b, size_t nb,
              uint32_t *out, cudaStream_t s)
 {
     const size_t len = na + nb;
-    const int n = std::max(1, ceil_log2(len));
-    if (n > kLogMaxNtt) fail(CAT_EINVAL, "operands too long for one transform");
+    const int np = points_log(len);
+    if (np > kLogMaxPts) fail(CAT_EINVAL, "operands too long for one transform");
     const bool square = (a == b && na == nb);
     Operand x{a, 0, na}, y{b, 0, nb};
-    if (n <= kFusedMaxLog) {
-        ntt_mul_small(c, n, 1, x, y, square, plain_sink(out, 0, len), s);
+    if (np <= kFusedMaxLog) {
+        ntt_mul_small(c, np, 1, x, y, square, plain_sink(out, 0, len), s);
     } else if (square) {
-        ntt_mul_multipass(c, n, PAIR_SQUARE, 1, x, x, plain_sink(out, 0, len), s);
+        ntt_mul_multipass(c, np, PAIR_SQUARE, 1, x, x, plain_sink(out, 0, len), s);
     } else {
-        ntt_mul_multipass(c, n, PAIR_FIRST_TWO, 1, x, y, plain_sink(out, 0, len), s);
+        ntt_mul_multipass(c, np, PAIR_FIRST_TWO, 1, x, y, plain_sink(out, 0, len), s);
     }
 }
 
@@ -1198,20 +1507,20 @@ void mul_broadcast(Ctx &c, const uint32_t *x, size_t xstride, size_t xlen, size_
                    const uint32_t *y, size_t ylen, const Sink &sink, cudaStream_t s)
 {
     if (nprod == 0) return;
-    const int n = std::max(1, ceil_log2(xlen + ylen));
-    if (n > kLogMaxNtt) fail(CAT_EINVAL, "operands too long for one transform");
+    const int np = points_log(xlen + ylen);
+    if (np > kLogMaxPts) fail(CAT_EINVAL, "operands too long for one transform");
     Operand ox{x, xstride, xlen}, oy{y, 0, ylen};
     if (nprod == 1 && x == y && xlen == ylen) {  // a square: one forward transform
-        if (n <= kFusedMaxLog)
-            ntt_mul_small(c, n, 1, ox, ox, true, sink, s);
+        if (np <= kFusedMaxLog)
+            ntt_mul_small(c, np, 1, ox, ox, true, sink, s);
         else
-            ntt_mul_multipass(c, n, PAIR_SQUARE, 1, ox, ox, sink, s);
+            ntt_mul_multipass(c, np, PAIR_SQUARE, 1, ox, ox, sink, s);
         return;
     }
-    if (n <= kFusedMaxLog)
-        ntt_mul_small(c, n, nprod, ox, oy, false, sink, s);
+    if (np <= kFusedMaxLog)
+        ntt_mul_small(c, np, nprod, ox, oy, false, sink, s);
     else
-        ntt_mul_multipass(c, n, PAIR_BROADCAST, nprod, ox, oy, sink, s);
+        ntt_mul_multipass(c, np, PAIR_BROADCAST, nprod, ox, oy, sink, s);
 }
 
 // ------------------------------------------------ long products by pieces
@@ -1225,16 +1534,13 @@ __global__ void __launch_bounds__(kTileThreads) add_tiles(uint32_t *acc, size_t 
     __shared__ uint32_t wsm[32];
     const size_t jt = (size_t)blockIdx.x * kTile;
     const int j0 = threadIdx.x * kLimbsPerThread;
-    CoefRun run;
-#pragma unroll
-    for (int i = 0; i < kLimbsPerThread; i++) {
+    auto limb = [&](int i) -> uint64_t {
         const size_t j = jt + j0 + i;
-        run.c0[i] = j < tn ? t[j] : 0u;
-        run.c1[i] = run.c2[i] = 0u;
-    }
+        return j < tn ? t[j] : 0u;
+    };
     const int tile_len = (int)(R - jt < (size_t)kTile ? R - jt : (size_t)kTile);
     uint32_t map;
-    tile_carry(run, 0u, 0u, 0u, tile_len, acc + jt, tile_len, dec, acc + jt, tile_len, wsm, &map);
+    tile_carry<-1, 1>(limb, tile_len, acc + jt, tile_len, dec, acc + jt, tile_len, wsm, &map);
     if (threadIdx.x == 0) tile_maps[blockIdx.x] = (uint8_t)map;
 }
 
@@ -1250,12 +1556,8 @@ void add_into(Ctx &c, uint32_t *acc, size_t R, const uint32_t *t, size_t tn, boo
     const int tok = prof_begin(c, "add_tiles", s);
     add_tiles<<<(unsigned)tiles, kTileThreads, 0, s>>>(acc, R, t, tn, dec, maps.get());
     CAT_LAUNCH("add_tiles");
-    carry_tile_scan<<<1, 1024, 0, s>>>(maps.get(), tiles);
-    CAT_LAUNCH("carry_tile_scan");
-    carry_fix<<<(unsigned)((tiles + 255) / 256), 256, 0, s>>>(maps.get(), tiles, tiles, 0, acc, 0,
-                                                              R, dec);
-    CAT_LAUNCH("carry_fix");
     prof_end(c, tok, s, 8.0 * (double)R + 4.0 * (double)tn);
+    carry_finish(c, maps.get(), 1, tiles, Sink{acc, 0, R, dec, nullptr, 0, 0}, s);
 }
 
 // acc[0 .. R) += x y for operands of any length: pieces of Mx and My limbs
@@ -1294,18 +1596,17 @@ void mul_acc(Ctx &c, const uint32_t *x, size_t xlen, const uint32_t *y, size_t y
 // words), and belongs at offset iM, so it overlaps the next chunk's product by
 // ny limbs.  Limb j of the result sums t1 = slot k's word j - kM (k = j / M,
 // the last slot also covers its tail) and t2 = slot k-1's word M + (j - kM)
-// when j - kM < ny.  Per tile: run words c0[i] = t1(j0 + i) and c1[i] =
-// t2(j0 + i + 1), so tile_carry's c1[j - 1] term adds t2(j) to limb j.
-__device__ __forceinline__ void overlap_terms(const uint32_t *T, size_t M, size_t ny,
-                                              size_t chunks, size_t j, uint32_t &t1,
-                                              uint32_t &t2)
+// when j - kM < ny.
+__device__ __forceinline__ uint64_t overlap_sum(const uint32_t *T, size_t M, size_t ny,
+                                                size_t chunks, size_t j)
 {
     size_t k = j / M;
     const bool past = k >= chunks;
     if (past) k = chunks - 1;
     const size_t r = j - k * M;
-    t1 = r < M + ny ? T[k * (M + ny) + r] : 0u;
-    t2 = (!past && k >= 1 && r < ny) ? T[(k - 1) * (M + ny) + M + r] : 0u;
+    const uint32_t t1 = r < M + ny ? T[k * (M + ny) + r] : 0u;
+    const uint32_t t2 = (!past && k >= 1 && r < ny) ? T[(k - 1) * (M + ny) + M + r] : 0u;
+    return (uint64_t)t1 + t2;
 }
 
 __global__ void __launch_bounds__(kTileThreads) overlap_tiles(const uint32_t *T, size_t M,
@@ -1314,26 +1615,14 @@ __global__ void __launch_bounds__(kTileThreads) overlap_tiles(const uint32_t *T,
                                                               uint8_t *tile_maps)
 {
     __shared__ uint32_t wsm[32];
-    __shared__ uint32_t hsm[96];
     const size_t jt = (size_t)blockIdx.x * kTile;
     const size_t j0 = jt + threadIdx.x * kLimbsPerThread;
-    CoefRun run;
-#pragma unroll
-    for (int i = 0; i < kLimbsPerThread; i++) {
-        uint32_t a = 0, b = 0, dummy = 0;
-        if (j0 + i < R) overlap_terms(T, M, ny, chunks, j0 + i, a, dummy);
-        if (j0 + i + 1 < R) overlap_terms(T, M, ny, chunks, j0 + i + 1, dummy, b);
-        run.c0[i] = a;
-        run.c1[i] = b;
-        run.c2[i] = 0u;
-    }
-    uint32_t first1 = 0, dummy = 0;
-    if (threadIdx.x == 0 && jt < R) overlap_terms(T, M, ny, chunks, jt, dummy, first1);
-    uint32_t h1, h2a, h2b;
-    run_halo(run, first1, 0u, 0u, hsm, h1, h2a, h2b);
+    auto limb = [&](int i) -> uint64_t {
+        return j0 + i < R ? overlap_sum(T, M, ny, chunks, j0 + i) : 0u;
+    };
     const int tile_len = (int)(R - jt < (size_t)kTile ? R - jt : (size_t)kTile);
     uint32_t map;
-    tile_carry(run, h1, 0u, 0u, tile_len, out + jt, tile_len, false, nullptr, 0, wsm, &map);
+    tile_carry<0, 0>(limb, tile_len, out + jt, tile_len, false, nullptr, 0, wsm, &map);
     if (threadIdx.x == 0) tile_maps[blockIdx.x] = (uint8_t)map;
 }
 
@@ -1358,12 +1647,8 @@ void mul_chunked(Ctx &c, const uint32_t *x, size_t nx, const uint32_t *y, size_t
     overlap_tiles<<<(unsigned)tiles, kTileThreads, 0, s>>>(T.get(), M, ny, chunks, out, R,
                                                             maps.get());
     CAT_LAUNCH("overlap_tiles");
-    carry_tile_scan<<<1, 1024, 0, s>>>(maps.get(), tiles);
-    CAT_LAUNCH("carry_tile_scan");
-    carry_fix<<<(unsigned)((tiles + 255) / 256), 256, 0, s>>>(maps.get(), tiles, tiles, 0, out, 0,
-                                                              R, false);
-    CAT_LAUNCH("carry_fix");
     prof_end(c, tok, s, 4.0 * (double)(chunks * slot) + 4.0 * (double)R);
+    carry_finish(c, maps.get(), 1, tiles, plain_sink(out, 0, R), s);
 }
 
 // --------------------------------------- multiplication without allocation
@@ -1378,10 +1663,10 @@ void mul_chunked(Ctx &c, const uint32_t *x, size_t nx, const uint32_t *y, size_t
 
 constexpr int kNoAllocLog = 16;
 constexpr size_t kNoAllocMaxLimbs = (size_t)1 << kNoAllocLog;   // na + nb limit
-constexpr size_t kNoAllocL = kNoAllocMaxLimbs;
-// words: F (3 primes x 2 transforms x L), G (3 x L), tile maps, top index
-constexpr size_t kNoAllocF = 6 * kNoAllocL;
-constexpr size_t kNoAllocG = 3 * kNoAllocL;
+constexpr size_t kNoAllocN = kNoAllocMaxLimbs / 2;  // points
+// words: F (5 primes x 2 transforms x N), G (5 x N), tile maps, top index
+constexpr size_t kNoAllocF = 2 * kNumPrimes * kNoAllocN;
+constexpr size_t kNoAllocG = kNumPrimes * kNoAllocN;
 constexpr size_t kNoAllocMapWords = 64;
 constexpr size_t kNoAllocWords = kNoAllocF + kNoAllocG + kNoAllocMapWords + 2;
 
@@ -1450,55 +1735,18 @@ static void noalloc_mul(const NoAllocDevice &d, const uint32_t *a, size_t na, co
     local.twiddles = d.twiddles;
     local.col_tw_tables = false;  // the passes compute their twiddles: nothing allocated
     const size_t len = na + nb;
-    const int n = std::max(1, ceil_log2(len));
+    const int np = points_log(len);
     Operand x{a, 0, na}, y{b, 0, nb};
-    if (n <= kFusedMaxLog) {
-        ntt_mul_small(local, n, 1, x, y, false, plain_sink(out, 0, len), s);
+    if (np <= kFusedMaxLog) {
+        ntt_mul_small(local, np, 1, x, y, false, plain_sink(out, 0, len), s);
         return;
     }
-    const NttPlan P = make_plan(local, n);
-    const size_t L = (size_t)1 << n;
-    uint32_t *F = d.scratch;
-    uint32_t *G = d.scratch + kNoAllocF;
-    uint8_t *maps = (uint8_t *)(d.scratch + kNoAllocF + kNoAllocG);
-    const size_t fp = 2 * L, gp = L;
-    col_pass(local, 0, true, F, fp, L, n, P.rcol[0], x.p, 0, x.len, s);
-    col_pass(local, 0, true, F + L, fp, L, n, P.rcol[0], y.p, 0, y.len, s);
-    int m = n - P.rcol[0];
-    for (int i = 1; i < P.ncol; i++) {
-        col_pass(local, 0, true, F, fp, fp, m, P.rcol[i], nullptr, 0, 0, s);
-        m -= P.rcol[i];
-    }
-    RowArgs ra;
-    ra.F = F;
-    ra.fpstride = fp;
-    ra.G = G;
-    ra.gpstride = gp;
-    ra.n = n;
-    ra.mode = PAIR_FIRST_TWO;
-    ra.prescaled = 0;  // computed twiddles: the row pass normalises
-    ra.tw = d.twiddles;
-    ra.scale = make_scale(0, n);
-    launch_row(0, P.rrow, 1, n, s, ra);
-    for (int i = P.ncol - 1; i >= 0; i--) {
-        int mi = n;
-        for (int j = 0; j < i; j++) mi -= P.rcol[j];
-        col_pass(local, 0, false, G, gp, gp, mi, P.rcol[i], nullptr, 0, 0, s);
-    }
-    const size_t tiles = L / kTile;
-    CrtArgs ca;
-    ca.G = G;
-    ca.gpstride = gp;
-    ca.n = n;
-    ca.sink = plain_sink(out, 0, len);
-    ca.tile_maps = maps;
-    launch_crt(0, (unsigned)tiles, s, ca);
-    CAT_LAUNCH("crt_carry_tiles");
-    carry_tile_scan<<<1, 1024, 0, s>>>(maps, tiles);
-    CAT_LAUNCH("carry_tile_scan");
-    carry_fix<<<(unsigned)((tiles + 255) / 256), 256, 0, s>>>(maps, tiles, tiles, n, out, 0, len,
-                                                            false);
-    CAT_LAUNCH("carry_fix");
+    MulScratch m;
+    m.fixed = true;
+    m.F = d.scratch;
+    m.G = d.scratch + kNoAllocF;
+    m.maps = (uint8_t *)(d.scratch + kNoAllocF + kNoAllocG);
+    ntt_mul_multipass(local, np, PAIR_FIRST_TWO, 1, x, y, plain_sink(out, 0, len), s, std::move(m));
 }
 
 }  // namespace cat

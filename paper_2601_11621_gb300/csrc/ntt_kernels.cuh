@@ -162,12 +162,16 @@ __device__ __forceinline__ void dit_stages(uint32_t (&x)[NA][1 << E], int glow, 
 // `out`.  COLFAST: consecutive threads take consecutive columns (strided
 // columns in global memory); otherwise consecutive threads take consecutive
 // groups of one column (contiguous rows in global memory).  No barrier.
-template <int LR, int C, int B, int E, bool FWD, int NA, bool COLFAST, int PS, class IN, class OUT>
+// THREADS: the block's threads (0: blockDim.x).
+template <int LR, int C, int B, int E, bool FWD, int NA, bool COLFAST, int PS, int THREADS = 0,
+          class IN, class OUT>
 __device__ __forceinline__ void round_io(const IN &in, const OUT &out, const TwRef &T, uint32_t q)
 {
     constexpr int NGC = (1 << LR) >> E;  // groups per column
     constexpr int NG = C * NGC;
-    for (int g = threadIdx.x; g < NG; g += blockDim.x) {
+    const int step = THREADS ? THREADS : (int)blockDim.x;
+#pragma unroll 1
+    for (int g = threadIdx.x; g < NG; g += step) {
         const int c = COLFAST ? (g & (C - 1)) : (g / NGC);
         const int gg = COLFAST ? (g / C) : (g & (NGC - 1));
         const int glow = gg & ((1 << B) - 1);
@@ -223,44 +227,6 @@ struct SmemIO {
     }
 };
 
-// All-shared-memory transforms (used by the one-block multiply) of C arrays
-// of 2^LR words each, back to back (swizzled); every group holds one array's
-// points, so a round has C 2^(LR - E) groups for the block's threads.  Caller
-// synchronises before; these return synchronised.
-template <int LR, int C, int PS>
-__device__ __forceinline__ void dif_smem(uint32_t *s, const TwRef &T, uint32_t q)
-{
-    constexpr int NR = rounds_of(LR);
-    SmemIO<LR, C, false> S{s};
-    round_io<LR, C, dif_base(LR, 0), round_size(LR, 0), true, 1, false, PS>(S, S, T, q);
-    __syncthreads();
-    if constexpr (NR >= 2) {
-        round_io<LR, C, dif_base(LR, 1), round_size(LR, 1), true, 1, false, PS>(S, S, T, q);
-        __syncthreads();
-    }
-    if constexpr (NR >= 3) {
-        round_io<LR, C, dif_base(LR, 2), round_size(LR, 2), true, 1, false, PS>(S, S, T, q);
-        __syncthreads();
-    }
-}
-
-template <int LR, int C, int PS>
-__device__ __forceinline__ void dit_smem(uint32_t *s, const TwRef &Ti, uint32_t q)
-{
-    constexpr int NR = rounds_of(LR);
-    SmemIO<LR, C, false> S{s};
-    round_io<LR, C, dit_base(LR, 0), dit_size(LR, 0), false, 1, false, PS>(S, S, Ti, q);
-    __syncthreads();
-    if constexpr (NR >= 2) {
-        round_io<LR, C, dit_base(LR, 1), dit_size(LR, 1), false, 1, false, PS>(S, S, Ti, q);
-        __syncthreads();
-    }
-    if constexpr (NR >= 3) {
-        round_io<LR, C, dit_base(LR, 2), dit_size(LR, 2), false, 1, false, PS>(S, S, Ti, q);
-        __syncthreads();
-    }
-}
-
 // ---------------------------------------------------------- column passes
 
 // A column pass block holds C columns of 2^LR rows: 16 columns at 2^10 rows
@@ -313,14 +279,16 @@ struct ColArgs {
     const uint32_t *src;   // first forward pass: limb source (else null)
     size_t src_tstride;    // limbs between consecutive transforms' sources
     size_t src_len;        // valid limbs per transform (rest are zero)
+    int src_al;            // every source starts on a 16-byte boundary
+    CoefMuls coef;         // the sources' input multipliers
     const uint2 *tw;
     // the pass's inter-pass twiddles, w^(col bitrev(row)) in the multiplier
     // form the pass applies, point (row, col) of a 2^m block at row 2^(m-LR) +
     // col, 2^m per prime; null: the pass computes them
     const uint32_t *twtab;
     // first forward pass of adjacent pairs: the odd transforms' (operand b's)
-    // table, its entries times 2^(32-m) (the pointwise product's 2^-m
-    // normalisation taken in advance), or null
+    // table, its entries times 2^32 S (the pointwise product's scale S taken
+    // in advance), or null
     const uint32_t *twtab_odd;
 };
 
@@ -377,18 +345,11 @@ __device__ __forceinline__ void store_v(uint32_t *p, const uint32_t (&w)[V])
 
 // Column tile in global memory: element (row, col) at p[row * S + col0 + col],
 // group c covering columns c V .. c V + V - 1 (V-word aligned: S, col0 and
-// the array bases are multiples of 16 words).  With `src`, elements come from
-// limbs instead (zero past src_len, reduced), word by word, since a caller's
-// limbs need not be aligned.
-template <int PS, int V, bool ZT = false>
+// the array bases are multiples of V words).
+template <int V>
 struct ColIn {
-    // ZT: the first round of the first pass of an operand of at most half the
-    // transform's length, whose points k >= 2^(E-1) lie in the zero upper half
-    static constexpr bool kZeroTop = ZT;
     const uint32_t *p;
-    const uint32_t *src;
-    uint32_t S, col0, src_len;  // offsets within one transform fit in 32 bits
-    uint32_t q, wp1;
+    uint32_t S, col0;  // offsets within one transform fit in 32 bits
     template <int E, int B, int NA>
     __device__ __forceinline__ void load(uint32_t (&x)[NA][1 << E], int base, int c) const
     {
@@ -396,22 +357,54 @@ struct ColIn {
         const uint32_t i0 = (uint32_t)base * S + col0 + (uint32_t)c * V;
 #pragma unroll
         for (int k = 0; k < (1 << E); k++) {
-            if (ZT && k >= (1 << (E - 1))) {
+            uint32_t w[V];
+            load_v<V>(p + i0 + (uint32_t)k * (S << B), w);
 #pragma unroll
-                for (int a = 0; a < V; a++) x[a][k] = 0u;
-                continue;
+            for (int a = 0; a < V; a++) x[a][k] = w[a];
+        }
+    }
+};
+
+// The same elements from an operand's limbs: coefficient i from words 2i and
+// 2i + 1 (zero past src_len).  A group inside the operand whose words are
+// 16-byte aligned takes one 16-byte load per pair of columns, the others word
+// by word; the choice is made once per group, so that its loads go out
+// together.  ZT: the first round of the first pass of an operand of at most
+// half the transform's length, whose points k >= 2^(E-1) lie in the zero
+// upper half.
+template <int PS, int V, bool ZT>
+struct ColSrcIn {
+    static constexpr bool kZeroTop = ZT;
+    const uint32_t *src;
+    uint32_t S, col0, src_len;
+    bool al;
+    uint32_t q;
+    CoefMul m;
+    template <int E, int B, int NA>
+    __device__ __forceinline__ void load(uint32_t (&x)[NA][1 << E], int base, int c) const
+    {
+        static_assert(NA == V && V == 2, "one array per column of the group");
+        const uint32_t i0 = 2u * ((uint32_t)base * S + col0 + (uint32_t)c * V);
+        constexpr int K = ZT ? (1 << (E - 1)) : (1 << E);
+        uint4 w[K];
+        if (al && i0 + (uint32_t)(K - 1) * (2u * S << B) + 4u <= src_len) {
+#pragma unroll
+            for (int k = 0; k < K; k++)
+                w[k] = *reinterpret_cast<const uint4 *>(src + i0 + (uint32_t)k * (2u * S << B));
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                const uint32_t i = i0 + (uint32_t)k * (2u * S << B);
+                w[k].x = i < src_len ? src[i] : 0u;
+                w[k].y = i + 1 < src_len ? src[i + 1] : 0u;
+                w[k].z = i + 2 < src_len ? src[i + 2] : 0u;
+                w[k].w = i + 3 < src_len ? src[i + 3] : 0u;
             }
-            const uint32_t idx = i0 + (uint32_t)k * (S << B);
-            if (src) {
+        }
 #pragma unroll
-                for (int a = 0; a < V; a++)
-                    x[a][k] = idx + a < src_len ? reduce_in<PS>(src[idx + a], q, wp1) : 0u;
-            } else {
-                uint32_t w[V];
-                load_v<V>(p + idx, w);
-#pragma unroll
-                for (int a = 0; a < V; a++) x[a][k] = w[a];
-            }
+        for (int k = 0; k < (1 << E); k++) {
+            x[0][k] = k < K ? coef_in<PS>(w[k].x, w[k].y, m, q) : 0u;
+            x[1][k] = k < K ? coef_in<PS>(w[k].z, w[k].w, m, q) : 0u;
         }
     }
 };
@@ -554,7 +547,9 @@ struct ColOut {
 
 // Forward column pass: a 2^LR-point DIF down each of C consecutive columns of
 // one block (row stride S = 2^(m-LR)), then the twiddle w_M^(col * bitrev(row)).
-template <int LR, int PS, int V, bool ZT>
+// SRC: 0 in place, 1 from the operands' limbs, 2 the same with the upper half
+// zero.
+template <int LR, int PS, int V, int SRC>
 __global__ void __launch_bounds__(kColFwdThreads, CAT_COL_FWD_MINB) ntt_col_fwd(ColArgs a)
 {
     extern __shared__ uint32_t sm[];
@@ -571,8 +566,14 @@ __global__ void __launch_bounds__(kColFwdThreads, CAT_COL_FWD_MINB) ntt_col_fwd(
     uint32_t *base = a.data + p * a.pstride + (blk << a.m);
     const uint2 *T = tw_table(a.tw, PS, p, 0);
     const TwRef TR{T, p};
-    const ColIn<PS, V, ZT> in{base, a.src ? a.src + blk * a.src_tstride : nullptr, (uint32_t)Sr,
-                              (uint32_t)col0, (uint32_t)a.src_len, q, c_wp1[PS][p]};
+    const auto in = [&] {
+        if constexpr (SRC != 0)
+            return ColSrcIn<PS, V, SRC == 2>{a.src + blk * a.src_tstride, (uint32_t)Sr,
+                                             (uint32_t)col0, (uint32_t)a.src_len, a.src_al != 0, q,
+                                             a.coef.c[p]};
+        else
+            return ColIn<V>{base, (uint32_t)Sr, (uint32_t)col0};
+    }();
     ColTw<LR, PS, NR, kColFwdThreads, V> tw{T, q, c_qinv[PS][p], set_log_root(PS) - a.m, {}};
     const uint32_t *tt = ((blk & 1) && a.twtab_odd) ? a.twtab_odd : a.twtab;
     if (tt) {
@@ -582,23 +583,23 @@ __global__ void __launch_bounds__(kColFwdThreads, CAT_COL_FWD_MINB) ntt_col_fwd(
     tw.init((uint32_t)col0);
     const ColOutTw<LR, PS, NR, V> out{base, (uint32_t)Sr, (uint32_t)col0, tw};
     if constexpr (NR == 1) {
-        round_io<LR, CV, 0, LR, true, V, true, PS>(in, out, TR, q);
+        round_io<LR, CV, 0, LR, true, V, true, PS, kColFwdThreads>(in, out, TR, q);
     } else {
         const SmemIO<LR, CV, true> sio{sm};
-        round_io<LR, CV, dif_base(LR, 0, NR), round_size(LR, 0, NR), true, V, true, PS>(in, sio,
+        round_io<LR, CV, dif_base(LR, 0, NR), round_size(LR, 0, NR), true, V, true, PS, kColFwdThreads>(in, sio,
                                                                                        TR, q);
         __syncthreads();
         if constexpr (NR >= 3) {
-            round_io<LR, CV, dif_base(LR, 1, NR), round_size(LR, 1, NR), true, V, true, PS>(
+            round_io<LR, CV, dif_base(LR, 1, NR), round_size(LR, 1, NR), true, V, true, PS, kColFwdThreads>(
                 sio, sio, TR, q);
             __syncthreads();
         }
         if constexpr (NR >= 4) {
-            round_io<LR, CV, dif_base(LR, 2, NR), round_size(LR, 2, NR), true, V, true, PS>(
+            round_io<LR, CV, dif_base(LR, 2, NR), round_size(LR, 2, NR), true, V, true, PS, kColFwdThreads>(
                 sio, sio, TR, q);
             __syncthreads();
         }
-        round_io<LR, CV, 0, round_size(LR, NR - 1, NR), true, V, true, PS>(sio, out, TR, q);
+        round_io<LR, CV, 0, round_size(LR, NR - 1, NR), true, V, true, PS, kColFwdThreads>(sio, out, TR, q);
     }
 }
 
@@ -628,22 +629,22 @@ __global__ void __launch_bounds__(kColInvThreads, CAT_COL_INV_MINB) ntt_col_inv(
     const ColInTw<LR, PS, NR, V> in{base, (uint32_t)Sr, (uint32_t)col0, tw};
     const ColOut<V> out{base, (uint32_t)Sr, (uint32_t)col0};
     if constexpr (NR == 1) {
-        round_io<LR, CV, 0, LR, false, V, true, PS>(in, out, TRi, q);
+        round_io<LR, CV, 0, LR, false, V, true, PS, kColInvThreads>(in, out, TRi, q);
     } else {
         const SmemIO<LR, CV, true> sio{sm};
-        round_io<LR, CV, 0, dit_size(LR, 0, NR), false, V, true, PS>(in, sio, TRi, q);
+        round_io<LR, CV, 0, dit_size(LR, 0, NR), false, V, true, PS, kColInvThreads>(in, sio, TRi, q);
         __syncthreads();
         if constexpr (NR >= 3) {
-            round_io<LR, CV, dit_base(LR, 1, NR), dit_size(LR, 1, NR), false, V, true, PS>(
+            round_io<LR, CV, dit_base(LR, 1, NR), dit_size(LR, 1, NR), false, V, true, PS, kColInvThreads>(
                 sio, sio, TRi, q);
             __syncthreads();
         }
         if constexpr (NR >= 4) {
-            round_io<LR, CV, dit_base(LR, 2, NR), dit_size(LR, 2, NR), false, V, true, PS>(
+            round_io<LR, CV, dit_base(LR, 2, NR), dit_size(LR, 2, NR), false, V, true, PS, kColInvThreads>(
                 sio, sio, TRi, q);
             __syncthreads();
         }
-        round_io<LR, CV, dit_base(LR, NR - 1, NR), dit_size(LR, NR - 1, NR), false, V, true, PS>(
+        round_io<LR, CV, dit_base(LR, NR - 1, NR), dit_size(LR, NR - 1, NR), false, V, true, PS, kColInvThreads>(
             sio, out, TRi, q);
     }
 }
@@ -662,9 +663,9 @@ struct RowArgs {
     size_t fpstride;
     uint32_t *G;        // products (transform domain, then inverse rows)
     size_t gpstride;
-    int n;              // log2 L
+    int np;             // log2 points
     int mode;           // which transforms product k multiplies
-    int prescaled;      // operand b's transform already carries 2^(32-n): no scale
+    int prescaled;      // operand b's transform already carries 2^32 S: no scale
     const uint2 *tw;
     Scale scale;
 };
@@ -730,86 +731,55 @@ struct RowOutPair {
     }
 };
 
-template <int LR>
-struct RowOut {
-    uint32_t *p;
-    template <int E, int B, int NA>
-    __device__ __forceinline__ void store(uint32_t (&x)[NA][1 << E], int base, int c) const
-    {
-#pragma unroll
-        for (int k = 0; k < (1 << E); k++) p[(c << LR) + base + (k << B)] = x[0][k];
-    }
-};
-
 // Last forward pass of both operands (or one, squaring), pointwise product
 // and first inverse pass, on 2^(12-LR) consecutive rows of 2^LR points of
 // product k.  The last forward round, the product and the first inverse round
-// share one register round (their stage bits coincide).  YH (broadcast
-// products): the common operand's transform is already complete in its slot
-// (ntt_row_fwd), in the order the product loop reads it, so only x is
-// transformed here.
-template <int LR, bool SQ, int PS, bool YH, bool NS = false>
-__device__ __forceinline__ void row_mul_body(const RowArgs &a, uint32_t *sm)
+// share one register round (their stage bits coincide).  `in` reads the rows
+// (PAIR: two rows of an operand per group), y is the common operand's
+// finished transform (YH, broadcast products, whose x alone is transformed
+// here; ntt_row_fwd left it in the order the product loop reads it), g takes
+// the rows of the product.
+template <int LR, bool SQ, int PS, bool YH, bool NS, bool PAIR, class IN>
+__device__ __forceinline__ void row_mul_core(const IN &in, const uint32_t *y, uint32_t *g,
+                                             const uint2 *tw, uint2 sc, uint32_t *sm)
 {
     constexpr int NR = rounds_of(LR);
     constexpr int NA = (SQ || YH) ? 1 : 2;
     constexpr int EL = round_size(LR, NR - 1);
-    constexpr int RB = row_log_rows(LR), C = 1 << RB;
+    constexpr int C = 1 << row_log_rows(LR);
     static_assert(EL == dit_size(LR, 0), "mirrored rounds");
     const int p = blockIdx.y;
     const uint32_t q = c_q[PS][p], qinv = c_qinv[PS][p];
-    const size_t blocks = (size_t)1 << (a.n - LR - RB);  // row blocks per product
-    const size_t k = blockIdx.x / blocks;
-    const size_t off = (blockIdx.x % blocks) << (LR + RB);
-    size_t ta, tb;
-    if (a.mode == PAIR_ADJACENT) { ta = 2 * k; tb = 2 * k + 1; }
-    else if (a.mode == PAIR_SQUARE) { ta = k; tb = k; }
-    else if (a.mode == PAIR_BROADCAST) { ta = k; tb = gridDim.x / blocks; }  // y after the x's
-    else { ta = 0; tb = 1; }
-    const uint32_t *fa = a.F + p * a.fpstride + (ta << a.n) + off;
-    const uint32_t *fb = a.F + p * a.fpstride + (tb << a.n) + off;
-    const TwRef T{tw_table(a.tw, PS, p, 0), p};
-    const TwRef Ti{tw_table(a.tw, PS, p, 1), p};
-    const uint2 sc = p == 0 ? a.scale.c[0] : (p == 1 ? a.scale.c[1] : a.scale.c[2]);
+    const TwRef T{tw_table(tw, PS, p, 0), p};
+    const TwRef Ti{tw_table(tw, PS, p, 1), p};
     const SmemIO<LR, C, false> sio{sm};
-    // forward rounds but the last, two rows per group when every thread still
-    // gets a group
-    constexpr int CF = C / 2 > 0 ? C / 2 : 1;
-    constexpr bool kPairFwd =
-        CAT_ROW_PAIR_FWD && C >= 2 && CF * ((1 << LR) >> round_size(LR, 0)) >= kRowThreads &&
-        (NR == 2 || CF * ((1 << LR) >> round_size(LR, 1)) >= kRowThreads);
-    if constexpr (kPairFwd) {
+    // forward rounds but the last
+    constexpr int CF = PAIR ? C / 2 : C;
+    constexpr int NF = PAIR ? 2 * NA : NA;
+    {
         const SmemIO<LR, CF, false> sp{sm};
-        round_io<LR, CF, dif_base(LR, 0), round_size(LR, 0), true, 2 * NA, false, PS>(
-            RowInPair<LR, CF>{fa, fb}, sp, T, q);
+        round_io<LR, CF, dif_base(LR, 0), round_size(LR, 0), true, NF, false, PS, kRowThreads>(
+            in, sp, T, q);
         __syncthreads();
         if constexpr (NR == 3) {
-            round_io<LR, CF, dif_base(LR, 1), round_size(LR, 1), true, 2 * NA, false, PS>(sp, sp, T,
-                                                                                       q);
-            __syncthreads();
-        }
-    } else {
-        round_io<LR, C, dif_base(LR, 0), round_size(LR, 0), true, NA, false, PS>(
-            RowIn<LR>{fa, fb}, sio, T, q);
-        __syncthreads();
-        if constexpr (NR == 3) {
-            round_io<LR, C, dif_base(LR, 1), round_size(LR, 1), true, NA, false, PS>(sio, sio, T,
-                                                                                   q);
+            round_io<LR, CF, dif_base(LR, 1), round_size(LR, 1), true, NF, false, PS, kRowThreads>(
+                sp, sp, T, q);
             __syncthreads();
         }
     }
     // last forward round + pointwise product + first inverse round
     constexpr int NGC = (1 << LR) >> EL;
-    for (int g = threadIdx.x; g < C * NGC; g += blockDim.x) {
-        const int c = g / NGC;
-        const int base = (g & (NGC - 1)) << EL;
+#pragma unroll 1
+    for (int gi = threadIdx.x; gi < C * NGC; gi += kRowThreads) {
+        const int c = gi / NGC;
+        const int base = (gi & (NGC - 1)) << EL;
         uint32_t x[NA][1 << EL];
         sio.template load<EL, 0, NA>(x, base, c);
         dif_stages<EL, 0, NA, PS>(x, 0, T, q);
         uint32_t yv[1 << EL];
         if constexpr (YH) {
             static_assert(EL >= 2, "the common transform is read 16 bytes at a time");
-            const uint4 *y4 = reinterpret_cast<const uint4 *>(fb + (c << LR) + base);
+            const uint4 *y4 = reinterpret_cast<const uint4 *>(y + (c << LR) + base);
 #pragma unroll
             for (int j = 0; j < (1 << EL) / 4; j++) {
                 const uint4 v = y4[j];
@@ -825,7 +795,6 @@ __device__ __forceinline__ void row_mul_body(const RowArgs &a, uint32_t *sm)
         sio.template store<EL, 0, 1>(z, base, c);
     }
     __syncthreads();
-    uint32_t *g = a.G + p * a.gpstride + (k << a.n) + off;
     // rows in pairs when the block has two rows or more and the paired rounds
     // still give every thread a group; the single-array layout (row r at
     // r 2^LR) is the paired layout's (array a at a CH 2^LR, column c at c 2^LR)
@@ -833,26 +802,53 @@ __device__ __forceinline__ void row_mul_body(const RowArgs &a, uint32_t *sm)
     constexpr bool kPair =
         CAT_ROW_PAIR && C >= 2 && CH * ((1 << LR) >> dit_size(LR, 1)) >= kRowThreads &&
         (NR == 2 || CH * ((1 << LR) >> dit_size(LR, 2)) >= kRowThreads);
-    if constexpr (kPair) {
-        const SmemIO<LR, CH, false> sp{sm};
-        if constexpr (NR == 2) {
-            round_io<LR, CH, dit_base(LR, 1), dit_size(LR, 1), false, 2, false, PS>(
-                sp, RowOutPair<LR, CH>{g}, Ti, q);
-        } else {
-            round_io<LR, CH, dit_base(LR, 1), dit_size(LR, 1), false, 2, false, PS>(sp, sp, Ti, q);
-            __syncthreads();
-            round_io<LR, CH, dit_base(LR, 2), dit_size(LR, 2), false, 2, false, PS>(
-                sp, RowOutPair<LR, CH>{g}, Ti, q);
-        }
-    } else if constexpr (NR == 2) {
-        round_io<LR, C, dit_base(LR, 1), dit_size(LR, 1), false, 1, false, PS>(sio, RowOut<LR>{g},
-                                                                               Ti, q);
+    constexpr int CI = kPair ? CH : C, NI = kPair ? 2 : 1;
+    const SmemIO<LR, CI, false> sp{sm};
+    const RowOutPair<LR, CI> ro{g};
+    if constexpr (NR == 2) {
+        round_io<LR, CI, dit_base(LR, 1), dit_size(LR, 1), false, NI, false, PS, kRowThreads>(
+            sp, ro, Ti, q);
     } else {
-        round_io<LR, C, dit_base(LR, 1), dit_size(LR, 1), false, 1, false, PS>(sio, sio, Ti, q);
+        round_io<LR, CI, dit_base(LR, 1), dit_size(LR, 1), false, NI, false, PS, kRowThreads>(
+            sp, sp, Ti, q);
         __syncthreads();
-        round_io<LR, C, dit_base(LR, 2), dit_size(LR, 2), false, 1, false, PS>(sio, RowOut<LR>{g},
-                                                                               Ti, q);
+        round_io<LR, CI, dit_base(LR, 2), dit_size(LR, 2), false, NI, false, PS, kRowThreads>(
+            sp, ro, Ti, q);
     }
+}
+
+// Whether the forward rounds but the last take two rows per group: when every
+// thread still gets one.
+template <int LR>
+__host__ __device__ constexpr bool row_pair_fwd()
+{
+    constexpr int NR = rounds_of(LR);
+    constexpr int C = 1 << row_log_rows(LR), CF = C / 2;
+    return CAT_ROW_PAIR_FWD && C >= 2 && CF * ((1 << LR) >> round_size(LR, 0)) >= kRowThreads &&
+           (NR == 2 || CF * ((1 << LR) >> round_size(LR, 1)) >= kRowThreads);
+}
+
+template <int LR, bool SQ, int PS, bool YH, bool NS = false>
+__device__ __forceinline__ void row_mul_body(const RowArgs &a, uint32_t *sm)
+{
+    constexpr int RB = row_log_rows(LR), C = 1 << RB;
+    const int p = blockIdx.y;
+    const size_t blocks = (size_t)1 << (a.np - LR - RB);  // row blocks per product
+    const size_t k = blockIdx.x / blocks;
+    const size_t off = (blockIdx.x % blocks) << (LR + RB);
+    size_t ta, tb;
+    if (a.mode == PAIR_ADJACENT) { ta = 2 * k; tb = 2 * k + 1; }
+    else if (a.mode == PAIR_SQUARE) { ta = k; tb = k; }
+    else if (a.mode == PAIR_BROADCAST) { ta = k; tb = gridDim.x / blocks; }  // y after the x's
+    else { ta = 0; tb = 1; }
+    const uint32_t *fa = a.F + p * a.fpstride + (ta << a.np) + off;
+    const uint32_t *fb = a.F + p * a.fpstride + (tb << a.np) + off;
+    uint32_t *g = a.G + p * a.gpstride + (k << a.np) + off;
+    if constexpr (row_pair_fwd<LR>())
+        row_mul_core<LR, SQ, PS, YH, NS, true>(RowInPair<LR, C / 2>{fa, fb}, fb, g, a.tw,
+                                               a.scale.c[p], sm);
+    else
+        row_mul_core<LR, SQ, PS, YH, NS, false>(RowIn<LR>{fa, fb}, fb, g, a.tw, a.scale.c[p], sm);
 }
 
 template <int LR, bool SQ, int PS>
@@ -863,7 +859,7 @@ __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_mul(RowArgs
 }
 
 // Products whose operand b transform already carries the normalisation
-// 2^(32-n) (its first pass took the scaled twiddle table): the pointwise
+// 2^32 S (its first pass took the scaled twiddle table): the pointwise
 // product is one Montgomery product.
 template <int LR, int PS>
 __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_mul_ns(RowArgs a)
@@ -901,24 +897,21 @@ __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_fwd(RowArgs
     const TwRef T{tw_table(a.tw, PS, p, 0), p};
     const SmemIO<LR, C, false> sio{sm};
     constexpr int CF = C / 2 > 0 ? C / 2 : 1;
-    constexpr bool kPairFwd =
-        CAT_ROW_PAIR_FWD && C >= 2 && CF * ((1 << LR) >> round_size(LR, 0)) >= kRowThreads &&
-        (NR == 2 || CF * ((1 << LR) >> round_size(LR, 1)) >= kRowThreads);
-    if constexpr (kPairFwd) {
+    if constexpr (row_pair_fwd<LR>()) {
         const SmemIO<LR, CF, false> sp{sm};
-        round_io<LR, CF, dif_base(LR, 0), round_size(LR, 0), true, 2, false, PS>(
+        round_io<LR, CF, dif_base(LR, 0), round_size(LR, 0), true, 2, false, PS, kRowThreads>(
             RowInPair<LR, CF>{fy, fy}, sp, T, q);
         __syncthreads();
         if constexpr (NR == 3) {
-            round_io<LR, CF, dif_base(LR, 1), round_size(LR, 1), true, 2, false, PS>(sp, sp, T, q);
+            round_io<LR, CF, dif_base(LR, 1), round_size(LR, 1), true, 2, false, PS, kRowThreads>(sp, sp, T, q);
             __syncthreads();
         }
     } else {
-        round_io<LR, C, dif_base(LR, 0), round_size(LR, 0), true, 1, false, PS>(
+        round_io<LR, C, dif_base(LR, 0), round_size(LR, 0), true, 1, false, PS, kRowThreads>(
             RowIn<LR>{fy, fy}, sio, T, q);
         __syncthreads();
         if constexpr (NR == 3) {
-            round_io<LR, C, dif_base(LR, 1), round_size(LR, 1), true, 1, false, PS>(sio, sio, T, q);
+            round_io<LR, C, dif_base(LR, 1), round_size(LR, 1), true, 1, false, PS, kRowThreads>(sio, sio, T, q);
             __syncthreads();
         }
     }
@@ -934,4 +927,74 @@ __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_fwd(RowArgs
         for (int j = 0; j < (1 << EL) / 4; j++)
             o4[j] = make_uint4(x[0][4 * j], x[0][4 * j + 1], x[0][4 * j + 2], x[0][4 * j + 3]);
     }
+}
+
+// ------------------------------------------ whole transforms from limbs
+
+struct RowLimbArgs {
+    const uint32_t *A, *B;
+    size_t a_tstride, b_tstride;  // limbs between consecutive products' operands
+    uint32_t a_len, b_len;
+    int a_al, b_al;               // every operand starts on an 8-byte boundary
+    uint32_t *G;
+    size_t gpstride;
+    const uint2 *tw;
+    Scale scale;
+    CoefMuls ca, cb;              // cb carries the pointwise scale
+};
+
+// One row of 2^LR coefficients per operand, from limbs (operand a, operand b).
+template <int LR, bool ZT>
+struct RowLimbIn {
+    static constexpr bool kZeroTop = ZT;
+    const uint32_t *pa, *pb;
+    uint32_t la, lb;
+    bool al_a, al_b;
+    uint32_t q;
+    CoefMul ca, cb;
+    template <int E, int B>
+    __device__ __forceinline__ void load1(uint32_t (&x)[1 << E], int base, const uint32_t *r,
+                                          uint32_t len, bool al, const CoefMul &m) const
+    {
+        constexpr int K = ZT ? (1 << (E - 1)) : (1 << E);
+        uint2 w[K];
+        if (al && 2u * (uint32_t)(base + ((K - 1) << B)) + 2u <= len) {
+#pragma unroll
+            for (int k = 0; k < K; k++)
+                w[k] = *reinterpret_cast<const uint2 *>(r + 2 * (base + (k << B)));
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                const uint32_t i = 2u * (uint32_t)(base + (k << B));
+                w[k].x = i < len ? r[i] : 0u;
+                w[k].y = i + 1 < len ? r[i + 1] : 0u;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < (1 << E); k++) x[k] = k < K ? coef_in<0>(w[k].x, w[k].y, m, q) : 0u;
+    }
+    template <int E, int B, int NA>
+    __device__ __forceinline__ void load(uint32_t (&x)[NA][1 << E], int base, int) const
+    {
+        load1<E, B>(x[0], base, pa, la, al_a, ca);
+        if (NA > 1) load1<E, B>(x[NA - 1], base, pb, lb, al_b, cb);
+    }
+};
+
+// Products of 2^12 points without column passes: one block transforms both
+// operands of product blockIdx.x modulo prime blockIdx.y from their limbs,
+// multiplies and transforms back.  The remaindering kernel follows.  (A
+// one-block multiply of 2^12 points would hold 96 KiB: two blocks per SM.)
+template <bool SQ, bool ZT>
+__global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_limbs(RowLimbArgs a)
+{
+    extern __shared__ uint32_t sm[];
+    constexpr int LR = kRowMaxLog;
+    const int p = blockIdx.y;
+    const size_t k = blockIdx.x;
+    const RowLimbIn<LR, ZT> in{a.A + k * a.a_tstride, a.B + k * a.b_tstride, a.a_len, a.b_len,
+                               a.a_al != 0,           a.b_al != 0,           c_q[0][p],
+                               a.ca.c[p],             a.cb.c[p]};
+    row_mul_core<LR, SQ, 0, false, !SQ, false>(in, nullptr, a.G + p * a.gpstride + (k << LR), a.tw,
+                                               a.scale.c[p], sm);
 }

@@ -4,8 +4,8 @@
 // (about 10^5 at a time) and by keeping partial products outside the working
 // set (Sec. 3.2, Algorithm 2 and its remarks on chunking; Sec. 6.2 on memory).
 // This file is that mode for a context whose HBM budget cannot hold the
-// in-core reconstruction (level arrays plus the three-prime transforms of a
-// whole tree level, ~120 bytes per result limb):
+// in-core reconstruction (level arrays plus the five-prime transforms of a
+// whole tree level, at most ~120 bytes per result limb):
 //   - the grouped primes move to pinned host memory;
 //   - each group's primes are multiplied in chunks of K consecutive primes,
 //     every chunk by the device product tree, its root copied to pinned host
@@ -79,9 +79,10 @@ size_t pow2_ceil(size_t x)
 }
 
 // Device bytes one in-core product of na + nb limbs holds at its peak: both
-// operands, the product, and the transform scratch (three residues of two
-// operands and of the product per point, 36 bytes, for the transform of the
-// product's length or of the longest piece), with headroom.
+// operands, the product, and the transform scratch (five residues of two
+// operands and of the product per point of two limbs, 30 bytes per limb, for
+// the transform of the product's length or of the longest piece), with
+// headroom (a product in chunks holds up to 48 bytes per limb).
 size_t mul_need(const Ctx &c, size_t na, size_t nb)
 {
     const size_t n = na + nb;
@@ -107,6 +108,11 @@ HostBig host_one()
     return h;
 }
 
+// Device bytes of a product by pieces of M limbs: two pieces, their product,
+// two windows, and the transform scratch of a piece product (60 M; products
+// of up to 4,096 limbs run in one block and take none), with headroom.
+size_t piece_need(size_t M) { return 36 * M + (2 * M > 4096 ? 64 * M : 0) + (8u << 10); }
+
 // a * b for host operands, by pieces of M limbs: piece products A_i B_j for
 // i + j = s are added into a device window holding limbs [sM, sM + 2M + 2) of
 // the sum (2M + 2 limbs always hold it: the pending sum is below (pieces + 1)
@@ -115,8 +121,8 @@ HostBig host_one()
 // shifts down by M limbs into the other buffer.
 HostBig mul_pieces(Ctx &c, const HostBig &a, const HostBig &b, cudaStream_t s)
 {
-    size_t M = pow2_floor(avail(c) / 112);
-    M = std::min(M, (size_t)1 << (c.max_log - 1));
+    size_t M = (size_t)1 << (c.max_log - 1);
+    while (M >= 1024 && piece_need(M) > avail(c)) M >>= 1;
     if (M < 1024) fail(CAT_ENOMEM, "HBM budget too small for a product by pieces");
     const size_t na = a.n, nb = b.n, nA = (na + M - 1) / M, nB = (nb + M - 1) / M;
     const size_t total = na + nb, W = 2 * M + 2;
@@ -186,7 +192,7 @@ HostBig tree_host(Ctx &c, std::vector<HostBig> v, cudaStream_t s)
 // The product of count 32-bit values in host memory: chunks of K values, each
 // by the device product tree (its root to the host), then a balanced tree
 // over the chunk roots.  The tree of K values holds about 8 K bytes of level
-// arrays and 36 K bytes of transform scratch at its top level; K is the
+// arrays and 30 K bytes of transform scratch at its top level; K is the
 // largest power of two that fits 80 K bytes into the budget.
 HostBig chunk_product(Ctx &c, const uint32_t *vals, size_t count, cudaStream_t s)
 {

@@ -43,7 +43,7 @@ uint64_t now_ns()
 
 // Device bytes a request may hold while it is computed: a fixed part (sieve
 // segments, small tables: measured at most 1.35 MB) and a part per limb of
-// the result bound (level arrays, three-prime transforms, leaves: measured at
+// the result bound (level arrays, five-prime transforms, leaves: measured at
 // most 124 bytes per limb from n = 10^4 to 3 * 10^8, all three kinds), with
 // headroom; a batch's estimate is the sum over its requests.
 constexpr uint64_t kFootprintFixed = 2u << 20;

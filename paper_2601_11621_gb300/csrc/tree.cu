@@ -54,9 +54,13 @@ size_t trim(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s)
     return normalized_length(c, x, n - k, s);
 }
 
-// Relative cost of a butterfly in the prime set of a 2^n-point transform
+// Relative cost of a butterfly in the prime set of a product of 2^n limbs
 // (measured: set 1 ~1.1x and set 2 ~1.5x the lazy set 0).
-static double set_cost(int n) { return n <= kLogSet0 ? 1.0 : (n <= kLogSet1 ? 1.1 : 1.5); }
+static double set_cost(int n)
+{
+    const int ps = set_for(n - 1);
+    return ps == 0 ? 1.0 : (ps == 1 ? 1.1 : 1.5);
+}
 
 static int clog2(size_t x)
 {

@@ -1,0 +1,55 @@
+"""The transform's 64-bit coefficients at the edges of its paths (through the
+C ABI, bit-exact): the largest coefficients every prime set must hold, and
+operands of odd lengths and odd alignment on both sides of each path's limit
+(one block up to 4,096 product limbs, a row pass alone up to 8,192, column
+passes above)."""
+import numpy as np
+import pytest
+
+from paper_2601_11621_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def host(t):
+    return t.detach().cpu().numpy().view(np.uint32)
+
+
+# 2^22, 2^25 and 2^26 limbs fill the transforms of the three prime sets
+@pytest.mark.parametrize("k", [2, 16, 2048, 4096, 8192, 1 << 22, 1 << 25, 1 << 26])
+def test_largest_coefficients(ctx, cat_lib, k):
+    """(2^(32 k) - 1)^2 = 2^(64 k) - 2^(32 k + 1) + 1 by two operands (not the
+    squaring path): every coefficient is the largest of its position."""
+    import torch
+    a = torch.full((k,), -1, dtype=torch.int32, device="cuda")
+    got = cat_lib.bigint_mul(ctx, a, a.clone())
+    want = torch.zeros(2 * k, dtype=torch.int32, device="cuda")
+    want[0] = 1
+    want[k] = -2
+    want[k + 1:] = -1
+    assert got.numel() == 2 * k and torch.equal(got, want)
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("na,nb", [(1, 1), (1, 2), (3, 3), (33, 30), (2047, 2048), (4095, 1),
+                                   (4096, 1), (4097, 3), (3001, 2999), (4097, 4095), (8191, 1),
+                                   (1, 8191), (8192, 1), (5001, 3193), (9001, 9002)])
+def test_odd_lengths_and_alignment(ctx, cat_lib, orc, na, nb, offset):
+    """Operands of odd lengths (a last coefficient of one limb), starting
+    `offset` limbs into their buffers, whose neighbouring words are not zero."""
+    import torch
+    a, b = W.random_limbs32(na, seed=na), W.random_limbs32(nb, seed=nb + 1)
+    ta = torch.full((na + 8,), -1, dtype=torch.int32, device="cuda")
+    tb = torch.full((nb + 8,), -1, dtype=torch.int32, device="cuda")
+    ta[offset:offset + na] = torch.from_numpy(a.view(np.int32)).cuda()
+    tb[offset:offset + nb] = torch.from_numpy(b.view(np.int32)).cuda()
+    got = host(cat_lib.bigint_mul(ctx, ta[offset:offset + na], tb[offset:offset + nb]))
+    assert np.array_equal(got, orc.mul(a, b))
+
+
+@pytest.mark.parametrize("n", [4096, 2049, 4097 // 2, 3000, 3501])
+def test_square_by_the_row_pass(ctx, cat_lib, orc, n):
+    import torch
+    a = W.random_limbs32(n, seed=n)
+    t = torch.from_numpy(a.view(np.int32)).cuda()
+    assert np.array_equal(host(cat_lib.bigint_mul(ctx, t, t)), orc.mul(a, a))
