@@ -26,6 +26,8 @@
 // row pass alone, straight from the operands' limbs.
 #include "cat_internal.cuh"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <mutex>
 
@@ -754,9 +756,107 @@ struct SmemRun {
     }
 };
 
-// One product per block: per prime the forward transforms of both operands,
-// the pointwise product and the inverse transform in shared memory (register
-// rounds, the middle one fused as in the row pass), then remaindering and
+// One prime of a product inside a block of T threads: the forward transforms
+// of both operands into X and X + N (N = 2^LR), the pointwise product and the
+// inverse transform, whose residues end up in X, in NR register rounds each
+// way (the middle one fused as in the row pass).  Returns synchronised.
+template <int LR, bool ZT, int NR, int T>
+__device__ __forceinline__ void block_transform(const FusedArgs &a, const uint32_t *ga,
+                                                const uint32_t *gb, int p, uint32_t *X)
+{
+    constexpr int N = 1 << LR;
+    const uint32_t q = c_q[0][p], qinv = c_qinv[0][p];
+    const TwRef T0{tw_table(a.tw, 0, p, 0), p};
+    const TwRef Ti{tw_table(a.tw, 0, p, 1), p};
+    const uint2 sc = a.scale.c[p];
+    // operand b (when there is one) takes the normalisation in advance
+    const RawIn<ZT> ri{ga,
+                       gb ? gb : ga,
+                       a.a_len,
+                       gb ? a.b_len : a.a_len,
+                       a.a_al != 0,
+                       gb ? a.b_al != 0 : a.a_al != 0,
+                       q,
+                       a.ca.c[p],
+                       gb ? a.cb.c[p] : a.ca.c[p]};
+    const SmemIO<LR, 2, false> xy{X};
+    round_io<LR, 2, dif_base(LR, 0, NR), round_size(LR, 0, NR), true, 1, false, 0, T>(ri, xy, T0,
+                                                                                      q);
+    __syncthreads();
+    const SmemIO<LR, 1, false> zs{X};
+    if constexpr (NR == 1) {
+        // up to 16 points: elementwise in the swizzled space (X and Y share
+        // the permutation), then back
+        for (int i = threadIdx.x; i < N; i += T)
+            X[i] = gb ? mul_mont<0>(X[i], X[N + i], q, qinv) : pmul<0>(X[i], X[N + i], sc, q, qinv);
+        __syncthreads();
+        round_io<LR, 1, 0, LR, false, 1, false, 0, T>(zs, zs, Ti, q);
+        __syncthreads();
+    } else {
+        if constexpr (NR >= 3) {
+            round_io<LR, 2, dif_base(LR, 1, NR), round_size(LR, 1, NR), true, 1, false, 0, T>(
+                xy, xy, T0, q);
+            __syncthreads();
+        }
+        if constexpr (NR >= 4) {
+            round_io<LR, 2, dif_base(LR, 2, NR), round_size(LR, 2, NR), true, 1, false, 0, T>(
+                xy, xy, T0, q);
+            __syncthreads();
+        }
+        // The last forward round of both operands, the pointwise product and
+        // the first inverse round share one register round (their stage bits
+        // coincide), as in the row pass.
+        constexpr int EL = round_size(LR, NR - 1, NR);
+        static_assert(EL == dit_size(LR, 0, NR), "mirrored rounds");
+        const SmemIO<LR, 1, false> pair{X};  // NA = 2: X and Y = X + N
+#pragma unroll 1
+        for (int g = threadIdx.x; g < (N >> EL); g += T) {
+            const int base = g << EL;
+            uint32_t x[2][1 << EL];
+            pair.template load<EL, 0, 2>(x, base, 0);
+            dif_stages<EL, 0, 2, 0>(x, 0, T0, q);
+            uint32_t zz[1][1 << EL];
+#pragma unroll
+            for (int j = 0; j < (1 << EL); j++)
+                zz[0][j] = gb ? mul_mont<0>(x[0][j], x[1][j], q, qinv)
+                              : pmul<0>(x[0][j], x[1][j], sc, q, qinv);
+            dit_stages<EL, 0, 1, 0>(zz, 0, Ti, q);
+            zs.template store<EL, 0, 1>(zz, base, 0);
+        }
+        __syncthreads();
+        round_io<LR, 1, dit_base(LR, 1, NR), dit_size(LR, 1, NR), false, 1, false, 0, T>(zs, zs, Ti,
+                                                                                         q);
+        __syncthreads();
+        if constexpr (NR >= 3) {
+            round_io<LR, 1, dit_base(LR, 2, NR), dit_size(LR, 2, NR), false, 1, false, 0, T>(
+                zs, zs, Ti, q);
+            __syncthreads();
+        }
+        if constexpr (NR >= 4) {
+            round_io<LR, 1, dit_base(LR, 3, NR), dit_size(LR, 3, NR), false, 1, false, 0, T>(
+                zs, zs, Ti, q);
+            __syncthreads();
+        }
+    }
+}
+
+// The carries of one product's 2^(LR+1) limbs and its output, from the
+// coefficients' words in shared memory (SmemRun's layout), by T threads.
+template <int LR, int T>
+__device__ __forceinline__ void block_limbs(const FusedArgs &a, size_t k, const uint32_t *words,
+                                            uint32_t *wsm)
+{
+    constexpr int N = 1 << LR;
+    constexpr int LPT = 2 * N / T > kLimbsPerThread ? 2 * N / T : kLimbsPerThread;
+    const Sink &o = a.sink;
+    uint32_t map;
+    tile_carry<-1, -1, LPT>(SmemRun<N>{words, (int)threadIdx.x * (LPT / 2)}, 2 * N,
+                            o.out + sink_node(o, k) * o.out_tstride, (long)o.out_len, o.dec,
+                            o.add ? o.add + k * o.add_tstride : nullptr, (long)o.add_len, wsm,
+                            &map);
+}
+
+// One product per block: its five primes in turn, then remaindering and
 // carries over one tile.
 // Layout (words): six arrays of N = 2^LR; prime p's transforms use arrays p
 // (operand a, then the product, whose residues stay there) and p + 1 (operand
@@ -773,86 +873,68 @@ __global__ void __launch_bounds__(fused_threads(LR), 1024 / fused_threads(LR))
     const size_t k = blockIdx.x;
     const uint32_t *ga = a.A + k * a.a_tstride;
     const uint32_t *gb = a.B ? a.B + k * a.b_tstride : nullptr;
-    constexpr int NR = rounds_of(LR);
 #pragma unroll 1
-    for (int p = 0; p < kNumPrimes; p++) {
-        const uint32_t q = c_q[0][p], qinv = c_qinv[0][p];
-        const TwRef T0{tw_table(a.tw, 0, p, 0), p};
-        const TwRef Ti{tw_table(a.tw, 0, p, 1), p};
-        const uint2 sc = a.scale.c[p];
-        uint32_t *X = sm + p * N;
-        // operand b (when there is one) takes the normalisation in advance
-        const RawIn<ZT> ri{ga,     gb ? gb : ga,           a.a_len,
-                           gb ? a.b_len : a.a_len, a.a_al != 0, gb ? a.b_al != 0 : a.a_al != 0, q,
-                           a.ca.c[p], gb ? a.cb.c[p] : a.ca.c[p]};
-        const SmemIO<LR, 2, false> xy{X};
-        round_io<LR, 2, dif_base(LR, 0), round_size(LR, 0), true, 1, false, 0, T>(ri, xy, T0, q);
-        __syncthreads();
-        const SmemIO<LR, 1, false> zs{X};
-        if constexpr (NR == 1) {
-            // up to 16 points: elementwise in the swizzled space (X and Y share
-            // the permutation), then back
-            for (int i = threadIdx.x; i < N; i += T)
-                X[i] = gb ? mul_mont<0>(X[i], X[N + i], q, qinv)
-                          : pmul<0>(X[i], X[N + i], sc, q, qinv);
-            __syncthreads();
-            round_io<LR, 1, 0, LR, false, 1, false, 0, T>(zs, zs, Ti, q);
-            __syncthreads();
-        } else {
-            if constexpr (NR == 3) {
-                round_io<LR, 2, dif_base(LR, 1), round_size(LR, 1), true, 1, false, 0, T>(xy, xy,
-                                                                                         T0, q);
-                __syncthreads();
-            }
-            // The last forward round of both operands, the pointwise product and
-            // the first inverse round share one register round (their stage bits
-            // coincide), as in the row pass.
-            constexpr int EL = round_size(LR, NR - 1);
-            static_assert(EL == dit_size(LR, 0), "mirrored rounds");
-            const SmemIO<LR, 1, false> pair{X};  // NA = 2: X and Y = X + N
-#pragma unroll 1
-            for (int g = threadIdx.x; g < (N >> EL); g += T) {
-                const int base = g << EL;
-                uint32_t x[2][1 << EL];
-                pair.template load<EL, 0, 2>(x, base, 0);
-                dif_stages<EL, 0, 2, 0>(x, 0, T0, q);
-                uint32_t zz[1][1 << EL];
-#pragma unroll
-                for (int j = 0; j < (1 << EL); j++)
-                    zz[0][j] = gb ? mul_mont<0>(x[0][j], x[1][j], q, qinv)
-                                  : pmul<0>(x[0][j], x[1][j], sc, q, qinv);
-                dit_stages<EL, 0, 1, 0>(zz, 0, Ti, q);
-                zs.template store<EL, 0, 1>(zz, base, 0);
-            }
-            __syncthreads();
-            round_io<LR, 1, dit_base(LR, 1), dit_size(LR, 1), false, 1, false, 0, T>(zs, zs, Ti, q);
-            __syncthreads();
-            if constexpr (NR == 3) {
-                round_io<LR, 1, dit_base(LR, 2), dit_size(LR, 2), false, 1, false, 0, T>(zs, zs, Ti,
-                                                                                        q);
-                __syncthreads();
-            }
-        }
-    }
+    for (int p = 0; p < kNumPrimes; p++)
+        block_transform<LR, ZT, rounds_of(LR), T>(a, ga, gb, p, sm + p * N);
     // the coefficients' words in place of their residues
-    const Sink &o = a.sink;
     for (int j = threadIdx.x; j < N; j += T) {
         uint32_t *x = sm + swz(j);
         uint32_t r[kNumPrimes], w[5];
 #pragma unroll
         for (int p = 0; p < kNumPrimes; p++) r[p] = x[p * N];
-        if (o.dec) crt5_dec<0>(r, w);
+        if (a.sink.dec) crt5_dec<0>(r, w);
         else crt5<0>(r, w);
 #pragma unroll
         for (int p = 0; p < 5; p++) x[p * N] = w[p];
     }
     __syncthreads();
-    constexpr int LPT = 2 * N / T > kLimbsPerThread ? 2 * N / T : kLimbsPerThread;
-    uint32_t map;
-    tile_carry<-1, -1, LPT>(SmemRun<N>{sm, (int)threadIdx.x * (LPT / 2)}, 2 * N,
-                            o.out + sink_node(o, k) * o.out_tstride, (long)o.out_len, o.dec,
-                            o.add ? o.add + k * o.add_tstride : nullptr, (long)o.add_len, wsm,
-                            &map);
+    block_limbs<LR, T>(a, k, sm, wsm);
+}
+
+// The same for few products at a time: a cluster of five blocks per product,
+// one prime each, so that a product's primes run side by side instead of in
+// turn, in blocks of twice the threads with rounds of at most three stages
+// (a shorter serial chain per thread).  Every block then remainders a fifth
+// of the coefficients from all five blocks' residues (distributed shared
+// memory) into the first block's shared memory, which carries and writes out.
+// The cluster barriers are the hardware's; the blocks of a cluster always run
+// together.
+constexpr int kClusterMinLog = 5;  // shorter products: the schoolbook sizes
+__host__ __device__ constexpr int cluster_threads(int lr)
+{
+    const int t = (1 << lr) / 4;
+    return t < 32 ? 32 : t;
+}
+
+template <int LR, bool ZT>
+__global__ void __cluster_dims__(kNumPrimes, 1, 1) __launch_bounds__(cluster_threads(LR))
+    ntt_mul_cluster(FusedArgs a)
+{
+    namespace cg = cooperative_groups;
+    extern __shared__ uint32_t sm[];
+    __shared__ uint32_t wsm[32];
+    constexpr int N = 1 << LR;
+    constexpr int T = cluster_threads(LR);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int p = blockIdx.x % kNumPrimes;  // the block's rank in its cluster
+    const size_t k = blockIdx.x / kNumPrimes;
+    const uint32_t *ga = a.A + k * a.a_tstride;
+    const uint32_t *gb = a.B ? a.B + k * a.b_tstride : nullptr;
+    block_transform<LR, ZT, (LR + 2) / 3, T>(a, ga, gb, p, sm);
+    cluster.sync();
+    uint32_t *words = sm + 2 * N;
+    uint32_t *out = cluster.map_shared_rank(words, 0);
+    for (int j = p * T + (int)threadIdx.x; j < N; j += kNumPrimes * T) {
+        uint32_t r[kNumPrimes], w[5];
+#pragma unroll
+        for (int i = 0; i < kNumPrimes; i++) r[i] = cluster.map_shared_rank(sm, i)[swz(j)];
+        if (a.sink.dec) crt5_dec<0>(r, w);
+        else crt5<0>(r, w);
+#pragma unroll
+        for (int i = 0; i < 5; i++) out[i * N + swz(j)] = w[i];
+    }
+    cluster.sync();  // no block reads another's shared memory after this
+    if (p == 0) block_limbs<LR, T>(a, k, words, wsm);
 }
 
 // ------------------------------------------------------------ host side
@@ -1392,18 +1474,46 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
     carry_finish(c, m.maps, nprod, tiles, sink, s);
 }
 
-template <int LR>
-static void launch_fused(unsigned grid, cudaStream_t s, const FusedArgs &a)
+template <int LR, bool ZT>
+static void launch_fused_t(size_t nprod, bool spread, cudaStream_t s, const FusedArgs &a)
 {
-    const size_t smem = 6 * ((size_t)1 << LR) * sizeof(uint32_t);
-    // operands of at most half the transform (every tree level)
-    if (std::max(a.a_len, a.B ? a.b_len : 0u) <= (1u << LR)) {
-        set_smem(ntt_mul_fused<LR, true>, smem);
-        ntt_mul_fused<LR, true><<<grid, fused_threads(LR), smem, s>>>(a);
-    } else {
-        set_smem(ntt_mul_fused<LR, false>, smem);
-        ntt_mul_fused<LR, false><<<grid, fused_threads(LR), smem, s>>>(a);
+    if constexpr (LR >= kClusterMinLog) {
+        if (spread) {
+            const size_t smem = 7 * ((size_t)1 << LR) * sizeof(uint32_t);
+            set_smem(ntt_mul_cluster<LR, ZT>, smem);
+            ntt_mul_cluster<LR, ZT>
+                <<<(unsigned)(nprod * kNumPrimes), cluster_threads(LR), smem, s>>>(a);
+            return;
+        }
     }
+    const size_t smem = 6 * ((size_t)1 << LR) * sizeof(uint32_t);
+    set_smem(ntt_mul_fused<LR, ZT>, smem);
+    ntt_mul_fused<LR, ZT><<<(unsigned)nprod, fused_threads(LR), smem, s>>>(a);
+}
+
+// Whether a batch of one-block products takes a cluster of five blocks per
+// product: while the clusters' threads fit the chip at once, at most 256
+// products.  Measured (us per launch, one block : cluster): one product of
+// 2^10 points 20.7 : 8.6, of 2^8 21.0 : 8.3, of 2^5 10.2 : 6.4; 256 products of
+// 2^10 points 25.0 : 22.8 and 512 37.3 : 37.5; of 2^11 points 64 products
+// 27.0 : 20.7, 128 27.1 : 27.1, 256 35.8 : 44.5; of 2^5 points 256 products
+// 10.4 : 8.6, 512 10.4 : 12.5.
+static bool spread_primes(size_t nprod, int lr, int num_sms)
+{
+    if (nprod == 1) return true;
+    return nprod <= 256 &&
+           nprod * kNumPrimes * (size_t)cluster_threads(lr) <= (size_t)num_sms * 2048;
+}
+
+template <int LR>
+static void launch_fused(size_t nprod, int num_sms, cudaStream_t s, const FusedArgs &a)
+{
+    const bool spread = spread_primes(nprod, LR, num_sms);
+    // operands of at most half the transform (every tree level)
+    if (std::max(a.a_len, a.B ? a.b_len : 0u) <= (1u << LR))
+        launch_fused_t<LR, true>(nprod, spread, s, a);
+    else
+        launch_fused_t<LR, false>(nprod, spread, s, a);
 }
 
 static void ntt_mul_small(Ctx &c, int np, size_t nprod, Operand x, Operand y, bool square,
@@ -1423,20 +1533,19 @@ static void ntt_mul_small(Ctx &c, int np, size_t nprod, Operand x, Operand y, bo
     a.scale = make_scale(0, np);
     a.ca = make_coef(0, sink.dec);
     a.cb = make_coef_scaled(0, np, sink.dec);
-    const unsigned grid = (unsigned)nprod;
     const int tok = prof_begin(c, "ntt_mul_fused", s);
     switch (np) {
-    case 1: launch_fused<1>(grid, s, a); break;
-    case 2: launch_fused<2>(grid, s, a); break;
-    case 3: launch_fused<3>(grid, s, a); break;
-    case 4: launch_fused<4>(grid, s, a); break;
-    case 5: launch_fused<5>(grid, s, a); break;
-    case 6: launch_fused<6>(grid, s, a); break;
-    case 7: launch_fused<7>(grid, s, a); break;
-    case 8: launch_fused<8>(grid, s, a); break;
-    case 9: launch_fused<9>(grid, s, a); break;
-    case 10: launch_fused<10>(grid, s, a); break;
-    case 11: launch_fused<11>(grid, s, a); break;
+    case 1: launch_fused<1>(nprod, c.num_sms, s, a); break;
+    case 2: launch_fused<2>(nprod, c.num_sms, s, a); break;
+    case 3: launch_fused<3>(nprod, c.num_sms, s, a); break;
+    case 4: launch_fused<4>(nprod, c.num_sms, s, a); break;
+    case 5: launch_fused<5>(nprod, c.num_sms, s, a); break;
+    case 6: launch_fused<6>(nprod, c.num_sms, s, a); break;
+    case 7: launch_fused<7>(nprod, c.num_sms, s, a); break;
+    case 8: launch_fused<8>(nprod, c.num_sms, s, a); break;
+    case 9: launch_fused<9>(nprod, c.num_sms, s, a); break;
+    case 10: launch_fused<10>(nprod, c.num_sms, s, a); break;
+    case 11: launch_fused<11>(nprod, c.num_sms, s, a); break;
     default: fail(CAT_EINVAL, "one-block transform size out of range");
     }
     CAT_LAUNCH("ntt_mul_fused");

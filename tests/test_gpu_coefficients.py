@@ -53,3 +53,22 @@ def test_square_by_the_row_pass(ctx, cat_lib, orc, n):
     a = W.random_limbs32(n, seed=n)
     t = torch.from_numpy(a.view(np.int32)).cuda()
     assert np.array_equal(host(cat_lib.bigint_mul(ctx, t, t)), orc.mul(a, a))
+
+
+@pytest.mark.parametrize("slot", [8, 16, 64, 256, 1024, 2048])
+@pytest.mark.parametrize("nprod", [2, 121, 122, 257])
+def test_levels_on_both_sides_of_the_cluster_rule(ctx, cat_lib, orc, slot, nprod):
+    """Product trees whose level at `slot` limbs has nprod products: few go by
+    clusters of blocks, many by one block each (the rule's limits are 256
+    products, and 121 of 2,048-limb operands on 152 SMs).  The tree's levels
+    run from 8 limbs up, so every size between is covered too."""
+    count = nprod * 2 * slot - 5
+    if count > 150_000:
+        count = 150_000 + nprod
+    v = W.random_values(count, seed=slot + nprod)
+    got = host(cat_lib.product_tree(ctx, v))
+    q = orc.check_primes(seed=slot, count=1, lower=1 << 61, bits=62)[0]
+    want = 1
+    for x in v.tolist():
+        want = want * x % q
+    assert orc.limbs_mod(got, q) == want
