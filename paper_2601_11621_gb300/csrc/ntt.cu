@@ -614,40 +614,41 @@ __global__ void __launch_bounds__(kTileThreads) crt_carry_tiles(CrtArgs a)
     if (threadIdx.x == 0) a.tile_maps[blockIdx.x] = (uint8_t)map;
 }
 
-// Carry into each tile of a product (one block per product), in place of the
-// tiles' compact maps: each thread folds the maps of its stretch of
-// consecutive tiles, a block scan carries between the stretches, and each
-// thread replays its stretch, writing every tile's carry-in.
-__global__ void __launch_bounds__(1024) carry_tile_scan(uint8_t *tile_maps, size_t tiles)
+// The carries between the tiles of each product, from the tiles' compact
+// maps: block b of a product folds the maps of the tiles before its own
+// blockDim.x (each thread a stretch of b consecutive ones, then a block scan),
+// scans its own tiles' maps from there, and every thread adds its tile's
+// carry-in to the tile's first limbs (rarely more than one), in base 2^32 or
+// (dec) 10^9.  One launch for any length: the refolded maps are at most 64 KB
+// per block (64 blocks at 2^27 limbs) and stay in L2.  Before, one block per
+// product scanned all its tiles and a second launch fixed them: 31 + 6 us at
+// 2^26 limbs and 6 + 6 us for short products.
+__global__ void __launch_bounds__(1024) carry_resolve(const uint8_t *maps, size_t tiles, int nb,
+                                                      uint32_t *out, size_t out_tstride,
+                                                      size_t out_len, bool dec,
+                                                      const uint32_t *out_index)
 {
     __shared__ uint32_t wsm[32];
-    uint8_t *m = tile_maps + blockIdx.x * tiles;
-    const size_t per = (tiles + blockDim.x - 1) / blockDim.x;
-    const size_t i0 = threadIdx.x * per, i1 = std::min(tiles, i0 + per);
-    uint32_t f = kUnitId;
-    for (size_t i = i0; i < i1; i++) f = unit_compose(m[i], f);
-    uint32_t total;
-    uint32_t c = block_carry_scan(f, wsm, &total);
-    for (size_t i = i0; i < i1; i++) {
-        const uint32_t g = m[i];
-        m[i] = (uint8_t)c;  // now the tile's carry-in
-        c = unit_eval(g, c);
+    const size_t k = blockIdx.x / nb, b = blockIdx.x % nb;
+    const uint8_t *m = maps + k * tiles;
+    uint32_t c0 = 0, total;
+    if (b) {
+        const uint8_t *st = m + (size_t)threadIdx.x * b;
+        uint32_t f = kUnitId;
+        for (size_t i = 0; i < b; i++) f = unit_compose(st[i], f);
+        block_carry_scan(f, wsm, &total);
+        c0 = unit_eval(total, 0u);
+        __syncthreads();
     }
-}
-
-// Add each tile's carry-in to its first limbs (rarely more than one), in
-// base 2^32 or (dec) 10^9.
-__global__ void carry_fix(const uint8_t *tile_cin, size_t tiles_total, size_t tiles,
-                          uint32_t *out, size_t out_tstride, size_t out_len, bool dec,
-                          const uint32_t *out_index = nullptr)
-{
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= tiles_total) return;
-    uint32_t c = tile_cin[t];
-    if (!c) return;
-    const size_t k = t / tiles, tt = t % tiles;
+    const size_t t = b * blockDim.x + threadIdx.x;
+    uint32_t f = t < tiles ? m[t] : kUnitId;
+    // the block's first tile takes c0: its map becomes the constant f(c0)
+    if (threadIdx.x == 0) f = (unit_eval(f, c0) << 4) | 4u;
+    uint32_t c = block_carry_scan(f, wsm, &total);
+    if (threadIdx.x == 0) c = c0;
+    if (!c || t >= tiles) return;
     uint32_t *o = out + (out_index ? (size_t)out_index[k] : k) * out_tstride;
-    size_t j = tt * kTile;
+    size_t j = t * kTile;
     const size_t end = std::min(j + kTile, out_len);
     for (; c && j < end; j++) {
         const uint64_t v = (uint64_t)o[j] + c;
@@ -1000,8 +1001,8 @@ static void launch_col(bool fwd, dim3 grid, cudaStream_t s, const ColArgs &a)
 {
     const size_t smem = ((size_t)1 << (LR + col_log_c(LR))) * sizeof(uint32_t);
     // the first pass of operands of at most half the transform (every tree
-    // level) knows its upper half is zero
-    const bool zt = fwd && a.src && a.src_len <= ((size_t)1 << a.m);  // limbs: two per point
+    // level; lengths count limbs, two per point) knows its upper half is zero
+    const bool zt = fwd && a.src && std::max(a.src_len, a.src_y_len) <= ((size_t)1 << a.m);
     if (zt) {
         set_smem(ntt_col_fwd<LR, PS, kColV, 2>, smem);
         ntt_col_fwd<LR, PS, kColV, 2><<<grid, kColFwdThreads, smem, s>>>(a);
@@ -1083,17 +1084,40 @@ void drop_col_twiddles(Ctx &c)
     c.col_tw.clear();
 }
 
+// One operand source of a batched product.
+struct Operand {
+    const uint32_t *p;
+    size_t tstride;  // limbs between consecutive transforms (for batches)
+    size_t len;      // valid limbs per transform
+};
+constexpr Operand kNoSource{nullptr, 0, 0};
+
+// One column pass over `total` points (blocks of 2^m points, 2^r rows).
+//
 // scaled (first forward passes): 1 = every transform of the call is an
 // operand b, 2 = the odd ones are (adjacent pairs); their twiddles then carry
 // the pointwise step's normalisation.  Returns whether they did (the scaled
 // table exists), i.e. whether the row pass must skip the normalisation.
+//
+// x: the sources of a first forward pass (p null otherwise); y, when given,
+// the source of the call's last transform (the second operand of a product or
+// the common one of broadcast products), so that both operands of a single
+// product share one launch.
 static bool col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, size_t total,
-                     int m, int r, const uint32_t *src, size_t src_tstride, size_t src_len,
-                     bool dec, cudaStream_t s, int scaled = 0)
+                     int m, int r, const Operand &x, const Operand *y, bool dec, cudaStream_t s,
+                     int scaled = 0)
 {
+    const uint32_t *src = x.p;
+    auto aligned16 = [](const Operand &o) {
+        return (reinterpret_cast<uintptr_t>(o.p) & 15) == 0 && (o.tstride & 3) == 0;
+    };
     ColArgs a;
     a.coef = make_coef(ps, dec);
-    a.src_al = (reinterpret_cast<uintptr_t>(src) & 15) == 0 && (src_tstride & 3) == 0;
+    a.src_al = aligned16(x);
+    a.last = y ? (total >> m) - 1 : ~(size_t)0;
+    a.src_y = y ? y->p : nullptr;
+    a.src_y_len = y ? y->len : 0;
+    a.src_y_al = y && aligned16(*y);
     a.twtab_odd = nullptr;
     // (measured per C(2,050,572,903): tables in every pass beat computed
     // twiddles at every block size, the first forward passes' large tables
@@ -1113,15 +1137,18 @@ static bool col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, s
     a.pstride = pstride;
     a.m = m;
     a.src = src;
-    a.src_tstride = src_tstride;
-    a.src_len = src_len;
+    a.src_tstride = x.tstride;
+    a.src_len = x.len;
     a.tw = c.twiddles;
     const size_t ctas = total >> (r + col_log_c(r));
     dim3 grid((unsigned)ctas, kNumPrimes);
     // algorithmic bytes: every point of the five prime arrays read and
     // written once (the first forward pass reads limbs instead)
     double bytes = 8.0 * kNumPrimes * (double)total;
-    if (src) bytes = 4.0 * kNumPrimes * (double)total + 4.0 * (double)src_len * (double)(total >> m);
+    if (src)
+        bytes = 4.0 * kNumPrimes * (double)total +
+                4.0 * (double)x.len * (double)((total >> m) - (y ? 1 : 0)) +
+                (y ? 4.0 * (double)y->len : 0.0);
     const int tok = prof_begin(c, fwd ? (src ? "ntt_col_fwd_first" : "ntt_col_fwd") : "ntt_col_inv", s);
     if (ps == 0) {
         switch (r) {
@@ -1309,13 +1336,6 @@ static void launch_row_limbs(size_t nprod, bool square, cudaStream_t s, const Ro
     CAT_LAUNCH("ntt_row_limbs");
 }
 
-// One operand source of a batched product.
-struct Operand {
-    const uint32_t *p;
-    size_t tstride;  // limbs between consecutive transforms (for batches)
-    size_t len;      // valid limbs per transform
-};
-
 // Scratch of one batch of multi-pass products: from the context's pool, or
 // the fixed arrays of the no-allocation multiply.
 struct MulScratch {
@@ -1327,21 +1347,17 @@ struct MulScratch {
 };
 
 // The carries of nprod products of `tiles` tiles each, whose compact tile
-// maps are in maps: the carry into every tile, then added to its first limbs.
-static void carry_finish(Ctx &c, uint8_t *maps, size_t nprod, size_t tiles, const Sink &sink,
+// maps are in maps.
+static void carry_finish(Ctx &c, const uint8_t *maps, size_t nprod, size_t tiles, const Sink &sink,
                          cudaStream_t s)
 {
-    int tok = prof_begin(c, "carry_tile_scan", s);
-    carry_tile_scan<<<(unsigned)nprod, 1024, 0, s>>>(maps, tiles);
-    CAT_LAUNCH("carry_tile_scan");
-    prof_end(c, tok, s, 2.0 * (double)(nprod * tiles));
-    const size_t tt = nprod * tiles;
-    tok = prof_begin(c, "carry_fix", s);
-    carry_fix<<<(unsigned)((tt + 255) / 256), 256, 0, s>>>(maps, tt, tiles, sink.out,
-                                                             sink.out_tstride, sink.out_len,
-                                                             sink.dec, sink.out_index);
-    CAT_LAUNCH("carry_fix");
-    prof_end(c, tok, s, (double)tt);
+    const int tok = prof_begin(c, "carry_resolve", s);
+    const size_t threads = std::min<size_t>(1024, (tiles + 31) / 32 * 32);
+    const size_t nb = (tiles + threads - 1) / threads;
+    carry_resolve<<<(unsigned)(nprod * nb), (unsigned)threads, 0, s>>>(
+        maps, tiles, (int)nb, sink.out, sink.out_tstride, sink.out_len, sink.dec, sink.out_index);
+    CAT_LAUNCH("carry_resolve");
+    prof_end(c, tok, s, (double)(nprod * tiles));
 }
 
 // Batched products of transforms of 2^np >= 2^12 points.
@@ -1404,19 +1420,27 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
         // forward column passes (operand b's first pass takes the pointwise
         // step's normalisation into its twiddles when it has a table)
         bool prescaled = false;
-        if (mode == PAIR_FIRST_TWO) {
-            col_pass(c, PS, true, F, fp, N, np, P.rcol[0], x.p, 0, x.len, dec, s);
-            prescaled = col_pass(c, PS, true, F + N, fp, N, np, P.rcol[0], y.p, 0, y.len, dec, s, 1);
-        } else if (mode == PAIR_BROADCAST) {
-            col_pass(c, PS, true, F, fp, nprod * N, np, P.rcol[0], x.p, x.tstride, x.len, dec, s);
-            col_pass(c, PS, true, F + nprod * N, fp, N, np, P.rcol[0], y.p, 0, y.len, dec, s);
+        const int r0 = P.rcol[0];
+        // one launch for the operands of a single or a broadcast product,
+        // unless only one of them fills its transform's upper half and the
+        // transform is long enough for the zero half to pay for a launch
+        const bool two = mode == PAIR_FIRST_TWO || mode == PAIR_BROADCAST;
+        const bool together =
+            two && (np <= 17 || (x.len <= N) == (y.len <= N));
+        if (together) {
+            prescaled = col_pass(c, PS, true, F, fp, fp, np, r0, x, &y, dec, s,
+                                 mode == PAIR_FIRST_TWO ? 2 : 0);
+        } else if (two) {
+            col_pass(c, PS, true, F, fp, fp - N, np, r0, x, nullptr, dec, s);
+            prescaled = col_pass(c, PS, true, F + fp - N, fp, N, np, r0, y, nullptr, dec, s,
+                                 mode == PAIR_FIRST_TWO ? 1 : 0);
         } else {
-            prescaled = col_pass(c, PS, true, F, fp, fp, np, P.rcol[0], x.p, x.tstride, x.len, dec,
-                                 s, mode == PAIR_ADJACENT ? 2 : 0);
+            prescaled = col_pass(c, PS, true, F, fp, fp, np, r0, x, nullptr, dec, s,
+                                 mode == PAIR_ADJACENT ? 2 : 0);
         }
-        int mm = np - P.rcol[0];
+        int mm = np - r0;
         for (int i = 1; i < P.ncol; i++) {
-            col_pass(c, PS, true, F, fp, fp, mm, P.rcol[i], nullptr, 0, 0, false, s);
+            col_pass(c, PS, true, F, fp, fp, mm, P.rcol[i], kNoSource, nullptr, false, s);
             mm -= P.rcol[i];
         }
         // fused row pass
@@ -1452,7 +1476,7 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
         for (int i = P.ncol - 1; i >= 0; i--) {
             int mi = np;
             for (int j = 0; j < i; j++) mi -= P.rcol[j];
-            col_pass(c, PS, false, m.G, gp, gp, mi, P.rcol[i], nullptr, 0, 0, false, s);
+            col_pass(c, PS, false, m.G, gp, gp, mi, P.rcol[i], kNoSource, nullptr, false, s);
         }
     }
     // remaindering and carries

@@ -280,6 +280,10 @@ struct ColArgs {
     size_t src_tstride;    // limbs between consecutive transforms' sources
     size_t src_len;        // valid limbs per transform (rest are zero)
     int src_al;            // every source starts on a 16-byte boundary
+    size_t last;           // the transform whose source is src_y (or none)
+    const uint32_t *src_y;
+    size_t src_y_len;
+    int src_y_al;
     CoefMuls coef;         // the sources' input multipliers
     const uint2 *tw;
     // the pass's inter-pass twiddles, w^(col bitrev(row)) in the multiplier
@@ -567,11 +571,16 @@ __global__ void __launch_bounds__(kColFwdThreads, CAT_COL_FWD_MINB) ntt_col_fwd(
     const uint2 *T = tw_table(a.tw, PS, p, 0);
     const TwRef TR{T, p};
     const auto in = [&] {
-        if constexpr (SRC != 0)
-            return ColSrcIn<PS, V, SRC == 2>{a.src + blk * a.src_tstride, (uint32_t)Sr,
-                                             (uint32_t)col0, (uint32_t)a.src_len, a.src_al != 0, q,
+        if constexpr (SRC != 0) {
+            const bool y = blk == a.last;
+            return ColSrcIn<PS, V, SRC == 2>{y ? a.src_y : a.src + blk * a.src_tstride,
+                                             (uint32_t)Sr,
+                                             (uint32_t)col0,
+                                             (uint32_t)(y ? a.src_y_len : a.src_len),
+                                             (y ? a.src_y_al : a.src_al) != 0,
+                                             q,
                                              a.coef.c[p]};
-        else
+        } else
             return ColIn<V>{base, (uint32_t)Sr, (uint32_t)col0};
     }();
     ColTw<LR, PS, NR, kColFwdThreads, V> tw{T, q, c_qinv[PS][p], set_log_root(PS) - a.m, {}};

@@ -72,3 +72,19 @@ def test_levels_on_both_sides_of_the_cluster_rule(ctx, cat_lib, orc, slot, nprod
     for x in v.tolist():
         want = want * x % q
     assert orc.limbs_mod(got, q) == want
+
+
+@pytest.mark.parametrize("s", [1500, 700_000, 3 << 20])
+def test_carry_through_many_tiles(ctx, cat_lib, s):
+    """a (1 + 2^(32 s)) with a = 1 and then s limbs of ones from limb s: the sum
+    at limb s overflows and its carry runs through the next s limbs, across
+    the tiles (2,048 limbs) and, at the largest, across the 1,024 tiles that
+    one block of the carry kernel resolves."""
+    a = np.zeros(2 * s, dtype=np.uint32)
+    a[0] = 1
+    a[s:] = 0xFFFFFFFF
+    b = np.zeros(s + 1, dtype=np.uint32)
+    b[0] = b[s] = 1
+    got = host(cat_lib.bigint_mul(ctx, a, b))
+    v = int.from_bytes(a.astype("<u4").tobytes(), "little")
+    assert int.from_bytes(got.astype("<u4").tobytes(), "little") == v + (v << (32 * s))
