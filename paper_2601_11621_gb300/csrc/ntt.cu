@@ -487,6 +487,7 @@ __device__ __forceinline__ void tile_carry(const SUM &sum, int tile_len, uint32_
                                            long out_count, bool dec_rt, const uint32_t *add,
                                            long add_count, uint32_t *wsm, uint32_t *tile_map)
 {
+    static_assert(LPT % 4 == 0, "limbs are stored 16 bytes at a time");
     const bool dec = DEC < 0 ? dec_rt : DEC == 1;
     if (ADD == 0) add = nullptr;
     const int j0 = threadIdx.x * LPT;
@@ -670,37 +671,38 @@ struct FusedArgs {
     const uint32_t *A;
     size_t a_tstride;
     uint32_t a_len;
-    const uint32_t *B;  // null: square A; b_tstride 0: the same B for every product
+    const uint32_t *B;  // b_tstride 0: the same B for every product
     size_t b_tstride;
     uint32_t b_len;
     int a_al, b_al;     // every operand starts on an 8-byte boundary
+    size_t nprod;
     Sink sink;
     const uint2 *tw;
-    Scale scale;
-    CoefMuls ca, cb;    // cb carries the pointwise scale (unused when squaring)
+    CoefMuls ca, cb;    // cb carries the pointwise scale
 };
 
-constexpr int kFusedMaxLog = 11;   // 2^11 points: products of 2^12 limbs
-constexpr int kFusedThreads = 256;
+constexpr int kFusedMaxLog = 11;  // 2^11 points: products of 2^12 limbs
 
-// Threads of the one-block multiply of 2^lr points: one group of 16 points of
-// each operand's transform per thread and round, at least one warp.
+// Points of all products of a one-block multiply of 2^lr points (several
+// short products share a block, at most one per thread) and its threads, one
+// group of 16 points of both operands each.
+__host__ __device__ constexpr int fused_points(int lr)
+{
+    return lr >= 9 ? 1 << lr : (lr >= 4 ? 512 : 32 << lr);
+}
 __host__ __device__ constexpr int fused_threads(int lr)
 {
-    const int t = (1 << lr) / 8;
-    return t < 32 ? 32 : (t > kFusedThreads ? kFusedThreads : t);
+    return fused_points(lr) >= 512 ? fused_points(lr) / 16 : 32;
 }
 
-// The one-block multiply's first forward round input: coefficient i of an
-// operand, words 2i and 2i + 1 of its limbs (zero past the end), from global
-// memory; column 0 is operand a, column 1 operand b (a again when squaring).
-// The five primes read the operands one after the other; the blocks' limbs
-// stay in L1 and L2 meanwhile, which leaves the shared memory to more blocks.
-// ZT: both operands fill at most the lower half.
+// The first forward round's input of product c of a block: both operands
+// (NA = 2), or, with the operands as columns, operand a (c = 0) or b (c = 1)
+// of one product.
 template <bool ZT>
 struct RawIn {
     static constexpr bool kZeroTop = ZT;
     const uint32_t *a, *b;
+    size_t sa, sb;  // limbs between consecutive products' operands
     uint32_t la, lb;
     bool al_a, al_b;
     uint32_t q;
@@ -708,198 +710,200 @@ struct RawIn {
     template <int E, int B, int NA>
     __device__ __forceinline__ void load(uint32_t (&x)[NA][1 << E], int base, int c) const
     {
-        const uint32_t *r = c ? b : a;
-        const uint32_t len = c ? lb : la;
-        const bool al = c ? al_b : al_a;
-        CoefMul m;
-        m.w0.x = c ? cb.w0.x : ca.w0.x;
-        m.w0.y = c ? cb.w0.y : ca.w0.y;
-        m.w1.x = c ? cb.w1.x : ca.w1.x;
-        m.w1.y = c ? cb.w1.y : ca.w1.y;
-        constexpr int K = ZT ? (1 << (E - 1)) : (1 << E);
-        uint32_t lo[K], hi[K];
-        if (al && 2u * (uint32_t)(base + ((K - 1) << B)) + 2u <= len) {
-#pragma unroll
-            for (int k = 0; k < K; k++) {
-                const uint2 v = *reinterpret_cast<const uint2 *>(r + 2 * (base + (k << B)));
-                lo[k] = v.x;
-                hi[k] = v.y;
-            }
+        if constexpr (NA == 2) {
+            load_coefs<E, B, ZT>(x[0], a + c * sa, base, la, al_a, ca, q);
+            load_coefs<E, B, ZT>(x[1], b + c * sb, base, lb, al_b, cb, q);
         } else {
-#pragma unroll
-            for (int k = 0; k < K; k++) {
-                const uint32_t w = 2u * (uint32_t)(base + (k << B));
-                lo[k] = w < len ? r[w] : 0u;
-                hi[k] = w + 1 < len ? r[w + 1] : 0u;
-            }
+            CoefMul m;
+            m.w0.x = c ? cb.w0.x : ca.w0.x;
+            m.w0.y = c ? cb.w0.y : ca.w0.y;
+            m.w1.x = c ? cb.w1.x : ca.w1.x;
+            m.w1.y = c ? cb.w1.y : ca.w1.y;
+            load_coefs<E, B, ZT>(x[0], c ? b : a, base, c ? lb : la, c ? al_b : al_a, m, q);
         }
-#pragma unroll
-        for (int k = 0; k < (1 << E); k++) x[0][k] = k < K ? coef_in<0>(lo[k], hi[k], m, q) : 0u;
     }
 };
 
-// Limb sums of a run of the one-block multiply, straight from the
-// coefficients' words in shared memory (word p of coefficient j at
-// s[p N + swz(j)]).
-template <int N>
+// The first product's operands k0, and prime p's input.
+template <bool ZT>
+__device__ __forceinline__ RawIn<ZT> raw_in(const FusedArgs &a, size_t k0, int p, uint32_t q)
+{
+    return RawIn<ZT>{a.A + k0 * a.a_tstride,
+                     a.B + k0 * a.b_tstride,
+                     a.a_tstride,
+                     a.b_tstride,
+                     a.a_len,
+                     a.b_len,
+                     a.a_al != 0,
+                     a.b_al != 0,
+                     q,
+                     a.ca.c[p],
+                     a.cb.c[p]};
+}
+
+// Forward rounds rd .. NR - 2 in shared memory, C columns and NA arrays.
+template <int LR, int C, int NR, int NA, int T, int RD, class IO>
+__device__ __forceinline__ void forward_rounds(const IO &io, const TwRef &T0, uint32_t q, int cols)
+{
+    if constexpr (RD < NR - 1) {
+        round_io<LR, C, dif_base(LR, RD, NR), round_size(LR, RD, NR), true, NA, false, 0, T>(
+            io, io, T0, q, cols);
+        __syncthreads();
+        forward_rounds<LR, C, NR, NA, T, RD + 1>(io, T0, q, cols);
+    }
+}
+
+// Inverse rounds rd .. NR - 1.
+template <int LR, int C, int NR, int T, int RD, class IO>
+__device__ __forceinline__ void inverse_rounds(const IO &io, const TwRef &Ti, uint32_t q, int cols)
+{
+    if constexpr (RD < NR) {
+        round_io<LR, C, dit_base(LR, RD, NR), dit_size(LR, RD, NR), false, 1, false, 0, T>(
+            io, io, Ti, q, cols);
+        __syncthreads();
+        inverse_rounds<LR, C, NR, T, RD + 1>(io, Ti, q, cols);
+    }
+}
+
+// The last forward round of both operands (arrays io and io + C 2^LR), the
+// pointwise product and the first inverse round share one register round
+// (their stage bits coincide), as in the row pass; the product replaces
+// operand a.
+template <int LR, int C, int NR, int T, class IO>
+__device__ __forceinline__ void middle_round(const IO &io, const TwRef &T0, const TwRef &Ti,
+                                             uint32_t q, uint32_t qinv, int cols)
+{
+    constexpr int EL = round_size(LR, NR - 1, NR);
+    static_assert(EL == dit_size(LR, 0, NR), "mirrored rounds");
+    constexpr int NGC = (1 << LR) >> EL;
+#pragma unroll 1
+    for (int g = threadIdx.x; g < cols * NGC; g += T) {
+        const int c = g / NGC, base = (g & (NGC - 1)) << EL;
+        uint32_t x[2][1 << EL];
+        io.template load<EL, 0, 2>(x, base, c);
+        dif_stages<EL, 0, 2, 0>(x, 0, T0, q);
+        uint32_t z[1][1 << EL];
+#pragma unroll
+        for (int j = 0; j < (1 << EL); j++) z[0][j] = mul_mont<0>(x[0][j], x[1][j], q, qinv);
+        dit_stages<EL, 0, 1, 0>(z, 0, Ti, q);
+        io.template store<EL, 0, 1>(z, base, c);
+    }
+    __syncthreads();
+}
+
+// The limbs of a block's products from their coefficients' words in shared
+// memory: word p of coefficient j at s[p PN + swz(j)], products of N = 2^LR
+// coefficients back to back, a run of LPT limbs per thread, first limb j0.
+template <int N, int PN>
 struct SmemRun {
     const uint32_t *s;
     int j0;  // first coefficient
-    __device__ __forceinline__ uint32_t word(int p, int j) const
+    __device__ __forceinline__ uint32_t word(int p, int j, int back) const
     {
-        return j >= 0 ? s[p * N + swz(j)] : 0u;
+        // coefficient j - back of the same product, or none
+        return (j & (N - 1)) >= back ? s[p * PN + swz(j - back)] : 0u;
     }
     __device__ __forceinline__ uint64_t operator()(int i) const
     {
         const int j = j0 + (i >> 1);
-        if (i & 1) return (uint64_t)word(1, j) + word(3, j - 1);
-        return (uint64_t)word(0, j) + word(2, j - 1) + word(4, j - 2);
+        if (i & 1) return (uint64_t)word(1, j, 0) + word(3, j, 1);
+        return (uint64_t)word(0, j, 0) + word(2, j, 1) + word(4, j, 2);
     }
 };
 
-// One prime of a product inside a block of T threads: the forward transforms
-// of both operands into X and X + N (N = 2^LR), the pointwise product and the
-// inverse transform, whose residues end up in X, in NR register rounds each
-// way (the middle one fused as in the row pass).  Returns synchronised.
-template <int LR, bool ZT, int NR, int T>
-__device__ __forceinline__ void block_transform(const FusedArgs &a, const uint32_t *ga,
-                                                const uint32_t *gb, int p, uint32_t *X)
+// The carries and the output of a block's products k0 .. k0 + cols - 1.
+template <int LPT, int N, int PN>
+__device__ __forceinline__ void block_limbs(const FusedArgs &a, size_t k0, int cols,
+                                            const uint32_t *words, uint32_t *wsm)
 {
-    constexpr int N = 1 << LR;
-    const uint32_t q = c_q[0][p], qinv = c_qinv[0][p];
-    const TwRef T0{tw_table(a.tw, 0, p, 0), p};
-    const TwRef Ti{tw_table(a.tw, 0, p, 1), p};
-    const uint2 sc = a.scale.c[p];
-    // operand b (when there is one) takes the normalisation in advance
-    const RawIn<ZT> ri{ga,
-                       gb ? gb : ga,
-                       a.a_len,
-                       gb ? a.b_len : a.a_len,
-                       a.a_al != 0,
-                       gb ? a.b_al != 0 : a.a_al != 0,
-                       q,
-                       a.ca.c[p],
-                       gb ? a.cb.c[p] : a.ca.c[p]};
-    const SmemIO<LR, 2, false> xy{X};
-    round_io<LR, 2, dif_base(LR, 0, NR), round_size(LR, 0, NR), true, 1, false, 0, T>(ri, xy, T0,
-                                                                                      q);
-    __syncthreads();
-    const SmemIO<LR, 1, false> zs{X};
-    if constexpr (NR == 1) {
-        // up to 16 points: elementwise in the swizzled space (X and Y share
-        // the permutation), then back
-        for (int i = threadIdx.x; i < N; i += T)
-            X[i] = gb ? mul_mont<0>(X[i], X[N + i], q, qinv) : pmul<0>(X[i], X[N + i], sc, q, qinv);
-        __syncthreads();
-        round_io<LR, 1, 0, LR, false, 1, false, 0, T>(zs, zs, Ti, q);
-        __syncthreads();
-    } else {
-        if constexpr (NR >= 3) {
-            round_io<LR, 2, dif_base(LR, 1, NR), round_size(LR, 1, NR), true, 1, false, 0, T>(
-                xy, xy, T0, q);
-            __syncthreads();
-        }
-        if constexpr (NR >= 4) {
-            round_io<LR, 2, dif_base(LR, 2, NR), round_size(LR, 2, NR), true, 1, false, 0, T>(
-                xy, xy, T0, q);
-            __syncthreads();
-        }
-        // The last forward round of both operands, the pointwise product and
-        // the first inverse round share one register round (their stage bits
-        // coincide), as in the row pass.
-        constexpr int EL = round_size(LR, NR - 1, NR);
-        static_assert(EL == dit_size(LR, 0, NR), "mirrored rounds");
-        const SmemIO<LR, 1, false> pair{X};  // NA = 2: X and Y = X + N
-#pragma unroll 1
-        for (int g = threadIdx.x; g < (N >> EL); g += T) {
-            const int base = g << EL;
-            uint32_t x[2][1 << EL];
-            pair.template load<EL, 0, 2>(x, base, 0);
-            dif_stages<EL, 0, 2, 0>(x, 0, T0, q);
-            uint32_t zz[1][1 << EL];
-#pragma unroll
-            for (int j = 0; j < (1 << EL); j++)
-                zz[0][j] = gb ? mul_mont<0>(x[0][j], x[1][j], q, qinv)
-                              : pmul<0>(x[0][j], x[1][j], sc, q, qinv);
-            dit_stages<EL, 0, 1, 0>(zz, 0, Ti, q);
-            zs.template store<EL, 0, 1>(zz, base, 0);
-        }
-        __syncthreads();
-        round_io<LR, 1, dit_base(LR, 1, NR), dit_size(LR, 1, NR), false, 1, false, 0, T>(zs, zs, Ti,
-                                                                                         q);
-        __syncthreads();
-        if constexpr (NR >= 3) {
-            round_io<LR, 1, dit_base(LR, 2, NR), dit_size(LR, 2, NR), false, 1, false, 0, T>(
-                zs, zs, Ti, q);
-            __syncthreads();
-        }
-        if constexpr (NR >= 4) {
-            round_io<LR, 1, dit_base(LR, 3, NR), dit_size(LR, 3, NR), false, 1, false, 0, T>(
-                zs, zs, Ti, q);
-            __syncthreads();
-        }
-    }
-}
-
-// The carries of one product's 2^(LR+1) limbs and its output, from the
-// coefficients' words in shared memory (SmemRun's layout), by T threads.
-template <int LR, int T>
-__device__ __forceinline__ void block_limbs(const FusedArgs &a, size_t k, const uint32_t *words,
-                                            uint32_t *wsm)
-{
-    constexpr int N = 1 << LR;
-    constexpr int LPT = 2 * N / T > kLimbsPerThread ? 2 * N / T : kLimbsPerThread;
     const Sink &o = a.sink;
+    const int j0 = threadIdx.x * LPT;     // first limb of the run
+    const int c = j0 / (2 * N);           // its product
+    const size_t k = k0 + c;
+    static_assert(2 * N % LPT == 0, "a run lies within one product");
+    const bool live = c < cols;
+    // the product's limbs start at limb `base` of the tile
+    const long base = (long)c * 2 * N;
+    uint32_t *out = live ? o.out + sink_node(o, k) * o.out_tstride - base : nullptr;
+    const uint32_t *add = live && o.add ? o.add + k * o.add_tstride - base : nullptr;
     uint32_t map;
-    tile_carry<-1, -1, LPT>(SmemRun<N>{words, (int)threadIdx.x * (LPT / 2)}, 2 * N,
-                            o.out + sink_node(o, k) * o.out_tstride, (long)o.out_len, o.dec,
-                            o.add ? o.add + k * o.add_tstride : nullptr, (long)o.add_len, wsm,
-                            &map);
+    tile_carry<-1, -1, LPT>(SmemRun<N, PN>{words, j0 / 2}, cols * 2 * N, out,
+                            base + (long)o.out_len, o.dec, add, base + (long)o.add_len, wsm, &map);
 }
 
-// One product per block: its five primes in turn, then remaindering and
-// carries over one tile.
-// Layout (words): six arrays of N = 2^LR; prime p's transforms use arrays p
-// (operand a, then the product, whose residues stay there) and p + 1 (operand
-// b; the next prime overwrites it): 24 N bytes, four blocks of 2^11 points per
-// SM.  The coefficients' words then replace the residues in place.
+// Whole products in one block: the five primes in turn (per prime both
+// forward transforms, the pointwise product and the inverse transform in
+// shared memory), then remaindering and carries.
+// A block holds one product of 2^10 or 2^11 points or as many shorter ones as
+// fill 2^9, one group of 16 points of both operands per thread: every thread
+// has a group in every round of four stages, both operands share the stage
+// twiddles, and up to 2^9 points the block is a single warp, whose barriers
+// cost next to nothing.  Sixteen warps per SM at up to 128 registers do
+// better here than 32 warps with half of them idle between the barriers of
+// the middle and inverse rounds: the levels of 2^8 .. 2^11 points of
+// C(2,050,572,903) 11.4 -> 10.5 ms (2^24 limbs of products take 260 us at 2^7
+// points, 285, 335, 354 and 365 at 2^11).
+// Layout (words): six arrays of PN; prime p's transforms use arrays p
+// (operands a, then the products, whose residues stay there) and p + 1
+// (operands b; the next prime overwrites them): 24 PN bytes, four blocks of
+// 2^11 points per SM.  The coefficients' words then replace the residues in
+// place.  The products' limbs form one tile: no carry leaves a product, so the
+// scan needs no boundaries between them.
 template <int LR, bool ZT>
-__global__ void __launch_bounds__(fused_threads(LR), 1024 / fused_threads(LR))
+__global__ void __launch_bounds__(fused_threads(LR), 512 / fused_threads(LR))
     ntt_mul_fused(FusedArgs a)
 {
     extern __shared__ uint32_t sm[];
     __shared__ uint32_t wsm[32];
-    constexpr int N = 1 << LR;
-    constexpr int T = fused_threads(LR);
-    const size_t k = blockIdx.x;
-    const uint32_t *ga = a.A + k * a.a_tstride;
-    const uint32_t *gb = a.B ? a.B + k * a.b_tstride : nullptr;
+    constexpr int N = 1 << LR, PN = fused_points(LR), P = PN / N;
+    constexpr int T = fused_threads(LR), NR = rounds_of(LR);
+    const size_t k0 = (size_t)blockIdx.x * P;
+    const int cols = (int)(a.nprod - k0 < (size_t)P ? a.nprod - k0 : (size_t)P);
 #pragma unroll 1
-    for (int p = 0; p < kNumPrimes; p++)
-        block_transform<LR, ZT, rounds_of(LR), T>(a, ga, gb, p, sm + p * N);
+    for (int p = 0; p < kNumPrimes; p++) {
+        const uint32_t q = c_q[0][p], qinv = c_qinv[0][p];
+        const TwRef T0{tw_table(a.tw, 0, p, 0), p};
+        const TwRef Ti{tw_table(a.tw, 0, p, 1), p};
+        const SmemIO<LR, P, false, true> io{sm + p * PN};
+        round_io<LR, P, dif_base(LR, 0, NR), round_size(LR, 0, NR), true, 2, false, 0, T>(
+            raw_in<ZT>(a, k0, p, q), io, T0, q, cols);
+        __syncthreads();
+        if constexpr (NR == 1) {
+            // up to 16 points: elementwise in the swizzled space, then back
+            for (int i = threadIdx.x; i < PN; i += T)
+                io.s[i] = mul_mont<0>(io.s[i], io.s[PN + i], q, qinv);
+            __syncthreads();
+            inverse_rounds<LR, P, NR, T, 0>(io, Ti, q, cols);
+        } else {
+            forward_rounds<LR, P, NR, 2, T, 1>(io, T0, q, cols);
+            middle_round<LR, P, NR, T>(io, T0, Ti, q, qinv, cols);
+            inverse_rounds<LR, P, NR, T, 1>(io, Ti, q, cols);
+        }
+    }
     // the coefficients' words in place of their residues
-    for (int j = threadIdx.x; j < N; j += T) {
+    for (int j = threadIdx.x; j < cols * N; j += T) {
         uint32_t *x = sm + swz(j);
         uint32_t r[kNumPrimes], w[5];
 #pragma unroll
-        for (int p = 0; p < kNumPrimes; p++) r[p] = x[p * N];
+        for (int p = 0; p < kNumPrimes; p++) r[p] = x[p * PN];
         if (a.sink.dec) crt5_dec<0>(r, w);
         else crt5<0>(r, w);
 #pragma unroll
-        for (int p = 0; p < 5; p++) x[p * N] = w[p];
+        for (int p = 0; p < 5; p++) x[p * PN] = w[p];
     }
     __syncthreads();
-    block_limbs<LR, T>(a, k, sm, wsm);
+    constexpr int LPT = 2 * PN / T;  // 32 limbs
+    block_limbs<LPT, N, PN>(a, k0, cols, sm, wsm);
 }
 
 // The same for few products at a time: a cluster of five blocks per product,
 // one prime each, so that a product's primes run side by side instead of in
-// turn, in blocks of twice the threads with rounds of at most three stages
-// (a shorter serial chain per thread).  Every block then remainders a fifth
-// of the coefficients from all five blocks' residues (distributed shared
-// memory) into the first block's shared memory, which carries and writes out.
-// The cluster barriers are the hardware's; the blocks of a cluster always run
-// together.
+// turn, the operands as two columns, in blocks of N / 4 threads with rounds of
+// at most three stages (a shorter serial chain per thread).  Every block then
+// remainders a fifth of the coefficients from all five blocks' residues
+// (distributed shared memory) into the first block's shared memory, which
+// carries and writes out.  The cluster barriers are the hardware's; the blocks
+// of a cluster always run together.
 constexpr int kClusterMinLog = 5;  // shorter products: the schoolbook sizes
 __host__ __device__ constexpr int cluster_threads(int lr)
 {
@@ -915,13 +919,21 @@ __global__ void __cluster_dims__(kNumPrimes, 1, 1) __launch_bounds__(cluster_thr
     extern __shared__ uint32_t sm[];
     __shared__ uint32_t wsm[32];
     constexpr int N = 1 << LR;
-    constexpr int T = cluster_threads(LR);
+    constexpr int T = cluster_threads(LR), NR = (LR + 2) / 3;
     cg::cluster_group cluster = cg::this_cluster();
     const int p = blockIdx.x % kNumPrimes;  // the block's rank in its cluster
     const size_t k = blockIdx.x / kNumPrimes;
-    const uint32_t *ga = a.A + k * a.a_tstride;
-    const uint32_t *gb = a.B ? a.B + k * a.b_tstride : nullptr;
-    block_transform<LR, ZT, (LR + 2) / 3, T>(a, ga, gb, p, sm);
+    const uint32_t q = c_q[0][p], qinv = c_qinv[0][p];
+    const TwRef T0{tw_table(a.tw, 0, p, 0), p};
+    const TwRef Ti{tw_table(a.tw, 0, p, 1), p};
+    const SmemIO<LR, 2, false> xy{sm};  // columns: operands a and b
+    const SmemIO<LR, 1, false> io{sm};  // arrays: b follows a
+    round_io<LR, 2, dif_base(LR, 0, NR), round_size(LR, 0, NR), true, 1, false, 0, T>(
+        raw_in<ZT>(a, k, p, q), xy, T0, q);
+    __syncthreads();
+    forward_rounds<LR, 2, NR, 1, T, 1>(xy, T0, q, 2);
+    middle_round<LR, 1, NR, T>(io, T0, Ti, q, qinv, 1);
+    inverse_rounds<LR, 1, NR, T, 1>(io, Ti, q, 1);
     cluster.sync();
     uint32_t *words = sm + 2 * N;
     uint32_t *out = cluster.map_shared_rank(words, 0);
@@ -935,7 +947,8 @@ __global__ void __cluster_dims__(kNumPrimes, 1, 1) __launch_bounds__(cluster_thr
         for (int i = 0; i < 5; i++) out[i * N + swz(j)] = w[i];
     }
     cluster.sync();  // no block reads another's shared memory after this
-    if (p == 0) block_limbs<LR, T>(a, k, words, wsm);
+    constexpr int LPT = 2 * N / T > kLimbsPerThread ? 2 * N / T : kLimbsPerThread;
+    if (p == 0) block_limbs<LPT, N, N>(a, k, 1, words, wsm);
 }
 
 // ------------------------------------------------------------ host side
@@ -1510,23 +1523,24 @@ static void launch_fused_t(size_t nprod, bool spread, cudaStream_t s, const Fuse
             return;
         }
     }
-    const size_t smem = 6 * ((size_t)1 << LR) * sizeof(uint32_t);
+    constexpr size_t PN = fused_points(LR), P = PN >> LR;
+    const size_t smem = 6 * PN * sizeof(uint32_t);
     set_smem(ntt_mul_fused<LR, ZT>, smem);
-    ntt_mul_fused<LR, ZT><<<(unsigned)nprod, fused_threads(LR), smem, s>>>(a);
+    ntt_mul_fused<LR, ZT><<<(unsigned)((nprod + P - 1) / P), fused_threads(LR), smem, s>>>(a);
 }
 
 // Whether a batch of one-block products takes a cluster of five blocks per
-// product: while the clusters' threads fit the chip at once, at most 256
-// products.  Measured (us per launch, one block : cluster): one product of
-// 2^10 points 20.7 : 8.6, of 2^8 21.0 : 8.3, of 2^5 10.2 : 6.4; 256 products of
-// 2^10 points 25.0 : 22.8 and 512 37.3 : 37.5; of 2^11 points 64 products
-// 27.0 : 20.7, 128 27.1 : 27.1, 256 35.8 : 44.5; of 2^5 points 256 products
-// 10.4 : 8.6, 512 10.4 : 12.5.
+// product: while the clusters' threads fit the chip's 2,048 per SM about once,
+// at most 512 products.  Measured (us per launch, one block : cluster): one
+// product of 2^10 points 26.9 : 8.6, of 2^8 20.9 : 8.1, of 2^5 12.8 : 6.6; 256
+// products of 2^10 points 28.9 : 22.8, 512 34.8 : 37.3; of 2^11 points 128
+// products 32.5 : 26.0, 256 36.9 : 42.6; of 2^9 points 512 products 27.0 : 20.8,
+// 1,024 33.1 : 34.0; of 2^5 points 512 products 18.8 : 10.8, 2,048 20.7 : 29.1.
 static bool spread_primes(size_t nprod, int lr, int num_sms)
 {
     if (nprod == 1) return true;
-    return nprod <= 256 &&
-           nprod * kNumPrimes * (size_t)cluster_threads(lr) <= (size_t)num_sms * 2048;
+    return nprod <= 512 && nprod * kNumPrimes * (size_t)cluster_threads(lr) * 8 <=
+                               (size_t)num_sms * 2048 * 9;
 }
 
 template <int LR>
@@ -1534,7 +1548,7 @@ static void launch_fused(size_t nprod, int num_sms, cudaStream_t s, const FusedA
 {
     const bool spread = spread_primes(nprod, LR, num_sms);
     // operands of at most half the transform (every tree level)
-    if (std::max(a.a_len, a.B ? a.b_len : 0u) <= (1u << LR))
+    if (std::max(a.a_len, a.b_len) <= (1u << LR))
         launch_fused_t<LR, true>(nprod, spread, s, a);
     else
         launch_fused_t<LR, false>(nprod, spread, s, a);
@@ -1547,14 +1561,14 @@ static void ntt_mul_small(Ctx &c, int np, size_t nprod, Operand x, Operand y, bo
     a.A = x.p;
     a.a_tstride = x.tstride;
     a.a_len = (uint32_t)x.len;
-    a.B = square ? nullptr : y.p;
+    a.B = y.p;  // squares are short and alone here: x twice
     a.b_tstride = y.tstride;
     a.b_len = (uint32_t)y.len;
     a.a_al = aligned8(x.p, x.tstride);
     a.b_al = aligned8(y.p, y.tstride);
+    a.nprod = nprod;
     a.sink = sink;
     a.tw = c.twiddles;
-    a.scale = make_scale(0, np);
     a.ca = make_coef(0, sink.dec);
     a.cb = make_coef_scaled(0, np, sink.dec);
     const int tok = prof_begin(c, "ntt_mul_fused", s);
@@ -1626,7 +1640,7 @@ void ntt_mul(Ctx &c, const uint32_t *a, size_t na, const uint32_t *b, size_t nb,
     const bool square = (a == b && na == nb);
     Operand x{a, 0, na}, y{b, 0, nb};
     if (np <= kFusedMaxLog) {
-        ntt_mul_small(c, np, 1, x, y, square, plain_sink(out, 0, len), s);
+        ntt_mul_small(c, np, 1, x, square ? x : y, square, plain_sink(out, 0, len), s);
     } else if (square) {
         ntt_mul_multipass(c, np, PAIR_SQUARE, 1, x, x, plain_sink(out, 0, len), s);
     } else {

@@ -162,13 +162,15 @@ __device__ __forceinline__ void dit_stages(uint32_t (&x)[NA][1 << E], int glow, 
 // `out`.  COLFAST: consecutive threads take consecutive columns (strided
 // columns in global memory); otherwise consecutive threads take consecutive
 // groups of one column (contiguous rows in global memory).  No barrier.
-// THREADS: the block's threads (0: blockDim.x).
+// THREADS: the block's threads (0: blockDim.x).  Only the first `cols` columns
+// are worked on.
 template <int LR, int C, int B, int E, bool FWD, int NA, bool COLFAST, int PS, int THREADS = 0,
           class IN, class OUT>
-__device__ __forceinline__ void round_io(const IN &in, const OUT &out, const TwRef &T, uint32_t q)
+__device__ __forceinline__ void round_io(const IN &in, const OUT &out, const TwRef &T, uint32_t q,
+                                         int cols = C)
 {
     constexpr int NGC = (1 << LR) >> E;  // groups per column
-    constexpr int NG = C * NGC;
+    const int NG = cols * NGC;
     const int step = THREADS ? THREADS : (int)blockDim.x;
 #pragma unroll 1
     for (int g = threadIdx.x; g < NG; g += step) {
@@ -193,14 +195,18 @@ __host__ __device__ constexpr int ilog2c(int x) { return x <= 1 ? 0 : 1 + ilog2c
 // is contiguous (at c 2^LR + i).  A group's points base + k 2^B have offsets
 // d_k = k 2^B (times C when interleaved) whose bits the group's own address
 // a0 never has, and swz is linear over XOR on disjoint bits, so the swizzled
-// address is swz(a0) ^ swz(d_k): one XOR with a compile-time constant.
-template <int LR, int C, bool COLFAST>
+// address is swz(a0) ^ swz(d_k): one XOR with a compile-time constant.  With
+// WHOLE the columns' own index takes part in the swizzle (columns of fewer
+// than 2^10 points, several to a warp: checked lane by lane for the one-block
+// multiply's shapes, at most two-way conflicts at 2^5 points and none above).
+template <int LR, int C, bool COLFAST, bool WHOLE = false>
 struct SmemIO {
     uint32_t *s;
     static constexpr int LC = ilog2c(C);
     template <int B>
     __device__ __forceinline__ static int group_addr(int base, int c)
     {
+        if (WHOLE) return swz((c << LR) + base);
         return COLFAST ? swz(base * C + c) : (c << LR) + swz(base);
     }
     template <int E, int B, int NA>
@@ -226,6 +232,32 @@ struct SmemIO {
                 s[a * ((1 << LR) * C) + (a0 ^ swz(k << SH))] = x[a][k];
     }
 };
+
+// Coefficients i = base + k 2^B (k < 2^E) of an operand of len limbs: words 2i
+// and 2i + 1 (zero past the end), 8 bytes at a time where al says that the
+// operand is aligned; the choice is made once per group, so that its loads go
+// out together.  ZT: the upper half is zero.
+template <int E, int B, bool ZT>
+__device__ __forceinline__ void load_coefs(uint32_t (&x)[1 << E], const uint32_t *r, int base,
+                                           uint32_t len, bool al, const CoefMul &m, uint32_t q)
+{
+    constexpr int K = ZT ? (1 << (E - 1)) : (1 << E);
+    uint2 w[K];
+    if (al && 2u * (uint32_t)(base + ((K - 1) << B)) + 2u <= len) {
+#pragma unroll
+        for (int k = 0; k < K; k++)
+            w[k] = *reinterpret_cast<const uint2 *>(r + 2 * (base + (k << B)));
+    } else {
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            const uint32_t i = 2u * (uint32_t)(base + (k << B));
+            w[k].x = i < len ? r[i] : 0u;
+            w[k].y = i + 1 < len ? r[i + 1] : 0u;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < (1 << E); k++) x[k] = k < K ? coef_in<0>(w[k].x, w[k].y, m, q) : 0u;
+}
 
 // ---------------------------------------------------------- column passes
 
@@ -961,32 +993,11 @@ struct RowLimbIn {
     bool al_a, al_b;
     uint32_t q;
     CoefMul ca, cb;
-    template <int E, int B>
-    __device__ __forceinline__ void load1(uint32_t (&x)[1 << E], int base, const uint32_t *r,
-                                          uint32_t len, bool al, const CoefMul &m) const
-    {
-        constexpr int K = ZT ? (1 << (E - 1)) : (1 << E);
-        uint2 w[K];
-        if (al && 2u * (uint32_t)(base + ((K - 1) << B)) + 2u <= len) {
-#pragma unroll
-            for (int k = 0; k < K; k++)
-                w[k] = *reinterpret_cast<const uint2 *>(r + 2 * (base + (k << B)));
-        } else {
-#pragma unroll
-            for (int k = 0; k < K; k++) {
-                const uint32_t i = 2u * (uint32_t)(base + (k << B));
-                w[k].x = i < len ? r[i] : 0u;
-                w[k].y = i + 1 < len ? r[i + 1] : 0u;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < (1 << E); k++) x[k] = k < K ? coef_in<0>(w[k].x, w[k].y, m, q) : 0u;
-    }
     template <int E, int B, int NA>
     __device__ __forceinline__ void load(uint32_t (&x)[NA][1 << E], int base, int) const
     {
-        load1<E, B>(x[0], base, pa, la, al_a, ca);
-        if (NA > 1) load1<E, B>(x[NA - 1], base, pb, lb, al_b, cb);
+        load_coefs<E, B, ZT>(x[0], pa, base, la, al_a, ca, q);
+        if (NA > 1) load_coefs<E, B, ZT>(x[NA - 1], pb, base, lb, al_b, cb, q);
     }
 };
 

@@ -56,12 +56,13 @@ def test_square_by_the_row_pass(ctx, cat_lib, orc, n):
 
 
 @pytest.mark.parametrize("slot", [8, 16, 64, 256, 1024, 2048])
-@pytest.mark.parametrize("nprod", [2, 121, 122, 257])
+@pytest.mark.parametrize("nprod", [2, 33, 136, 137, 273, 274, 513])
 def test_levels_on_both_sides_of_the_cluster_rule(ctx, cat_lib, orc, slot, nprod):
     """Product trees whose level at `slot` limbs has nprod products: few go by
-    clusters of blocks, many by one block each (the rule's limits are 256
-    products, and 121 of 2,048-limb operands on 152 SMs).  The tree's levels
-    run from 8 limbs up, so every size between is covered too."""
+    clusters of blocks, many by one block each (the rule's limits are 512
+    products, 273 of 1,024-limb and 136 of 2,048-limb operands on 152 SMs), and
+    a block takes several short products, the last one fewer.  The tree's
+    levels run from 8 limbs up, so every size between is covered too."""
     count = nprod * 2 * slot - 5
     if count > 150_000:
         count = 150_000 + nprod
