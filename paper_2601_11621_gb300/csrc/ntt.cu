@@ -483,7 +483,7 @@ __device__ __forceinline__ void run_halo(CoefRun &r, uint32_t *hsm)
 // carry-in is assumed 0.  DEC / ADD: 1 or 0 when known at compile time, -1
 // when the runtime flag (dec, add != null) decides.  LPT: limbs per run.
 template <int DEC, int ADD, int LPT = kLimbsPerThread, class SUM>
-__device__ __forceinline__ void tile_carry(const SUM &sum, int tile_len, uint32_t *out,
+__device__ __forceinline__ void tile_carry(SUM &&sum, int tile_len, uint32_t *out,
                                            long out_count, bool dec_rt, const uint32_t *add,
                                            long add_count, uint32_t *wsm, uint32_t *tile_map)
 {
@@ -793,21 +793,51 @@ __device__ __forceinline__ void middle_round(const IO &io, const TwRef &T0, cons
 
 // The limbs of a block's products from their coefficients' words in shared
 // memory: word p of coefficient j at s[p PN + swz(j)], products of N = 2^LR
-// coefficients back to back, a run of LPT limbs per thread, first limb j0.
+// coefficients back to back, a run of limbs per thread from the first
+// coefficient j0 (a multiple of 4).  The limbs are asked for in order; every
+// fourth coefficient reads the next four coefficients' words, 16 bytes each.
 template <int N, int PN>
 struct SmemRun {
     const uint32_t *s;
-    int j0;  // first coefficient
-    __device__ __forceinline__ uint32_t word(int p, int j, int back) const
+    int j0;
+    uint32_t w[5][4];
+    uint32_t h2, h3, h4a, h4b;  // the words that the run before hands over (CoefRun)
+    __device__ __forceinline__ SmemRun(const uint32_t *words, int first) : s(words), j0(first) {}
+    __device__ __forceinline__ uint64_t operator()(int i)
     {
-        // coefficient j - back of the same product, or none
-        return (j & (N - 1)) >= back ? s[p * PN + swz(j - back)] : 0u;
-    }
-    __device__ __forceinline__ uint64_t operator()(int i) const
-    {
-        const int j = j0 + (i >> 1);
-        if (i & 1) return (uint64_t)word(1, j, 0) + word(3, j, 1);
-        return (uint64_t)word(0, j, 0) + word(2, j, 1) + word(4, j, 2);
+        const int j = (i >> 1) & 3;
+        if ((i & 7) == 0) {
+            if (i) {
+                h2 = w[2][3];
+                h3 = w[3][3];
+                h4a = w[4][2];
+                h4b = w[4][3];
+            } else {
+                // coefficients j0 - 1 and j0 - 2 of the same product, if any
+                // (read here, not at construction: a thread without limbs may
+                // have a j0 past the arrays)
+                const bool one = (j0 & (N - 1)) >= 1, two = (j0 & (N - 1)) >= 2;
+                h2 = one ? s[2 * PN + swz(j0 - 1)] : 0u;
+                h3 = one ? s[3 * PN + swz(j0 - 1)] : 0u;
+                h4b = one ? s[4 * PN + swz(j0 - 1)] : 0u;
+                h4a = two ? s[4 * PN + swz(j0 - 2)] : 0u;
+            }
+#pragma unroll
+            for (int p = 0; p < 5; p++) {
+                if (N >= 4) {
+                    const uint4 v =
+                        *reinterpret_cast<const uint4 *>(s + p * PN + swz(j0 + (i >> 1)));
+                    w[p][0] = v.x; w[p][1] = v.y; w[p][2] = v.z; w[p][3] = v.w;
+                } else {
+#pragma unroll
+                    for (int t = 0; t < 4; t++)
+                        w[p][t] = t < N ? s[p * PN + swz(j0 + t)] : 0u;
+                }
+            }
+        }
+        if (i & 1) return (uint64_t)w[1][j] + (j >= 1 ? w[3][j - 1] : h3);
+        return (uint64_t)w[0][j] + (j >= 1 ? w[2][j - 1] : h2) +
+               (j >= 2 ? w[4][j - 2] : (j == 0 ? h4a : h4b));
     }
 };
 

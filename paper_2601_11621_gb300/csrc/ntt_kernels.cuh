@@ -63,20 +63,19 @@ __host__ __device__ constexpr int dit_base(int lr, int rd, int nr)
 }
 __host__ __device__ constexpr int dit_base(int lr, int rd) { return dit_base(lr, rd, rounds_of(lr)); }
 
-// Shared-memory address swizzle: the bank bits of address a are XORed with a
-// GF(2)-linear image f(t) of its row-of-32 index t = (a >> 5) mod 32, f
-// sending the bits of t to 1, 10, 20, 24, 16.  In a round with base bit
-// B < 5 the lanes of a warp differ in address bits [0, B) and in bits at and
-// above B + E; f is chosen so that those five bits always land on five
-// independent bank bits for the round shapes used here (E = 3 or 4 with
-// B = 0, 3 or 4 on contiguous rows; the group bit 7 of 16-column tiles; in the
-// column passes' interleaved tiles every shape from E = 2 to 4 at the bases
-// they use, checked lane by lane), so no round has a bank conflict.  Rounds
-// with B >= 5 are conflict-free under any such XOR.
+// Shared-memory address swizzle: the four-word chunks of address a (bits 2-4,
+// the bank's upper bits) are XORed with a GF(2)-linear image of its row-of-32
+// index t = (a >> 5) mod 32, which sends the bits of t to 1, 2, 4, 6, 0.  Four
+// consecutive words stay together, so that the rounds at stage bits [0, E) move
+// 16 bytes per access; in the others a warp's lanes differ in address bits
+// [0, B) and in bits at and above B + E, which the image spreads over the
+// banks: no conflicts in any round of the row and column passes and of the
+// one-block multiply from 2^6 points (every shape's accesses enumerated on the
+// CPU), at most two-way ones in a few rounds of 2^5 .. 2^7 points.
 __host__ __device__ constexpr int swz(int a)
 {
     const int t = (a >> 5) & 31;
-    return a ^ t ^ ((t & 6) << 2) ^ ((t & 8) << 1);
+    return a ^ (((t & 7) ^ ((t & 8) >> 2) ^ ((t & 8) >> 1)) << 2);
 }
 
 // The twiddles of one direction of one prime: the stage table in global
@@ -195,41 +194,73 @@ __host__ __device__ constexpr int ilog2c(int x) { return x <= 1 ? 0 : 1 + ilog2c
 // is contiguous (at c 2^LR + i).  A group's points base + k 2^B have offsets
 // d_k = k 2^B (times C when interleaved) whose bits the group's own address
 // a0 never has, and swz is linear over XOR on disjoint bits, so the swizzled
-// address is swz(a0) ^ swz(d_k): one XOR with a compile-time constant.  With
-// WHOLE the columns' own index takes part in the swizzle (columns of fewer
-// than 2^10 points, several to a warp: checked lane by lane for the one-block
-// multiply's shapes, at most two-way conflicts at 2^5 points and none above).
+// address is swz(a0) ^ swz(d_k).  Of that the bank bits take an XOR with one of
+// at most 32 constants (eight in most rounds, one where the offsets lie above
+// the swizzle's bits), shared by the points that agree in it, and the higher
+// bits, which are zero in a0, an immediate offset.  With WHOLE the columns' own
+// index takes part in the swizzle (columns of fewer than 2^10 points, several
+// to a warp).  Together with the 16-byte accesses and the 32-bit offsets into
+// global memory (word_at), against one XOR per point and 4-byte accesses:
+// C(2,050,572,903) 90.2 -> 87.8 ms.
 template <int LR, int C, bool COLFAST, bool WHOLE = false>
 struct SmemIO {
     uint32_t *s;
     static constexpr int LC = ilog2c(C);
-    template <int B>
-    __device__ __forceinline__ static int group_addr(int base, int c)
+    static constexpr int SIZE = (1 << LR) * C;
+    // byte address of the group's first point
+    __device__ __forceinline__ static uint32_t group_addr(int base, int c)
     {
-        if (WHOLE) return swz((c << LR) + base);
-        return COLFAST ? swz(base * C + c) : (c << LR) + swz(base);
+        const int a = WHOLE     ? swz((c << LR) + base)
+                      : COLFAST ? swz(base * C + c)
+                                : (c << LR) + swz(base);
+        return (uint32_t)a * 4u;
+    }
+    // the address of point d (its offset from the group's first) of array a
+    __device__ __forceinline__ char *at(uint32_t g0, int d, int a) const
+    {
+        return reinterpret_cast<char *>(s) + (g0 ^ (uint32_t)(4 * (swz(d) & 31))) +
+               4 * ((d & ~31) + a * SIZE);
     }
     template <int E, int B, int NA>
     __device__ __forceinline__ void load(uint32_t (&x)[NA][1 << E], int base, int c) const
     {
-        constexpr int SH = COLFAST ? B + LC : B;
-        const int a0 = group_addr<B>(base, c);
+        const uint32_t g0 = group_addr(base, c);
+        if constexpr (B == 0 && !COLFAST && E >= 2) {  // consecutive points
 #pragma unroll
-        for (int a = 0; a < NA; a++)
+            for (int k = 0; k < (1 << E); k += 4)
 #pragma unroll
-            for (int k = 0; k < (1 << E); k++)
-                x[a][k] = s[a * ((1 << LR) * C) + (a0 ^ swz(k << SH))];
+                for (int a = 0; a < NA; a++) {
+                    const uint4 v = *reinterpret_cast<const uint4 *>(at(g0, k, a));
+                    x[a][k] = v.x; x[a][k + 1] = v.y; x[a][k + 2] = v.z; x[a][k + 3] = v.w;
+                }
+        } else {
+            constexpr int SH = COLFAST ? B + LC : B;
+#pragma unroll
+            for (int a = 0; a < NA; a++)
+#pragma unroll
+                for (int k = 0; k < (1 << E); k++)
+                    x[a][k] = *reinterpret_cast<const uint32_t *>(at(g0, k << SH, a));
+        }
     }
     template <int E, int B, int NA>
     __device__ __forceinline__ void store(uint32_t (&x)[NA][1 << E], int base, int c) const
     {
-        constexpr int SH = COLFAST ? B + LC : B;
-        const int a0 = group_addr<B>(base, c);
+        const uint32_t g0 = group_addr(base, c);
+        if constexpr (B == 0 && !COLFAST && E >= 2) {
 #pragma unroll
-        for (int a = 0; a < NA; a++)
+            for (int k = 0; k < (1 << E); k += 4)
 #pragma unroll
-            for (int k = 0; k < (1 << E); k++)
-                s[a * ((1 << LR) * C) + (a0 ^ swz(k << SH))] = x[a][k];
+                for (int a = 0; a < NA; a++)
+                    *reinterpret_cast<uint4 *>(at(g0, k, a)) =
+                        make_uint4(x[a][k], x[a][k + 1], x[a][k + 2], x[a][k + 3]);
+        } else {
+            constexpr int SH = COLFAST ? B + LC : B;
+#pragma unroll
+            for (int a = 0; a < NA; a++)
+#pragma unroll
+                for (int k = 0; k < (1 << E); k++)
+                    *reinterpret_cast<uint32_t *>(at(g0, k << SH, a)) = x[a][k];
+        }
     }
 };
 
@@ -338,6 +369,17 @@ struct ColArgs {
 #endif
 constexpr int kColV = CAT_COL_V;
 
+// Word i of a transform at the block-uniform address p: the byte offset stays
+// in 32 bits (transforms of up to 2^26 points, operands of up to 2^27 limbs
+// below 2^30 words), so that an access takes the uniform base and one 32-bit
+// register instead of a 64-bit sum per point.
+template <class T>
+__device__ __forceinline__ T *word_at(T *p, uint32_t i)
+{
+    using C = std::conditional_t<std::is_const_v<T>, const char, char>;
+    return reinterpret_cast<T *>(reinterpret_cast<C *>(p) + 4u * i);
+}
+
 template <int V>
 __device__ __forceinline__ void load_v(const uint32_t *p, uint32_t (&w)[V])
 {
@@ -394,7 +436,7 @@ struct ColIn {
 #pragma unroll
         for (int k = 0; k < (1 << E); k++) {
             uint32_t w[V];
-            load_v<V>(p + i0 + (uint32_t)k * (S << B), w);
+            load_v<V>(word_at(p, i0 + (uint32_t)k * (S << B)), w);
 #pragma unroll
             for (int a = 0; a < V; a++) x[a][k] = w[a];
         }
@@ -426,7 +468,8 @@ struct ColSrcIn {
         if (al && i0 + (uint32_t)(K - 1) * (2u * S << B) + 4u <= src_len) {
 #pragma unroll
             for (int k = 0; k < K; k++)
-                w[k] = *reinterpret_cast<const uint4 *>(src + i0 + (uint32_t)k * (2u * S << B));
+                w[k] = *reinterpret_cast<const uint4 *>(
+                    word_at(src, i0 + (uint32_t)k * (2u * S << B)));
         } else {
 #pragma unroll
             for (int k = 0; k < K; k++) {
@@ -497,7 +540,7 @@ struct ColTw {
             for (int j = 0; j < (1 << E); j++) {
                 const int k = bitrev_c(j, E);
                 uint32_t w[V];
-                load_v_ro<V>(tab + (uint32_t)(base + k) * S + gcol, w);
+                load_v_ro<V>(word_at(tab, (uint32_t)(base + k) * S + gcol), w);
                 f(k, w);
             }
             return;
@@ -536,7 +579,7 @@ struct ColOutTw {
             uint32_t w[V];
 #pragma unroll
             for (int a = 0; a < V; a++) w[a] = mul_mont<PS>(x[a][k], v[a], tw.q, tw.qinv);
-            store_v<V>(p + i0 + (uint32_t)k * S, w);
+            store_v<V>(word_at(p, i0 + (uint32_t)k * S), w);
         });
     }
 };
@@ -555,7 +598,7 @@ struct ColInTw {
         const uint32_t i0 = (uint32_t)base * S + gcol;
         tw.template each<E>(gcol, base, [&](int k, const uint32_t(&v)[V]) {
             uint32_t w[V];
-            load_v<V>(p + i0 + (uint32_t)k * S, w);
+            load_v<V>(word_at(p, i0 + (uint32_t)k * S), w);
 #pragma unroll
             for (int a = 0; a < V; a++) x[a][k] = mul_mont<PS>(w[a], v[a], tw.q, tw.qinv);
         });
@@ -576,7 +619,7 @@ struct ColOut {
             uint32_t w[V];
 #pragma unroll
             for (int a = 0; a < V; a++) w[a] = x[a][k];
-            store_v<V>(p + i0 + (uint32_t)k * (S << B), w);
+            store_v<V>(word_at(p, i0 + (uint32_t)k * (S << B)), w);
         }
     }
 };
