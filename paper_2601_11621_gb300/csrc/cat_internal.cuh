@@ -212,36 +212,21 @@ __device__ __forceinline__ uint32_t shoup(uint32_t a, uint32_t w, uint32_t wp, u
     return a * w - __umulhi(a, wp) * q;
 }
 
+// Montgomery product a b 2^-32 mod q in [0, 2q), for a b < 2^32 q and q < 2^31:
+// with m = -(a b) q^-1 mod 2^32, a b + m q is a multiple of 2^32, so its high
+// word is exact.  One wide product, one low product and one wide multiply-add
+// (10 cycles of the multiply pipe and no adds; by high products and their
+// difference it was 12 cycles and two adds).
+__device__ __forceinline__ uint32_t mont2(uint32_t a, uint32_t b, uint32_t q, uint32_t qinv)
+{
+    const uint64_t p = (uint64_t)a * b;
+    const uint32_t m = (uint32_t)p * (0u - qinv);
+    return (uint32_t)(((uint64_t)m * q + p) >> 32);
+}
+
 // x - m when x >= m, for x < 2m <= 2^32: when x < m the difference wraps to
 // at least 2^32 - m > x, so the smaller candidate is always the answer.
 __device__ __forceinline__ uint32_t csub(uint32_t x, uint32_t m) { return min(x, x - m); }
-
-// Modular add, subtract and Montgomery products for q < 2^31 (S) in the
-// min-of-two form, or for any q < 2^32.  Inputs below q, results below q.
-template <bool S>
-__device__ __forceinline__ uint32_t add_m(uint32_t a, uint32_t b, uint32_t q)
-{
-    if (S) return csub(a + b, q);
-    return add_mod(a, b, q);
-}
-
-template <bool S>
-__device__ __forceinline__ uint32_t sub_m(uint32_t a, uint32_t b, uint32_t q)
-{
-    if (S) return csub(a - b + q, q);
-    return sub_mod(a, b, q);
-}
-
-template <bool S>
-__device__ __forceinline__ uint32_t mont(uint32_t a, uint32_t b, uint32_t q, uint32_t qinv)
-{
-    if (S) {
-        const uint32_t hi = __umulhi(a, b);
-        const uint32_t m = (a * b) * qinv;
-        return csub(hi - __umulhi(m, q) + q, q);
-    }
-    return mont_mul(a, b, q, qinv);
-}
 
 // ------------------------------------------- the transform data per set
 //
@@ -258,6 +243,22 @@ __device__ __forceinline__ uint32_t mul_w(uint32_t a, uint2 w, uint32_t q)
     else return mont_mul_pre(a, w.x, w.y, q);
 }
 
+// The sum a + b less m when it reaches m (a, b < m, 2m <= 2^32), and the
+// difference a - b + m as 2a - (a + b - m): with the corrected sum's second
+// candidate at hand that is one instruction (a shift-add), where a - b + m
+// takes two.  A set-0 butterfly of either direction comes to 7 instructions
+// instead of 8, the multiply pipe's three of 8 cycles (a high product takes
+// four cycles there, a low one two) and four adds: C(2,050,572,903) 87.8 ->
+// 84.4 ms.  In set 1, with two corrections per butterfly, the shift-add lands
+// on the multiply pipe and is slower (2^25 x 2^25 limbs 2.94 -> 3.11 ms).
+__device__ __forceinline__ void sum_diff(uint32_t a, uint32_t b, uint32_t m, uint32_t &sum,
+                                         uint32_t &diff)
+{
+    const uint32_t t = a + b, u = t - m;
+    sum = min(t, u);
+    diff = 2 * a - u;
+}
+
 // Forward (decimation-in-frequency) butterfly (x, y) <- (x + y, (x - y) w)
 // on forward-range residues.
 template <int PS>
@@ -265,8 +266,9 @@ __device__ __forceinline__ void bf_dif(uint32_t &x, uint32_t &y, uint2 w, uint32
 {
     const uint32_t a = x, b = y;
     if constexpr (PS == 0) {
-        x = csub(a + b, 2 * q);                 // [0, 4q) -> [0, 2q)
-        y = shoup(a - b + 2 * q, w.x, w.y, q);  // (0, 4q) times w -> [0, 2q)
+        uint32_t d;
+        sum_diff(a, b, 2 * q, x, d);  // [0, 4q) -> [0, 2q), (0, 4q)
+        y = shoup(d, w.x, w.y, q);    // times w -> [0, 2q)
     } else if constexpr (PS == 1) {
         x = csub(a + b, q);
         y = csub(shoup(a - b + q, w.x, w.y, q), q);
@@ -282,11 +284,15 @@ __device__ __forceinline__ void bf_dif1(uint32_t &x, uint32_t &y, uint32_t q)
 {
     const uint32_t a = x, b = y;
     if constexpr (PS == 0) {
-        x = csub(a + b, 2 * q);
-        y = csub(a - b + 2 * q, 2 * q);
+        uint32_t d;
+        sum_diff(a, b, 2 * q, x, d);
+        y = csub(d, 2 * q);
+    } else if constexpr (PS == 1) {
+        x = csub(a + b, q);
+        y = csub(a - b + q, q);
     } else {
-        x = add_m<PS == 1>(a, b, q);
-        y = sub_m<PS == 1>(a, b, q);
+        x = add_mod(a, b, q);
+        y = sub_mod(a, b, q);
     }
 }
 
@@ -296,14 +302,19 @@ template <int PS>
 __device__ __forceinline__ void bf_dit(uint32_t &x, uint32_t &y, uint2 w, uint32_t q)
 {
     if constexpr (PS == 0) {
-        const uint32_t a = csub(x, 2 * q);          // [0, 2q)
-        const uint32_t t = shoup(y, w.x, w.y, q);   // [0, 2q)
-        x = a + t;                                  // [0, 4q)
-        y = a - t + 2 * q;                          // (0, 4q)
+        const uint32_t a = csub(x, 2 * q);  // [0, 2q)
+        // a + t with t = shoup(y, w) in [0, 2q): the sum rides on the product's
+        // multiply-adds; a - t + 2q = 2a + 2q - (a + t)
+        x = y * w.x + a - __umulhi(y, w.y) * q;  // [0, 4q)
+        y = 2 * a + 2 * q - x;                   // (0, 4q)
+    } else if constexpr (PS == 1) {
+        const uint32_t a = x, t = mul_w<PS>(y, w, q);
+        x = csub(a + t, q);
+        y = csub(a - t + q, q);
     } else {
         const uint32_t a = x, t = mul_w<PS>(y, w, q);
-        x = add_m<PS == 1>(a, t, q);
-        y = sub_m<PS == 1>(a, t, q);
+        x = add_mod(a, t, q);
+        y = sub_mod(a, t, q);
     }
 }
 
@@ -313,11 +324,9 @@ __device__ __forceinline__ void bf_dit1(uint32_t &x, uint32_t &y, uint32_t q)
     if constexpr (PS == 0) {
         const uint32_t a = csub(x, 2 * q), t = csub(y, 2 * q);
         x = a + t;
-        y = a - t + 2 * q;
+        y = 2 * a + 2 * q - x;
     } else {
-        const uint32_t a = x, b = y;
-        x = add_m<PS == 1>(a, b, q);
-        y = sub_m<PS == 1>(a, b, q);
+        bf_dif1<PS>(x, y, q);  // the same sum and difference
     }
 }
 
@@ -347,17 +356,14 @@ __device__ __forceinline__ uint32_t coef_in(uint32_t lo, uint32_t hi, const Coef
 // Pointwise product of two forward-range residues times the scale factor S:
 // x y 2^-32 by Montgomery's reduction, then times sc = 2^32 S (Shoup) for
 // sets 0 and 1 or sc = 2^64 S (Montgomery) for set 2, giving x y S.
-// For set 0, x y < 4 q^2 < 2^32 q keeps hi(x y) - hi(m q) in (-q, q).
+// For set 0, x y < 4 q^2 < 2^32 q keeps the Montgomery product below 2q.
 template <int PS>
 __device__ __forceinline__ uint32_t pmul(uint32_t x, uint32_t y, uint2 sc, uint32_t q,
                                          uint32_t qinv)
 {
-    if constexpr (PS == 0) {
-        const uint32_t hi = __umulhi(x, y);
-        const uint32_t m = (x * y) * qinv;
-        return shoup(hi - __umulhi(m, q) + q, sc.x, sc.y, q);
-    } else if constexpr (PS == 1) {
-        return csub(shoup(mont<true>(x, y, q, qinv), sc.x, sc.y, q), q);
+    if constexpr (PS < 2) {
+        const uint32_t r = shoup(mont2(x, y, q, qinv), sc.x, sc.y, q);
+        return PS == 0 ? r : csub(r, q);
     } else {
         return mont_mul(mont_mul(x, y, q, qinv), sc.x, q, qinv);
     }

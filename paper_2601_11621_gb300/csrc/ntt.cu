@@ -203,16 +203,14 @@ __device__ __forceinline__ uint32_t tw_pow_mont(const uint2 *T, uint32_t E, uint
 }
 
 // x v for any 32-bit x and a Montgomery-form multiplier vm = v 2^32 mod q,
-// into the set's forward range (set 0: hi(x vm) - hi(m q) + q lies in (0, 2q)).
+// into the set's forward range (x vm < 2^32 q).
 template <int PS>
 __device__ __forceinline__ uint32_t mul_mont(uint32_t x, uint32_t vm, uint32_t q, uint32_t qinv)
 {
     if constexpr (PS == 0) {
-        const uint32_t hi = __umulhi(x, vm);
-        const uint32_t m = (x * vm) * qinv;
-        return hi - __umulhi(m, q) + q;
+        return mont2(x, vm, q, qinv);
     } else if constexpr (PS == 1) {
-        return mont<true>(x, vm, q, qinv);
+        return csub(mont2(x, vm, q, qinv), q);
     } else {
         return mont_mul(x, vm, q, qinv);
     }
