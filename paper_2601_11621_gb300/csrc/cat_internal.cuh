@@ -195,14 +195,6 @@ __device__ __forceinline__ uint32_t mont_mul_pre(uint32_t a, uint32_t w, uint32_
     return hi < u ? r + q : r;
 }
 
-// x mod q for any 32-bit x (3q > 2^32, so at most two subtractions).
-__device__ __forceinline__ uint32_t reduce32(uint32_t x, uint32_t q)
-{
-    if (x >= q) x -= q;
-    if (x >= q) x -= q;
-    return x;
-}
-
 // Shoup's product: a w - floor(a wp / 2^32) q with wp = floor(w 2^32 / q)
 // equals a w mod q or that plus q, for any a < 2^32 and w < q < 2^31
 // (the quotient estimate is short by at most one), so it lies in [0, 2q) and
@@ -338,8 +330,7 @@ struct CoefMul {
     uint2 w0, w1;
 };
 
-// The residue of lo w0 + hi w1 in the forward range.  Set 2 takes w0 = 1 only
-// (lo < 2^32 < 3q).
+// The residue of lo w0 + hi w1 in the forward range.
 template <int PS>
 __device__ __forceinline__ uint32_t coef_in(uint32_t lo, uint32_t hi, const CoefMul &c, uint32_t q)
 {
@@ -349,7 +340,8 @@ __device__ __forceinline__ uint32_t coef_in(uint32_t lo, uint32_t hi, const Coef
         return csub(csub(shoup(lo, c.w0.x, c.w0.y, q), q) + csub(shoup(hi, c.w1.x, c.w1.y, q), q),
                     q);
     } else {
-        return add_mod(reduce32(lo, q), mont_mul_pre(hi, c.w1.x, c.w1.y, q), q);
+        return add_mod(mont_mul_pre(lo, c.w0.x, c.w0.y, q), mont_mul_pre(hi, c.w1.x, c.w1.y, q),
+                       q);
     }
 }
 
@@ -417,7 +409,6 @@ struct Ctx {
     // context is released; contexts with a budget compute the twiddles)
     struct ColTwTable {
         int ps, m, lr, dir;
-        bool scaled;  // entries times 2^(32-m): operand b's first forward pass
         uint32_t *p;
     };
     std::vector<ColTwTable> col_tw;

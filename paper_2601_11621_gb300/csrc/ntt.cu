@@ -139,40 +139,26 @@ static Scale make_scale(int set, int np)
 }
 
 // The operands' input multipliers (coef_in): 1 and the word base (2^32, or
-// 10^9 for decimal digits).
+// 10^9 for decimal digits), both times the pointwise scale 2^32 S of 2^np
+// points for the operand that takes it in advance (np >= 0).
 struct CoefMuls {
     CoefMul c[kNumPrimes];
 };
 
-static CoefMuls make_coef(int set, bool dec)
+static CoefMuls make_coef(int set, bool dec, int np = -1)
 {
+    auto form = [&](uint32_t w, uint32_t q) {
+        if (set_shoup(set)) return make_uint2(w, shoup_c(w, q));
+        const uint32_t m = to_mont_c(w, q);
+        return make_uint2(m, m * inv32(q));
+    };
     CoefMuls m;
     for (int i = 0; i < kNumPrimes; i++) {
         const uint32_t q = ntt_prime(set, i);
         const uint32_t b = (uint32_t)((dec ? (uint64_t)kDecBase : (1ull << 32)) % q);
-        if (set_shoup(set)) {
-            m.c[i].w0 = make_uint2(1u, shoup_c(1u, q));
-            m.c[i].w1 = make_uint2(b, shoup_c(b, q));
-        } else {
-            const uint32_t bm = to_mont_c(b, q);
-            m.c[i].w0 = make_uint2(1u, 0u);
-            m.c[i].w1 = make_uint2(bm, bm * inv32(q));
-        }
-    }
-    return m;
-}
-
-// The same times the pointwise scale 2^32 S (sets in Shoup's form): operand b
-// of a product whose pointwise step is then one Montgomery product.
-static CoefMuls make_coef_scaled(int set, int np, bool dec)
-{
-    CoefMuls m;
-    for (int i = 0; i < kNumPrimes; i++) {
-        const uint32_t q = ntt_prime(set, i);
-        const uint32_t b = (uint32_t)((dec ? (uint64_t)kDecBase : (1ull << 32)) % q);
-        const uint32_t r = scale_value(set, i, np), rb = mulmod_u64(r, b, q);
-        m.c[i].w0 = make_uint2(r, shoup_c(r, q));
-        m.c[i].w1 = make_uint2(rb, shoup_c(rb, q));
+        const uint32_t r = np < 0 ? 1u : scale_value(set, i, np);
+        m.c[i].w0 = form(r, q);
+        m.c[i].w1 = form(mulmod_u64(r, b, q), q);
     }
     return m;
 }
@@ -1064,56 +1050,41 @@ static void launch_col(bool fwd, dim3 grid, cudaStream_t s, const ColArgs &a)
 // ps, direction dir): entry row 2^(m-r) + col = w^((col bitrev_r(row)) << shift)
 // in Montgomery form, the value the pass would otherwise compute for that
 // point (tw_pow_mont, exactly as the stepping reaches it).
-// With scale (per prime, nonzero), every entry is multiplied by it mod q.
-struct TwScale {
-    uint32_t c[kNumPrimes];
-};
-
 template <int PS>
-__global__ void col_twiddle_table(const uint2 *tw, int m, int r, int dir, TwScale scale,
-                                  uint32_t *tab)
+__global__ void col_twiddle_table(const uint2 *tw, int m, int r, int dir, uint32_t *tab)
 {
     const int p = blockIdx.y;
     const uint32_t q = c_q[PS][p], qinv = c_qinv[PS][p];
-    const uint32_t sp = scale.c[p];
     const uint2 *T = tw_table(tw, PS, p, dir);
     const int shift = set_log_root(PS) - m;
     const uint32_t cols = 1u << (m - r);
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < (1u << m);
          i += gridDim.x * blockDim.x) {
         const uint32_t row = i >> (m - r), col = i & (cols - 1);
-        uint32_t v = tw_pow_mont<PS>(T, (col * bitrev(row, r)) << shift, q, qinv);
-        if (sp) v = (uint32_t)((uint64_t)v * sp % q);
-        tab[((size_t)p << m) + i] = v;
+        tab[((size_t)p << m) + i] =
+            tw_pow_mont<PS>(T, (col * bitrev(row, r)) << shift, q, qinv);
     }
 }
 
 // A column pass's twiddle table, built on first use; null when the context
 // computes its twiddles (a budgeted context, or no room for the table).
-// scaled: the entries times 2^32 S mod q (S the pointwise scale of 2^m
-// points), for operand b of a product whose pointwise step then needs no
-// normalisation (forward first passes, m = np).
-static const uint32_t *col_twiddles(Ctx &c, int ps, int m, int r, int dir, cudaStream_t s,
-                                    bool scaled = false)
+static const uint32_t *col_twiddles(Ctx &c, int ps, int m, int r, int dir, cudaStream_t s)
 {
     if (!c.col_tw_tables || c.budget || c.shared_budget) return nullptr;
     for (const Ctx::ColTwTable &t : c.col_tw)
-        if (t.ps == ps && t.m == m && t.lr == r && t.dir == dir && t.scaled == scaled) return t.p;
+        if (t.ps == ps && t.m == m && t.lr == r && t.dir == dir) return t.p;
     uint32_t *p = nullptr;
     if (cudaMalloc(&p, ((size_t)kNumPrimes << m) * sizeof(uint32_t)) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    TwScale sc{};
-    if (scaled)
-        for (int i = 0; i < kNumPrimes; i++) sc.c[i] = scale_value(ps, i, m);
     const unsigned blocks = (unsigned)std::min<size_t>(((size_t)1 << m) / 256 + 1, 4096);
     const dim3 grid(blocks, kNumPrimes);
-    if (ps == 0) col_twiddle_table<0><<<grid, 256, 0, s>>>(c.twiddles, m, r, dir, sc, p);
-    else if (ps == 1) col_twiddle_table<1><<<grid, 256, 0, s>>>(c.twiddles, m, r, dir, sc, p);
-    else col_twiddle_table<2><<<grid, 256, 0, s>>>(c.twiddles, m, r, dir, sc, p);
+    if (ps == 0) col_twiddle_table<0><<<grid, 256, 0, s>>>(c.twiddles, m, r, dir, p);
+    else if (ps == 1) col_twiddle_table<1><<<grid, 256, 0, s>>>(c.twiddles, m, r, dir, p);
+    else col_twiddle_table<2><<<grid, 256, 0, s>>>(c.twiddles, m, r, dir, p);
     CAT_LAUNCH("col_twiddle_table");
-    c.col_tw.push_back(Ctx::ColTwTable{ps, m, r, dir, scaled, p});
+    c.col_tw.push_back(Ctx::ColTwTable{ps, m, r, dir, p});
     return p;
 }
 
@@ -1135,16 +1106,15 @@ constexpr Operand kNoSource{nullptr, 0, 0};
 
 // One column pass over `total` points (blocks of 2^m points, 2^r rows).
 //
-// scaled (first forward passes): 1 = every transform of the call is an
-// operand b, 2 = the odd ones are (adjacent pairs); their twiddles then carry
-// the pointwise step's normalisation.  Returns whether they did (the scaled
-// table exists), i.e. whether the row pass must skip the normalisation.
+// scaled (first forward passes): 1 = the call's last transform (or its only
+// one) is an operand b, 2 = the odd ones are (adjacent pairs); their input
+// multipliers then carry the pointwise scale.
 //
 // x: the sources of a first forward pass (p null otherwise); y, when given,
 // the source of the call's last transform (the second operand of a product or
 // the common one of broadcast products), so that both operands of a single
 // product share one launch.
-static bool col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, size_t total,
+static void col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, size_t total,
                      int m, int r, const Operand &x, const Operand *y, bool dec, cudaStream_t s,
                      int scaled = 0)
 {
@@ -1154,26 +1124,18 @@ static bool col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, s
     };
     ColArgs a;
     a.coef = make_coef(ps, dec);
+    a.coef_b = scaled ? make_coef(ps, dec, m) : a.coef;
+    a.odd_b = scaled == 2;
     a.src_al = aligned16(x);
-    a.last = y ? (total >> m) - 1 : ~(size_t)0;
-    a.src_y = y ? y->p : nullptr;
-    a.src_y_len = y ? y->len : 0;
-    a.src_y_al = y && aligned16(*y);
-    a.twtab_odd = nullptr;
+    a.last = y || scaled == 1 ? (unsigned)(total >> m) - 1u : ~0u;
+    a.src_y = y ? y->p : x.p;
+    a.src_y_len = y ? y->len : x.len;
+    a.src_y_al = aligned16(y ? *y : x);
     // (measured per C(2,050,572,903): tables in every pass beat computed
     // twiddles at every block size, the first forward passes' large tables
     // included, once the table loads go through the read-only path)
     const int tmax = src ? c.col_tw_first_max_log : c.col_tw_max_log;
     a.twtab = m <= tmax ? col_twiddles(c, ps, m, r, fwd ? 0 : 1, s) : nullptr;
-    bool prescaled = false;
-    if (scaled && a.twtab) {
-        const uint32_t *sct = col_twiddles(c, ps, m, r, 0, s, true);
-        if (sct) {
-            if (scaled == 1) a.twtab = sct;
-            else a.twtab_odd = sct;
-            prescaled = true;
-        }
-    }
     a.data = data;
     a.pstride = pstride;
     a.m = m;
@@ -1182,6 +1144,7 @@ static bool col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, s
     a.src_len = x.len;
     a.tw = c.twiddles;
     const size_t ctas = total >> (r + col_log_c(r));
+    a.nblk = (unsigned)(total >> m);
     dim3 grid((unsigned)ctas, kNumPrimes);
     // algorithmic bytes: every point of the five prime arrays read and
     // written once (the first forward pass reads limbs instead)
@@ -1232,17 +1195,12 @@ static bool col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, s
     }
     CAT_LAUNCH(fwd ? "ntt_col_fwd" : "ntt_col_inv");
     prof_end(c, tok, s, bytes);
-    return prescaled;
 }
 
 template <int LR, int PS>
 static void launch_row_t(dim3 grid, cudaStream_t s, const RowArgs &a, bool pre)
 {
-    if (a.prescaled && a.mode != PAIR_SQUARE && !pre) {  // operand b carries the scale
-        const size_t smem = ((size_t)2 << kRowMaxLog) * sizeof(uint32_t);
-        set_smem(ntt_row_mul_ns<LR, PS>, smem);
-        ntt_row_mul_ns<LR, PS><<<grid, kRowThreads, smem, s>>>(a);
-    } else if (pre) {  // broadcast products, the common transform complete
+    if (pre) {  // broadcast products, the common transform complete
         const size_t smem = ((size_t)1 << kRowMaxLog) * sizeof(uint32_t);
         set_smem(ntt_row_mul_bcast<LR, PS>, smem);
         ntt_row_mul_bcast<LR, PS><<<grid, kRowThreads, smem, s>>>(a);
@@ -1448,7 +1406,7 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
         ra.tw = c.twiddles;
         ra.scale = make_scale(PS, np);
         ra.ca = make_coef(PS, dec);
-        ra.cb = make_coef_scaled(PS, np, dec);
+        ra.cb = make_coef(PS, dec, np);
         tok = prof_begin(c, "ntt_row_limbs", s);
         launch_row_limbs(nprod, mode == PAIR_SQUARE, s, ra);
         prof_end(c, tok, s, 4.0 * kNumPrimes * (double)gp + unit, unit);
@@ -1458,9 +1416,8 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
             m.F = m.Fb.get();
         }
         uint32_t *F = m.F;
-        // forward column passes (operand b's first pass takes the pointwise
-        // step's normalisation into its twiddles when it has a table)
-        bool prescaled = false;
+        // forward column passes (operand b's input multipliers take the
+        // pointwise scale)
         const int r0 = P.rcol[0];
         // one launch for the operands of a single or a broadcast product,
         // unless only one of them fills its transform's upper half and the
@@ -1469,15 +1426,13 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
         const bool together =
             two && (np <= 17 || (x.len <= N) == (y.len <= N));
         if (together) {
-            prescaled = col_pass(c, PS, true, F, fp, fp, np, r0, x, &y, dec, s,
-                                 mode == PAIR_FIRST_TWO ? 2 : 0);
+            col_pass(c, PS, true, F, fp, fp, np, r0, x, &y, dec, s, 1);
         } else if (two) {
             col_pass(c, PS, true, F, fp, fp - N, np, r0, x, nullptr, dec, s);
-            prescaled = col_pass(c, PS, true, F + fp - N, fp, N, np, r0, y, nullptr, dec, s,
-                                 mode == PAIR_FIRST_TWO ? 1 : 0);
+            col_pass(c, PS, true, F + fp - N, fp, N, np, r0, y, nullptr, dec, s, 1);
         } else {
-            prescaled = col_pass(c, PS, true, F, fp, fp, np, r0, x, nullptr, dec, s,
-                                 mode == PAIR_ADJACENT ? 2 : 0);
+            col_pass(c, PS, true, F, fp, fp, np, r0, x, nullptr, dec, s,
+                     mode == PAIR_ADJACENT ? 2 : 0);
         }
         int mm = np - r0;
         for (int i = 1; i < P.ncol; i++) {
@@ -1496,7 +1451,6 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
         ra.gpstride = gp;
         ra.np = np;
         ra.mode = mode;
-        ra.prescaled = prescaled ? 1 : 0;
         ra.tw = c.twiddles;
         ra.scale = make_scale(PS, np);
         // broadcast products: y's transform completed once, in its slot, so that
@@ -1598,7 +1552,7 @@ static void ntt_mul_small(Ctx &c, int np, size_t nprod, Operand x, Operand y, bo
     a.sink = sink;
     a.tw = c.twiddles;
     a.ca = make_coef(0, sink.dec);
-    a.cb = make_coef_scaled(0, np, sink.dec);
+    a.cb = make_coef(0, sink.dec, np);
     const int tok = prof_begin(c, "ntt_mul_fused", s);
     switch (np) {
     case 1: launch_fused<1>(nprod, c.num_sms, s, a); break;

@@ -343,21 +343,36 @@ struct ColArgs {
     size_t src_tstride;    // limbs between consecutive transforms' sources
     size_t src_len;        // valid limbs per transform (rest are zero)
     int src_al;            // every source starts on a 16-byte boundary
-    size_t last;           // the transform whose source is src_y (or none)
+    unsigned last;         // the transform whose source is src_y (or none)
     const uint32_t *src_y;
     size_t src_y_len;
     int src_y_al;
-    CoefMuls coef;         // the sources' input multipliers
+    CoefMuls coef;         // the sources' input multipliers,
+    CoefMuls coef_b;       // those of transform `last`, or (odd_b) of the odd ones
+    int odd_b;
+    unsigned nblk;         // blocks of 2^m points
     const uint2 *tw;
     // the pass's inter-pass twiddles, w^(col bitrev(row)) in the multiplier
     // form the pass applies, point (row, col) of a 2^m block at row 2^(m-LR) +
     // col, 2^m per prime; null: the pass computes them
     const uint32_t *twtab;
-    // first forward pass of adjacent pairs: the odd transforms' (operand b's)
-    // table, its entries times 2^32 S (the pointwise product's scale S taken
-    // in advance), or null
-    const uint32_t *twtab_odd;
 };
+
+// The 2^m-point block and the column group of a block of threads.  ACROSS: the
+// same columns of all blocks one after the other, so that both operands of a
+// product and all products of a level read a twiddle word from memory once;
+// else a block's columns one after the other.  Measured per
+// C(2,050,572,903): first forward passes across 16.16 -> 16.01 ms, the other
+// passes 15.2 -> 15.7, so only the first ones go across.
+template <bool ACROSS>
+__device__ __forceinline__ void col_place(unsigned nblk, unsigned groups, unsigned &blk,
+                                          unsigned &group)
+{
+    const unsigned d = ACROSS ? nblk : groups;
+    const unsigned hi = blockIdx.x / d, lo = blockIdx.x - hi * d;
+    blk = ACROSS ? lo : hi;
+    group = ACROSS ? hi : lo;
+}
 
 // Column tiles hold V adjacent columns per thread group: the group's V
 // columns c V + a (a < V) are the V arrays of the register round (NA = V), so
@@ -639,29 +654,28 @@ __global__ void __launch_bounds__(kColFwdThreads, CAT_COL_FWD_MINB) ntt_col_fwd(
     const int p = blockIdx.y;
     const uint32_t q = c_q[PS][p];
     const size_t Sr = (size_t)1 << (a.m - LR);
-    const size_t groups = Sr >> LC;
-    const size_t blk = blockIdx.x / groups;
-    const size_t col0 = (blockIdx.x % groups) << LC;
-    uint32_t *base = a.data + p * a.pstride + (blk << a.m);
+    unsigned blk, group;
+    col_place<SRC != 0>(a.nblk, (unsigned)(Sr >> LC), blk, group);
+    const size_t col0 = (size_t)group << LC;
+    uint32_t *base = a.data + p * a.pstride + ((size_t)blk << a.m);
     const uint2 *T = tw_table(a.tw, PS, p, 0);
     const TwRef TR{T, p};
     const auto in = [&] {
         if constexpr (SRC != 0) {
-            const bool y = blk == a.last;
+            const bool y = blk == a.last, b = y || (a.odd_b && (blk & 1));
             return ColSrcIn<PS, V, SRC == 2>{y ? a.src_y : a.src + blk * a.src_tstride,
                                              (uint32_t)Sr,
                                              (uint32_t)col0,
                                              (uint32_t)(y ? a.src_y_len : a.src_len),
                                              (y ? a.src_y_al : a.src_al) != 0,
                                              q,
-                                             a.coef.c[p]};
+                                             b ? a.coef_b.c[p] : a.coef.c[p]};
         } else
             return ColIn<V>{base, (uint32_t)Sr, (uint32_t)col0};
     }();
     ColTw<LR, PS, NR, kColFwdThreads, V> tw{T, q, c_qinv[PS][p], set_log_root(PS) - a.m, {}};
-    const uint32_t *tt = ((blk & 1) && a.twtab_odd) ? a.twtab_odd : a.twtab;
-    if (tt) {
-        tw.tab = tt + ((size_t)p << a.m);
+    if (a.twtab) {
+        tw.tab = a.twtab + ((size_t)p << a.m);
         tw.S = (uint32_t)Sr;
     }
     tw.init((uint32_t)col0);
@@ -698,10 +712,10 @@ __global__ void __launch_bounds__(kColInvThreads, CAT_COL_INV_MINB) ntt_col_inv(
     const int p = blockIdx.y;
     const uint32_t q = c_q[PS][p];
     const size_t Sr = (size_t)1 << (a.m - LR);
-    const size_t groups = Sr >> LC;
-    const size_t blk = blockIdx.x / groups;
-    const size_t col0 = (blockIdx.x % groups) << LC;
-    uint32_t *base = a.data + p * a.pstride + (blk << a.m);
+    unsigned blk, group;
+    col_place<false>(a.nblk, (unsigned)(Sr >> LC), blk, group);
+    const size_t col0 = (size_t)group << LC;
+    uint32_t *base = a.data + p * a.pstride + ((size_t)blk << a.m);
     const uint2 *Ti = tw_table(a.tw, PS, p, 1);
     const TwRef TRi{Ti, p};
     ColTw<LR, PS, NR, kColInvThreads, V> tw{Ti, q, c_qinv[PS][p], set_log_root(PS) - a.m, {}};
@@ -749,9 +763,8 @@ struct RowArgs {
     size_t gpstride;
     int np;             // log2 points
     int mode;           // which transforms product k multiplies
-    int prescaled;      // operand b's transform already carries 2^32 S: no scale
     const uint2 *tw;
-    Scale scale;
+    Scale scale;        // squares only: operand b carries the scale otherwise
 };
 
 // Consecutive rows in global memory (operands a, b): point i of row c at
@@ -823,7 +836,7 @@ struct RowOutPair {
 // finished transform (YH, broadcast products, whose x alone is transformed
 // here; ntt_row_fwd left it in the order the product loop reads it), g takes
 // the rows of the product.
-template <int LR, bool SQ, int PS, bool YH, bool NS, bool PAIR, class IN>
+template <int LR, bool SQ, int PS, bool YH, bool PAIR, class IN>
 __device__ __forceinline__ void row_mul_core(const IN &in, const uint32_t *y, uint32_t *g,
                                              const uint2 *tw, uint2 sc, uint32_t *sm)
 {
@@ -873,8 +886,8 @@ __device__ __forceinline__ void row_mul_core(const IN &in, const uint32_t *y, ui
         uint32_t z[1][1 << EL];
 #pragma unroll
         for (int j = 0; j < (1 << EL); j++)
-            z[0][j] = NS ? mul_mont<PS>(x[0][j], x[NA - 1][j], q, qinv)
-                         : pmul<PS>(x[0][j], YH ? yv[j] : x[NA - 1][j], sc, q, qinv);
+            z[0][j] = SQ ? pmul<PS>(x[0][j], x[0][j], sc, q, qinv)
+                         : mul_mont<PS>(x[0][j], YH ? yv[j] : x[NA - 1][j], q, qinv);
         dit_stages<EL, 0, 1, PS>(z, 0, Ti, q);
         sio.template store<EL, 0, 1>(z, base, c);
     }
@@ -912,7 +925,7 @@ __host__ __device__ constexpr bool row_pair_fwd()
            (NR == 2 || CF * ((1 << LR) >> round_size(LR, 1)) >= kRowThreads);
 }
 
-template <int LR, bool SQ, int PS, bool YH, bool NS = false>
+template <int LR, bool SQ, int PS, bool YH>
 __device__ __forceinline__ void row_mul_body(const RowArgs &a, uint32_t *sm)
 {
     constexpr int RB = row_log_rows(LR), C = 1 << RB;
@@ -929,10 +942,10 @@ __device__ __forceinline__ void row_mul_body(const RowArgs &a, uint32_t *sm)
     const uint32_t *fb = a.F + p * a.fpstride + (tb << a.np) + off;
     uint32_t *g = a.G + p * a.gpstride + (k << a.np) + off;
     if constexpr (row_pair_fwd<LR>())
-        row_mul_core<LR, SQ, PS, YH, NS, true>(RowInPair<LR, C / 2>{fa, fb}, fb, g, a.tw,
-                                               a.scale.c[p], sm);
+        row_mul_core<LR, SQ, PS, YH, true>(RowInPair<LR, C / 2>{fa, fb}, fb, g, a.tw, a.scale.c[p],
+                                           sm);
     else
-        row_mul_core<LR, SQ, PS, YH, NS, false>(RowIn<LR>{fa, fb}, fb, g, a.tw, a.scale.c[p], sm);
+        row_mul_core<LR, SQ, PS, YH, false>(RowIn<LR>{fa, fb}, fb, g, a.tw, a.scale.c[p], sm);
 }
 
 template <int LR, bool SQ, int PS>
@@ -940,16 +953,6 @@ __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_mul(RowArgs
 {
     extern __shared__ uint32_t sm[];
     row_mul_body<LR, SQ, PS, false>(a, sm);
-}
-
-// Products whose operand b transform already carries the normalisation
-// 2^32 S (its first pass took the scaled twiddle table): the pointwise
-// product is one Montgomery product.
-template <int LR, int PS>
-__global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_mul_ns(RowArgs a)
-{
-    extern __shared__ uint32_t sm[];
-    row_mul_body<LR, false, PS, false, true>(a, sm);
 }
 
 // Broadcast products x_k y whose y transform ntt_row_fwd has completed.
@@ -1058,6 +1061,6 @@ __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_limbs(RowLi
     const RowLimbIn<LR, ZT> in{a.A + k * a.a_tstride, a.B + k * a.b_tstride, a.a_len, a.b_len,
                                a.a_al != 0,           a.b_al != 0,           c_q[0][p],
                                a.ca.c[p],             a.cb.c[p]};
-    row_mul_core<LR, SQ, 0, false, !SQ, false>(in, nullptr, a.G + p * a.gpstride + (k << LR), a.tw,
+    row_mul_core<LR, SQ, 0, false, false>(in, nullptr, a.G + p * a.gpstride + (k << LR), a.tw,
                                                a.scale.c[p], sm);
 }
