@@ -1,14 +1,14 @@
 // autotune.cu -- measures the device-dependent choices of the product tree's
 // multiplications on the current GPU and applies them to a context:
 //   - the row-pass size (2^9 .. 2^12 points) of the multi-pass transform for
-//     every transform size 2^13 .. 2^27, the rest of the transform going to
-//     one or two column passes;
+//     every product size 2^13 .. 2^27 limbs, the rest of the transform going
+//     to one or two column passes;
 //   - the largest tree-level slot (32 .. 256 limbs) whose products the
 //     schoolbook (Comba) kernels finish faster than the transform.
 // Each candidate multiplies a synthetic tree level of 2^24 limbs (one product
 // of 2^n limbs above that; seeded words) and is timed with CUDA events on the
-// context's stream; the fastest wins.  The largest trial holds about 6 GB of
-// scratch and 4.5 GB of column twiddle tables (dropped after every trial).
+// context's stream; the fastest wins.  The largest trial holds about 5 GB of
+// scratch and 4 GB of column twiddle tables (dropped after every trial).
 // The table is written as text, tagged with the device's name and SM count,
 // and read back by contexts created later on the same kind of device.
 #include "cat_internal.cuh"
@@ -26,6 +26,7 @@
 namespace cat {
 
 bool plan_row_ok(int n, int rrow);
+int default_row(int np);
 
 namespace {
 
@@ -69,10 +70,6 @@ float time_ms(cudaStream_t s, F &&f)
     return t[2];
 }
 
-// The default row-pass size of a 2^n-point transform (the plan without a
-// tuned value).
-int default_row(int n) { return std::min(12, n - 4); }
-
 std::string device_tag(int device)
 {
     cudaDeviceProp p;
@@ -98,7 +95,8 @@ void autotune(Ctx &c, cudaStream_t s)
         const size_t slot = (size_t)1 << (n - 1), nprod = std::max<size_t>(1, kTuneLimbs >> n);
         // the default plan first; another size replaces it only when at least
         // 1 % faster, so that near-ties keep the default
-        const int def = default_row(n);
+        // (2^13 limbs take the row pass alone whatever the table says)
+        const int def = std::max(9, default_row(n - 1));
         c.row_log[n] = 0;
         int best = def;
         // each trial's column twiddle tables (built by its warm-up run) are

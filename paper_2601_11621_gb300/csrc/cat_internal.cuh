@@ -399,7 +399,9 @@ struct Ctx {
     std::string last_error;
     uint2 *twiddles = nullptr;  // [set][prime][dir][kTwPerDir] multiplier pairs
     int num_sms = 0;
-    size_t comba_max_slot = 128;  // tree levels with slots up to this use schoolbook
+    // tree levels with slots up to this use schoolbook (us per level of 2^24
+    // limbs, schoolbook : transform: slots of 64 limbs 150 : 229, 128 263 : 241)
+    size_t comba_max_slot = 64;
     int max_log = kLogMaxNtt;     // longest product (log2 limbs) of one transform; longer by pieces
     // row-pass size (log2 points) of the multi-pass transform of products of
     // 2^n limbs, as tuned on this device (cat_autotune); 0 = the default plan

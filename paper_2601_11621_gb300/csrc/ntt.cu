@@ -974,6 +974,21 @@ struct NttPlan {
     int rrow = 0;
 };
 
+// The default row-pass size of a transform of 2^np points: as long as the
+// columns fit one pass, rows of 2^12 points (at least 2^4 column rows), but
+// 2^10 where that leaves 2^5 or 2^6 column rows; above 2^22 points, where the
+// columns take two passes whatever the rows, rows of 2^9.  Measured (ms per
+// level of 2^27 limbs, rows of 2^9 : 2^10 : 2^11 : 2^12): np = 17 3.74 : 3.74 :
+// 3.81 : 3.92, 18 4.00 : 3.87 : 3.93 : 3.95, 20 5.10 : 4.42 : 4.29 : 4.16, 22
+// 5.17 : 5.19 : 5.42 : 4.76, 23 5.14 : 5.21 : 5.33 : 5.46, 25 5.27 : 5.26 : 5.48 :
+// 5.53.
+int default_row(int np)
+{
+    if (np > 22) return 9;
+    if (np == 17 || np == 18) return 10;
+    return std::min(12, np - kColMinLog);
+}
+
 // The plan of a product of 2^n limbs (2^np points, np = n - 1 >= 12): a row
 // pass of up to 2^12 points and column passes of at most 2^10 rows, split as
 // evenly as possible.  2^12 points take the row pass alone.  A row-pass size
@@ -1001,7 +1016,7 @@ static NttPlan make_plan(const Ctx &c, int np)
         P.rrow = np;
         return P;
     }
-    P.rrow = std::min(kRowMaxLog, np - kColMinLog);
+    P.rrow = default_row(np);
     if (n <= kLogMaxNtt && c.row_log[n] && plan_row_ok(n, c.row_log[n])) P.rrow = c.row_log[n];
     int rem = np - P.rrow;
     P.ncol = (rem + kColMaxLog - 1) / kColMaxLog;
