@@ -9,7 +9,7 @@
 
 namespace cat {
 
-void exclusive_scan_u32(Ctx &c, uint32_t *data, size_t n, cudaStream_t s);
+void exclusive_scan_u32(Ctx &c, uint32_t *data, size_t n, cudaStream_t s, uint32_t *sum = nullptr);
 
 __device__ __forceinline__ int dec_digits(uint32_t p)
 {

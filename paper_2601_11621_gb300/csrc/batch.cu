@@ -23,7 +23,7 @@
 namespace cat {
 
 DevBuf<uint32_t> sieve_primes(Ctx &c, uint64_t limit, uint64_t *count, cudaStream_t s);
-void exclusive_scan_u32(Ctx &c, uint32_t *data, size_t n, cudaStream_t s);
+void exclusive_scan_u32(Ctx &c, uint32_t *data, size_t n, cudaStream_t s, uint32_t *sum = nullptr);
 
 namespace {
 

@@ -178,7 +178,10 @@ int cat_ctx_profile(const cat_ctx *ctx, size_t i, const char **name, uint64_t *l
 int catalan_factor(cat_ctx *ctx, uint64_t n, int kind, cat_factorization *out, void *stream)
 {
     if (!ctx || !out) return CAT_EINVAL;
-    return guarded(ctx, [&] { cat::factor(ctx->c, n, kind, out, as_stream(stream)); });
+    return guarded(ctx, [&] {
+        cat::factor(ctx->c, n, kind, out, as_stream(stream));
+        CAT_CUDA(cudaStreamSynchronize(as_stream(stream)));
+    });
 }
 
 void cat_factor_free(cat_ctx *ctx, cat_factorization *f)
@@ -314,7 +317,10 @@ int cat_ratio_factor(cat_ctx *ctx, const uint64_t *a, int ka, const uint64_t *b,
 {
     cat::Ratio r;
     if (!ctx || !out || !make_ratio(a, ka, b, kb, &r)) return CAT_EINVAL;
-    return guarded(ctx, [&] { cat::factor_ratio(ctx->c, r, out, as_stream(stream)); });
+    return guarded(ctx, [&] {
+        cat::factor_ratio(ctx->c, r, out, as_stream(stream));
+        CAT_CUDA(cudaStreamSynchronize(as_stream(stream)));
+    });
 }
 
 int cat_ratio_exact(cat_ctx *ctx, const uint64_t *a, int ka, const uint64_t *b, int kb,

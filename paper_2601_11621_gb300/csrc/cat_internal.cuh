@@ -386,6 +386,8 @@ struct ProfPending {
     double unit_bytes;
 };
 
+struct Phase1Info;
+
 struct Ctx {
     int device = 0;
     size_t budget = 0;   // 0 = unlimited
@@ -423,10 +425,25 @@ struct Ctx {
     // word, allocated once per context
     uint64_t *host_word = nullptr;
     unsigned long long *dev_word = nullptr;
+    // the primes below 2^16, ascending (every sieve's seeds are a prefix), on
+    // the device and the host, and Phase 1's read-back (pinned)
+    uint32_t *seeds = nullptr;
+    std::vector<uint32_t> host_seeds;
+    struct Phase1Info *host_info = nullptr;
     bool profiling = false;
     std::vector<ProfEntry> prof;
     std::vector<ProfPending> pending;
     std::vector<cudaEvent_t> event_pool;
+};
+
+// Phase 1 of a binomial kind, read back in one copy: the large primes kept by
+// the sieve, all odd primes up to the limit, whether an exponent came out
+// negative, and the groups of the seed primes by ascending exponent (group g
+// at [off[g], off[g+1]) of the grouped seeds; exponents are at most 31).
+constexpr int kMaxSeedGroups = 32;
+struct Phase1Info {
+    uint32_t kept, total, negative, ngroups;
+    uint32_t exp[kMaxSeedGroups], off[kMaxSeedGroups + 1];
 };
 
 // Launch bracketing for the profiler: prof_begin returns a token (or -1 when
@@ -647,8 +664,8 @@ struct Ratio {
     uint32_t a[kMaxRatioTerms], b[kMaxRatioTerms];
 };
 
-// Phase 1 on the device.  The arrays of *out come from the context's pool
-// and are released by factor_free.
+// Phase 1 on the device, complete on stream s.  The arrays of *out come from
+// the context's pool and are released by factor_free.
 void factor(Ctx &c, uint64_t n, int kind, cat_factorization *out, cudaStream_t s);
 void factor_ratio(Ctx &c, const Ratio &r, cat_factorization *out, cudaStream_t s);
 void factor_free(Ctx &c, cat_factorization *f);

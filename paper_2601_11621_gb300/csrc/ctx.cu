@@ -269,6 +269,16 @@ void ctx_init(Ctx &c, int device, size_t budget)
     }
     pool_for(device);
     build_twiddles(c);
+    std::vector<bool> composite(1u << 16);
+    for (uint32_t p = 2; p < (1u << 16); p++) {
+        if (composite[p]) continue;
+        c.host_seeds.push_back(p);
+        for (uint32_t j = p * p; p < 256 && j < (1u << 16); j += p) composite[j] = true;
+    }
+    CAT_CUDA(cudaMalloc(&c.seeds, c.host_seeds.size() * sizeof(uint32_t)));
+    CAT_CUDA(cudaMemcpy(c.seeds, c.host_seeds.data(), c.host_seeds.size() * sizeof(uint32_t),
+                        cudaMemcpyHostToDevice));
+    CAT_CUDA(cudaMallocHost(&c.host_info, sizeof(Phase1Info)));
     CAT_CUDA(cudaMallocHost(&c.host_word, 4 * sizeof(uint64_t)));
     CAT_CUDA(cudaMalloc(&c.dev_word, sizeof(unsigned long long)));
 }
@@ -284,6 +294,14 @@ void ctx_release(Ctx &c)
     if (c.dev_word) {
         cudaFree(c.dev_word);
         c.dev_word = nullptr;
+    }
+    if (c.seeds) {
+        cudaFree(c.seeds);
+        c.seeds = nullptr;
+    }
+    if (c.host_info) {
+        cudaFreeHost(c.host_info);
+        c.host_info = nullptr;
     }
     if (c.host_word) {
         cudaFreeHost(c.host_word);

@@ -8,14 +8,13 @@
 
 namespace cat {
 
-// v_p(m!) = sum_k floor(m / p^k)
+// v_p(m!) = sum_k floor(m / p^k), floor(m / p^(k+1)) = floor(floor(m / p^k) / p)
 __device__ __forceinline__ uint32_t legendre32(uint32_t m, uint32_t p)
 {
     uint32_t s = 0;
-    uint64_t pk = p;
-    while (pk <= m) {
-        s += m / (uint32_t)pk;
-        pk *= p;
+    while (m >= p) {
+        m /= p;
+        s += m;
     }
     return s;
 }

@@ -3,13 +3,14 @@
 // exponent of each prime by Legendre's formula (Sec. 2), and the grouping of
 // the primes with e > 0 by exponent into CSR form.
 //
-// Sieve.  Seed primes up to sqrt(limit) come from one thread block.  The odd
-// numbers up to the limit are cut into segments of 2^18 (one bit each, 32 KiB
-// of shared memory per block).  Primes 3..31 are struck word by word from
-// precomputed bit patterns; primes 37..511 are struck by whole warps (one
-// multiple per lane); larger seed primes by one thread each.  Each segment's
-// bitmap and prime count go to global memory; an exclusive scan of the
-// counts gives every segment its first output position.
+// Sieve.  The seed primes up to sqrt(limit) < 2^16 are a prefix of the
+// context's table.  The odd numbers up to the limit are cut into segments of
+// 2^13 .. 2^18 (one bit each, at most 32 KiB of shared memory per block).
+// Primes 3..31 are struck word by word from bit patterns; primes 37..511 are
+// struck by whole warps (one multiple per lane); larger seed primes by one
+// thread each.  The bitmap and a prime count per unit of 2^13 odd numbers go
+// to global memory; an exclusive scan of the counts gives every unit its first
+// output position.
 //
 // Exponents.  2n < 2^32, so every term floor(m / p^k) is a 32-bit division;
 // primes above sqrt(m) take one division per factorial.  c_p = v_p(n+1) is
@@ -24,7 +25,9 @@
 // exponent 0 or 1 (one base-p carry), found with one division inside the
 // sieve; the sieve keeps only the primes with exponent 1 and they are written
 // in order straight into the e = 1 group.  Only the seed primes (below
-// sqrt(2n) <= 65536) go through Legendre's formula and the radix grouping.
+// sqrt(2n) <= 65536) go through Legendre's formula, and one block sorts them
+// by exponent.  Such a Phase 1 is four launches and one read-back (what the
+// CSR's size depends on).
 #include "cat_internal.cuh"
 #include "legendre.cuh"
 
@@ -33,64 +36,26 @@
 
 namespace cat {
 
-void exclusive_scan_u32(Ctx &c, uint32_t *data, size_t n, cudaStream_t s);
+void exclusive_scan_u32(Ctx &c, uint32_t *data, size_t n, cudaStream_t s, uint32_t *sum = nullptr);
 
-constexpr int kSegBits = 1 << 18;           // odd numbers per segment
-constexpr int kSegWords = kSegBits / 32;    // 8192 words
+constexpr int kUnitLog = 13;                     // odd numbers per counting unit (log2)
+constexpr int kUnitWords = (1 << kUnitLog) / 32;  // 256 words
+constexpr int kMaxSegLog = 18;                   // odd numbers per segment, at most (log2)
+constexpr int kMaxSegUnits = 1 << (kMaxSegLog - kUnitLog);
 constexpr int kSieveThreads = 512;
 constexpr uint32_t kMediumPrime = 37;       // first prime struck by atomics
 constexpr uint32_t kLargePrime = 512;       // thread-per-prime from here (measured best)
 
-// ---------------------------------------------------------------- seeds
-
-// All primes <= root (root < 2^16) in ascending order, by one block.
-__global__ void __launch_bounds__(1024) seed_sieve(uint32_t root, uint32_t *seeds,
-                                                   uint32_t *nseeds)
-{
-    __shared__ uint32_t bm[2048];  // bit x set = x composite, x < 65536
-    __shared__ uint32_t pre[1024];
-    for (int i = threadIdx.x; i < 2048; i += blockDim.x) bm[i] = 0;
-    __syncthreads();
-    if (threadIdx.x == 0) atomicOr(&bm[0], 3u);  // 0 and 1
-    for (uint32_t p = 2; p * p <= root; p++)
-        for (uint32_t j = p * p + threadIdx.x * p; j <= root; j += blockDim.x * p)
-            atomicOr(&bm[j >> 5], 1u << (j & 31));
-    __syncthreads();
-    // thread t owns numbers [64 t, 64 t + 64)
-    const uint32_t lo = threadIdx.x * 64;
-    uint32_t w0 = ~bm[2 * threadIdx.x], w1 = ~bm[2 * threadIdx.x + 1];
-    if (lo > root) { w0 = 0; w1 = 0; }
-    else if (lo + 64 > root + 1) {
-        const uint32_t keep = root + 1 - lo;  // 1..64 numbers kept
-        if (keep < 32) { w0 &= (1u << keep) - 1; w1 = 0; }
-        else if (keep < 64) { w1 &= (1u << (keep - 32)) - 1; }
-    }
-    const uint32_t cnt = __popc(w0) + __popc(w1);
-    pre[threadIdx.x] = cnt;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        uint32_t v = threadIdx.x >= (unsigned)off ? pre[threadIdx.x - off] : 0;
-        __syncthreads();
-        pre[threadIdx.x] += v;
-        __syncthreads();
-    }
-    uint32_t pos = pre[threadIdx.x] - cnt;
-    for (int b = 0; b < 32; b++)
-        if (w0 >> b & 1) seeds[pos++] = lo + b;
-    for (int b = 0; b < 32; b++)
-        if (w1 >> b & 1) seeds[pos++] = lo + 32 + b;
-    if (threadIdx.x == 1023) *nseeds = pre[1023];
-}
-
 // ------------------------------------------------------------ segments
 
 struct SieveArgs {
-    const uint32_t *seeds;  // ascending primes <= sqrt(limit)
+    const uint32_t *seeds;  // ascending odd primes <= sqrt(limit)
     uint32_t i_med, i_large, nseeds;  // index ranges: [0,i_med) small (3..31 are
                                        // patterned), [i_med,i_large) medium, rest large
     uint32_t imax;          // largest odd index i with 2i+1 <= limit
-    uint32_t *bits;         // out: per segment, bit set = prime
-    uint32_t *counts;       // out: primes per segment
+    int seg_log;            // log2 odd numbers per segment
+    uint32_t *bits;         // out: bit set = prime
+    uint32_t *counts;       // out: primes per unit
     // unit_kind >= 0: keep only the primes p > root (p^2 > 2 unit_n) whose
     // exponent in the quantity of that kind is 1 (all others are 0 there);
     // counts then count the kept primes, and *total gets every odd prime.
@@ -103,13 +68,16 @@ __constant__ uint32_t c_small_primes[10] = {3, 5, 7, 11, 13, 17, 19, 23, 29, 31}
 
 __global__ void __launch_bounds__(kSieveThreads) sieve_segments(SieveArgs a)
 {
-    __shared__ uint32_t bm[kSegWords];
-    __shared__ uint32_t red[kSieveThreads / 32], red_all[kSieveThreads / 32];
+    extern __shared__ uint32_t bm[];
+    __shared__ uint32_t unit_count[kMaxSegUnits], all_count;
     const uint32_t seg = blockIdx.x;
-    const uint32_t ibase = seg * (uint32_t)kSegBits;  // odd index of bit 0
+    const int seg_words = 1 << (a.seg_log - 5);
+    const uint32_t ibase = seg << a.seg_log;  // odd index of bit 0
+    if (threadIdx.x < kMaxSegUnits) unit_count[threadIdx.x] = 0;
+    if (threadIdx.x == 0) all_count = 0;
     // words of this segment at or below the last odd index (the last segment,
     // or the only one of a small limit, is sieved only that far)
-    const uint32_t used = (uint32_t)std::min<uint64_t>(kSegWords, (a.imax - ibase) / 32 + 1);
+    const uint32_t used = (uint32_t)std::min<uint64_t>(seg_words, (a.imax - ibase) / 32 + 1);
     const uint64_t used_bits = 32ull * used;
     // primes 3..31: bit b of word w is odd number x = 2(ibase + 32 w + b) + 1;
     // p | x  <=>  ibase + 32 w + b = (p - 1)/2 (mod p)
@@ -171,9 +139,11 @@ __global__ void __launch_bounds__(kSieveThreads) sieve_segments(SieveArgs a)
         bm[0] = w0;
     }
     __syncthreads();
-    uint32_t cnt = 0, all = 0;
-    uint32_t *out = a.bits + (size_t)seg * kSegWords;
-    for (int w = threadIdx.x; w < kSegWords; w += blockDim.x) {
+    uint32_t all = 0;
+    uint32_t *out = a.bits + (size_t)seg * seg_words;
+    // (a warp's 32 words lie in one unit: units and segments are multiples of
+    // 256 words, the block's threads a multiple of 32)
+    for (int w = threadIdx.x; w < seg_words; w += blockDim.x) {
         const uint64_t i0 = (uint64_t)ibase + 32u * w;
         uint32_t v = w < (int)used ? ~bm[w] : 0u;
         if (i0 > a.imax) v = 0;
@@ -199,102 +169,93 @@ __global__ void __launch_bounds__(kSieveThreads) sieve_segments(SieveArgs a)
             }
         }
         out[w] = v;
-        cnt += __popc(v);
+        const uint32_t cnt = __reduce_add_sync(0xffffffffu, __popc(v));
+        if (lane == 0 && cnt) atomicAdd(&unit_count[w / kUnitWords], cnt);
     }
-    for (int off = 16; off; off >>= 1) {
-        cnt += __shfl_down_sync(0xffffffffu, cnt, off);
-        all += __shfl_down_sync(0xffffffffu, all, off);
-    }
-    if (lane == 0) {
-        red[wid] = cnt;
-        red_all[wid] = all;
-    }
+    all = __reduce_add_sync(0xffffffffu, all);
+    if (lane == 0 && all) atomicAdd(&all_count, all);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t t = 0, ta = 0;
-        for (int k = 0; k < nw; k++) {
-            t += red[k];
-            ta += red_all[k];
-        }
-        a.counts[seg] = t;
-        if (a.unit_kind >= 0) atomicAdd(a.total, ta);
-    }
+    const int units = seg_words / kUnitWords;
+    if ((int)threadIdx.x < units) a.counts[seg * units + threadIdx.x] = unit_count[threadIdx.x];
+    if (threadIdx.x == 0 && a.unit_kind >= 0) atomicAdd(a.total, all_count);
 }
 
 // ----------------------------------------------------------- exponents
 
+// The primes of a unit, in order, by one warp: 32 words at a time (one per
+// lane), a warp scan of the bit counts placing each lane's primes in the
+// warp's shared stage (32 x 32 words); f(tot) then takes the stage's tot
+// primes.  f must not change the stage's order; the warp is converged.
+template <class F>
+__device__ __forceinline__ void unit_primes(const uint32_t *bits, uint32_t unit, uint32_t *st,
+                                            F &&f)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t *b = bits + (size_t)unit * kUnitWords;
+    uint32_t w[kUnitWords / 32];
+#pragma unroll
+    for (int it = 0; it < kUnitWords / 32; it++) w[it] = b[it * 32 + lane];
+#pragma unroll
+    for (int it = 0; it < kUnitWords / 32; it++) {
+        const uint32_t c = __popc(w[it]);
+        uint32_t incl = c;
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += v;
+        }
+        const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
+        uint32_t at = incl - c;
+        const uint32_t ibase = (unit << kUnitLog) + 32u * (it * 32 + lane);
+        for (uint32_t m = w[it]; m; m &= m - 1) st[at++] = 2 * (ibase + __ffs(m) - 1) + 1;
+        __syncwarp();
+        f(tot);
+        __syncwarp();
+    }
+}
+
+constexpr int kExpandThreads = 256;
+constexpr int kExpandWarps = kExpandThreads / 32;
+
 struct ExpandArgs {
     const uint32_t *bits;
-    const uint32_t *seg_offsets;  // exclusive scan of the per-segment counts
-    Ratio r;                      // the quantity (a kind of n, or a factorial ratio)
-    int has_two;                  // limit >= 2: item 0 is the prime 2
-    uint64_t *items;              // out: (e << 32) | p, all primes ascending
+    const uint32_t *unit_offsets;  // exclusive scan of the per-unit counts
+    uint32_t units;
+    Ratio r;                       // the quantity (a kind of n, or a factorial ratio)
+    uint64_t *items;               // out: (e << 32) | p, all primes ascending (item 0: 2)
     unsigned int *max_e;
     unsigned int *negative;
 };
 
-// One block per segment: list its primes in order with their exponents.
-__global__ void __launch_bounds__(kSieveThreads) expand_exponents(ExpandArgs a)
+// One warp per unit: its primes in order with their exponents, one prime per
+// lane at a time (a lane per word, with as many primes as the word holds, left
+// most lanes waiting: 163 -> 43 us at the limit 10^7 with three terms).
+__global__ void __launch_bounds__(kExpandThreads) expand_exponents(ExpandArgs a)
 {
-    __shared__ uint32_t pre[kSieveThreads];
-    __shared__ uint32_t red[kSieveThreads / 32];
-    constexpr int kWordsPerThread = kSegWords / kSieveThreads;  // 16
-    const uint32_t seg = blockIdx.x;
-    const uint32_t *bits = a.bits + (size_t)seg * kSegWords + threadIdx.x * kWordsPerThread;
-    uint32_t w[kWordsPerThread];
-    uint32_t cnt = 0;
-#pragma unroll
-    for (int k = 0; k < kWordsPerThread; k++) {
-        w[k] = bits[k];
-        cnt += __popc(w[k]);
-    }
-    pre[threadIdx.x] = cnt;
-    __syncthreads();
-    for (int off = 1; off < kSieveThreads; off <<= 1) {
-        const uint32_t v = threadIdx.x >= (unsigned)off ? pre[threadIdx.x - off] : 0;
-        __syncthreads();
-        pre[threadIdx.x] += v;
-        __syncthreads();
-    }
-    size_t pos = (size_t)a.seg_offsets[seg] + pre[threadIdx.x] - cnt + (a.has_two ? 1 : 0);
-    const uint32_t ibase = seg * (uint32_t)kSegBits + threadIdx.x * kWordsPerThread * 32;
+    __shared__ uint32_t stage[kExpandWarps][32 * 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t unit = blockIdx.x * kExpandWarps + wid;
     uint32_t emax = 0, neg = 0;
-#pragma unroll
-    for (int k = 0; k < kWordsPerThread; k++) {
-        uint32_t v = w[k];
-        while (v) {
-            const int b = __ffs(v) - 1;
-            v &= v - 1;
-            const uint32_t p = 2 * (ibase + 32 * k + b) + 1;
-            const int64_t e = exponent_of(p, a.r);
-            if (e < 0) neg = 1;
-            const uint32_t eu = e < 0 ? 0u : (uint32_t)e;
-            emax = max(emax, eu);
-            a.items[pos++] = ((uint64_t)eu << 32) | p;
-        }
-    }
-    if (seg == 0 && threadIdx.x == 0 && a.has_two) {
-        const int64_t e = exponent_of(2, a.r);
+    auto put = [&](size_t at, uint32_t p) {
+        const int64_t e = exponent_of(p, a.r);
         if (e < 0) neg = 1;
         const uint32_t eu = e < 0 ? 0u : (uint32_t)e;
         emax = max(emax, eu);
-        a.items[0] = ((uint64_t)eu << 32) | 2u;
+        a.items[at] = ((uint64_t)eu << 32) | p;
+    };
+    if (unit < a.units) {
+        size_t pos = (size_t)a.unit_offsets[unit] + 1;
+        uint32_t *st = stage[wid];
+        unit_primes(a.bits, unit, st, [&](uint32_t tot) {
+            for (uint32_t k = lane; k < tot; k += 32) put(pos + k, st[k]);
+            pos += tot;
+        });
+        if (unit == 0 && lane == 0) put(0, 2u);
     }
-    for (int off = 16; off; off >>= 1) {
-        emax = max(emax, __shfl_down_sync(0xffffffffu, emax, off));
-        neg |= __shfl_down_sync(0xffffffffu, neg, off);
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) red[wid] = emax | (neg ? 0x80000000u : 0u);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t m = 0, ng = 0;
-        for (int k = 0; k < kSieveThreads / 32; k++) {
-            m = max(m, red[k] & 0x7fffffffu);
-            ng |= red[k] >> 31;
-        }
-        atomicMax(a.max_e, m);
-        if (ng) atomicOr(a.negative, 1u);
+    emax = __reduce_max_sync(0xffffffffu, emax);
+    neg = __reduce_or_sync(0xffffffffu, neg);
+    if (lane == 0) {
+        if (emax) atomicMax(a.max_e, emax);
+        if (neg) atomicOr(a.negative, 1u);
     }
 }
 
@@ -405,72 +366,132 @@ __global__ void group_starts(const uint64_t *items, size_t count, uint64_t *star
     }
 }
 
-// One block per segment: the primes of its bitmap in ascending order, written
-// to primes[first + seg_offsets[seg] + ...]; with_two also puts 2 at primes[0].
-// Each warp owns 1024 consecutive words and takes them 32 at a time (one word
-// a lane): a warp scan of the bit counts places each lane's primes in a
-// per-warp shared stage, which the warp then copies out contiguously.
-constexpr int kExpandThreads = 256;
-constexpr int kExpandWarps = kExpandThreads / 32;
-constexpr int kWordsPerWarp = kSegWords / kExpandWarps;  // 1024
-constexpr int kExpandIters = kWordsPerWarp / 32;          // 32
-
+// The primes of the bitmap in ascending order, written to primes[first + ...]
+// (with_two: 2 at primes[0]); one warp per unit.
 __global__ void __launch_bounds__(kExpandThreads) expand_primes(const uint32_t *bits,
-                                                               const uint32_t *seg_offsets,
-                                                               uint32_t *primes, uint32_t first,
-                                                               int with_two)
+                                                               const uint32_t *unit_offsets,
+                                                               uint32_t units, uint32_t *primes,
+                                                               uint32_t first, int with_two)
 {
     __shared__ uint32_t stage[kExpandWarps][32 * 32];
-    __shared__ uint32_t wsum[kExpandWarps];
-    const uint32_t seg = blockIdx.x;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint32_t word0 = (uint32_t)wid * kWordsPerWarp;
-    const uint32_t *b = bits + (size_t)seg * kSegWords + word0;
-    uint32_t w[kExpandIters];
-    uint32_t cnt = 0;
-#pragma unroll
-    for (int it = 0; it < kExpandIters; it++) {
-        w[it] = b[it * 32 + lane];
-        cnt += __popc(w[it]);
-    }
-    for (int off = 16; off; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
-    if (lane == 0) wsum[wid] = cnt;
-    __syncthreads();
-    size_t pos = (size_t)seg_offsets[seg] + first;
-    for (int k = 0; k < wid; k++) pos += wsum[k];
+    const uint32_t unit = blockIdx.x * kExpandWarps + wid;
+    if (with_two && blockIdx.x == 0 && threadIdx.x == 0) primes[0] = 2;
+    if (unit >= units) return;
+    size_t pos = (size_t)unit_offsets[unit] + first;
     uint32_t *st = stage[wid];
-#pragma unroll
-    for (int it = 0; it < kExpandIters; it++) {
-        const uint32_t c = __popc(w[it]);
-        uint32_t incl = c;
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += v;
-        }
-        const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
-        uint32_t at = incl - c;
-        const uint32_t ibase = seg * (uint32_t)kSegBits + 32u * (word0 + it * 32 + lane);
-        for (uint32_t m = w[it]; m; m &= m - 1) st[at++] = 2 * (ibase + __ffs(m) - 1) + 1;
-        __syncwarp();
+    unit_primes(bits, unit, st, [&](uint32_t tot) {
         for (uint32_t k = lane; k < tot; k += 32) primes[pos + k] = st[k];
         pos += tot;
-        __syncwarp();
-    }
-    if (with_two && seg == 0 && threadIdx.x == 0) primes[0] = 2;
+    });
 }
 
-// The exponents of the seed primes (all primes <= sqrt(2n)), one thread each.
-__global__ void seed_items(const uint32_t *seeds, uint32_t ns, Ratio r, uint64_t *items,
-                           unsigned int *max_e, unsigned int *negative)
+// The seed primes of a binomial kind grouped by exponent, by one block: the
+// exponents (one prime per thread at a time), then a stable counting sort
+// (every thread counts a stretch of consecutive seeds per exponent, one warp
+// per exponent scans its counts over the threads), primes with e = 0 dropped.
+// Exponents are at most 31 (p^e <= 2n).  sorted takes the grouped primes, info
+// the groups beside the sieve's counts.
+constexpr int kSeedThreads = 512;
+constexpr int kMaxSeeds = 6542;  // primes below 2^16
+constexpr int kSeedsPerThread = (kMaxSeeds + kSeedThreads - 1) / kSeedThreads;
+constexpr size_t kSeedSmem = (size_t)kMaxSeedGroups * kSeedThreads * 2;
+
+__global__ void __launch_bounds__(kSeedThreads) group_seeds(const uint32_t *seeds, uint32_t ns,
+                                                           Ratio r, const uint32_t *kept,
+                                                           const uint32_t *total, uint32_t *sorted,
+                                                           Phase1Info *info)
 {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ns) return;
-    const uint32_t p = seeds[i];
-    const int64_t e = exponent_of(p, r);
-    if (e < 0) atomicOr(negative, 1u);
-    const uint32_t eu = e < 0 ? 0u : (uint32_t)e;
-    atomicMax(max_e, eu);
-    items[i] = ((uint64_t)eu << 32) | p;
+    extern __shared__ uint16_t cnt[];  // [exponent][thread]
+    __shared__ uint8_t ex[kMaxSeeds];
+    __shared__ uint32_t bin_total[kMaxSeedGroups], bin_base[kMaxSeedGroups], negative;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    for (int i = tid; i < kMaxSeedGroups * kSeedThreads; i += kSeedThreads) cnt[i] = 0;
+    if (tid == 0) negative = 0;
+    __syncthreads();
+    for (uint32_t i = tid; i < ns; i += kSeedThreads) {
+        const int64_t e = exponent_of(seeds[i], r);
+        if (e < 0) atomicOr(&negative, 1u);
+        ex[i] = e < 0 ? 0 : (uint8_t)e;
+    }
+    __syncthreads();
+    const uint32_t i0 = tid * kSeedsPerThread, i1 = min(ns, i0 + kSeedsPerThread);
+    for (uint32_t i = i0; i < i1; i++) cnt[ex[i] * kSeedThreads + tid]++;
+    __syncthreads();
+    for (int e = wid; e < kMaxSeedGroups; e += kSeedThreads / 32) {
+        uint32_t run = 0;
+        for (int t = lane; t < kSeedThreads; t += 32) {
+            const uint32_t c = cnt[e * kSeedThreads + t];
+            uint32_t incl = c;
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += v;
+            }
+            cnt[e * kSeedThreads + t] = (uint16_t)(run + incl - c);
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) bin_total[e] = run;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        uint32_t at = 0, ng = 0;
+        for (int e = 1; e < kMaxSeedGroups; e++) {
+            bin_base[e] = at;
+            if (bin_total[e]) {
+                info->exp[ng] = e;
+                info->off[ng] = at;
+                ng++;
+            }
+            at += bin_total[e];
+        }
+        info->off[ng] = at;
+        info->ngroups = ng;
+        info->negative = negative;
+        info->kept = *kept;
+        info->total = *total;
+    }
+    __syncthreads();
+    for (uint32_t i = i0; i < i1; i++) {
+        const uint32_t e = ex[i];
+        if (e) sorted[bin_base[e] + cnt[e * kSeedThreads + tid]++] = seeds[i];
+    }
+}
+
+// The CSR of a binomial kind: blocks [0, expand_blocks) write the large primes
+// behind the n1 seeds with e = 1; the last block writes the grouped seeds
+// around them and the group table.
+struct CsrArgs {
+    const uint32_t *bits, *unit_offsets;
+    uint32_t units, expand_blocks;
+    const uint32_t *sorted;   // grouped seeds
+    uint32_t nsorted, n1, nl; // all of them, those with e = 1, the large primes
+    uint32_t *primes;
+    uint32_t ng;
+    uint64_t *exps, *offs;
+    uint64_t h_exps[kMaxSeedGroups + 1], h_offs[kMaxSeedGroups + 2];
+};
+
+__global__ void __launch_bounds__(kExpandThreads) write_csr(CsrArgs a)
+{
+    __shared__ uint32_t stage[kExpandWarps][32 * 32];
+    if (blockIdx.x == a.expand_blocks) {
+        for (uint32_t i = threadIdx.x; i < a.nsorted; i += kExpandThreads)
+            a.primes[i < a.n1 ? i : i + a.nl] = a.sorted[i];
+        for (uint32_t i = threadIdx.x; i <= a.ng; i += kExpandThreads) {
+            a.exps[i] = a.h_exps[i];
+            a.offs[i] = a.h_offs[i];
+        }
+        return;
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t unit = blockIdx.x * kExpandWarps + wid;
+    if (unit >= a.units) return;
+    size_t pos = (size_t)a.unit_offsets[unit] + a.n1;
+    uint32_t *st = stage[wid];
+    unit_primes(a.bits, unit, st, [&](uint32_t tot) {
+        for (uint32_t k = lane; k < tot; k += 32) a.primes[pos + k] = st[k];
+        pos += tot;
+    });
 }
 
 // ------------------------------------------------------------ host side
@@ -483,15 +504,35 @@ static uint64_t isqrt64(uint64_t x)
     return r;
 }
 
-// The segmented sieve up to `limit` (>= 2): per-segment bitmaps of the odd
-// primes and the exclusive scan of their counts.  sieved = pi(limit).
-// With unit_kind >= 0 (a binomial kind of n, limit = 2n) the bitmaps keep only
-// the primes above sqrt(2n) with exponent 1, the offsets scan their counts
-// (kept in total), and the seeds are exactly the primes up to sqrt(2n).
+// A device word, read back (through the context's pinned word).
+static uint64_t read_word(Ctx &c, const uint32_t *d, cudaStream_t s)
+{
+    uint32_t *h = reinterpret_cast<uint32_t *>(c.host_word);
+    CAT_CUDA(cudaMemcpyAsync(h, d, 4, cudaMemcpyDeviceToHost, s));
+    CAT_CUDA(cudaStreamSynchronize(s));
+    return *h;
+}
+
+// log2 odd numbers per segment: 2^18 (32 KiB of bitmap) when that still gives
+// every SM several rounds of its four resident blocks, down to 2^13 for short
+// sieves, so that their few numbers spread over the SMs (limits 2 10^5: 26 ->
+// 17 us, 10^7: 37 -> 18, 10^8: 73 -> 61, 2 10^8: 97 either way).
+static int segment_log(uint32_t odds, int num_sms)
+{
+    int lg = kMaxSegLog;
+    while (lg > kUnitLog && (odds >> lg) < 8u * (uint32_t)num_sms) lg--;
+    return lg;
+}
+
+// The segmented sieve up to `limit` (>= 2): the bitmap of the odd primes and
+// the exclusive scan of the units' counts, whose sum goes to words[0]; nothing
+// is read back.  With unit_kind >= 0 (a binomial kind of n, limit = 2n) the
+// bitmap keeps only the primes above sqrt(2n) with exponent 1, words[1] gets
+// the number of all odd primes, and the seeds are exactly the primes up to
+// sqrt(2n).
 struct SieveOut {
-    DevBuf<uint32_t> bits, offsets, seeds;
-    uint32_t nsegs = 0, nseeds = 0;
-    uint64_t sieved = 0, kept = 0;
+    DevBuf<uint32_t> bits, offsets, words;
+    uint32_t units = 0, nseeds = 0;
 };
 
 static SieveOut run_sieve(Ctx &c, uint64_t limit, cudaStream_t s, int unit_kind = -1,
@@ -499,51 +540,31 @@ static SieveOut run_sieve(Ctx &c, uint64_t limit, cudaStream_t s, int unit_kind 
 {
     SieveOut o;
     const uint64_t root = isqrt64(limit);
-    o.seeds = DevBuf<uint32_t>(c, 8192, s);
-    DevBuf<uint32_t> &seeds = o.seeds;
-    DevBuf<uint32_t> nseeds(c, 2, s);
-    CAT_CUDA(cudaMemsetAsync(nseeds.get(), 0, 8, s));
-    seed_sieve<<<1, 1024, 0, s>>>((uint32_t)root, seeds.get(), nseeds.get());
-    CAT_LAUNCH("seed_sieve");
-    uint32_t ns = 0;
-    CAT_CUDA(cudaMemcpyAsync(&ns, nseeds.get(), 4, cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaStreamSynchronize(s));
-    o.nseeds = ns;
-    std::vector<uint32_t> hs(ns);
-    if (ns)
-        CAT_CUDA(cudaMemcpyAsync(hs.data(), seeds.get(), 4 * ns, cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaStreamSynchronize(s));
+    auto below = [&](uint64_t x) {  // seeds <= x
+        return (uint32_t)(std::upper_bound(c.host_seeds.begin(), c.host_seeds.end(), x) -
+                          c.host_seeds.begin());
+    };
+    o.nseeds = below(root);
     // odd seeds only for the segment sieve
-    const uint32_t *odd = seeds.get() + (ns > 0 && hs[0] == 2 ? 1 : 0);
-    const uint32_t nodd = ns > 0 ? ns - 1 : 0;
-    uint32_t i_med = 0, i_large = 0;
-    for (uint32_t k = 0; k < nodd; k++) {
-        const uint32_t p = hs[k + 1];
-        if (p < kMediumPrime) i_med = k + 1;
-        if (p < kLargePrime) i_large = k + 1;
-    }
-    // segments over odd indices 0..imax (odd number 2i+1 <= limit)
+    const uint32_t nodd = o.nseeds ? o.nseeds - 1 : 0;
+    const uint32_t i_med = std::min(nodd, below(kMediumPrime - 1) - 1);
+    const uint32_t i_large = std::min(nodd, below(kLargePrime - 1) - 1);
+    // odd indices 0..imax (odd number 2i+1 <= limit)
     const uint32_t imax = (uint32_t)((limit - 1) / 2);
-    o.nsegs = imax / kSegBits + 1;
-    o.bits = DevBuf<uint32_t>(c, (size_t)o.nsegs * kSegWords, s);
-    o.offsets = DevBuf<uint32_t>(c, o.nsegs, s);
-    SieveArgs sa{odd, i_med, i_large, nodd, imax, o.bits.get(), o.offsets.get(),
-                 unit_kind, unit_n, (uint32_t)root, nseeds.get() + 1};
+    const int lg = segment_log(imax, c.num_sms);
+    const uint32_t nsegs = (imax >> lg) + 1;
+    o.units = nsegs << (lg - kUnitLog);
+    o.bits = DevBuf<uint32_t>(c, (size_t)o.units * kUnitWords, s);
+    o.offsets = DevBuf<uint32_t>(c, o.units, s);
+    o.words = DevBuf<uint32_t>(c, 2, s);
+    CAT_CUDA(cudaMemsetAsync(o.words.get(), 0, 8, s));
+    SieveArgs sa{c.seeds + 1, i_med, i_large, nodd, imax, lg, o.bits.get(), o.offsets.get(),
+                 unit_kind, unit_n, (uint32_t)root, o.words.get() + 1};
     const int tok = prof_begin(c, "sieve_segments", s);
-    sieve_segments<<<o.nsegs, kSieveThreads, 0, s>>>(sa);
+    sieve_segments<<<nsegs, std::min(kSieveThreads, 1 << (lg - 5)), (size_t)4 << (lg - 5), s>>>(sa);
     CAT_LAUNCH("sieve_segments");
-    prof_end(c, tok, s, 4.0 * (double)o.nsegs * kSegWords);
-    uint32_t last_count = 0;
-    CAT_CUDA(cudaMemcpyAsync(&last_count, o.offsets.get() + o.nsegs - 1, 4,
-                             cudaMemcpyDeviceToHost, s));
-    exclusive_scan_u32(c, o.offsets.get(), o.nsegs, s);
-    uint32_t last_off = 0, total = 0;
-    CAT_CUDA(cudaMemcpyAsync(&last_off, o.offsets.get() + o.nsegs - 1, 4,
-                             cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaMemcpyAsync(&total, nseeds.get() + 1, 4, cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaStreamSynchronize(s));
-    o.kept = (uint64_t)last_off + last_count;
-    o.sieved = (unit_kind >= 0 ? (uint64_t)total : o.kept) + 1;  // plus the prime 2
+    prof_end(c, tok, s, 4.0 * (double)o.units * kUnitWords);
+    exclusive_scan_u32(c, o.offsets.get(), o.units, s, o.words.get());
     return o;
 }
 
@@ -634,59 +655,59 @@ static Grouped group_items(Ctx &c, DevBuf<uint64_t> &items, size_t count, uint32
 // Catalan or central binomial kinds with n >= 2.  Every prime above sqrt(2n)
 // has exponent 0 or 1; the sieve keeps those with 1 and they are written in
 // order straight into the e = 1 group, after the seed primes with e = 1.  The
-// seed primes (<= sqrt(2n), fewer than 6600) take Legendre's formula and the
-// radix grouping; their groups with e >= 2 follow.
-static void factor_unit(Ctx &c, const Ratio &r, uint64_t limit, DevBuf<uint32_t> &primes_out,
-                        std::vector<uint64_t> &h_exps, std::vector<uint64_t> &h_offs,
-                        uint64_t &sieved, uint64_t &npos, cudaStream_t s)
+// seed primes (<= sqrt(2n), at most 6542) are grouped by one block; their
+// groups with e >= 2 follow.
+static void factor_unit(Ctx &c, const Ratio &r, uint64_t limit, cat_factorization *out,
+                        cudaStream_t s)
 {
     SieveOut sv = run_sieve(c, limit, s, r.kind, r.n);
-    sieved = sv.sieved;
     const uint32_t ns = sv.nseeds;
-    DevBuf<uint64_t> items(c, std::max<uint32_t>(ns, 1), s);
-    DevBuf<unsigned int> flags(c, 2, s);
-    CAT_CUDA(cudaMemsetAsync(flags.get(), 0, 8, s));
-    if (ns) {
-        seed_items<<<(ns + 255) / 256, 256, 0, s>>>(sv.seeds.get(), ns, r, items.get(),
-                                                    flags.get(), flags.get() + 1);
-        CAT_LAUNCH("seed_items");
-    }
-    unsigned int hf[2];
-    CAT_CUDA(cudaMemcpyAsync(hf, flags.get(), 8, cudaMemcpyDeviceToHost, s));
+    DevBuf<uint32_t> sorted(c, std::max<uint32_t>(ns, 1), s);
+    DevBuf<Phase1Info> d_info(c, 1, s);
+    int tok = prof_begin(c, "group_seeds", s);
+    group_seeds<<<1, kSeedThreads, kSeedSmem, s>>>(c.seeds, ns, r, sv.words.get(),
+                                                   sv.words.get() + 1, sorted.get(), d_info.get());
+    CAT_LAUNCH("group_seeds");
+    prof_end(c, tok, s, 8.0 * (double)ns);
+    Phase1Info &h = *c.host_info;
+    CAT_CUDA(cudaMemcpyAsync(&h, d_info.get(), sizeof(h), cudaMemcpyDeviceToHost, s));
     CAT_CUDA(cudaStreamSynchronize(s));
-    if (hf[1]) fail(CAT_ENOTINTEGRAL, "a prime exponent is negative");
-    Grouped g = group_items(c, items, ns, hf[0], s);
-    const uint64_t nl = sv.kept;
-    const uint64_t n1 = (!g.exps.empty() && g.exps[0] == 1) ? g.offs[1] : 0;
-    npos = g.count + nl;
-    h_exps.clear();
-    h_offs.assign(1, 0);
-    if (npos == 0) return;
-    primes_out = DevBuf<uint32_t>(c, npos, s);
-    uint32_t *d = primes_out.get();
-    if (n1)
-        CAT_CUDA(cudaMemcpyAsync(d, g.primes.get(), 4 * n1, cudaMemcpyDeviceToDevice, s));
-    if (nl) {
-        const int tok = prof_begin(c, "expand_primes", s);
-        expand_primes<<<sv.nsegs, kExpandThreads, 0, s>>>(sv.bits.get(), sv.offsets.get(),
-                                                           d + n1, 0, 0);
-        CAT_LAUNCH("expand_primes");
-        prof_end(c, tok, s, 4.0 * (double)sv.nsegs * kSegWords + 4.0 * (double)nl);
+    if (h.negative) fail(CAT_ENOTINTEGRAL, "a prime exponent is negative");
+    CsrArgs a{};
+    a.nl = h.kept;
+    a.n1 = h.ngroups && h.exp[0] == 1 ? h.off[1] : 0;
+    a.nsorted = h.off[h.ngroups];
+    const uint64_t npos = (uint64_t)a.nsorted + a.nl;
+    if (a.n1 + a.nl) a.h_exps[a.ng++] = 1;
+    for (uint32_t k = a.n1 ? 1 : 0; k < h.ngroups; k++) {
+        a.h_offs[a.ng] = (uint64_t)h.off[k] + a.nl;
+        a.h_exps[a.ng++] = h.exp[k];
     }
-    if (g.count > n1)
-        CAT_CUDA(cudaMemcpyAsync(d + n1 + nl, g.primes.get() + n1, 4 * (g.count - n1),
-                                 cudaMemcpyDeviceToDevice, s));
-    h_offs.clear();
-    if (n1 + nl) {
-        h_exps.push_back(1);
-        h_offs.push_back(0);
-    }
-    for (size_t k = n1 ? 1 : 0; k < g.exps.size(); k++) {
-        h_exps.push_back(g.exps[k]);
-        h_offs.push_back(g.offs[k] + nl);
-    }
-    h_offs.push_back(npos);
-    CAT_CUDA(cudaStreamSynchronize(s));  // the copies read g.primes before it is freed
+    a.h_offs[a.ng] = npos;
+    DevBuf<uint32_t> primes(c, std::max<uint64_t>(npos, 1), s);
+    DevBuf<uint64_t> d_exps(c, a.ng + 1, s), d_offs(c, a.ng + 1, s);
+    a.bits = sv.bits.get();
+    a.unit_offsets = sv.offsets.get();
+    a.units = sv.units;
+    a.expand_blocks = a.nl ? (sv.units + kExpandWarps - 1) / kExpandWarps : 0;
+    a.sorted = sorted.get();
+    a.primes = primes.get();
+    a.exps = d_exps.get();
+    a.offs = d_offs.get();
+    tok = prof_begin(c, "write_csr", s);
+    write_csr<<<a.expand_blocks + 1, kExpandThreads, 0, s>>>(a);
+    CAT_LAUNCH("write_csr");
+    prof_end(c, tok, s, 4.0 * (double)sv.units * kUnitWords + 4.0 * (double)npos);
+    out->host_exps = new uint64_t[a.ng + 1];
+    out->host_offsets = new uint64_t[a.ng + 1];
+    std::copy(a.h_exps, a.h_exps + a.ng + 1, out->host_exps);
+    std::copy(a.h_offs, a.h_offs + a.ng + 1, out->host_offsets);
+    out->num_groups = a.ng;
+    out->num_primes = npos;
+    out->primes_sieved = (uint64_t)h.total + 1;  // plus the prime 2
+    out->exps = d_exps.release();
+    out->offsets = d_offs.release();
+    out->primes = primes.release();
 }
 
 // Phase 1 for any Ratio: primes up to the largest factorial argument (2n for
@@ -703,28 +724,28 @@ void factor_ratio(Ctx &c, const Ratio &r, cat_factorization *out, cudaStream_t s
         for (int i = 0; i < r.ka; i++) limit = std::max<uint64_t>(limit, r.a[i]);
         for (int j = 0; j < r.kb; j++) limit = std::max<uint64_t>(limit, r.b[j]);
     }
+    if ((kind == CAT_CATALAN || kind == CAT_CENTRAL_BINOMIAL) && n >= 2) {
+        factor_unit(c, r, limit, out, s);
+        return;
+    }
     std::vector<uint64_t> h_exps, h_offs{0};
     DevBuf<uint32_t> primes_out;
     uint64_t sieved = 0, npos = 0;
-    if ((kind == CAT_CATALAN || kind == CAT_CENTRAL_BINOMIAL) && n >= 2) {
-        factor_unit(c, r, limit, primes_out, h_exps, h_offs, sieved, npos, s);
-    } else if (limit >= 2) {
+    if (limit >= 2) {
         SieveOut sv = run_sieve(c, limit, s);
-        const uint32_t nsegs = sv.nsegs;
-        sieved = sv.sieved;
+        sieved = read_word(c, sv.words.get(), s) + 1;  // plus the prime 2
         // exponents
         DevBuf<uint64_t> items(c, sieved, s);
         DevBuf<unsigned int> flags(c, 2, s);
         CAT_CUDA(cudaMemsetAsync(flags.get(), 0, 8, s));
-        ExpandArgs ea{sv.bits.get(), sv.offsets.get(), r, 1, items.get(), flags.get(),
+        ExpandArgs ea{sv.bits.get(), sv.offsets.get(), sv.units, r, items.get(), flags.get(),
                       flags.get() + 1};
         const int tok = prof_begin(c, "expand_exponents", s);
-        expand_exponents<<<nsegs, kSieveThreads, 0, s>>>(ea);
+        expand_exponents<<<(sv.units + kExpandWarps - 1) / kExpandWarps, kExpandThreads, 0, s>>>(
+            ea);
         CAT_LAUNCH("expand_exponents");
-        prof_end(c, tok, s, 4.0 * (double)nsegs * kSegWords + 8.0 * (double)sieved);
-        sv.bits.reset();
-        sv.offsets.reset();
-        sv.seeds.reset();
+        prof_end(c, tok, s, 4.0 * (double)sv.units * kUnitWords + 8.0 * (double)sieved);
+        sv = SieveOut{};
         unsigned int hf[2];
         CAT_CUDA(cudaMemcpyAsync(hf, flags.get(), 8, cudaMemcpyDeviceToHost, s));
         CAT_CUDA(cudaStreamSynchronize(s));
@@ -761,13 +782,14 @@ DevBuf<uint32_t> sieve_primes(Ctx &c, uint64_t limit, uint64_t *count, cudaStrea
     *count = 0;
     if (limit < 2) return DevBuf<uint32_t>(c, 1, s);
     SieveOut sv = run_sieve(c, limit, s);
-    DevBuf<uint32_t> primes(c, sv.sieved, s);
+    const uint64_t sieved = read_word(c, sv.words.get(), s) + 1;
+    DevBuf<uint32_t> primes(c, sieved, s);
     const int tok = prof_begin(c, "expand_primes", s);
-    expand_primes<<<sv.nsegs, kExpandThreads, 0, s>>>(sv.bits.get(), sv.offsets.get(),
-                                                       primes.get(), 1, 1);
+    expand_primes<<<(sv.units + kExpandWarps - 1) / kExpandWarps, kExpandThreads, 0, s>>>(
+        sv.bits.get(), sv.offsets.get(), sv.units, primes.get(), 1, 1);
     CAT_LAUNCH("expand_primes");
-    prof_end(c, tok, s, 4.0 * (double)sv.nsegs * kSegWords + 4.0 * (double)sv.sieved);
-    *count = sv.sieved;
+    prof_end(c, tok, s, 4.0 * (double)sv.units * kUnitWords + 4.0 * (double)sieved);
+    *count = sieved;
     return primes;
 }
 

@@ -50,8 +50,9 @@ __global__ void __launch_bounds__(kScanThreads) scan_block_sums(const uint32_t *
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-// Single block: exclusive scan of n values (any n), chunk by chunk.
-__global__ void __launch_bounds__(kScanThreads) scan_single(uint32_t *d, size_t n)
+// Single block: exclusive scan of n values (any n), chunk by chunk; their sum
+// goes to *sum (when set).
+__global__ void __launch_bounds__(kScanThreads) scan_single(uint32_t *d, size_t n, uint32_t *sum)
 {
     __shared__ uint32_t wsm[32];
     uint32_t run = 0;
@@ -73,6 +74,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_single(uint32_t *d, size_t 
         run += total;
         __syncthreads();
     }
+    if (sum && threadIdx.x == 0) *sum = run;
 }
 
 __global__ void __launch_bounds__(kScanThreads) scan_apply(uint32_t *d, size_t n,
@@ -95,19 +97,23 @@ __global__ void __launch_bounds__(kScanThreads) scan_apply(uint32_t *d, size_t n
     }
 }
 
-void exclusive_scan_u32(Ctx &c, uint32_t *data, size_t n, cudaStream_t s)
+// sum (a device word), when given, takes the sum of all n values.
+void exclusive_scan_u32(Ctx &c, uint32_t *data, size_t n, cudaStream_t s, uint32_t *sum)
 {
-    if (n == 0) return;
+    if (n == 0) {
+        if (sum) CAT_CUDA(cudaMemsetAsync(sum, 0, 4, s));
+        return;
+    }
     const size_t blocks = (n + kScanChunk - 1) / kScanChunk;
     if (blocks <= 4) {
-        scan_single<<<1, kScanThreads, 0, s>>>(data, n);
+        scan_single<<<1, kScanThreads, 0, s>>>(data, n, sum);
         CAT_LAUNCH("scan_single");
         return;
     }
     DevBuf<uint32_t> sums(c, blocks, s);
     scan_block_sums<<<(unsigned)blocks, kScanThreads, 0, s>>>(data, n, sums.get());
     CAT_LAUNCH("scan_block_sums");
-    scan_single<<<1, kScanThreads, 0, s>>>(sums.get(), blocks);
+    scan_single<<<1, kScanThreads, 0, s>>>(sums.get(), blocks, sum);
     CAT_LAUNCH("scan_single");
     scan_apply<<<(unsigned)blocks, kScanThreads, 0, s>>>(data, n, sums.get());
     CAT_LAUNCH("scan_apply");
