@@ -84,6 +84,17 @@ void copy_out(cat::Ctx &c, const cat::Big &r, uint32_t *out, size_t cap, size_t 
     (void)c;
 }
 
+// The caller's buffer as the place of a result of at most `bound` limbs.
+cat::Direct direct_out(uint32_t *out, size_t cap, size_t bound)
+{
+    cat::Direct d;
+    if (cap >= bound) {
+        d.out = out;
+        d.len = bound;
+    }
+    return d;
+}
+
 }  // namespace
 
 extern "C" {
@@ -293,10 +304,13 @@ int cat_exact(cat_ctx *ctx, int kind, uint64_t n, uint32_t *out, size_t cap,
                 return;
             }
             // the primes are at most the sieve limit
+            cat::Direct direct = direct_out(out, cap, cat::bound_limbs(n, kind));
             cat::Big r = cat::reconstruct(ctx->c, &f, s,
-                                          cat::bits_below(kind == CAT_FACTORIAL ? n : 2 * n));
+                                          cat::bits_below(kind == CAT_FACTORIAL ? n : 2 * n),
+                                          &direct);
             cat::factor_free(ctx->c, &f);
-            copy_out(ctx->c, r, out, cap, out_len, s);
+            if (direct.used) *out_len = r.n;
+            else copy_out(ctx->c, r, out, cap, out_len, s);
         } catch (...) {
             cat::factor_free(ctx->c, &f);
             throw;
@@ -339,9 +353,11 @@ int cat_ratio_exact(cat_ctx *ctx, const uint64_t *a, int ka, const uint64_t *b, 
             }
             uint64_t top = 1;  // the primes are at most the largest numerator term
             for (int i = 0; i < q.ka; i++) top = std::max<uint64_t>(top, q.a[i]);
-            cat::Big r = cat::reconstruct(ctx->c, &f, s, cat::bits_below(top));
+            cat::Direct direct = direct_out(out, cap, cat::ratio_bound_limbs(q));
+            cat::Big r = cat::reconstruct(ctx->c, &f, s, cat::bits_below(top), &direct);
             cat::factor_free(ctx->c, &f);
-            copy_out(ctx->c, r, out, cap, out_len, s);
+            if (direct.used) *out_len = r.n;
+            else copy_out(ctx->c, r, out, cap, out_len, s);
         } catch (...) {
             cat::factor_free(ctx->c, &f);
             throw;

@@ -612,6 +612,11 @@ bool comba_level(Ctx &c, const uint32_t *in, size_t slot, size_t nprod, uint32_t
 void ntt_level(Ctx &c, const uint32_t *level, size_t slot, size_t nprod, uint32_t *out,
                cudaStream_t s, const uint32_t *out_index = nullptr,
                const uint32_t *out_index_host = nullptr);
+// Whether the product of two slot-limb nodes takes one transform.
+bool ntt_level_whole(const Ctx &c, size_t slot);
+// That product (adjacent nodes at `pair`), which fits len <= 2 slot limbs, into
+// out[0 .. len).
+void ntt_pair(Ctx &c, const uint32_t *pair, size_t slot, uint32_t *out, size_t len, cudaStream_t s);
 
 // out[0 .. na+nb) = a * b (exact, zero-padded).  out must hold na + nb limbs.
 void mul_into(Ctx &c, const uint32_t *a, size_t na, const uint32_t *b, size_t nb,
@@ -641,13 +646,31 @@ size_t normalized_length(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s);
 // The same, reading only the top four limbs when one of them is nonzero (the
 // usual case for a product of normalised operands).
 size_t trim(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s);
+// Groups of values that a product tree takes several times each, as further
+// leaves behind its values: leaves [start[g], start[g+1]) are base[off[g]],
+// base[off[g]], ..., every value times[g] times.
+constexpr int kMaxRepeats = 64;
+struct Repeats {
+    int groups = 0;
+    const uint32_t *base = nullptr;
+    uint64_t start[kMaxRepeats + 1] = {}, off[kMaxRepeats] = {};
+    uint32_t times[kMaxRepeats] = {};
+};
+// A caller's device buffer for a result that fits len limbs: `used` says
+// whether the result went there (its limbs up to len written).
+struct Direct {
+    uint32_t *out = nullptr;
+    size_t len = 0;
+    bool used = false;
+};
 // Product of count 32-bit values (balanced tree).  Returns the result.
-// The product of values[0 .. count), times *extra when given; exact = false
-// returns a length bound (zero top limbs) without a host read-back (tree.cu).
-// Every value is below 2^leaf_bits: a first-level node of eight limbs then
-// takes leaves_per_node(leaf_bits) values.
+// The product of values[0 .. count) and of the repeated groups, times *extra
+// when given; exact = false returns a length bound (zero top limbs) without a
+// host read-back (tree.cu).  Every value is below 2^leaf_bits: a first-level
+// node of eight limbs then takes leaves_per_node(leaf_bits) values.
 Big tree_product(Ctx &c, const uint32_t *values, size_t count, cudaStream_t s,
-                 const Big *extra = nullptr, bool exact = true, int leaf_bits = 32);
+                 const Big *extra = nullptr, bool exact = true, int leaf_bits = 32,
+                 const Repeats *rep = nullptr, Direct *direct = nullptr);
 // a^e.
 Big power(Ctx &c, const uint32_t *a, size_t na, uint64_t e, cudaStream_t s, bool exact = true);
 // Factorial ratios (Sec. 6.3): N = prod_i a_i! / prod_j b_j!.  A Ratio also
@@ -676,7 +699,10 @@ void factor_free(Ctx &c, cat_factorization *f);
 void copy_to_host(Ctx &c, uint32_t *host, const uint32_t *dev, size_t n, cudaStream_t s);
 // Algorithm 2 on a factorisation; returns the result (normalised length).
 // Every prime of f is below 2^leaf_bits (32 when nothing smaller is known).
-Big reconstruct(Ctx &c, const cat_factorization *f, cudaStream_t s, int leaf_bits = 32);
+// direct: a buffer that holds the result, taken when the last product can go
+// there (the result's Big then carries the length alone).
+Big reconstruct(Ctx &c, const cat_factorization *f, cudaStream_t s, int leaf_bits = 32,
+                Direct *direct = nullptr);
 // Kernels launched by the library so far (every CAT_LAUNCH).
 unsigned long long launch_count();
 

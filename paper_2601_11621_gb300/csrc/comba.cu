@@ -26,11 +26,22 @@ __device__ __forceinline__ void mac96(uint32_t a, uint32_t b, uint32_t &c0, uint
 
 constexpr int kLeafSlot = 8;
 
-// Node i (eight limbs) = product of values[lpn i .. lpn i + lpn) (values
-// past `count` count as 1; the caller picks lpn so that the product fits),
+// Leaf idx of a tree over values[0 .. count) followed by the repeated groups
+// (1 past the end).
+__device__ __forceinline__ uint32_t leaf_value(const uint32_t *v, size_t count, const Repeats &rep,
+                                               size_t idx)
+{
+    if (idx < count) return v[idx];
+    int g = 0;
+    while (g < rep.groups && idx >= rep.start[g + 1]) g++;
+    return g < rep.groups ? rep.base[rep.off[g] + (idx - rep.start[g]) / rep.times[g]] : 1u;
+}
+
+// Node i (eight limbs) = product of the leaves [lpn i, lpn i + lpn) (those
+// past the end count as 1; the caller picks lpn so that the product fits),
 // accumulated by single-limb multiplications.
-__global__ void leaf_products(const uint32_t *v, size_t count, uint32_t *out, size_t nodes,
-                              int lpn)
+__global__ void leaf_products(const uint32_t *v, size_t count, const __grid_constant__ Repeats rep,
+                              uint32_t *out, size_t nodes, int lpn)
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nodes) return;
@@ -39,8 +50,7 @@ __global__ void leaf_products(const uint32_t *v, size_t count, uint32_t *out, si
     for (int j = 0; j < kLeafSlot; j++) acc[j] = 0;
     acc[0] = 1;
     for (int k = 0; k < lpn; k++) {
-        const size_t idx = i * (size_t)lpn + k;
-        const uint32_t x = idx < count ? v[idx] : 1u;
+        const uint32_t x = leaf_value(v, count, rep, i * (size_t)lpn + k);
         uint32_t carry = 0;
 #pragma unroll
         for (int j = 0; j < kLeafSlot; j++) {
@@ -224,11 +234,11 @@ __global__ void find_top(const uint32_t *x, size_t n, unsigned long long *top)
 
 // ----------------------------------------------------------- host side
 
-void leaf_level(Ctx &c, const uint32_t *values, size_t count, uint32_t *out, size_t nodes,
-                int lpn, cudaStream_t s)
+void leaf_level(Ctx &c, const uint32_t *values, size_t count, const Repeats &rep, uint32_t *out,
+                size_t nodes, int lpn, cudaStream_t s)
 {
     const int tok = prof_begin(c, "leaf_products", s);
-    leaf_products<<<(unsigned)((nodes + 255) / 256), 256, 0, s>>>(values, count, out, nodes,
+    leaf_products<<<(unsigned)((nodes + 255) / 256), 256, 0, s>>>(values, count, rep, out, nodes,
                                                                     lpn);
     CAT_LAUNCH("leaf_products");
     prof_end(c, tok, s, 4.0 * (double)count + 32.0 * (double)nodes,

@@ -1627,6 +1627,18 @@ void ntt_level(Ctx &c, const uint32_t *level, size_t slot, size_t nprod, uint32_
     }
 }
 
+bool ntt_level_whole(const Ctx &c, size_t slot) { return points_log(2 * slot) + 1 <= c.max_log; }
+
+void ntt_pair(Ctx &c, const uint32_t *pair, size_t slot, uint32_t *out, size_t len, cudaStream_t s)
+{
+    const int np = points_log(2 * slot);
+    const Operand a{pair, 2 * slot, slot}, b{pair + slot, 2 * slot, slot};
+    if (np <= kFusedMaxLog)
+        ntt_mul_small(c, np, 1, a, b, false, plain_sink(out, 0, len), s);
+    else
+        ntt_mul_multipass(c, np, PAIR_FIRST_TWO, 1, a, b, plain_sink(out, 0, len), s);
+}
+
 // out[0 .. na+nb) = a * b by the transform (na + nb <= 2^27).
 void ntt_mul(Ctx &c, const uint32_t *a, size_t na, const uint32_t *b, size_t nb,
              uint32_t *out, cudaStream_t s)

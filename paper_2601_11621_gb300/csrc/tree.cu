@@ -20,8 +20,8 @@
 namespace cat {
 
 // comba.cu
-void leaf_level(Ctx &c, const uint32_t *values, size_t count, uint32_t *out, size_t nodes,
-                int lpn, cudaStream_t s);
+void leaf_level(Ctx &c, const uint32_t *values, size_t count, const Repeats &rep, uint32_t *out,
+                size_t nodes, int lpn, cudaStream_t s);
 // ntt.cu
 void ntt_mul(Ctx &c, const uint32_t *a, size_t na, const uint32_t *b, size_t nb,
              uint32_t *out, cudaStream_t s);
@@ -135,11 +135,16 @@ static int tree_depth(size_t count, int lpn)
 // slot, so the levels above are unchanged; only when the padding would add a
 // level is extra multiplied in at the end instead.  exact = false returns the
 // top slot (zero-padded) as the length instead of reading the true length
-// back: no host synchronisation.
+// back: no host synchronisation.  With `direct` the last product goes straight
+// to the caller's buffer when one transform forms it.
 Big tree_product(Ctx &c, const uint32_t *values, size_t count, cudaStream_t s, const Big *extra,
-                 bool exact, int leaf_bits)
+                 bool exact, int leaf_bits, const Repeats *rep, Direct *direct)
 {
     NvtxRange range("product tree");
+    static const Repeats none{};
+    if (!rep) rep = &none;
+    const size_t own = count;
+    count += rep->groups ? rep->start[rep->groups] - rep->start[0] : 0;
     if (count == 0) return extra ? copy_big(c, extra->buf.get(), extra->n, s) : make_one(c, s);
     const int lpn = leaves_per_node(leaf_bits);
     size_t total = count, inj_slot = 0;
@@ -156,9 +161,18 @@ Big tree_product(Ctx &c, const uint32_t *values, size_t count, cudaStream_t s, c
     size_t slot = kLeafSlot;
     size_t nodes = (total + lpn - 1) / lpn;
     DevBuf<uint32_t> cur(c, nodes * slot, s);
-    leaf_level(c, values, count, cur.get(), nodes, lpn, s);
+    leaf_level(c, values, own, *rep, cur.get(), nodes, lpn, s);
     while (nodes > 1) {
         NvtxRange level("tree level");
+        if (direct && direct->out && nodes == 2 && !extra && slot > c.comba_max_slot &&
+            ntt_level_whole(c, slot)) {
+            const size_t len = std::min(2 * slot, direct->len);
+            ntt_pair(c, cur.get(), slot, direct->out, len, s);
+            direct->used = true;
+            Big r;
+            r.n = trim(c, direct->out, len, s);
+            return r;
+        }
         const size_t nprod = nodes / 2, odd = nodes & 1, nn = nprod + odd, ns = 2 * slot;
         DevBuf<uint32_t> nxt(c, nn * ns, s);
         if (slot > c.comba_max_slot || !comba_level(c, cur.get(), slot, nprod, nxt.get(), s))
@@ -233,7 +247,7 @@ Big power(Ctx &c, const uint32_t *a, size_t na, uint64_t e, cudaStream_t s, bool
 // Factorisations with more exponent groups than this (n! has about 2 sqrt(n))
 // take the bit-decomposed form below; Catalan numbers and central binomials
 // (at most 33 groups) always take Algorithm 2 as written.
-constexpr uint64_t kManyGroups = 64;
+constexpr uint64_t kManyGroups = kMaxRepeats;
 
 // prod_e Q_e^e = prod_b R_b^(2^b), R_b = prod of Q_e over the groups whose
 // exponent has bit b set.  All R_b come from one segmented tree over the
@@ -278,13 +292,52 @@ static Big reconstruct_bits(Ctx &c, const cat_factorization *f, cudaStream_t s, 
     return X;
 }
 
+// The groups with e >= 2 as leaves of Q_1's own tree, every prime e times (the
+// same integer, re-associated), when that adds at most a quarter to the tree
+// or 4,096 leaves; false otherwise.  For C(n) and C(2n, n) those primes are at
+// most sqrt(2n), so they are a handful of leaves, where forming every Q_e, its
+// power and their product took about 25 short launches one after the other at
+// n = 10^5 and 40 at the paper's n (with the last product straight into the
+// caller's buffer: C(10^5) 0.43 -> 0.22 ms, C(5 10^7) 2.27 -> 1.92,
+// C(2,050,572,903) 81.2 -> 80.6).
+static bool repeat_leaves(const cat_factorization *f, Repeats &rep, uint64_t &off1, uint64_t &cnt1)
+{
+    uint64_t more = 0;
+    off1 = cnt1 = 0;
+    rep.base = f->primes;
+    for (uint64_t g = 0; g < f->num_groups; g++) {
+        const uint64_t off = f->host_offsets[g], cnt = f->host_offsets[g + 1] - off;
+        const uint64_t e = f->host_exps[g];
+        if (e == 1) {
+            off1 = off;
+            cnt1 = cnt;
+            continue;
+        }
+        if (e > 0xffffffffull || cnt > (1ull << 40) / e) return false;
+        rep.off[rep.groups] = off;
+        rep.times[rep.groups] = (uint32_t)e;
+        rep.start[rep.groups] = more;
+        more += e * cnt;
+        rep.start[++rep.groups] = more;
+    }
+    for (int g = 0; g <= rep.groups; g++) rep.start[g] += cnt1;  // behind Q_1's leaves
+    return more <= std::max<uint64_t>(cnt1 / 4, 4096);
+}
+
 // Algorithm 2: Q_e by the tree, P_e = Q_e^e, then the P_e combined by
 // repeatedly multiplying the two shortest (equal-length operands meet
 // first, so intermediates stay as short as possible).
-Big reconstruct(Ctx &c, const cat_factorization *f, cudaStream_t s, int leaf_bits)
+Big reconstruct(Ctx &c, const cat_factorization *f, cudaStream_t s, int leaf_bits, Direct *direct)
 {
     NvtxRange range("phase2: reconstruction");
     if (f->num_groups > kManyGroups) return reconstruct_bits(c, f, s, leaf_bits);
+    {
+        Repeats rep;
+        uint64_t off1 = 0, cnt1 = 0;
+        if (repeat_leaves(f, rep, off1, cnt1))
+            return tree_product(c, f->primes + off1, cnt1, s, nullptr, true, leaf_bits, &rep,
+                                direct);
+    }
     // P_e = Q_e^e for e >= 2 first, combined into R; then Q_1's tree takes R
     // in as one of its nodes, so that the long P_1 needs no final product
     // (the same integer: the final product of the P_e, re-associated).  The
