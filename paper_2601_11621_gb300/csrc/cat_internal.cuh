@@ -552,6 +552,7 @@ struct DevBuf {
 struct Big {
     DevBuf<uint32_t> buf;
     size_t n = 0;
+    double bits = 0;  // where tracked: the value is below 2^bits
 };
 
 // A device copy job: `len` limbs from src to dst, then dst zero-filled up to
@@ -646,6 +647,10 @@ size_t normalized_length(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s);
 // The same, reading only the top four limbs when one of them is nonzero (the
 // usual case for a product of normalised operands).
 size_t trim(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s);
+// Normalises up to kMaxTops numbers at once (their n and bits, from their
+// lengths and top two limbs), with one read-back.
+constexpr int kMaxTops = 64;
+void normalize_all(Ctx &c, Big *const *x, int count, cudaStream_t s);
 // Groups of values that a product tree takes several times each, as further
 // leaves behind its values: leaves [start[g], start[g+1]) are base[off[g]],
 // base[off[g]], ..., every value times[g] times.

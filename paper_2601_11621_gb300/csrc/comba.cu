@@ -9,6 +9,8 @@
 // next level's slot of 2S limbs exactly.
 #include "cat_internal.cuh"
 
+#include <math.h>
+
 namespace cat {
 
 // c2:c1:c0 += a * b  (96-bit accumulator)
@@ -232,6 +234,36 @@ __global__ void find_top(const uint32_t *x, size_t n, unsigned long long *top)
     if ((threadIdx.x & 31) == 0 && best) atomicMax(top, best);
 }
 
+struct TopsArgs {
+    const uint32_t *x[kMaxTops];
+    uint64_t n[kMaxTops];
+    uint64_t *out;  // per number: normalised length, top two limbs
+};
+
+// One block per number, scanning down from the top for the highest nonzero
+// limb (usually in the first stretch).
+__global__ void __launch_bounds__(1024) number_tops(const __grid_constant__ TopsArgs a)
+{
+    __shared__ unsigned long long best;
+    const uint32_t *x = a.x[blockIdx.x];
+    if (threadIdx.x == 0) best = 0;
+    __syncthreads();
+    for (uint64_t top = a.n[blockIdx.x]; top > 0;) {
+        const uint64_t lo = top > blockDim.x ? top - blockDim.x : 0;
+        const uint64_t i = lo + threadIdx.x;
+        if (i < top && x[i]) atomicMax(&best, (unsigned long long)(i + 1));
+        __syncthreads();
+        if (best) break;  // the same for every thread: nothing is written until the next barrier
+        top = lo;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        a.out[2 * blockIdx.x] = best;
+        a.out[2 * blockIdx.x + 1] =
+            best ? (uint64_t)x[best - 1] << 32 | (best > 1 ? x[best - 2] : 0u) : 0u;
+    }
+}
+
 // ----------------------------------------------------------- host side
 
 void leaf_level(Ctx &c, const uint32_t *values, size_t count, const Repeats &rep, uint32_t *out,
@@ -268,6 +300,32 @@ bool comba_level(Ctx &c, const uint32_t *in, size_t slot, size_t nprod, uint32_t
     CAT_LAUNCH("comba_level");
     prof_end(c, tok, s, 16.0 * (double)slot * (double)nprod, 16.0 * (double)slot * (double)nprod);
     return true;
+}
+
+void normalize_all(Ctx &c, Big *const *x, int count, cudaStream_t s)
+{
+    if (count > kMaxTops) fail(CAT_EINVAL, "too many numbers");
+    if (count == 0) return;
+    DevBuf<uint64_t> d(c, 2 * (size_t)count, s);
+    TopsArgs a{};
+    for (int i = 0; i < count; i++) {
+        a.x[i] = x[i]->buf.get();
+        a.n[i] = x[i]->n;
+    }
+    a.out = d.get();
+    number_tops<<<count, 1024, 0, s>>>(a);
+    CAT_LAUNCH("number_tops");
+    CAT_CUDA(cudaMemcpyAsync(c.host_word, d.get(), 16 * (size_t)count, cudaMemcpyDeviceToHost, s));
+    CAT_CUDA(cudaStreamSynchronize(s));
+    for (int i = 0; i < count; i++) {
+        const uint64_t n = c.host_word[2 * i], top = c.host_word[2 * i + 1];
+        x[i]->n = n;
+        // below 2^(32 (n - 2)) (top + 1), top of 33 bits or more unless n = 1
+        x[i]->bits = n == 0 ? 0
+                     : n == 1
+                         ? log2((double)(top >> 32)) + 1e-9
+                         : 32.0 * (double)(n - 2) + log2((double)top) + 1e-9;
+    }
 }
 
 size_t normalized_length(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s)

@@ -279,7 +279,7 @@ void ctx_init(Ctx &c, int device, size_t budget)
     CAT_CUDA(cudaMemcpy(c.seeds, c.host_seeds.data(), c.host_seeds.size() * sizeof(uint32_t),
                         cudaMemcpyHostToDevice));
     CAT_CUDA(cudaMallocHost(&c.host_info, sizeof(Phase1Info)));
-    CAT_CUDA(cudaMallocHost(&c.host_word, 4 * sizeof(uint64_t)));
+    CAT_CUDA(cudaMallocHost(&c.host_word, 2 * kMaxTops * sizeof(uint64_t)));
     CAT_CUDA(cudaMalloc(&c.dev_word, sizeof(unsigned long long)));
 }
 

@@ -223,24 +223,41 @@ static Big mul_big(Ctx &c, const Big &x, const Big &y, cudaStream_t s, bool exac
     return r;
 }
 
+// x y for numbers whose bits are tracked: the product's length bound comes from
+// its bits (at most one limb above the true length), so that a chain of
+// products needs no read-back between its steps.
+static Big mul_bits(Ctx &c, const Big &x, const Big &y, cudaStream_t s)
+{
+    Big r = mul_big(c, x, y, s, false);
+    r.bits = x.bits + y.bits;
+    r.n = std::min<size_t>(r.n, (size_t)(r.bits / 32.0) + 1);
+    return r;
+}
+
 // a^e, left-to-right binary (the powering step of Algorithm 2).  Squarings reuse
 // one forward transform.  exact = false takes a (nonzero) as given, with zero
 // top limbs allowed, and returns a bound as the length: no host
-// synchronisation.
+// synchronisation; exact = true reads a's length and top limbs first and the
+// result's length last, and nothing between.
 Big power(Ctx &c, const uint32_t *a, size_t na, uint64_t e, cudaStream_t s, bool exact)
 {
     NvtxRange range("power");
-    if (exact) na = normalized_length(c, a, na, s);
-    if (e == 0) return make_one(c, s);
-    if (na == 0) return copy_big(c, a, 0, s);
     Big base = copy_big(c, a, na, s);
-    Big r = copy_big(c, a, na, s);
+    if (exact) {
+        Big *p = &base;
+        normalize_all(c, &p, 1, s);
+    }
+    if (e == 0) return make_one(c, s);
+    if (base.n == 0) return base;
+    Big r = copy_big(c, base.buf.get(), base.n, s);
+    r.bits = base.bits;
     int top = 63;
     while (!((e >> top) & 1)) top--;
     for (int bit = top - 1; bit >= 0; bit--) {
-        r = mul_big(c, r, r, s, exact);
-        if ((e >> bit) & 1) r = mul_big(c, r, base, s, exact);
+        r = exact ? mul_bits(c, r, r, s) : mul_big(c, r, r, s, false);
+        if ((e >> bit) & 1) r = exact ? mul_bits(c, r, base, s) : mul_big(c, r, base, s, false);
     }
+    if (exact) r.n = trim(c, r.buf.get(), r.n, s);
     return r;
 }
 
@@ -248,6 +265,67 @@ Big power(Ctx &c, const uint32_t *a, size_t na, uint64_t e, cudaStream_t s, bool
 // take the bit-decomposed form below; Catalan numbers and central binomials
 // (at most 33 groups) always take Algorithm 2 as written.
 constexpr uint64_t kManyGroups = kMaxRepeats;
+
+// Leaves of the bit segments (exponents fit 32 bits): segment b holds the
+// primes of the groups whose exponent has bit b set, group after group.
+struct BitSegments {
+    uint64_t start[33];
+};
+
+// at[b ng + g]: the first leaf of group g in segment b; block b scans the
+// groups, 1,024 at a time.
+__global__ void __launch_bounds__(1024) bit_offsets(const uint64_t *exps, const uint64_t *offs,
+                                                    uint32_t ng,
+                                                    const __grid_constant__ BitSegments seg,
+                                                    uint64_t *at)
+{
+    __shared__ uint64_t wsum[32];
+    const int b = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint64_t run = seg.start[b];
+    for (uint32_t g0 = 0; g0 < ng; g0 += 1024) {
+        const uint32_t g = g0 + threadIdx.x;
+        const uint64_t c = g < ng && (exps[g] >> b & 1) ? offs[g + 1] - offs[g] : 0;
+        uint64_t incl = c;
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint64_t v = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += v;
+        }
+        if (lane == 31) wsum[wid] = incl;
+        __syncthreads();
+        uint64_t before = 0, total = 0;
+        for (int w = 0; w < 32; w++) {
+            before += w < wid ? wsum[w] : 0;
+            total += wsum[w];
+        }
+        if (g < ng) at[(size_t)b * ng + g] = run + before + incl - c;
+        run += total;
+        __syncthreads();
+    }
+}
+
+// One thread per prime: its group by bisection, then one leaf per bit of the
+// exponent.
+__global__ void bit_leaves(const uint32_t *primes, uint64_t np, const uint64_t *exps,
+                           const uint64_t *offs, uint32_t ng, const uint64_t *at,
+                           uint32_t *leaves)
+{
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= np) return;
+    uint32_t lo = 0, hi = ng;  // offs[lo] <= i < offs[hi]
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (offs[mid] <= i) lo = mid;
+        else hi = mid;
+    }
+    const uint32_t p = primes[i];
+    const uint64_t k = i - offs[lo];
+    uint32_t e = (uint32_t)exps[lo];
+    while (e) {
+        const int b = __ffs(e) - 1;
+        e &= e - 1;
+        leaves[at[(size_t)b * ng + lo] + k] = p;
+    }
+}
 
 // prod_e Q_e^e = prod_b R_b^(2^b), R_b = prod of Q_e over the groups whose
 // exponent has bit b set.  All R_b come from one segmented tree over the
@@ -268,27 +346,36 @@ static Big reconstruct_bits(Ctx &c, const cat_factorization *f, cudaStream_t s, 
                 seg[b + 1] += f->host_offsets[g + 1] - f->host_offsets[g];
     for (int b = 0; b < B; b++) seg[b + 1] += seg[b];
     DevBuf<uint32_t> leaves(c, std::max<uint64_t>(seg[B], 1), s);
-    std::vector<CopyJob> jobs;
-    std::vector<uint64_t> at(seg.begin(), seg.end() - 1);
-    for (uint64_t g = 0; g < f->num_groups; g++) {
-        const uint64_t off = f->host_offsets[g], cnt = f->host_offsets[g + 1] - off;
-        if (!cnt) continue;
-        for (int b = 0; b < B; b++)
-            if ((f->host_exps[g] >> b) & 1) {
-                jobs.push_back(CopyJob{f->primes + off, leaves.get() + at[b], cnt, cnt});
-                at[b] += cnt;
-            }
+    {
+        const uint32_t ng = (uint32_t)f->num_groups;
+        DevBuf<uint64_t> at(c, (size_t)B * ng, s);
+        BitSegments sb{};
+        std::copy(seg.begin(), seg.end(), sb.start);
+        bit_offsets<<<B, 1024, 0, s>>>(f->exps, f->offsets, ng, sb, at.get());
+        CAT_LAUNCH("bit_offsets");
+        const int tok = prof_begin(c, "bit_leaves", s);
+        bit_leaves<<<(unsigned)((f->num_primes + 255) / 256), 256, 0, s>>>(
+            f->primes, f->num_primes, f->exps, f->offsets, ng, at.get(), leaves.get());
+        CAT_LAUNCH("bit_leaves");
+        prof_end(c, tok, s, 4.0 * (double)(f->num_primes + seg[B]));
     }
-    run_copy_jobs(c, jobs, s);
     std::vector<TreeRoot> R(B);
     segmented_tree(c, leaves.get(), seg, R, s, leaf_bits);
     leaves.reset();
-    for (int b = 0; b < B; b++) R[b].big.n = trim(c, R[b].big.buf.get(), R[b].big.n, s);
+    std::vector<Big *> roots;
+    for (int b = 0; b < B; b++) {
+        // a root's slot has a limb per leaf; its value ends with the leaves' bits
+        Big &r = R[b].big;
+        r.n = std::min<size_t>(r.n, (seg[b + 1] - seg[b]) * (uint64_t)leaf_bits / 32 + 1);
+        roots.push_back(&r);
+    }
+    normalize_all(c, roots.data(), B, s);
     Big X = std::move(R[B - 1].big);
     for (int b = B - 2; b >= 0; b--) {
-        X = mul_big(c, X, X, s);
-        if (seg[b + 1] > seg[b]) X = mul_big(c, X, R[b].big, s);
+        X = mul_bits(c, X, X, s);
+        if (seg[b + 1] > seg[b]) X = mul_bits(c, X, R[b].big, s);
     }
+    X.n = trim(c, X.buf.get(), X.n, s);
     return X;
 }
 
