@@ -386,7 +386,7 @@ struct ProfPending {
     double unit_bytes;
 };
 
-struct Phase1Info;
+struct HostPage;
 
 struct Ctx {
     int device = 0;
@@ -421,15 +421,16 @@ struct Ctx {
     // forward pass (which runs once per operand) and for the others (all by
     // default; smaller values are for measurements)
     int col_tw_first_max_log = kLogMaxPts, col_tw_max_log = kLogMaxPts;
-    // small read-backs (lengths of results): a pinned host word and a device
+    // small read-backs (lengths of results, Phase 1's counts): a pinned page
+    // that read_back's kernel writes, the number of the last one, and a device
     // word, allocated once per context
-    uint64_t *host_word = nullptr;
+    struct HostPage *page = nullptr;
+    uint64_t read_backs = 0;
     unsigned long long *dev_word = nullptr;
     // the primes below 2^16, ascending (every sieve's seeds are a prefix), on
-    // the device and the host, and Phase 1's read-back (pinned)
+    // the device and the host
     uint32_t *seeds = nullptr;
     std::vector<uint32_t> host_seeds;
-    struct Phase1Info *host_info = nullptr;
     bool profiling = false;
     std::vector<ProfEntry> prof;
     std::vector<ProfPending> pending;
@@ -445,6 +446,13 @@ struct Phase1Info {
     uint32_t kept, total, negative, ngroups;
     uint32_t exp[kMaxSeedGroups], off[kMaxSeedGroups + 1];
 };
+
+// Up to kPageWords words of device memory, read back when stream s has reached
+// this point: everything issued before is complete on return, as after a
+// stream synchronisation.  The words stay valid until the context's next
+// read_back.
+constexpr int kPageWords = 512;
+const uint32_t *read_back(Ctx &c, const void *dev, int words, cudaStream_t s);
 
 // Launch bracketing for the profiler: prof_begin returns a token (or -1 when
 // profiling is off); prof_end records the stop event and the launch's

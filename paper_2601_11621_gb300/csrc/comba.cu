@@ -315,10 +315,10 @@ void normalize_all(Ctx &c, Big *const *x, int count, cudaStream_t s)
     a.out = d.get();
     number_tops<<<count, 1024, 0, s>>>(a);
     CAT_LAUNCH("number_tops");
-    CAT_CUDA(cudaMemcpyAsync(c.host_word, d.get(), 16 * (size_t)count, cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaStreamSynchronize(s));
+    const uint32_t *h = read_back(c, d.get(), 4 * count, s);
     for (int i = 0; i < count; i++) {
-        const uint64_t n = c.host_word[2 * i], top = c.host_word[2 * i + 1];
+        const uint64_t n = (uint64_t)h[4 * i + 1] << 32 | h[4 * i];
+        const uint64_t top = (uint64_t)h[4 * i + 3] << 32 | h[4 * i + 2];
         x[i]->n = n;
         // below 2^(32 (n - 2)) (top + 1), top of 33 bits or more unless n = 1
         x[i]->bits = n == 0 ? 0
@@ -344,11 +344,8 @@ size_t normalized_length(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s)
     if (blocks > cap) blocks = cap;
     find_top<<<(unsigned)blocks, threads, 0, s>>>(x, n, top);
     CAT_LAUNCH("find_top");
-    unsigned long long local = 0;
-    unsigned long long *h = c.host_word ? reinterpret_cast<unsigned long long *>(c.host_word) : &local;
-    CAT_CUDA(cudaMemcpyAsync(h, top, sizeof(*h), cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaStreamSynchronize(s));
-    return (size_t)*h;
+    const uint32_t *h = read_back(c, top, 2, s);
+    return (size_t)((uint64_t)h[1] << 32 | h[0]);
 }
 
 }  // namespace cat

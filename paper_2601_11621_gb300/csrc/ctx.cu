@@ -6,6 +6,7 @@
 #include <stdio.h>
 #include <stdlib.h>
 
+#include <chrono>
 #include <string>
 #include <vector>
 
@@ -102,6 +103,50 @@ void dev_free(Ctx &c, void *p, size_t bytes, cudaStream_t s)
     cudaFreeAsync(p, s);
     c.in_use -= bytes;
     if (c.shared_in_use) c.shared_in_use->fetch_sub(bytes);
+}
+
+// -------------------------------------------------------------- read-backs
+
+// The page's words, and the number of the read-back they belong to.
+struct HostPage {
+    uint32_t words[kPageWords];
+    uint64_t done;
+};
+
+// Copies the words to the host page and, once they are visible there, sets its
+// number.
+__global__ void __launch_bounds__(kPageWords) publish(const uint32_t *src, int words,
+                                                      HostPage *page, uint64_t number)
+{
+    if ((int)threadIdx.x < words) page->words[threadIdx.x] = src[threadIdx.x];
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x == 0) *(volatile uint64_t *)&page->done = number;
+}
+
+// A kernel storing into the mapped page and a short wait on its number cost
+// less than a copy-engine transfer and a stream synchronisation (a call on
+// 1,000 x 700 limbs 26.5 -> 20.0 us, C(10^5) 205 -> 189, 3 10^6! 2.13 -> 2.00 ms).  The
+// wait is bounded: after a millisecond, or when the stream has failed, the
+// stream is synchronised, which waits without polling and reports errors.
+const uint32_t *read_back(Ctx &c, const void *dev, int words, cudaStream_t s)
+{
+    if (words > kPageWords) fail(CAT_EINVAL, "read-back too long");
+    const uint64_t number = ++c.read_backs;
+    const int threads = words <= 32 ? 32 : (words + 31) / 32 * 32;
+    publish<<<1, threads, 0, s>>>(static_cast<const uint32_t *>(dev), words, c.page, number);
+    CAT_LAUNCH("publish");
+    const auto t0 = std::chrono::steady_clock::now();
+    for (int i = 0;; i++) {
+        if (__atomic_load_n(&c.page->done, __ATOMIC_ACQUIRE) == number) return c.page->words;
+        if ((i & 255) == 255 &&
+            std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(1))
+            break;
+    }
+    CAT_CUDA(cudaStreamSynchronize(s));
+    if (__atomic_load_n(&c.page->done, __ATOMIC_ACQUIRE) != number)
+        fail(CAT_ECUDA, "a read-back did not arrive");
+    return c.page->words;
 }
 
 // --------------------------------------------------------------- profiler
@@ -278,8 +323,8 @@ void ctx_init(Ctx &c, int device, size_t budget)
     CAT_CUDA(cudaMalloc(&c.seeds, c.host_seeds.size() * sizeof(uint32_t)));
     CAT_CUDA(cudaMemcpy(c.seeds, c.host_seeds.data(), c.host_seeds.size() * sizeof(uint32_t),
                         cudaMemcpyHostToDevice));
-    CAT_CUDA(cudaMallocHost(&c.host_info, sizeof(Phase1Info)));
-    CAT_CUDA(cudaMallocHost(&c.host_word, 2 * kMaxTops * sizeof(uint64_t)));
+    CAT_CUDA(cudaHostAlloc(&c.page, sizeof(HostPage), cudaHostAllocMapped | cudaHostAllocPortable));
+    c.page->done = 0;
     CAT_CUDA(cudaMalloc(&c.dev_word, sizeof(unsigned long long)));
 }
 
@@ -299,13 +344,9 @@ void ctx_release(Ctx &c)
         cudaFree(c.seeds);
         c.seeds = nullptr;
     }
-    if (c.host_info) {
-        cudaFreeHost(c.host_info);
-        c.host_info = nullptr;
-    }
-    if (c.host_word) {
-        cudaFreeHost(c.host_word);
-        c.host_word = nullptr;
+    if (c.page) {
+        cudaFreeHost(c.page);
+        c.page = nullptr;
     }
 }
 

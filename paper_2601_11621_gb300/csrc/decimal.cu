@@ -188,9 +188,7 @@ int to_decimal_dev(Ctx &c, const uint32_t *x, size_t n, char *out, size_t cap, s
     // cur: the number in S chunks of base 10^9
     const size_t nch = normalized_length(c, cur.get(), S, s);
     const size_t top = nch - 1;
-    uint32_t lead_chunk = 0;
-    CAT_CUDA(cudaMemcpyAsync(&lead_chunk, cur.get() + top, 4, cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaStreamSynchronize(s));
+    const uint32_t lead_chunk = *read_back(c, cur.get() + top, 1, s);
     int lead = 1;
     for (uint32_t v = lead_chunk; v >= 10; v /= 10) lead++;
     const size_t total = (size_t)lead + 9 * top;

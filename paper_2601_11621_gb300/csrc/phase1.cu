@@ -33,6 +33,7 @@
 
 #include <algorithm>
 #include <math.h>
+#include <string.h>
 
 namespace cat {
 
@@ -504,15 +505,6 @@ static uint64_t isqrt64(uint64_t x)
     return r;
 }
 
-// A device word, read back (through the context's pinned word).
-static uint64_t read_word(Ctx &c, const uint32_t *d, cudaStream_t s)
-{
-    uint32_t *h = reinterpret_cast<uint32_t *>(c.host_word);
-    CAT_CUDA(cudaMemcpyAsync(h, d, 4, cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaStreamSynchronize(s));
-    return *h;
-}
-
 // log2 odd numbers per segment: 2^18 (32 KiB of bitmap) when that still gives
 // every SM several rounds of its four resident blocks, down to 2^13 for short
 // sieves, so that their few numbers spread over the SMs (limits 2 10^5: 26 ->
@@ -595,6 +587,7 @@ static Grouped group_items(Ctx &c, DevBuf<uint64_t> &items, size_t count, uint32
     int ebits = 0;
     while (ebits < 32 && (max_e >> ebits)) ebits++;
     DevBuf<uint64_t> alt(c, std::max<size_t>(count, 1), s);
+    DevBuf<uint32_t> kept(c, 1, s);
     uint64_t *src = items.get(), *dst = alt.get();
     int tok;
     for (int shift = 0, pass = 0; pass == 0 || shift < ebits; pass++) {
@@ -608,18 +601,13 @@ static Grouped group_items(Ctx &c, DevBuf<uint64_t> &items, size_t count, uint32
         rs_histogram<<<(unsigned)tiles, kRsThreads, 0, s>>>(ra);
         CAT_LAUNCH("rs_histogram");
         prof_end(c, tok, s, 8.0 * (double)count);
-        uint32_t lastc = 0, lasto = 0;
-        CAT_CUDA(cudaMemcpyAsync(&lastc, cnt.get() + nbins * tiles - 1, 4,
-                                 cudaMemcpyDeviceToHost, s));
-        exclusive_scan_u32(c, cnt.get(), nbins * tiles, s);
-        CAT_CUDA(cudaMemcpyAsync(&lasto, cnt.get() + nbins * tiles - 1, 4,
-                                 cudaMemcpyDeviceToHost, s));
+        exclusive_scan_u32(c, cnt.get(), nbins * tiles, s, kept.get());
         tok = prof_begin(c, "rs_scatter", s);
         rs_scatter<<<(unsigned)tiles, kRsThreads, 0, s>>>(ra);
         CAT_LAUNCH("rs_scatter");
         prof_end(c, tok, s, 16.0 * (double)count);
-        CAT_CUDA(cudaStreamSynchronize(s));
-        count = (size_t)lasto + lastc;
+        // only the first pass drops items
+        if (pass == 0) count = *read_back(c, kept.get(), 1, s);
         std::swap(src, dst);
         shift += bitsd;
         if (ebits == 0) break;
@@ -633,9 +621,7 @@ static Grouped group_items(Ctx &c, DevBuf<uint64_t> &items, size_t count, uint32
     group_starts<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(src, count, starts.get(),
                                                                   nst.get(), g.primes.get());
     CAT_LAUNCH("group_starts");
-    unsigned int ng = 0;
-    CAT_CUDA(cudaMemcpyAsync(&ng, nst.get(), 4, cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaStreamSynchronize(s));
+    const unsigned int ng = *read_back(c, nst.get(), 1, s);
     std::vector<uint64_t> hst(2 * (size_t)ng);
     CAT_CUDA(cudaMemcpyAsync(hst.data(), starts.get(), 16 * (size_t)ng, cudaMemcpyDeviceToHost,
                              s));
@@ -669,9 +655,8 @@ static void factor_unit(Ctx &c, const Ratio &r, uint64_t limit, cat_factorizatio
                                                    sv.words.get() + 1, sorted.get(), d_info.get());
     CAT_LAUNCH("group_seeds");
     prof_end(c, tok, s, 8.0 * (double)ns);
-    Phase1Info &h = *c.host_info;
-    CAT_CUDA(cudaMemcpyAsync(&h, d_info.get(), sizeof(h), cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaStreamSynchronize(s));
+    Phase1Info h;
+    memcpy(&h, read_back(c, d_info.get(), sizeof(h) / 4, s), sizeof(h));
     if (h.negative) fail(CAT_ENOTINTEGRAL, "a prime exponent is negative");
     CsrArgs a{};
     a.nl = h.kept;
@@ -733,7 +718,7 @@ void factor_ratio(Ctx &c, const Ratio &r, cat_factorization *out, cudaStream_t s
     uint64_t sieved = 0, npos = 0;
     if (limit >= 2) {
         SieveOut sv = run_sieve(c, limit, s);
-        sieved = read_word(c, sv.words.get(), s) + 1;  // plus the prime 2
+        sieved = (uint64_t)*read_back(c, sv.words.get(), 1, s) + 1;  // plus the prime 2
         // exponents
         DevBuf<uint64_t> items(c, sieved, s);
         DevBuf<unsigned int> flags(c, 2, s);
@@ -746,9 +731,7 @@ void factor_ratio(Ctx &c, const Ratio &r, cat_factorization *out, cudaStream_t s
         CAT_LAUNCH("expand_exponents");
         prof_end(c, tok, s, 4.0 * (double)sv.units * kUnitWords + 8.0 * (double)sieved);
         sv = SieveOut{};
-        unsigned int hf[2];
-        CAT_CUDA(cudaMemcpyAsync(hf, flags.get(), 8, cudaMemcpyDeviceToHost, s));
-        CAT_CUDA(cudaStreamSynchronize(s));
+        const uint32_t *hf = read_back(c, flags.get(), 2, s);
         if (hf[1]) fail(CAT_ENOTINTEGRAL, "a prime exponent is negative");
         Grouped g = group_items(c, items, sieved, hf[0], s);
         npos = g.count;
@@ -782,7 +765,7 @@ DevBuf<uint32_t> sieve_primes(Ctx &c, uint64_t limit, uint64_t *count, cudaStrea
     *count = 0;
     if (limit < 2) return DevBuf<uint32_t>(c, 1, s);
     SieveOut sv = run_sieve(c, limit, s);
-    const uint64_t sieved = read_word(c, sv.words.get(), s) + 1;
+    const uint64_t sieved = (uint64_t)*read_back(c, sv.words.get(), 1, s) + 1;
     DevBuf<uint32_t> primes(c, sieved, s);
     const int tok = prof_begin(c, "expand_primes", s);
     expand_primes<<<(sv.units + kExpandWarps - 1) / kExpandWarps, kExpandThreads, 0, s>>>(

@@ -45,10 +45,7 @@ size_t trim(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s)
 {
     if (n == 0) return 0;
     const size_t k = std::min<size_t>(n, 4);
-    uint32_t local[4];
-    uint32_t *h = c.host_word ? reinterpret_cast<uint32_t *>(c.host_word) : local;
-    CAT_CUDA(cudaMemcpyAsync(h, x + n - k, 4 * k, cudaMemcpyDeviceToHost, s));
-    CAT_CUDA(cudaStreamSynchronize(s));
+    const uint32_t *h = read_back(c, x + n - k, (int)k, s);
     for (size_t i = k; i-- > 0;)
         if (h[i]) return n - k + i + 1;
     return normalized_length(c, x, n - k, s);
