@@ -176,14 +176,19 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
 
 
 def _stream(stream):
+    """The handle of `stream`, or of the current device's current stream."""
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # the handle without a Stream object around it (0.3 us instead of 3)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None and t.numel() else ctypes.c_void_p(0)
+    return t.data_ptr() if t is not None and t.numel() else None
 
 
 class Context:
@@ -197,6 +202,14 @@ class Context:
             raise CatError(rc, "cat_ctx_create failed")
         self.handle = h
         self.device = device
+        self._torch_device = None
+
+    @property
+    def torch_device(self):
+        if self._torch_device is None:
+            import torch
+            self._torch_device = torch.device("cuda", self.device)
+        return self._torch_device
 
     def check(self, rc: int):
         if rc != 0:
@@ -259,6 +272,8 @@ def _limbs_tensor(x, device):
     """Accept a torch tensor (int32/uint32 limbs on the device) or a numpy array."""
     import torch
     if isinstance(x, torch.Tensor):
+        if x.dtype is torch.int32 and x.is_contiguous():
+            return x
         if x.dtype not in (torch.int32,) and str(x.dtype) != "torch.uint32":
             raise TypeError("limb tensors must be int32 (uint32 bits)")
         return x.contiguous().view(torch.int32)
@@ -285,13 +300,13 @@ def cat_bound_limbs(n: int, kind: int = CAT_CATALAN) -> int:
 
 
 def bigint_mul(ctx: Context, a, b, stream=None):
-    dev = f"cuda:{ctx.device}"
+    dev = ctx.torch_device
     ta, tb = _limbs_tensor(a, dev), _limbs_tensor(b, dev)
-    cap = ta.numel() + tb.numel()
-    out = _empty(cap, dev)
+    na, nb = ta.numel(), tb.numel()
+    out = _empty(na + nb, dev)
     n = ctypes.c_size_t()
-    ctx.check(load().bigint_mul(ctx.handle, _ptr(ta), ta.numel(), _ptr(tb), tb.numel(),
-                                _ptr(out), cap, ctypes.byref(n), _stream(stream)))
+    ctx.check(load().bigint_mul(ctx.handle, ta.data_ptr(), na, tb.data_ptr(), nb, out.data_ptr(),
+                                na + nb, ctypes.byref(n), _stream(stream)))
     return out[:n.value]
 
 
@@ -322,7 +337,7 @@ def cat_ratio_factor(ctx: Context, a, b, stream=None) -> "FactorResult":
 def cat_ratio_exact(ctx: Context, a, b, out=None, stream=None):
     """prod a_i! / prod b_j! as a device limb tensor (CAT_ENOTINTEGRAL when it is
     not an integer)."""
-    dev = f"cuda:{ctx.device}"
+    dev = ctx.torch_device
     (pa, ka), (pb, kb) = _u64_array(a), _u64_array(b)
     if out is None:
         out = _empty(cat_ratio_bound_limbs(a, b), dev)
@@ -335,7 +350,7 @@ def cat_ratio_exact(ctx: Context, a, b, out=None, stream=None):
 def cat_factor_text(ctx: Context, fr: "FactorResult", name: str, stream=None):
     """The factorisation in the text layout of Sec. 3.1 (uint8 device tensor)."""
     import torch
-    dev = f"cuda:{ctx.device}"
+    dev = ctx.torch_device
     n = ctypes.c_size_t()
     rc = load().cat_factor_text(ctx.handle, ctypes.byref(fr.f), name.encode(), None, 0,
                                 ctypes.byref(n), _stream(stream))
@@ -351,7 +366,7 @@ def cat_binary(ctx: Context, limbs, stream=None):
     """The result file bytes (01 01, then the little-endian magnitude) as a
     uint8 device tensor."""
     import torch
-    dev = f"cuda:{ctx.device}"
+    dev = ctx.torch_device
     t = _limbs_tensor(limbs, dev)
     out = torch.empty(4 * t.numel() + 2, dtype=torch.uint8, device=dev)
     n = ctypes.c_size_t()
@@ -371,7 +386,7 @@ def to_decimal(ctx: Context, limbs, out=None, stream=None):
     significant first ("0" for zero).  `out` may be a preallocated uint8
     device tensor of at least cat_decimal_bound(len(limbs)) bytes."""
     import torch
-    dev = f"cuda:{ctx.device}"
+    dev = ctx.torch_device
     t = _limbs_tensor(limbs, dev)
     if out is None:
         out = torch.empty(max(cat_decimal_bound(t.numel()), 1), dtype=torch.uint8, device=dev)
@@ -402,7 +417,7 @@ def bigint_mul_noalloc(a, b, out=None, stream=None, device: int = 0):
 
 
 def bigint_pow(ctx: Context, a, e: int, stream=None):
-    dev = f"cuda:{ctx.device}"
+    dev = ctx.torch_device
     ta = _limbs_tensor(a, dev)
     na = ta.numel()
     bits = na * 32
@@ -415,7 +430,7 @@ def bigint_pow(ctx: Context, a, e: int, stream=None):
 
 
 def product_tree(ctx: Context, values, stream=None):
-    dev = f"cuda:{ctx.device}"
+    dev = ctx.torch_device
     tv = _limbs_tensor(values, dev)
     cap = max(1, tv.numel())
     out = _empty(cap, dev)
@@ -433,14 +448,15 @@ class FactorResult:
         self.ctx = ctx
         self.f = f
         ng = f.num_groups
-        self.exps = np.array([f.host_exps[i] for i in range(ng)], dtype=np.uint64)
-        self.offsets = np.array([f.host_offsets[i] for i in range(ng + 1)], dtype=np.uint64)
+        self.exps = np.frombuffer(ctypes.string_at(f.host_exps, 8 * ng), dtype=np.uint64).copy()
+        self.offsets = np.frombuffer(ctypes.string_at(f.host_offsets, 8 * (ng + 1)),
+                                     dtype=np.uint64).copy()
         self.num_primes = f.num_primes
         self.primes_sieved = f.primes_sieved
 
     def primes(self):
         """Device copy of the grouped primes as an int32 tensor (uint32 bits)."""
-        out = _empty(self.num_primes, f"cuda:{self.ctx.device}")
+        out = _empty(self.num_primes, self.ctx.torch_device)
         self.ctx.check(load().cat_factor_copy_primes(self.ctx.handle, ctypes.byref(self.f),
                                                      _ptr(out), self.num_primes,
                                                      _stream(None)))
@@ -465,7 +481,7 @@ def catalan_factor(ctx: Context, n: int, kind: int = CAT_CATALAN, stream=None) -
 
 
 def cat_reconstruct(ctx: Context, fact: FactorResult, cap: int, stream=None):
-    out = _empty(cap, f"cuda:{ctx.device}")
+    out = _empty(cap, ctx.torch_device)
     n = ctypes.c_size_t()
     ctx.check(load().cat_reconstruct(ctx.handle, ctypes.byref(fact.f), _ptr(out), cap,
                                      ctypes.byref(n), _stream(stream)))
@@ -476,7 +492,7 @@ def cat_exact(ctx: Context, kind: int, n: int, out=None, stream=None):
     """The exact quantity as an int32 device tensor of uint32 limbs.  `out`
     may be a preallocated int32 device tensor of at least cat_bound_limbs."""
     if out is None:
-        out = _empty(cat_bound_limbs(n, kind), f"cuda:{ctx.device}")
+        out = _empty(cat_bound_limbs(n, kind), ctx.torch_device)
     m = ctypes.c_size_t()
     ctx.check(load().cat_exact(ctx.handle, kind, n, _ptr(out), out.numel(),
                                ctypes.byref(m), _stream(stream)))
@@ -549,7 +565,7 @@ def cat_exact_batch(ctx: Context, reqs, out=None, stream=None):
     if rc != 0:
         raise CatError(rc, "cat_batch_bound")
     if out is None:
-        out = _empty(total.value, f"cuda:{ctx.device}")
+        out = _empty(total.value, ctx.torch_device)
     offs = np.zeros(max(1, count), dtype=np.uint64)
     lens = np.zeros(max(1, count), dtype=np.uint64)
     u64p = ctypes.POINTER(ctypes.c_uint64)
