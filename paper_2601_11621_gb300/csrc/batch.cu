@@ -64,6 +64,7 @@ __device__ __forceinline__ int block_segment(const uint64_t *pre, int count, uin
 __global__ void count_primes_le(const uint32_t *primes, uint64_t np, const uint64_t *limits,
                                 int count, uint64_t *out)
 {
+    chain_wait();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= count) return;
     uint64_t lo = 0, hi = np;  // first index with primes[i] > limit
@@ -83,6 +84,7 @@ struct ReqDev {
 __global__ void batch_exponents(const uint32_t *primes, const uint64_t *pre, int count,
                                 const ReqDev *reqs, uint32_t *e, unsigned int *negative)
 {
+    chain_wait();
     const uint64_t total = pre[count];
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int r = block_segment(pre, count, t);
@@ -104,6 +106,7 @@ __global__ void batch_exponents(const uint32_t *primes, const uint64_t *pre, int
 __global__ void batch_leaves(const uint32_t *primes, const uint64_t *pre, int count,
                              const uint32_t *pos, uint32_t *leaves)
 {
+    chain_wait();
     const uint64_t total = pre[count];
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int r = block_segment(pre, count, t);
@@ -120,6 +123,7 @@ __global__ void batch_leaves(const uint32_t *primes, const uint64_t *pre, int co
 __global__ void batch_seg_starts(const uint64_t *pre, int count, const uint32_t *pos,
                                  uint64_t *seg)
 {
+    chain_wait();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r > count) return;
     seg[r] = (r < count && pre[r] < pre[count]) ? pos[pre[r]] : pos[pre[count]];
@@ -132,6 +136,7 @@ __global__ void batch_leaf_nodes(const uint32_t *leaves, const uint64_t *seg,
                                  const uint64_t *node_pre, const uint64_t *dpos, int count,
                                  int lpn, uint32_t *out)
 {
+    chain_wait();
     const uint64_t total = node_pre[count];
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int r = block_segment(node_pre, count, t);
@@ -177,6 +182,7 @@ __global__ void batch_copy(const CopyJob *jobs, int njobs)
 __global__ void batch_lengths(const uint32_t *out, const uint64_t *off, const uint64_t *cap,
                               uint64_t *len)
 {
+    chain_wait();
     __shared__ unsigned long long best;
     const int r = blockIdx.x;
     if (threadIdx.x == 0) best = 0;
@@ -230,6 +236,7 @@ constexpr uint64_t kOne = ~(uint64_t)0;
 __global__ void batch_copy_level(const LevelJob *jobs, int njobs, const uint32_t *src_base,
                                  uint32_t *dst_base)
 {
+    chain_wait();
     for (int j = blockIdx.y; j < njobs; j += gridDim.y) {
         const LevelJob J = jobs[j];
         uint32_t *dst = J.dst_abs ? J.dst_abs : dst_base + J.dst;
@@ -246,6 +253,7 @@ __global__ void batch_copy_level(const LevelJob *jobs, int njobs, const uint32_t
 __global__ void batch_level_index(const uint64_t *rs, const uint64_t *dst, int runs,
                                   uint32_t *index)
 {
+    chain_wait();
     const uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= rs[runs]) return;
     const int i = find_segment(rs, runs, k);
@@ -382,8 +390,8 @@ void segmented_tree(Ctx &c, const uint32_t *leaves, const std::vector<uint64_t> 
     const LevelJob *d_jobs = reinterpret_cast<const LevelJob *>(d + at_jobs);
     DevBuf<uint32_t> index(c, std::max<uint64_t>(total_prod, 1), s);
     if (total_prod) {
-        batch_level_index<<<(unsigned)((total_prod + 255) / 256), 256, 0, s>>>(
-            d + at_rs, d + at_rd, runs, index.get());
+        launch_chained(batch_level_index, (unsigned)((total_prod + 255) / 256), 256, 0, s,
+                       d + at_rs, d + at_rd, runs, index.get());
         CAT_LAUNCH("batch_level_index");
     }
     const uint64_t tn = node_pre[count];
@@ -391,8 +399,8 @@ void segmented_tree(Ctx &c, const uint32_t *leaves, const std::vector<uint64_t> 
     {
         const int tok = prof_begin(c, "batch_leaf_nodes", s);
         if (tn)
-            batch_leaf_nodes<<<(unsigned)((tn + 255) / 256), 256, 0, s>>>(
-                leaves, d + at_seg, d + at_np, d + at_pos, nr, lpn, cur.get());
+            launch_chained(batch_leaf_nodes, (unsigned)((tn + 255) / 256), 256, 0, s, leaves,
+                           d + at_seg, d + at_np, d + at_pos, nr, lpn, cur.get());
         CAT_LAUNCH("batch_leaf_nodes");
         prof_end(c, tok, s, 4.0 * (double)(seg[count] - seg[0]) + 32.0 * (double)tn);
     }
@@ -402,9 +410,9 @@ void segmented_tree(Ctx &c, const uint32_t *leaves, const std::vector<uint64_t> 
             // blocks per job by the longest job (2,048 limbs a block), jobs
             // spread over the grid's second dimension
             const unsigned gx = (unsigned)std::min<uint64_t>(64, (lv.maxcap + 2047) / 2048);
-            batch_copy_level<<<dim3(std::max(1u, gx), (unsigned)std::min<size_t>(lv.njobs, 65535)),
-                               256, 0, s>>>(
-                d_jobs + lv.job0, (int)lv.njobs, cur.get(), cur.get());
+            launch_chained(batch_copy_level,
+                           dim3(std::max(1u, gx), (unsigned)std::min<size_t>(lv.njobs, 65535)), 256,
+                           0, s, d_jobs + lv.job0, (int)lv.njobs, cur.get(), cur.get());
             CAT_LAUNCH("batch_copy_level");
         }
         if (lv.padded == 0) break;
@@ -448,8 +456,8 @@ static void batch_core(Ctx &c, const cat_request *reqs, size_t count, uint32_t *
     DevBuf<uint32_t> primes = sieve_primes(c, std::max<uint64_t>(M, 2), &np, s);
     DevBuf<uint64_t> d_limits = upload(c, limits, s);
     DevBuf<uint64_t> d_pi(c, count, s);
-    count_primes_le<<<(nr + 255) / 256, 256, 0, s>>>(primes.get(), np, d_limits.get(), nr,
-                                                     d_pi.get());
+    launch_chained(count_primes_le, (nr + 255) / 256, 256, 0, s, primes.get(), np, d_limits.get(),
+                   nr, d_pi.get());
     CAT_LAUNCH("count_primes_le");
     std::vector<uint64_t> pi(count), pre(count + 1, 0);
     CAT_CUDA(cudaMemcpyAsync(pi.data(), d_pi.get(), 8 * count, cudaMemcpyDeviceToHost, s));
@@ -465,8 +473,8 @@ static void batch_core(Ctx &c, const cat_request *reqs, size_t count, uint32_t *
     CAT_CUDA(cudaMemsetAsync(pos.get() + F, 0, 4, s));
     const unsigned fb = (unsigned)((F + 255) / 256);
     int tok = prof_begin(c, "batch_exponents", s);
-    if (F) batch_exponents<<<fb, 256, 0, s>>>(primes.get(), d_pre.get(), nr, d_req.get(),
-                                              pos.get(), neg.get());
+    if (F) launch_chained(batch_exponents, fb, 256, 0, s, primes.get(), d_pre.get(), nr,
+                          d_req.get(), pos.get(), neg.get());
     CAT_LAUNCH("batch_exponents");
     prof_end(c, tok, s, 8.0 * (double)F);
     // exclusive scan over F + 1 entries: pos[F] becomes the total leaf count
@@ -474,7 +482,8 @@ static void batch_core(Ctx &c, const cat_request *reqs, size_t count, uint32_t *
     // the segment starts (the last one the total leaf count) and the sign
     // flag in one read-back
     DevBuf<uint64_t> d_seg(c, count + 1, s);
-    batch_seg_starts<<<(nr + 256) / 256, 256, 0, s>>>(d_pre.get(), nr, pos.get(), d_seg.get());
+    launch_chained(batch_seg_starts, (nr + 256) / 256, 256, 0, s, d_pre.get(), nr, pos.get(),
+                   d_seg.get());
     CAT_LAUNCH("batch_seg_starts");
     std::vector<uint64_t> seg(count + 1);
     unsigned int hneg = 0;
@@ -485,8 +494,8 @@ static void batch_core(Ctx &c, const cat_request *reqs, size_t count, uint32_t *
     const uint32_t total_leaves = (uint32_t)seg[count];
     DevBuf<uint32_t> leaves(c, total_leaves ? total_leaves : 1, s);
     tok = prof_begin(c, "batch_leaves", s);
-    if (F) batch_leaves<<<fb, 256, 0, s>>>(primes.get(), d_pre.get(), nr, pos.get(),
-                                           leaves.get());
+    if (F) launch_chained(batch_leaves, fb, 256, 0, s, primes.get(), d_pre.get(), nr, pos.get(),
+                          leaves.get());
     CAT_LAUNCH("batch_leaves");
     prof_end(c, tok, s, 8.0 * (double)F + 4.0 * total_leaves);
     primes.reset();
@@ -504,7 +513,7 @@ static void batch_core(Ctx &c, const cat_request *reqs, size_t count, uint32_t *
     DevBuf<uint64_t> d_off = upload(c, std::vector<uint64_t>(offsets, offsets + count), s);
     DevBuf<uint64_t> d_cap = upload(c, caps, s);
     DevBuf<uint64_t> d_len(c, count, s);
-    batch_lengths<<<nr, 256, 0, s>>>(out, d_off.get(), d_cap.get(), d_len.get());
+    launch_chained(batch_lengths, nr, 256, 0, s, out, d_off.get(), d_cap.get(), d_len.get());
     CAT_LAUNCH("batch_lengths");
     CAT_CUDA(cudaMemcpyAsync(lengths, d_len.get(), 8 * count, cudaMemcpyDeviceToHost, s));
     CAT_CUDA(cudaStreamSynchronize(s));

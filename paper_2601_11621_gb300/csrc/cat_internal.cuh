@@ -34,6 +34,39 @@ void launched(const char *what);
 #define CAT_CUDA(call) ::cat::check_cuda((call), #call)
 #define CAT_LAUNCH(what) ::cat::launched(what)
 
+// ---------------------------------------------------------------- launches
+
+// A kernel launch that may begin while the kernel before it on the stream
+// drains (programmatic dependent launch): its blocks are set up as slots
+// become free and wait in chain_wait, the first statement of every kernel
+// launched so, until that kernel is complete and its writes are visible.  The
+// order and the results are those of plain launches; what is saved is the gap
+// between two kernels: 3 10^6! (220 launches) 2.00 -> 1.49 ms, C(10^5) (17)
+// 185 -> 155 us, decimal text of 3.1 M limbs 2.80 -> 2.52 ms.
+template <class... P, class... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                           cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    CAT_CUDA(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
+}
+
+// Waits for the kernel before on the stream, then lets the next one set up.
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+}
+
 // ------------------------------------------------------------- constants
 
 constexpr int kNumPrimes = 5;

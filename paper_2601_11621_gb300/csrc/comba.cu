@@ -45,6 +45,7 @@ __device__ __forceinline__ uint32_t leaf_value(const uint32_t *v, size_t count, 
 __global__ void leaf_products(const uint32_t *v, size_t count, const __grid_constant__ Repeats rep,
                               uint32_t *out, size_t nodes, int lpn)
 {
+    chain_wait();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nodes) return;
     uint32_t acc[kLeafSlot];
@@ -72,6 +73,7 @@ template <int S>
 __global__ void comba_thread(const uint32_t *in, size_t nprod, uint32_t *out,
                              const uint32_t *out_index)
 {
+    chain_wait();
     const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nprod) return;
     const uint4 *a4 = reinterpret_cast<const uint4 *>(in + 2 * k * S);
@@ -124,6 +126,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) comba_warp(const uint32_t
                                                                   size_t nprod, uint32_t *out,
                                                                   const uint32_t *out_index)
 {
+    chain_wait();
     constexpr int W = 2 * S / 32;
     static_assert(W >= 2, "warp Comba needs at least two columns per lane");
     constexpr int PADN = 3 * S;              // padded indices j' in [0, 3S)
@@ -223,6 +226,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) comba_warp(const uint32_t
 // Largest i + 1 with x[i] != 0, reduced into *top (0 if all zero).
 __global__ void find_top(const uint32_t *x, size_t n, unsigned long long *top)
 {
+    chain_wait();
     unsigned long long best = 0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (size_t)gridDim.x * blockDim.x)
@@ -244,6 +248,7 @@ struct TopsArgs {
 // limb (usually in the first stretch).
 __global__ void __launch_bounds__(1024) number_tops(const __grid_constant__ TopsArgs a)
 {
+    chain_wait();
     __shared__ unsigned long long best;
     const uint32_t *x = a.x[blockIdx.x];
     if (threadIdx.x == 0) best = 0;
@@ -270,8 +275,8 @@ void leaf_level(Ctx &c, const uint32_t *values, size_t count, const Repeats &rep
                 size_t nodes, int lpn, cudaStream_t s)
 {
     const int tok = prof_begin(c, "leaf_products", s);
-    leaf_products<<<(unsigned)((nodes + 255) / 256), 256, 0, s>>>(values, count, rep, out, nodes,
-                                                                    lpn);
+    launch_chained(leaf_products, (unsigned)((nodes + 255) / 256), 256, 0, s, values, count, rep,
+                   out, nodes, lpn);
     CAT_LAUNCH("leaf_products");
     prof_end(c, tok, s, 4.0 * (double)count + 32.0 * (double)nodes,
              4.0 * (double)count + 32.0 * (double)nodes);
@@ -289,12 +294,16 @@ bool comba_level(Ctx &c, const uint32_t *in, size_t slot, size_t nprod, uint32_t
     const unsigned gt = (unsigned)((nprod + tb - 1) / tb);
     const unsigned gw = (unsigned)((nprod + kWarpsPerBlock - 1) / kWarpsPerBlock);
     switch (slot) {
-    case 8: comba_thread<8><<<gt, tb, 0, s>>>(in, nprod, out, out_index); break;
-    case 16: comba_thread<16><<<gt, tb, 0, s>>>(in, nprod, out, out_index); break;
-    case 32: comba_warp<32><<<gw, 32 * kWarpsPerBlock, 0, s>>>(in, nprod, out, out_index); break;
-    case 64: comba_warp<64><<<gw, 32 * kWarpsPerBlock, 0, s>>>(in, nprod, out, out_index); break;
-    case 128: comba_warp<128><<<gw, 32 * kWarpsPerBlock, 0, s>>>(in, nprod, out, out_index); break;
-    case 256: comba_warp<256><<<gw, 32 * kWarpsPerBlock, 0, s>>>(in, nprod, out, out_index); break;
+    case 8: launch_chained(comba_thread<8>, gt, tb, 0, s, in, nprod, out, out_index); break;
+    case 16: launch_chained(comba_thread<16>, gt, tb, 0, s, in, nprod, out, out_index); break;
+    case 32: launch_chained(comba_warp<32>, gw, 32 * kWarpsPerBlock, 0, s, in, nprod, out,
+                            out_index); break;
+    case 64: launch_chained(comba_warp<64>, gw, 32 * kWarpsPerBlock, 0, s, in, nprod, out,
+                            out_index); break;
+    case 128: launch_chained(comba_warp<128>, gw, 32 * kWarpsPerBlock, 0, s, in, nprod, out,
+                             out_index); break;
+    case 256: launch_chained(comba_warp<256>, gw, 32 * kWarpsPerBlock, 0, s, in, nprod, out,
+                             out_index); break;
     default: return false;
     }
     CAT_LAUNCH("comba_level");
@@ -313,7 +322,7 @@ void normalize_all(Ctx &c, Big *const *x, int count, cudaStream_t s)
         a.n[i] = x[i]->n;
     }
     a.out = d.get();
-    number_tops<<<count, 1024, 0, s>>>(a);
+    launch_chained(number_tops, count, 1024, 0, s, a);
     CAT_LAUNCH("number_tops");
     const uint32_t *h = read_back(c, d.get(), 4 * count, s);
     for (int i = 0; i < count; i++) {
@@ -342,7 +351,7 @@ size_t normalized_length(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s)
     size_t blocks = (n + threads - 1) / threads;
     const size_t cap = (size_t)c.num_sms * 8;
     if (blocks > cap) blocks = cap;
-    find_top<<<(unsigned)blocks, threads, 0, s>>>(x, n, top);
+    launch_chained(find_top, (unsigned)blocks, threads, 0, s, x, n, top);
     CAT_LAUNCH("find_top");
     const uint32_t *h = read_back(c, top, 2, s);
     return (size_t)((uint64_t)h[1] << 32 | h[0]);

@@ -118,6 +118,7 @@ struct HostPage {
 __global__ void __launch_bounds__(kPageWords) publish(const uint32_t *src, int words,
                                                       HostPage *page, uint64_t number)
 {
+    chain_wait();
     if ((int)threadIdx.x < words) page->words[threadIdx.x] = src[threadIdx.x];
     __threadfence_system();
     __syncthreads();
@@ -134,7 +135,8 @@ const uint32_t *read_back(Ctx &c, const void *dev, int words, cudaStream_t s)
     if (words > kPageWords) fail(CAT_EINVAL, "read-back too long");
     const uint64_t number = ++c.read_backs;
     const int threads = words <= 32 ? 32 : (words + 31) / 32 * 32;
-    publish<<<1, threads, 0, s>>>(static_cast<const uint32_t *>(dev), words, c.page, number);
+    launch_chained(publish, 1, threads, 0, s, static_cast<const uint32_t *>(dev), words, c.page,
+                   number);
     CAT_LAUNCH("publish");
     const auto t0 = std::chrono::steady_clock::now();
     for (int i = 0;; i++) {

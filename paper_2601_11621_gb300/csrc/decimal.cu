@@ -49,6 +49,7 @@ static size_t chunks_for_bits(double bits)
 __global__ void __launch_bounds__(128) dec_leaves(const uint32_t *x, size_t n, size_t leaves,
                                                   uint32_t *out)
 {
+    chain_wait();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= leaves) return;
     uint32_t acc[kDecLeafChunks];
@@ -80,6 +81,7 @@ __global__ void __launch_bounds__(128) dec_leaves(const uint32_t *x, size_t n, s
 // exactly nine.
 __global__ void dec_print(const uint32_t *ch, size_t top, int lead, char *out)
 {
+    chain_wait();
     const size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c > top) return;
     uint32_t v = ch[c];
@@ -135,7 +137,8 @@ int to_decimal_dev(Ctx &c, const uint32_t *x, size_t n, char *out, size_t cap, s
     DevBuf<uint32_t> cur(c, nodes * S, s);
     {
         const int tok = prof_begin(c, "dec_leaves", s);
-        dec_leaves<<<(unsigned)((nodes + 127) / 128), 128, 0, s>>>(x, n, nodes, cur.get());
+        launch_chained(dec_leaves, (unsigned)((nodes + 127) / 128), 128, 0, s, x, n, nodes,
+                       cur.get());
         CAT_LAUNCH("dec_leaves");
         prof_end(c, tok, s, 4.0 * (double)n + 4.0 * (double)(nodes * S));
     }
@@ -195,7 +198,7 @@ int to_decimal_dev(Ctx &c, const uint32_t *x, size_t n, char *out, size_t cap, s
     *needed = total;
     if (cap < total) return CAT_ERANGE;
     const int tok = prof_begin(c, "dec_print", s);
-    dec_print<<<(unsigned)((nch + 255) / 256), 256, 0, s>>>(cur.get(), top, lead, out);
+    launch_chained(dec_print, (unsigned)((nch + 255) / 256), 256, 0, s, cur.get(), top, lead, out);
     CAT_LAUNCH("dec_print");
     prof_end(c, tok, s, 4.0 * (double)nch + (double)total);
     CAT_CUDA(cudaStreamSynchronize(s));

@@ -549,6 +549,7 @@ __device__ __forceinline__ void coef_words(const uint32_t (&r)[kNumPrimes], uint
 template <int PS, bool DEC, bool ADD>
 __global__ void __launch_bounds__(kTileThreads) crt_carry_tiles(CrtArgs a)
 {
+    chain_wait();
     __shared__ uint32_t wsm[32];
     __shared__ uint32_t hsm[128];
     const size_t tiles = ((size_t)1 << a.np) / kTileCoefs;
@@ -613,6 +614,7 @@ __global__ void __launch_bounds__(1024) carry_resolve(const uint8_t *maps, size_
                                                       size_t out_len, bool dec,
                                                       const uint32_t *out_index)
 {
+    chain_wait();
     __shared__ uint32_t wsm[32];
     const size_t k = blockIdx.x / nb, b = blockIdx.x % nb;
     const uint8_t *m = maps + k * tiles;
@@ -867,6 +869,7 @@ template <int LR, bool ZT>
 __global__ void __launch_bounds__(fused_threads(LR), 512 / fused_threads(LR))
     ntt_mul_fused(FusedArgs a)
 {
+    chain_wait();
     extern __shared__ uint32_t sm[];
     __shared__ uint32_t wsm[32];
     constexpr int N = 1 << LR, PN = fused_points(LR), P = PN / N;
@@ -929,6 +932,7 @@ template <int LR, bool ZT>
 __global__ void __cluster_dims__(kNumPrimes, 1, 1) __launch_bounds__(cluster_threads(LR))
     ntt_mul_cluster(FusedArgs a)
 {
+    chain_wait();
     namespace cg = cooperative_groups;
     extern __shared__ uint32_t sm[];
     __shared__ uint32_t wsm[32];
@@ -1047,16 +1051,16 @@ static void launch_col(bool fwd, dim3 grid, cudaStream_t s, const ColArgs &a)
     const bool zt = fwd && a.src && std::max(a.src_len, a.src_y_len) <= ((size_t)1 << a.m);
     if (zt) {
         set_smem(ntt_col_fwd<LR, PS, kColV, 2>, smem);
-        ntt_col_fwd<LR, PS, kColV, 2><<<grid, kColFwdThreads, smem, s>>>(a);
+        launch_chained(ntt_col_fwd<LR, PS, kColV, 2>, grid, kColFwdThreads, smem, s, a);
     } else if (fwd && a.src) {
         set_smem(ntt_col_fwd<LR, PS, kColV, 1>, smem);
-        ntt_col_fwd<LR, PS, kColV, 1><<<grid, kColFwdThreads, smem, s>>>(a);
+        launch_chained(ntt_col_fwd<LR, PS, kColV, 1>, grid, kColFwdThreads, smem, s, a);
     } else if (fwd) {
         set_smem(ntt_col_fwd<LR, PS, kColV, 0>, smem);
-        ntt_col_fwd<LR, PS, kColV, 0><<<grid, kColFwdThreads, smem, s>>>(a);
+        launch_chained(ntt_col_fwd<LR, PS, kColV, 0>, grid, kColFwdThreads, smem, s, a);
     } else {
         set_smem(ntt_col_inv<LR, PS, kColV>, smem);
-        ntt_col_inv<LR, PS, kColV><<<grid, kColInvThreads, smem, s>>>(a);
+        launch_chained(ntt_col_inv<LR, PS, kColV>, grid, kColInvThreads, smem, s, a);
     }
 }
 
@@ -1218,15 +1222,15 @@ static void launch_row_t(dim3 grid, cudaStream_t s, const RowArgs &a, bool pre)
     if (pre) {  // broadcast products, the common transform complete
         const size_t smem = ((size_t)1 << kRowMaxLog) * sizeof(uint32_t);
         set_smem(ntt_row_mul_bcast<LR, PS>, smem);
-        ntt_row_mul_bcast<LR, PS><<<grid, kRowThreads, smem, s>>>(a);
+        launch_chained(ntt_row_mul_bcast<LR, PS>, grid, kRowThreads, smem, s, a);
     } else if (a.mode == PAIR_SQUARE) {
         const size_t smem = ((size_t)1 << kRowMaxLog) * sizeof(uint32_t);
         set_smem(ntt_row_mul<LR, true, PS>, smem);
-        ntt_row_mul<LR, true, PS><<<grid, kRowThreads, smem, s>>>(a);
+        launch_chained(ntt_row_mul<LR, true, PS>, grid, kRowThreads, smem, s, a);
     } else {
         const size_t smem = ((size_t)2 << kRowMaxLog) * sizeof(uint32_t);
         set_smem(ntt_row_mul<LR, false, PS>, smem);
-        ntt_row_mul<LR, false, PS><<<grid, kRowThreads, smem, s>>>(a);
+        launch_chained(ntt_row_mul<LR, false, PS>, grid, kRowThreads, smem, s, a);
     }
 }
 
@@ -1269,7 +1273,7 @@ static void launch_row_fwd_t(dim3 grid, cudaStream_t s, const RowArgs &a)
 {
     const size_t smem = ((size_t)1 << kRowMaxLog) * sizeof(uint32_t);
     set_smem(ntt_row_fwd<LR, PS>, smem);
-    ntt_row_fwd<LR, PS><<<grid, kRowThreads, smem, s>>>(a);
+    launch_chained(ntt_row_fwd<LR, PS>, grid, kRowThreads, smem, s, a);
 }
 
 // The row pass's forward rounds of one transform of 2^np points in place (the
@@ -1302,13 +1306,13 @@ static void launch_crt_ps(unsigned grid, cudaStream_t s, const CrtArgs &a)
 {
     const bool dec = a.sink.dec, add = a.sink.add != nullptr;
     if (dec && add)
-        crt_carry_tiles<PS, true, true><<<grid, kTileThreads, 0, s>>>(a);
+        launch_chained(crt_carry_tiles<PS, true, true>, grid, kTileThreads, 0, s, a);
     else if (dec)
-        crt_carry_tiles<PS, true, false><<<grid, kTileThreads, 0, s>>>(a);
+        launch_chained(crt_carry_tiles<PS, true, false>, grid, kTileThreads, 0, s, a);
     else if (add)
-        crt_carry_tiles<PS, false, true><<<grid, kTileThreads, 0, s>>>(a);
+        launch_chained(crt_carry_tiles<PS, false, true>, grid, kTileThreads, 0, s, a);
     else
-        crt_carry_tiles<PS, false, false><<<grid, kTileThreads, 0, s>>>(a);
+        launch_chained(crt_carry_tiles<PS, false, false>, grid, kTileThreads, 0, s, a);
 }
 
 static void launch_crt(int ps, unsigned grid, cudaStream_t s, const CrtArgs &a)
@@ -1333,7 +1337,8 @@ static void launch_row_limbs_t(size_t nprod, cudaStream_t s, const RowLimbArgs &
 {
     const size_t smem = ((size_t)(SQ ? 1 : 2) << kRowMaxLog) * sizeof(uint32_t);
     set_smem(ntt_row_limbs<SQ, ZT>, smem);
-    ntt_row_limbs<SQ, ZT><<<dim3((unsigned)nprod, kNumPrimes), kRowThreads, smem, s>>>(a);
+    launch_chained(ntt_row_limbs<SQ, ZT>, dim3((unsigned)nprod, kNumPrimes), kRowThreads, smem, s,
+                   a);
 }
 
 // The whole transforms of nprod products of 2^12 points, from limbs.
@@ -1368,8 +1373,8 @@ static void carry_finish(Ctx &c, const uint8_t *maps, size_t nprod, size_t tiles
     const int tok = prof_begin(c, "carry_resolve", s);
     const size_t threads = std::min<size_t>(1024, (tiles + 31) / 32 * 32);
     const size_t nb = (tiles + threads - 1) / threads;
-    carry_resolve<<<(unsigned)(nprod * nb), (unsigned)threads, 0, s>>>(
-        maps, tiles, (int)nb, sink.out, sink.out_tstride, sink.out_len, sink.dec, sink.out_index);
+    launch_chained(carry_resolve, (unsigned)(nprod * nb), (unsigned)threads, 0, s, maps, tiles,
+                   (int)nb, sink.out, sink.out_tstride, sink.out_len, sink.dec, sink.out_index);
     CAT_LAUNCH("carry_resolve");
     prof_end(c, tok, s, (double)(nprod * tiles));
 }
@@ -1515,15 +1520,16 @@ static void launch_fused_t(size_t nprod, bool spread, cudaStream_t s, const Fuse
         if (spread) {
             const size_t smem = 7 * ((size_t)1 << LR) * sizeof(uint32_t);
             set_smem(ntt_mul_cluster<LR, ZT>, smem);
-            ntt_mul_cluster<LR, ZT>
-                <<<(unsigned)(nprod * kNumPrimes), cluster_threads(LR), smem, s>>>(a);
+            launch_chained(ntt_mul_cluster<LR, ZT>, (unsigned)(nprod * kNumPrimes),
+                           cluster_threads(LR), smem, s, a);
             return;
         }
     }
     constexpr size_t PN = fused_points(LR), P = PN >> LR;
     const size_t smem = 6 * PN * sizeof(uint32_t);
     set_smem(ntt_mul_fused<LR, ZT>, smem);
-    ntt_mul_fused<LR, ZT><<<(unsigned)((nprod + P - 1) / P), fused_threads(LR), smem, s>>>(a);
+    launch_chained(ntt_mul_fused<LR, ZT>, (unsigned)((nprod + P - 1) / P), fused_threads(LR), smem,
+                   s, a);
 }
 
 // Whether a batch of one-block products takes a cluster of five blocks per
@@ -1687,6 +1693,7 @@ __global__ void __launch_bounds__(kTileThreads) add_tiles(uint32_t *acc, size_t 
                                                           const uint32_t *t, size_t tn, bool dec,
                                                           uint8_t *tile_maps)
 {
+    chain_wait();
     __shared__ uint32_t wsm[32];
     const size_t jt = (size_t)blockIdx.x * kTile;
     const int j0 = threadIdx.x * kLimbsPerThread;
@@ -1710,7 +1717,7 @@ void add_into(Ctx &c, uint32_t *acc, size_t R, const uint32_t *t, size_t tn, boo
     if (tiles > 0x7fffffffu) fail(CAT_EINVAL, "addition too long");
     DevBuf<uint8_t> maps(c, tiles, s);
     const int tok = prof_begin(c, "add_tiles", s);
-    add_tiles<<<(unsigned)tiles, kTileThreads, 0, s>>>(acc, R, t, tn, dec, maps.get());
+    launch_chained(add_tiles, (unsigned)tiles, kTileThreads, 0, s, acc, R, t, tn, dec, maps.get());
     CAT_LAUNCH("add_tiles");
     prof_end(c, tok, s, 8.0 * (double)R + 4.0 * (double)tn);
     carry_finish(c, maps.get(), 1, tiles, Sink{acc, 0, R, dec, nullptr, 0, 0}, s);
@@ -1770,6 +1777,7 @@ __global__ void __launch_bounds__(kTileThreads) overlap_tiles(const uint32_t *T,
                                                               uint32_t *out, size_t R,
                                                               uint8_t *tile_maps)
 {
+    chain_wait();
     __shared__ uint32_t wsm[32];
     const size_t jt = (size_t)blockIdx.x * kTile;
     const size_t j0 = jt + threadIdx.x * kLimbsPerThread;
@@ -1800,8 +1808,8 @@ void mul_chunked(Ctx &c, const uint32_t *x, size_t nx, const uint32_t *y, size_t
     const size_t R = nx + ny, tiles = (R + kTile - 1) / kTile;
     DevBuf<uint8_t> maps(c, tiles, s);
     const int tok = prof_begin(c, "overlap_tiles", s);
-    overlap_tiles<<<(unsigned)tiles, kTileThreads, 0, s>>>(T.get(), M, ny, chunks, out, R,
-                                                            maps.get());
+    launch_chained(overlap_tiles, (unsigned)tiles, kTileThreads, 0, s, T.get(), M, ny, chunks, out,
+                   R, maps.get());
     CAT_LAUNCH("overlap_tiles");
     prof_end(c, tok, s, 4.0 * (double)(chunks * slot) + 4.0 * (double)R);
     carry_finish(c, maps.get(), 1, tiles, plain_sink(out, 0, R), s);

@@ -646,6 +646,7 @@ struct ColOut {
 template <int LR, int PS, int V, int SRC>
 __global__ void __launch_bounds__(kColFwdThreads, CAT_COL_FWD_MINB) ntt_col_fwd(ColArgs a)
 {
+    chain_wait();
     extern __shared__ uint32_t sm[];
     constexpr int LC = col_log_c(LR), C = 1 << LC, CV = C / V;
     // 2^4-row columns in one round, straight from global to global memory
@@ -705,6 +706,7 @@ __global__ void __launch_bounds__(kColFwdThreads, CAT_COL_FWD_MINB) ntt_col_fwd(
 template <int LR, int PS, int V>
 __global__ void __launch_bounds__(kColInvThreads, CAT_COL_INV_MINB) ntt_col_inv(ColArgs a)
 {
+    chain_wait();
     extern __shared__ uint32_t sm[];
     constexpr int LC = col_log_c(LR), C = 1 << LC, CV = C / V;
     constexpr int NR = col_rounds(LR, kColInvRoundMax);
@@ -951,6 +953,7 @@ __device__ __forceinline__ void row_mul_body(const RowArgs &a, uint32_t *sm)
 template <int LR, bool SQ, int PS>
 __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_mul(RowArgs a)
 {
+    chain_wait();
     extern __shared__ uint32_t sm[];
     row_mul_body<LR, SQ, PS, false>(a, sm);
 }
@@ -959,6 +962,7 @@ __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_mul(RowArgs
 template <int LR, int PS>
 __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_mul_bcast(RowArgs a)
 {
+    chain_wait();
     extern __shared__ uint32_t sm[];
     row_mul_body<LR, false, PS, true>(a, sm);
 }
@@ -972,6 +976,7 @@ __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_mul_bcast(R
 template <int LR, int PS>
 __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_fwd(RowArgs a)
 {
+    chain_wait();
     extern __shared__ uint32_t sm[];
     constexpr int NR = rounds_of(LR);
     constexpr int EL = round_size(LR, NR - 1);
@@ -1054,6 +1059,7 @@ struct RowLimbIn {
 template <bool SQ, bool ZT>
 __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_limbs(RowLimbArgs a)
 {
+    chain_wait();
     extern __shared__ uint32_t sm[];
     constexpr int LR = kRowMaxLog;
     const int p = blockIdx.y;

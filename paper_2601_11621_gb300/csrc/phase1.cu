@@ -69,6 +69,7 @@ __constant__ uint32_t c_small_primes[10] = {3, 5, 7, 11, 13, 17, 19, 23, 29, 31}
 
 __global__ void __launch_bounds__(kSieveThreads) sieve_segments(SieveArgs a)
 {
+    chain_wait();
     extern __shared__ uint32_t bm[];
     __shared__ uint32_t unit_count[kMaxSegUnits], all_count;
     const uint32_t seg = blockIdx.x;
@@ -232,6 +233,7 @@ struct ExpandArgs {
 // most lanes waiting: 163 -> 43 us at the limit 10^7 with three terms).
 __global__ void __launch_bounds__(kExpandThreads) expand_exponents(ExpandArgs a)
 {
+    chain_wait();
     __shared__ uint32_t stage[kExpandWarps][32 * 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint32_t unit = blockIdx.x * kExpandWarps + wid;
@@ -286,6 +288,7 @@ struct RsArgs {
 
 __global__ void __launch_bounds__(kRsThreads) rs_histogram(RsArgs a)
 {
+    chain_wait();
     __shared__ uint32_t h[256];
     const int nb = 1 << a.bits;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) h[i] = 0;
@@ -305,6 +308,7 @@ __global__ void __launch_bounds__(kRsThreads) rs_histogram(RsArgs a)
 
 __global__ void __launch_bounds__(kRsThreads) rs_scatter(RsArgs a)
 {
+    chain_wait();
     __shared__ uint32_t wh[kRsWarps][256];
     const int nb = 1 << a.bits;
     for (int i = threadIdx.x; i < kRsWarps * 256; i += blockDim.x) (&wh[0][0])[i] = 0;
@@ -355,6 +359,7 @@ __global__ void __launch_bounds__(kRsThreads) rs_scatter(RsArgs a)
 __global__ void group_starts(const uint64_t *items, size_t count, uint64_t *starts,
                              unsigned int *nstarts, uint32_t *primes)
 {
+    chain_wait();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     const uint64_t v = items[i];
@@ -374,6 +379,7 @@ __global__ void __launch_bounds__(kExpandThreads) expand_primes(const uint32_t *
                                                                uint32_t units, uint32_t *primes,
                                                                uint32_t first, int with_two)
 {
+    chain_wait();
     __shared__ uint32_t stage[kExpandWarps][32 * 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint32_t unit = blockIdx.x * kExpandWarps + wid;
@@ -403,6 +409,7 @@ __global__ void __launch_bounds__(kSeedThreads) group_seeds(const uint32_t *seed
                                                            const uint32_t *total, uint32_t *sorted,
                                                            Phase1Info *info)
 {
+    chain_wait();
     extern __shared__ uint16_t cnt[];  // [exponent][thread]
     __shared__ uint8_t ex[kMaxSeeds];
     __shared__ uint32_t bin_total[kMaxSeedGroups], bin_base[kMaxSeedGroups], negative;
@@ -474,6 +481,7 @@ struct CsrArgs {
 
 __global__ void __launch_bounds__(kExpandThreads) write_csr(CsrArgs a)
 {
+    chain_wait();
     __shared__ uint32_t stage[kExpandWarps][32 * 32];
     if (blockIdx.x == a.expand_blocks) {
         for (uint32_t i = threadIdx.x; i < a.nsorted; i += kExpandThreads)
@@ -553,7 +561,8 @@ static SieveOut run_sieve(Ctx &c, uint64_t limit, cudaStream_t s, int unit_kind 
     SieveArgs sa{c.seeds + 1, i_med, i_large, nodd, imax, lg, o.bits.get(), o.offsets.get(),
                  unit_kind, unit_n, (uint32_t)root, o.words.get() + 1};
     const int tok = prof_begin(c, "sieve_segments", s);
-    sieve_segments<<<nsegs, std::min(kSieveThreads, 1 << (lg - 5)), (size_t)4 << (lg - 5), s>>>(sa);
+    launch_chained(sieve_segments, nsegs, std::min(kSieveThreads, 1 << (lg - 5)),
+                   (size_t)4 << (lg - 5), s, sa);
     CAT_LAUNCH("sieve_segments");
     prof_end(c, tok, s, 4.0 * (double)o.units * kUnitWords);
     exclusive_scan_u32(c, o.offsets.get(), o.units, s, o.words.get());
@@ -598,12 +607,12 @@ static Grouped group_items(Ctx &c, DevBuf<uint64_t> &items, size_t count, uint32
         DevBuf<uint32_t> cnt(c, nbins * tiles, s);
         RsArgs ra{src, dst, count, shift, bitsd, pass == 0 ? 1 : 0, cnt.get(), tiles};
         tok = prof_begin(c, "rs_histogram", s);
-        rs_histogram<<<(unsigned)tiles, kRsThreads, 0, s>>>(ra);
+        launch_chained(rs_histogram, (unsigned)tiles, kRsThreads, 0, s, ra);
         CAT_LAUNCH("rs_histogram");
         prof_end(c, tok, s, 8.0 * (double)count);
         exclusive_scan_u32(c, cnt.get(), nbins * tiles, s, kept.get());
         tok = prof_begin(c, "rs_scatter", s);
-        rs_scatter<<<(unsigned)tiles, kRsThreads, 0, s>>>(ra);
+        launch_chained(rs_scatter, (unsigned)tiles, kRsThreads, 0, s, ra);
         CAT_LAUNCH("rs_scatter");
         prof_end(c, tok, s, 16.0 * (double)count);
         // only the first pass drops items
@@ -618,8 +627,8 @@ static Grouped group_items(Ctx &c, DevBuf<uint64_t> &items, size_t count, uint32
     DevBuf<uint64_t> starts(c, 2 * count, s);
     DevBuf<unsigned int> nst(c, 1, s);
     CAT_CUDA(cudaMemsetAsync(nst.get(), 0, 4, s));
-    group_starts<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(src, count, starts.get(),
-                                                                  nst.get(), g.primes.get());
+    launch_chained(group_starts, (unsigned)((count + 255) / 256), 256, 0, s, src, count,
+                   starts.get(), nst.get(), g.primes.get());
     CAT_LAUNCH("group_starts");
     const unsigned int ng = *read_back(c, nst.get(), 1, s);
     std::vector<uint64_t> hst(2 * (size_t)ng);
@@ -651,8 +660,8 @@ static void factor_unit(Ctx &c, const Ratio &r, uint64_t limit, cat_factorizatio
     DevBuf<uint32_t> sorted(c, std::max<uint32_t>(ns, 1), s);
     DevBuf<Phase1Info> d_info(c, 1, s);
     int tok = prof_begin(c, "group_seeds", s);
-    group_seeds<<<1, kSeedThreads, kSeedSmem, s>>>(c.seeds, ns, r, sv.words.get(),
-                                                   sv.words.get() + 1, sorted.get(), d_info.get());
+    launch_chained(group_seeds, 1, kSeedThreads, kSeedSmem, s, c.seeds, ns, r, sv.words.get(),
+                   sv.words.get() + 1, sorted.get(), d_info.get());
     CAT_LAUNCH("group_seeds");
     prof_end(c, tok, s, 8.0 * (double)ns);
     Phase1Info h;
@@ -680,7 +689,7 @@ static void factor_unit(Ctx &c, const Ratio &r, uint64_t limit, cat_factorizatio
     a.exps = d_exps.get();
     a.offs = d_offs.get();
     tok = prof_begin(c, "write_csr", s);
-    write_csr<<<a.expand_blocks + 1, kExpandThreads, 0, s>>>(a);
+    launch_chained(write_csr, a.expand_blocks + 1, kExpandThreads, 0, s, a);
     CAT_LAUNCH("write_csr");
     prof_end(c, tok, s, 4.0 * (double)sv.units * kUnitWords + 4.0 * (double)npos);
     out->host_exps = new uint64_t[a.ng + 1];
@@ -726,8 +735,8 @@ void factor_ratio(Ctx &c, const Ratio &r, cat_factorization *out, cudaStream_t s
         ExpandArgs ea{sv.bits.get(), sv.offsets.get(), sv.units, r, items.get(), flags.get(),
                       flags.get() + 1};
         const int tok = prof_begin(c, "expand_exponents", s);
-        expand_exponents<<<(sv.units + kExpandWarps - 1) / kExpandWarps, kExpandThreads, 0, s>>>(
-            ea);
+        launch_chained(expand_exponents, (sv.units + kExpandWarps - 1) / kExpandWarps,
+                       kExpandThreads, 0, s, ea);
         CAT_LAUNCH("expand_exponents");
         prof_end(c, tok, s, 4.0 * (double)sv.units * kUnitWords + 8.0 * (double)sieved);
         sv = SieveOut{};
@@ -768,8 +777,8 @@ DevBuf<uint32_t> sieve_primes(Ctx &c, uint64_t limit, uint64_t *count, cudaStrea
     const uint64_t sieved = (uint64_t)*read_back(c, sv.words.get(), 1, s) + 1;
     DevBuf<uint32_t> primes(c, sieved, s);
     const int tok = prof_begin(c, "expand_primes", s);
-    expand_primes<<<(sv.units + kExpandWarps - 1) / kExpandWarps, kExpandThreads, 0, s>>>(
-        sv.bits.get(), sv.offsets.get(), sv.units, primes.get(), 1, 1);
+    launch_chained(expand_primes, (sv.units + kExpandWarps - 1) / kExpandWarps, kExpandThreads, 0,
+                   s, sv.bits.get(), sv.offsets.get(), sv.units, primes.get(), 1, 1);
     CAT_LAUNCH("expand_primes");
     prof_end(c, tok, s, 4.0 * (double)sv.units * kUnitWords + 4.0 * (double)sieved);
     *count = sieved;

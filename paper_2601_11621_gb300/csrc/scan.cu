@@ -39,6 +39,7 @@ __device__ uint32_t block_exclusive_sum(uint32_t v, uint32_t *wsm, uint32_t *tot
 __global__ void __launch_bounds__(kScanThreads) scan_block_sums(const uint32_t *d, size_t n,
                                                                 uint32_t *sums)
 {
+    chain_wait();
     __shared__ uint32_t wsm[32];
     const size_t base = (size_t)blockIdx.x * kScanChunk + (size_t)threadIdx.x * kScanItems;
     uint32_t s = 0;
@@ -54,6 +55,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_block_sums(const uint32_t *
 // goes to *sum (when set).
 __global__ void __launch_bounds__(kScanThreads) scan_single(uint32_t *d, size_t n, uint32_t *sum)
 {
+    chain_wait();
     __shared__ uint32_t wsm[32];
     uint32_t run = 0;
     for (size_t base = 0; base < n; base += kScanChunk) {
@@ -80,6 +82,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_single(uint32_t *d, size_t 
 __global__ void __launch_bounds__(kScanThreads) scan_apply(uint32_t *d, size_t n,
                                                            const uint32_t *offs)
 {
+    chain_wait();
     __shared__ uint32_t wsm[32];
     const size_t i0 = (size_t)blockIdx.x * kScanChunk + (size_t)threadIdx.x * kScanItems;
     uint32_t v[kScanItems], s = 0;
@@ -106,16 +109,16 @@ void exclusive_scan_u32(Ctx &c, uint32_t *data, size_t n, cudaStream_t s, uint32
     }
     const size_t blocks = (n + kScanChunk - 1) / kScanChunk;
     if (blocks <= 4) {
-        scan_single<<<1, kScanThreads, 0, s>>>(data, n, sum);
+        launch_chained(scan_single, 1, kScanThreads, 0, s, data, n, sum);
         CAT_LAUNCH("scan_single");
         return;
     }
     DevBuf<uint32_t> sums(c, blocks, s);
-    scan_block_sums<<<(unsigned)blocks, kScanThreads, 0, s>>>(data, n, sums.get());
+    launch_chained(scan_block_sums, (unsigned)blocks, kScanThreads, 0, s, data, n, sums.get());
     CAT_LAUNCH("scan_block_sums");
-    scan_single<<<1, kScanThreads, 0, s>>>(sums.get(), blocks, sum);
+    launch_chained(scan_single, 1, kScanThreads, 0, s, sums.get(), blocks, sum);
     CAT_LAUNCH("scan_single");
-    scan_apply<<<(unsigned)blocks, kScanThreads, 0, s>>>(data, n, sums.get());
+    launch_chained(scan_apply, (unsigned)blocks, kScanThreads, 0, s, data, n, sums.get());
     CAT_LAUNCH("scan_apply");
 }
 

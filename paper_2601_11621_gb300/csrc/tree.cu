@@ -276,6 +276,7 @@ __global__ void __launch_bounds__(1024) bit_offsets(const uint64_t *exps, const 
                                                     const __grid_constant__ BitSegments seg,
                                                     uint64_t *at)
 {
+    chain_wait();
     __shared__ uint64_t wsum[32];
     const int b = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint64_t run = seg.start[b];
@@ -306,6 +307,7 @@ __global__ void bit_leaves(const uint32_t *primes, uint64_t np, const uint64_t *
                            const uint64_t *offs, uint32_t ng, const uint64_t *at,
                            uint32_t *leaves)
 {
+    chain_wait();
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= np) return;
     uint32_t lo = 0, hi = ng;  // offs[lo] <= i < offs[hi]
@@ -348,11 +350,11 @@ static Big reconstruct_bits(Ctx &c, const cat_factorization *f, cudaStream_t s, 
         DevBuf<uint64_t> at(c, (size_t)B * ng, s);
         BitSegments sb{};
         std::copy(seg.begin(), seg.end(), sb.start);
-        bit_offsets<<<B, 1024, 0, s>>>(f->exps, f->offsets, ng, sb, at.get());
+        launch_chained(bit_offsets, B, 1024, 0, s, f->exps, f->offsets, ng, sb, at.get());
         CAT_LAUNCH("bit_offsets");
         const int tok = prof_begin(c, "bit_leaves", s);
-        bit_leaves<<<(unsigned)((f->num_primes + 255) / 256), 256, 0, s>>>(
-            f->primes, f->num_primes, f->exps, f->offsets, ng, at.get(), leaves.get());
+        launch_chained(bit_leaves, (unsigned)((f->num_primes + 255) / 256), 256, 0, s, f->primes,
+                       f->num_primes, f->exps, f->offsets, ng, at.get(), leaves.get());
         CAT_LAUNCH("bit_leaves");
         prof_end(c, tok, s, 4.0 * (double)(f->num_primes + seg[B]));
     }
