@@ -321,6 +321,20 @@ __device__ __forceinline__ void bf_dif1(uint32_t &x, uint32_t &y, uint32_t q)
     }
 }
 
+// bf_dif1 whose outputs go into a Montgomery product that takes any 32-bit
+// value: no corrections, sum and difference in [0, 4q) (set 0) or [0, 2q).
+template <int PS>
+__device__ __forceinline__ void bf_dif1_any(uint32_t &x, uint32_t &y, uint32_t q)
+{
+    if constexpr (PS == 2) {
+        bf_dif1<PS>(x, y, q);
+    } else {
+        const uint32_t a = x, b = y;
+        x = a + b;
+        y = a - b + (PS == 0 ? 2 * q : q);
+    }
+}
+
 // Inverse (decimation-in-time) butterfly (x, y) <- (x + y w, x - y w) on
 // inverse-range residues.
 template <int PS>
@@ -343,11 +357,12 @@ __device__ __forceinline__ void bf_dit(uint32_t &x, uint32_t &y, uint2 w, uint32
     }
 }
 
-template <int PS>
+// FRESH: the inputs are products, in the forward range.
+template <int PS, bool FRESH>
 __device__ __forceinline__ void bf_dit1(uint32_t &x, uint32_t &y, uint32_t q)
 {
     if constexpr (PS == 0) {
-        const uint32_t a = csub(x, 2 * q), t = csub(y, 2 * q);
+        const uint32_t a = FRESH ? x : csub(x, 2 * q), t = FRESH ? y : csub(y, 2 * q);
         x = a + t;
         y = 2 * a + 2 * q - x;
     } else {

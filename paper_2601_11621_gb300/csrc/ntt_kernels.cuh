@@ -26,6 +26,13 @@ struct zero_top : std::false_type {};
 template <class T>
 struct zero_top<T, std::void_t<decltype(T::kZeroTop)>> : std::bool_constant<T::kZeroTop> {};
 
+// Whether an output of a register round multiplies its points by factors that
+// take any 32-bit value.
+template <class T, class = void>
+struct takes_any : std::false_type {};
+template <class T>
+struct takes_any<T, std::void_t<decltype(T::kTakesAny)>> : std::bool_constant<T::kTakesAny> {};
+
 // size of DIF round rd of nr rounds (counted from the top stage bits); when
 // the stages do not split evenly the last rounds take the extra ones, so that
 // the round at stage bits [0, E) (which carries the column twiddles) is the
@@ -99,8 +106,11 @@ __device__ __forceinline__ uint2 tw_at(const TwRef &T, int idx)
 // In a round with B = 0 the twiddle index is a compile-time constant, and the
 // butterflies with (k mod 2^st) = 0 have twiddle w^0 = 1: no multiply.  With
 // ZT the top stage's second inputs are zero, so its butterflies are
-// (x, 0) -> (x, x w): one product, no sum or difference.
-template <int E, int B, int NA, int PS, bool ZT = false>
+// (x, 0) -> (x, x w): one product, no sum or difference.  ANY: the outputs go
+// into products that take any 32-bit value, so the last stage, whose twiddles
+// are all 1, makes no corrections (and the inverse's first stage, whose inputs
+// are always products, needs none: together C(2,050,572,903) 80.7 -> 80.1 ms).
+template <int E, int B, int NA, int PS, bool ZT = false, bool ANY = false>
 __device__ __forceinline__ void dif_stages(uint32_t (&x)[NA][1 << E], int glow, const TwRef &T,
                                            uint32_t q)
 {
@@ -123,7 +133,10 @@ __device__ __forceinline__ void dif_stages(uint32_t (&x)[NA][1 << E], int glow, 
             }
             if (B == 0 && (k & ((1 << st) - 1)) == 0) {
 #pragma unroll
-                for (int a = 0; a < NA; a++) bf_dif1<PS>(x[a][k], x[a][k + (1 << st)], q);
+                for (int a = 0; a < NA; a++) {
+                    if (ANY && st == 0) bf_dif1_any<PS>(x[a][k], x[a][k + 1], q);
+                    else bf_dif1<PS>(x[a][k], x[a][k + (1 << st)], q);
+                }
                 continue;
             }
             const int p = glow + ((k & ((1 << st) - 1)) << B);
@@ -145,7 +158,10 @@ __device__ __forceinline__ void dit_stages(uint32_t (&x)[NA][1 << E], int glow, 
             if (k & (1 << st)) continue;
             if (B == 0 && (k & ((1 << st) - 1)) == 0) {
 #pragma unroll
-                for (int a = 0; a < NA; a++) bf_dit1<PS>(x[a][k], x[a][k + (1 << st)], q);
+                for (int a = 0; a < NA; a++) {
+                    if (st == 0) bf_dit1<PS, true>(x[a][k], x[a][k + 1], q);
+                    else bf_dit1<PS, false>(x[a][k], x[a][k + (1 << st)], q);
+                }
                 continue;
             }
             const int p = glow + ((k & ((1 << st) - 1)) << B);
@@ -180,7 +196,7 @@ __device__ __forceinline__ void round_io(const IN &in, const OUT &out, const TwR
         uint32_t x[NA][1 << E];
         in.template load<E, B, NA>(x, base, c);
         if (FWD)
-            dif_stages<E, B, NA, PS, zero_top<IN>::value>(x, glow, T, q);
+            dif_stages<E, B, NA, PS, zero_top<IN>::value, takes_any<OUT>::value>(x, glow, T, q);
         else
             dit_stages<E, B, NA, PS>(x, glow, T, q);
         out.template store<E, B, NA>(x, base, c);
@@ -581,6 +597,7 @@ struct ColTw {
 // Forward pass output: element (row, col) times w_M^(col * bitrev(row)).
 template <int LR, int PS, int NR, int V>
 struct ColOutTw {
+    static constexpr bool kTakesAny = true;
     uint32_t *p;
     uint32_t S, col0;
     ColTw<LR, PS, NR, kColFwdThreads, V> tw;
