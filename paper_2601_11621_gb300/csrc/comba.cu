@@ -1,7 +1,8 @@
 // comba.cu -- the lower levels of the balanced product tree (Sec. 3.2):
-// many independent small products, by column-wise schoolbook ("Comba")
-// multiplication with 96-bit column accumulators built from 32x32->64
-// multiply-add chains.
+// many independent small products by schoolbook multiplication: column-wise
+// ("Comba") with 96-bit column accumulators, by a thread (8 limbs) or a warp
+// per product, or row-wise by one or two threads per product where there are
+// enough products (comba_rows).
 //
 // Layout: a tree level is an array of nodes in fixed slots of S limbs (node i
 // at [i S, (i+1) S)), zero-padded.  A product of 2^k values below 2^32 always
@@ -221,6 +222,174 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) comba_warp(const uint32_t
     for (int w = 0; w < W; w++) o[w] = limb[w];
 }
 
+// ------------------------------------- one product per thread, row by row
+
+// The lowest P + 1 words of a running sum V as two rows of aligned 64-bit
+// pieces, V = sum_j e[j] 2^(32 j) + sum_j o[j] 2^(32 (j + 1)).  row() returns
+// V's lowest word after V <- floor(V / 2^32) + a B, the caller passing the old
+// o as e and the old e as o: the pieces of a row's products with B's even
+// words fall on e, those with its odd words on o one place further down, so
+// that the shift is the choice of the destination.  Each piece is one wide
+// multiply-add with carry in and out; V < 2^(32 (P + 1)) always, so the
+// carries end in o's top word.
+template <int P>
+__device__ __forceinline__ uint32_t comba_row(uint32_t (&e)[P], uint32_t (&o)[P], uint32_t a,
+                                              const uint32_t (&b)[P])
+{
+    asm volatile("add.cc.u32 %0, %0, %1;" : "+r"(e[0]) : "r"(o[1]));
+#pragma unroll
+    for (int k = 0; k + 2 < P; k += 2)
+        asm volatile("madc.lo.cc.u32 %0, %2, %3, %4;\n\t"
+                     "madc.hi.cc.u32 %1, %2, %3, %5;"
+                     : "=r"(o[k]), "=r"(o[k + 1])
+                     : "r"(a), "r"(b[k + 1]), "r"(o[k + 2]), "r"(o[k + 3]));
+    asm volatile("madc.lo.cc.u32 %0, %2, %3, 0;\n\t"
+                 "madc.hi.u32 %1, %2, %3, 0;"
+                 : "=r"(o[P - 2]), "=r"(o[P - 1]) : "r"(a), "r"(b[P - 1]));
+    asm volatile("mad.lo.cc.u32 %0, %2, %3, %0;\n\t"
+                 "madc.hi.cc.u32 %1, %2, %3, %1;"
+                 : "+r"(e[0]), "+r"(e[1]) : "r"(a), "r"(b[0]));
+#pragma unroll
+    for (int k = 2; k < P; k += 2)
+        asm volatile("madc.lo.cc.u32 %0, %2, %3, %0;\n\t"
+                     "madc.hi.cc.u32 %1, %2, %3, %1;"
+                     : "+r"(e[k]), "+r"(e[k + 1]) : "r"(a), "r"(b[k]));
+    asm volatile("addc.u32 %0, %0, 0;" : "+r"(o[P - 1]));
+    return e[0];
+}
+
+// A product's operands a, b (S words each) in shared memory, a at 0 and b at
+// kB; products are kStride (odd) words apart, so that a warp's accesses to the
+// same word of each fall in distinct banks (with two threads per product the
+// gap puts the second thread's words half the banks away).
+template <int S, int T>
+struct CombaRows {
+    static constexpr int kPer = 32 / T;  // products per warp
+    static constexpr int kB = S + (T == 2 ? 16 : 0);
+    static constexpr int kStride = kB + S + 1;
+    static constexpr size_t kBytes = 4 * (size_t)kPer * kStride;
+};
+
+// T threads per product, thread t with words [t P, t P + P) of b (P = S / T)
+// in registers, all of a's words in turn from shared memory.  Each row emits
+// one word; the words of thread 0 take the place of a's, those of thread 1 of
+// b's, and the two threads' numbers are added at the end.
+//
+// Bound by the multiply pipe (an S = 64 level: three instructions per wide
+// multiply-add, the pipe 92 % busy by their rates), where a warp per product
+// spends half of its multiply-adds on B's zero padding and four instructions
+// on each.  A level of 2^25 limbs, before -> after: slots of 16 69 -> 54 us
+// (a thread per product reading its 128 bytes alone), 32 220 -> 81 us, 64
+// 292 -> 186 us.
+template <int S, int T>
+__global__ void __launch_bounds__(32) comba_rows(const uint32_t *in, size_t nprod, uint32_t *out,
+                                                 const uint32_t *out_index)
+{
+    chain_wait();
+    using R = CombaRows<S, T>;
+    constexpr int P = S / T;
+    static_assert((T == 1 || T == 2) && P % 4 == 0 && S % 8 == 0, "shape");
+    extern __shared__ uint32_t comba_smem[];
+    const int lane = threadIdx.x;
+    const size_t k0 = (size_t)blockIdx.x * R::kPer;
+    const int np = nprod - k0 < (size_t)R::kPer ? (int)(nprod - k0) : R::kPer;
+    {
+        const uint32_t *src = in + 2 * k0 * S;
+        const int words = 2 * S * np;
+        for (int w = lane; w < words; w += 32) {
+            const int q = w / (2 * S), i = w % (2 * S);
+            const uint32_t to = (uint32_t)__cvta_generic_to_shared(
+                comba_smem + q * R::kStride + i + (i >= S ? R::kB - S : 0));
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(src + w));
+        }
+        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
+    }
+    // products past the last one work on whatever is in their words
+    const int t = T == 1 ? 0 : lane / R::kPer;
+    uint32_t *A = comba_smem + (lane % R::kPer) * R::kStride, *B = A + R::kB;
+    uint32_t *em = t ? B : A;
+    uint32_t b[P], e[P], o[P];
+#pragma unroll
+    for (int j = 0; j < P; j++) {
+        b[j] = B[t * P + j];
+        e[j] = o[j] = 0;
+    }
+    if (T > 1) __syncwarp();
+    uint32_t a0 = A[0], a1 = A[1];
+#pragma unroll 1
+    for (int i = 0; i < S; i += 2) {
+        // the next two words of a (those past the last are b's or the gap's, unused)
+        const uint32_t n0 = A[i + 2], n1 = A[i + 3];
+        if (T > 1) __syncwarp();
+        em[i] = comba_row<P>(e, o, a0, b);
+        em[i + 1] = comba_row<P>(o, e, a1, b);
+        a0 = n0;
+        a1 = n1;
+    }
+    // V / 2^32 = words e[1 .. P) and o[0 .. P), the roles as after an even row:
+    // o is the row that held the last emitted word
+    uint32_t top[P];
+    {
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < P; j++) {
+            const uint64_t v = (uint64_t)(j + 1 < P ? o[j + 1] : 0u) + e[j] + c;
+            top[j] = (uint32_t)v;
+            c = (uint32_t)(v >> 32);
+        }
+    }
+    if (T == 1) {
+#pragma unroll
+        for (int j = 0; j < P; j++) B[j] = top[j];
+    } else {
+        __syncwarp();
+        uint32_t c = 0;
+        if (t == 0) {
+            // words [P, S) += the other thread's first, then its next P meet top
+#pragma unroll 4
+            for (int j = 0; j < P; j++) {
+                const uint64_t v = (uint64_t)A[P + j] + B[j] + c;
+                A[P + j] = (uint32_t)v;
+                c = (uint32_t)(v >> 32);
+            }
+#pragma unroll
+            for (int j = 0; j < P; j++) {
+                const uint64_t v = (uint64_t)top[j] + B[P + j] + c;
+                B[j] = (uint32_t)v;
+                c = (uint32_t)(v >> 32);
+            }
+        }
+        c = __shfl_sync(0xffffffffu, c, lane % R::kPer);
+        if (t == 1) {
+#pragma unroll
+            for (int j = 0; j < P; j++) {
+                const uint64_t v = (uint64_t)top[j] + c;
+                B[P + j] = (uint32_t)v;
+                c = (uint32_t)(v >> 32);
+            }
+        }
+    }
+    __syncwarp();
+    for (int q = 0; q < np; q++) {
+        const size_t node = out_index ? (size_t)out_index[k0 + q] : k0 + q;
+        uint32_t *dst = out + 2 * node * S;
+        const uint32_t *from = comba_smem + q * R::kStride;
+#pragma unroll
+        for (int i = lane; i < 2 * S; i += 32) dst[i] = from[i + (i >= S ? R::kB - S : 0)];
+    }
+}
+
+template <int S, int T>
+void launch_rows(const uint32_t *in, size_t nprod, uint32_t *out, cudaStream_t s,
+                 const uint32_t *out_index)
+{
+    using R = CombaRows<S, T>;
+    static_assert(R::kBytes <= 48 * 1024, "no opt-in needed");
+    launch_chained(comba_rows<S, T>, (unsigned)((nprod + R::kPer - 1) / R::kPer), 32, R::kBytes, s,
+                   in, nprod, out, out_index);
+}
+
 // ------------------------------------------------------------ utilities
 
 // Largest i + 1 with x[i] != 0, reduced into *top (0 if all zero).
@@ -289,17 +458,31 @@ bool comba_level(Ctx &c, const uint32_t *in, size_t slot, size_t nprod, uint32_t
 {
     if (nprod == 0) return true;
     if (slot > 256) return false;
-    const int tok = prof_begin(c, slot <= 16 ? "comba_thread" : "comba_warp", s);
+    // Rows from two products per lane and SM on: below that a warp per product
+    // spreads the few products over more of the chip (8,189 products of 32 and
+    // 64 limbs: 5.2 and 11.3 us by warps, 6.0 and 11.8 us by rows; 16,381: 8.2
+    // and 20.7 us, 6.2 and 16.6 us).  A row's latency keeps one thread per
+    // product ahead at 32 limbs (2^19 products: 81 us, two threads 104 us) and
+    // two at 64, whose registers else leave nine warps per SM (2^18: 207 and
+    // 186 us).  Products of 16 limbs go by rows at any count.
+    const bool rows = slot == 16 || (slot <= 64 && nprod >= 64 * (size_t)c.num_sms);
+    const int tok = prof_begin(c, slot == 8 ? "comba_thread" : rows ? "comba_rows" : "comba_warp", s);
     const unsigned tb = 256;
     const unsigned gt = (unsigned)((nprod + tb - 1) / tb);
     const unsigned gw = (unsigned)((nprod + kWarpsPerBlock - 1) / kWarpsPerBlock);
     switch (slot) {
     case 8: launch_chained(comba_thread<8>, gt, tb, 0, s, in, nprod, out, out_index); break;
-    case 16: launch_chained(comba_thread<16>, gt, tb, 0, s, in, nprod, out, out_index); break;
-    case 32: launch_chained(comba_warp<32>, gw, 32 * kWarpsPerBlock, 0, s, in, nprod, out,
-                            out_index); break;
-    case 64: launch_chained(comba_warp<64>, gw, 32 * kWarpsPerBlock, 0, s, in, nprod, out,
-                            out_index); break;
+    case 16: launch_rows<16, 1>(in, nprod, out, s, out_index); break;
+    case 32:
+        if (rows) launch_rows<32, 1>(in, nprod, out, s, out_index);
+        else launch_chained(comba_warp<32>, gw, 32 * kWarpsPerBlock, 0, s, in, nprod, out,
+                            out_index);
+        break;
+    case 64:
+        if (rows) launch_rows<64, 2>(in, nprod, out, s, out_index);
+        else launch_chained(comba_warp<64>, gw, 32 * kWarpsPerBlock, 0, s, in, nprod, out,
+                            out_index);
+        break;
     case 128: launch_chained(comba_warp<128>, gw, 32 * kWarpsPerBlock, 0, s, in, nprod, out,
                              out_index); break;
     case 256: launch_chained(comba_warp<256>, gw, 32 * kWarpsPerBlock, 0, s, in, nprod, out,
