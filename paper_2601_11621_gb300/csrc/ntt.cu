@@ -564,7 +564,54 @@ struct CrtArgs {
     int np;             // log2 points
     Sink sink;          // product k's limbs (out_len <= 2^(np+1))
     uint8_t *tile_maps; // [product][tiles], compact carry maps
+    // when set, the products are summed, product k at coefficient k step
+    // (a multiple of 4), and a product reaches into the next one's stretch only
+    uint32_t step, nprod;
 };
+
+// The residues of N consecutive coefficients from j on (runs of 4 start at
+// multiples of 4) of the sum of the products step coefficients apart: product
+// k = j / step from its own coefficient r on, and the tail of product k - 1.
+template <int PS, int N>
+__device__ __forceinline__ void summed_residues(const CrtArgs &a, uint32_t j,
+                                                uint32_t (&x)[N][kNumPrimes])
+{
+    const uint32_t k = j / a.step, r = j - k * a.step;
+    const bool own = k < a.nprod, tail = k >= 1 && k <= a.nprod && a.step + r < (1u << a.np);
+    const uint32_t *go = a.G + ((size_t)k << a.np) + r;
+    const uint32_t *gt = a.G + ((size_t)(k - 1) << a.np) + a.step + r;
+#pragma unroll
+    for (int p = 0; p < kNumPrimes; p++) {
+        uint32_t u[N] = {}, v[N] = {};
+        if constexpr (N == 4) {
+            if (own) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(go + p * a.gpstride);
+                u[0] = w.x; u[1] = w.y; u[2] = w.z; u[3] = w.w;
+            }
+            if (tail) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(gt + p * a.gpstride);
+                v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
+            }
+        } else {
+            if (own) u[0] = go[p * a.gpstride];
+            if (tail) v[0] = gt[p * a.gpstride];
+        }
+        const uint32_t q = c_q[PS][p];
+#pragma unroll
+        for (int i = 0; i < N; i++) {
+            // below 2^32: set 0's residues lie in [0, 4q), the others' in
+            // [0, q), q < 2^30, 2^31 and 2^32
+            if constexpr (PS == 0) {
+                x[i][p] = min(u[i], u[i] - 2 * q) + min(v[i], v[i] - 2 * q);
+            } else if constexpr (PS == 1) {
+                x[i][p] = u[i] + v[i];
+            } else {
+                const uint32_t t = q - v[i];
+                x[i][p] = u[i] >= t ? u[i] - t : u[i] + v[i];
+            }
+        }
+    }
+}
 
 template <int PS, bool DEC>
 __device__ __forceinline__ void coef_words(const uint32_t (&r)[kNumPrimes], uint32_t (&w)[5])
@@ -579,13 +626,19 @@ __device__ __forceinline__ void coef_words(const uint32_t (&r)[kNumPrimes], uint
 // One tile of 1,024 coefficients (2,048 limbs) per block: each thread
 // remainders its run of four (one 16-byte load per prime: tiles, runs and the
 // prime arrays are multiples of 4 words apart) and sums them into limbs.
-template <int PS, bool DEC, bool ADD>
-__global__ void __launch_bounds__(kTileThreads, 5) crt_carry_tiles(CrtArgs a)
+//
+// SUM: one product from the products of a long operand's chunks.  The chunks'
+// coefficients meet as residues, so that every coefficient is remaindered and
+// carried once; before, the chunk products were written out as limbs and
+// added by a pass of their own (a 2^23 x 2^21 limb product: 556 -> 505 us;
+// 52,063 x 23,097 limbs, whose last chunk was a product by itself: 85 -> 56 us).
+template <int PS, bool DEC, bool ADD, bool SUM>
+__global__ void __launch_bounds__(kTileThreads, SUM ? 4 : 5) crt_carry_tiles(CrtArgs a)
 {
     chain_wait();
     __shared__ uint32_t wsm[32];
     __shared__ uint32_t hsm[128];
-    const size_t tiles = ((size_t)1 << a.np) / kTileCoefs;
+    const size_t tiles = SUM ? (size_t)gridDim.x : ((size_t)1 << a.np) / kTileCoefs;
     const size_t k = blockIdx.x / tiles;
     const size_t t = blockIdx.x % tiles;
     const size_t jt = t * kTileCoefs;
@@ -593,10 +646,14 @@ __global__ void __launch_bounds__(kTileThreads, 5) crt_carry_tiles(CrtArgs a)
     const uint32_t *g0 = a.G + (k << a.np) + jt;
     const int j0 = threadIdx.x * kCoefsPerThread;
     uint32_t r[kCoefsPerThread][kNumPrimes];
+    if constexpr (SUM) {
+        summed_residues<PS>(a, (uint32_t)jt + j0, r);
+    } else {
 #pragma unroll
-    for (int p = 0; p < kNumPrimes; p++) {
-        const uint4 x = *reinterpret_cast<const uint4 *>(g0 + p * a.gpstride + j0);
-        r[0][p] = x.x; r[1][p] = x.y; r[2][p] = x.z; r[3][p] = x.w;
+        for (int p = 0; p < kNumPrimes; p++) {
+            const uint4 x = *reinterpret_cast<const uint4 *>(g0 + p * a.gpstride + j0);
+            r[0][p] = x.x; r[1][p] = x.y; r[2][p] = x.z; r[3][p] = x.w;
+        }
     }
     // the tile's predecessor: coefficients jt - 2 and jt - 1 (none for tile 0),
     // by the first two threads side by side, loaded beside their runs so that
@@ -604,9 +661,16 @@ __global__ void __launch_bounds__(kTileThreads, 5) crt_carry_tiles(CrtArgs a)
     const bool pred = threadIdx.x < 2 && t > 0;
     uint32_t pr[kNumPrimes] = {};
     if (pred) {
+        if constexpr (SUM) {
+            uint32_t x[1][kNumPrimes];
+            summed_residues<PS>(a, (uint32_t)jt + threadIdx.x - 2, x);
 #pragma unroll
-        for (int p = 0; p < kNumPrimes; p++)
-            pr[p] = g0[(long)(p * a.gpstride) + (int)threadIdx.x - 2];
+            for (int p = 0; p < kNumPrimes; p++) pr[p] = x[0][p];
+        } else {
+#pragma unroll
+            for (int p = 0; p < kNumPrimes; p++)
+                pr[p] = g0[(long)(p * a.gpstride) + (int)threadIdx.x - 2];
+        }
     }
     CoefRun run;
 #pragma unroll
@@ -1151,6 +1215,9 @@ struct Operand {
     const uint32_t *p;
     size_t tstride;  // limbs between consecutive transforms (for batches)
     size_t len;      // valid limbs per transform
+    // the transform with fewer limbs than the others, if any
+    unsigned ragged = ~0u;
+    size_t ragged_len = 0;
 };
 constexpr Operand kNoSource{nullptr, 0, 0};
 
@@ -1192,6 +1259,8 @@ static void col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, s
     a.src = src;
     a.src_tstride = x.tstride;
     a.src_len = x.len;
+    a.ragged = x.ragged;
+    a.ragged_len = x.ragged_len;
     a.tw = c.twiddles;
     const size_t ctas = total >> (r + col_log_c(r));
     a.nblk = (unsigned)(total >> m);
@@ -1336,14 +1405,16 @@ template <int PS>
 static void launch_crt_ps(unsigned grid, cudaStream_t s, const CrtArgs &a)
 {
     const bool dec = a.sink.dec, add = a.sink.add != nullptr;
-    if (dec && add)
-        launch_chained(crt_carry_tiles<PS, true, true>, grid, kTileThreads, 0, s, a);
+    if (a.step)  // binary, without an addend (mul_chunked)
+        launch_chained(crt_carry_tiles<PS, false, false, true>, grid, kTileThreads, 0, s, a);
+    else if (dec && add)
+        launch_chained(crt_carry_tiles<PS, true, true, false>, grid, kTileThreads, 0, s, a);
     else if (dec)
-        launch_chained(crt_carry_tiles<PS, true, false>, grid, kTileThreads, 0, s, a);
+        launch_chained(crt_carry_tiles<PS, true, false, false>, grid, kTileThreads, 0, s, a);
     else if (add)
-        launch_chained(crt_carry_tiles<PS, false, true>, grid, kTileThreads, 0, s, a);
+        launch_chained(crt_carry_tiles<PS, false, true, false>, grid, kTileThreads, 0, s, a);
     else
-        launch_chained(crt_carry_tiles<PS, false, false>, grid, kTileThreads, 0, s, a);
+        launch_chained(crt_carry_tiles<PS, false, false, false>, grid, kTileThreads, 0, s, a);
 }
 
 static void launch_crt(int ps, unsigned grid, cudaStream_t s, const CrtArgs &a)
@@ -1417,8 +1488,12 @@ static void carry_finish(Ctx &c, const uint8_t *maps, size_t nprod, size_t tiles
 //  mode PAIR_SQUARE:    nprod squares of x's transforms;
 //  mode PAIR_BROADCAST: nprod products of x's transforms (tstride apart) with
 //                       one y, whose transform is computed once.
+// With step, the products (PAIR_BROADCAST, np >= 13) are summed into one, each
+// step coefficients (a multiple of 4) after the one before, and none reaches
+// past the next one's stretch of step.
 static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x, Operand y,
-                              const Sink &sink, cudaStream_t s, MulScratch &&m = MulScratch{})
+                              const Sink &sink, cudaStream_t s, MulScratch &&m = MulScratch{},
+                              uint32_t step = 0)
 {
     const NttPlan P = make_plan(c, np);
     const int PS = set_for(np);
@@ -1526,9 +1601,10 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
         }
     }
     // remaindering and carries
-    const size_t tiles = N / kTileCoefs;
+    const size_t sums = step ? 1 : nprod;
+    const size_t tiles = step ? (sink.out_len + kTile - 1) / kTile : N / kTileCoefs;
     if (!m.fixed) {
-        m.mb = DevBuf<uint8_t>(c, nprod * tiles, s);
+        m.mb = DevBuf<uint8_t>(c, sums * tiles, s);
         m.maps = m.mb.get();
     }
     CrtArgs ca;
@@ -1537,11 +1613,13 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
     ca.np = np;
     ca.sink = sink;
     ca.tile_maps = m.maps;
+    ca.step = step;
+    ca.nprod = (uint32_t)nprod;
     tok = prof_begin(c, "crt_carry_tiles", s);
-    launch_crt(PS, (unsigned)(nprod * tiles), s, ca);
+    launch_crt(PS, (unsigned)(sums * tiles), s, ca);
     CAT_LAUNCH("crt_carry_tiles");
-    prof_end(c, tok, s, 4.0 * kNumPrimes * (double)gp + 4.0 * (double)nprod * (double)sink.out_len);
-    carry_finish(c, m.maps, nprod, tiles, sink, s);
+    prof_end(c, tok, s, 4.0 * kNumPrimes * (double)gp + 4.0 * (double)sums * (double)sink.out_len);
+    carry_finish(c, m.maps, sums, tiles, sink, s);
 }
 
 template <int LR, bool ZT>
@@ -1823,11 +1901,25 @@ __global__ void __launch_bounds__(kTileThreads) overlap_tiles(const uint32_t *T,
 
 // out[0 .. nx + ny) = x y by chunks of M = 2^k - ny >= ny limbs of x, each
 // multiplied by y in one batch (y transformed once).
+//
+// Transforms of 2^13 points or more sum the chunk products as residues (M
+// rounded down to whole runs of four coefficients; at least ny still, 2^(k-1)
+// being a multiple of 8 limbs and not below ny); the last chunk is shorter.
+// The one-block and one-row products write limbs, which overlap_tiles adds.
 void mul_chunked(Ctx &c, const uint32_t *x, size_t nx, const uint32_t *y, size_t ny, int k,
                  uint32_t *out, cudaStream_t s)
 {
     const size_t L = (size_t)1 << k, M = L - ny, slot = L;
     if (ny == 0 || M < ny) fail(CAT_EINVAL, "chunk size below the short operand");
+    if (k - 1 > kRowMaxLog) {
+        const size_t m = M & ~(size_t)7, n = (nx + m - 1) / m;
+        Operand ox{x, m, m}, oy{y, 0, ny};
+        ox.ragged = (unsigned)(n - 1);
+        ox.ragged_len = nx - (n - 1) * m;
+        ntt_mul_multipass(c, k - 1, PAIR_BROADCAST, n, ox, oy, plain_sink(out, 0, nx + ny), s,
+                          MulScratch{}, (uint32_t)(m / 2));
+        return;
+    }
     const size_t full = nx / M, rem = nx - full * M, chunks = full + (rem ? 1 : 0);
     DevBuf<uint32_t> T(c, chunks * slot, s);
     if (full) mul_broadcast(c, x, M, M, full, y, ny, plain_sink(T.get(), slot, slot), s);

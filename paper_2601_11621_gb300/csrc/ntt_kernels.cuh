@@ -358,6 +358,8 @@ struct ColArgs {
     const uint32_t *src;   // first forward pass: limb source (else null)
     size_t src_tstride;    // limbs between consecutive transforms' sources
     size_t src_len;        // valid limbs per transform (rest are zero)
+    unsigned ragged;       // the transform of ragged_len limbs instead (or none)
+    size_t ragged_len;
     int src_al;            // every source starts on a 16-byte boundary
     unsigned last;         // the transform whose source is src_y (or none)
     const uint32_t *src_y;
@@ -684,7 +686,9 @@ __global__ void __launch_bounds__(kColFwdThreads, CAT_COL_FWD_MINB) ntt_col_fwd(
             return ColSrcIn<PS, V, SRC == 2>{y ? a.src_y : a.src + blk * a.src_tstride,
                                              (uint32_t)Sr,
                                              (uint32_t)col0,
-                                             (uint32_t)(y ? a.src_y_len : a.src_len),
+                                             (uint32_t)(y                 ? a.src_y_len
+                                                        : blk == a.ragged ? a.ragged_len
+                                                                          : a.src_len),
                                              (y ? a.src_y_al : a.src_al) != 0,
                                              q,
                                              b ? a.coef_b.c[p] : a.coef.c[p]};

@@ -67,8 +67,9 @@ static int clog2(size_t x)
 }
 
 // For a long x and a short y: the chunk transform size 2^k whose estimated
-// cost (transform points x log2 points x set cost, plus the overlap pass)
-// beats one product of nx + ny limbs, or 0 if none does.
+// cost (transform points x log2 points x set cost, plus the overlap pass, or
+// the column passes' traffic above 2^12 points) beats one product of nx + ny
+// limbs, or 0 if none does.
 static int chunk_log(const Ctx &c, size_t nx, size_t ny)
 {
     if (nx < 2 * ny || nx + ny <= 4096) return 0;
