@@ -652,7 +652,8 @@ static void batch_core(Ctx &c, const cat_request *reqs, size_t count, uint32_t *
         CAT_LAUNCH("tile_segments");
         const int tok = prof_begin(c, "batch_flags", s);
         launch_chained(batch_flags, (unsigned)ntiles, kFlatThreads, 0, s, primes.get(), inv.get(),
-                       d_pre.get(), nr, first.get(), d_req.get(), flags.get(), tiles.get(), xs, neg);
+                       d_pre.get(), nr, first.get(), d_req.get(), flags.get(), tiles.get(), xs,
+                       neg);
         CAT_LAUNCH("batch_flags");
         prof_end(c, tok, s, 4.0 * (double)F);
     }

@@ -466,7 +466,8 @@ bool comba_level(Ctx &c, const uint32_t *in, size_t slot, size_t nprod, uint32_t
     // two at 64, whose registers else leave nine warps per SM (2^18: 207 and
     // 186 us).  Products of 16 limbs go by rows at any count.
     const bool rows = slot == 16 || (slot <= 64 && nprod >= 64 * (size_t)c.num_sms);
-    const int tok = prof_begin(c, slot == 8 ? "comba_thread" : rows ? "comba_rows" : "comba_warp", s);
+    const char *name = slot == 8 ? "comba_thread" : rows ? "comba_rows" : "comba_warp";
+    const int tok = prof_begin(c, name, s);
     const unsigned tb = 256;
     const unsigned gt = (unsigned)((nprod + tb - 1) / tb);
     const unsigned gw = (unsigned)((nprod + kWarpsPerBlock - 1) / kWarpsPerBlock);

@@ -61,6 +61,13 @@ static cudaMemPool_t pool_for(int device)
     return g_pools[device];
 }
 
+bool has_room(const Ctx &c, size_t bytes)
+{
+    if (c.budget && c.in_use + bytes > c.budget) return false;
+    return !c.shared_in_use || !c.shared_budget ||
+           c.shared_in_use->load() + bytes <= c.shared_budget;
+}
+
 void *dev_alloc(Ctx &c, size_t bytes, cudaStream_t s)
 {
     if (bytes == 0) return nullptr;
@@ -79,7 +86,8 @@ void *dev_alloc(Ctx &c, size_t bytes, cudaStream_t s)
         }
         if (c.shared_peak) {
             size_t pk = c.shared_peak->load();
-            while (before + bytes > pk && !c.shared_peak->compare_exchange_weak(pk, before + bytes)) {
+            while (before + bytes > pk &&
+                   !c.shared_peak->compare_exchange_weak(pk, before + bytes)) {
             }
         }
     }

@@ -23,8 +23,9 @@
 // Exactness: a level's product coefficients are below min(len) (10^9)^2 <
 // 2^25 10^36 < 10^44 (a coefficient is two digits of base 10^9), inside the
 // five-prime range, and each node sum lo + hi 2^(32 w) < 2^(64 w) fits the
-// next level's chunk count, so no carry leaves a node.  The one product too long for a single transform (the top
-// level of very long numbers) goes by pieces (mul_acc).
+// next level's chunk count, so no carry leaves a node.  The one product too
+// long for a single transform (the top level of very long numbers) goes by
+// pieces (mul_acc).
 #include "cat_internal.cuh"
 
 #include <math.h>

@@ -65,7 +65,8 @@ void copy_to_host(Ctx &c, uint32_t *host, const uint32_t *dev, size_t n, cudaStr
         return;
     }
     const int tok = prof_begin(c, "to_host", s);
-    const bool wide = ((reinterpret_cast<uintptr_t>(d) | reinterpret_cast<uintptr_t>(dev)) & 15) == 0;
+    const bool wide =
+        ((reinterpret_cast<uintptr_t>(d) | reinterpret_cast<uintptr_t>(dev)) & 15) == 0;
     const size_t items = wide ? n / 4 : n;
     const unsigned blocks = (unsigned)std::min<size_t>(
         kToHostBlocks, std::max<size_t>(1, (items + kToHostThreads - 1) / kToHostThreads));

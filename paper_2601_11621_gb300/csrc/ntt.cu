@@ -36,7 +36,8 @@ namespace cat {
 // --------------------------------------------------------------- constants
 
 #define CAT_SET_ROW(f, s) \
-    {f(ntt_prime(s, 0)), f(ntt_prime(s, 1)), f(ntt_prime(s, 2)), f(ntt_prime(s, 3)), f(ntt_prime(s, 4))}
+    {f(ntt_prime(s, 0)), f(ntt_prime(s, 1)), f(ntt_prime(s, 2)), f(ntt_prime(s, 3)), \
+     f(ntt_prime(s, 4))}
 #define CAT_SET_CONST(f) {CAT_SET_ROW(f, 0), CAT_SET_ROW(f, 1), CAT_SET_ROW(f, 2)}
 #define CAT_Q(q) (q)
 __constant__ uint32_t c_q[kNumSets][kNumPrimes] = CAT_SET_CONST(CAT_Q);
@@ -60,7 +61,8 @@ void upload_low_twiddles(const uint2 *tables)
         for (int p = 0; p < kNumPrimes; p++)
             for (int d = 0; d < 2; d++)
                 for (int j = 0; j < 16; j++)
-                    h[set][p][d][j] = tables[(((size_t)set * kNumPrimes + p) * 2 + d) * kTwPerDir + j];
+                    h[set][p][d][j] =
+                        tables[(((size_t)set * kNumPrimes + p) * 2 + d) * kTwPerDir + j];
     CAT_CUDA(cudaMemcpyToSymbol(c_tw_low, h, sizeof(h)));
 }
 
@@ -1272,7 +1274,8 @@ static void col_pass(Ctx &c, int ps, bool fwd, uint32_t *data, size_t pstride, s
         bytes = 4.0 * kNumPrimes * (double)total +
                 4.0 * (double)x.len * (double)((total >> m) - (y ? 1 : 0)) +
                 (y ? 4.0 * (double)y->len : 0.0);
-    const int tok = prof_begin(c, fwd ? (src ? "ntt_col_fwd_first" : "ntt_col_fwd") : "ntt_col_inv", s);
+    const char *name = !fwd ? "ntt_col_inv" : src ? "ntt_col_fwd_first" : "ntt_col_fwd";
+    const int tok = prof_begin(c, name, s);
     if (ps == 0) {
         switch (r) {
         case 1: launch_col<1, 0>(fwd, grid, s, a); break;
@@ -1905,14 +1908,17 @@ __global__ void __launch_bounds__(kTileThreads) overlap_tiles(const uint32_t *T,
 // Transforms of 2^13 points or more sum the chunk products as residues (M
 // rounded down to whole runs of four coefficients; at least ny still, 2^(k-1)
 // being a multiple of 8 limbs and not below ny); the last chunk is shorter.
-// The one-block and one-row products write limbs, which overlap_tiles adds.
+// The one-block and one-row products write limbs, which overlap_tiles adds; so
+// do longer ones where a budget has no room for all chunks' residues at once
+// (10 bytes per limb of 2 n + 1 transforms: up to four chunks of which the
+// last is short take less one after the other).
 void mul_chunked(Ctx &c, const uint32_t *x, size_t nx, const uint32_t *y, size_t ny, int k,
                  uint32_t *out, cudaStream_t s)
 {
     const size_t L = (size_t)1 << k, M = L - ny, slot = L;
     if (ny == 0 || M < ny) fail(CAT_EINVAL, "chunk size below the short operand");
-    if (k - 1 > kRowMaxLog) {
-        const size_t m = M & ~(size_t)7, n = (nx + m - 1) / m;
+    const size_t m = M & ~(size_t)7, n = (nx + m - 1) / m;
+    if (k - 1 > kRowMaxLog && has_room(c, 10 * (2 * n + 1) * L + (nx + ny) / kTile + 1024)) {
         Operand ox{x, m, m}, oy{y, 0, ny};
         ox.ragged = (unsigned)(n - 1);
         ox.ragged_len = nx - (n - 1) * m;

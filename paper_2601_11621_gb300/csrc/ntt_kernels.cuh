@@ -53,14 +53,20 @@ __host__ __device__ constexpr int dif_base(int lr, int rd, int nr)
     for (int j = 0; j <= rd; j++) b -= round_size(lr, j, nr);
     return b;
 }
-__host__ __device__ constexpr int dif_base(int lr, int rd) { return dif_base(lr, rd, rounds_of(lr)); }
+__host__ __device__ constexpr int dif_base(int lr, int rd)
+{
+    return dif_base(lr, rd, rounds_of(lr));
+}
 
 // DIT round rd (counted from the bottom) mirrors DIF round NR-1-rd
 __host__ __device__ constexpr int dit_size(int lr, int rd, int nr)
 {
     return round_size(lr, nr - 1 - rd, nr);
 }
-__host__ __device__ constexpr int dit_size(int lr, int rd) { return dit_size(lr, rd, rounds_of(lr)); }
+__host__ __device__ constexpr int dit_size(int lr, int rd)
+{
+    return dit_size(lr, rd, rounds_of(lr));
+}
 
 __host__ __device__ constexpr int dit_base(int lr, int rd, int nr)
 {
@@ -68,7 +74,10 @@ __host__ __device__ constexpr int dit_base(int lr, int rd, int nr)
     for (int j = 0; j < rd; j++) b += dit_size(lr, j, nr);
     return b;
 }
-__host__ __device__ constexpr int dit_base(int lr, int rd) { return dit_base(lr, rd, rounds_of(lr)); }
+__host__ __device__ constexpr int dit_base(int lr, int rd)
+{
+    return dit_base(lr, rd, rounds_of(lr));
+}
 
 // Shared-memory address swizzle: the four-word chunks of address a (bits 2-4,
 // the bank's upper bits) are XORed with a GF(2)-linear image of its row-of-32
@@ -312,8 +321,10 @@ __device__ __forceinline__ void load_coefs(uint32_t (&x)[1 << E], const uint32_t
 // (64 KiB), otherwise 2^(13-LR) columns (8192 points, 32 KiB), so that
 // every thread has a group to work on even for short columns.
 // Launch shapes of the passes (compile-time knobs; the defaults are the
-// fastest measured per C(2,050,572,903) on GB300, 142.0 -> 125.7 ms with the
-// two-column groups below): threads per forward / inverse column-pass block,
+// fastest measured per C(2,050,572,903) on GB300: forward rounds of at most
+// three stages, inverse rounds of four, three row or forward blocks per SM
+// instead of four and four inverse blocks are all slower or equal): threads
+// per forward / inverse column-pass block,
 // the most stages per register round in those passes, and the minimum
 // resident blocks per SM of the row pass and of the forward column pass
 // (which cap their registers at 64: four blocks per SM).
@@ -344,9 +355,10 @@ constexpr int kColInvThreads = CAT_COL_INV_THREADS;
 constexpr int kColMinLog = 4;   // columns of at least 2^4 rows
 constexpr int kColMaxLog = 10;  // and at most 2^10
 // Most stages per register round in the forward and inverse column passes
-// (measured per C(2,050,572,903) with two-column groups: forward passes
-// 39.2 -> 35.0 ms with four-stage rounds at 64 registers, inverse passes
-// 17.7 ms with three-stage rounds against 18.9 with four).
+// (with three primes of 32-bit coefficients, per C(2,050,572,903): forward
+// passes 39.2 -> 35.0 ms with four-stage rounds at 64 registers, inverse
+// passes 17.7 ms with three-stage rounds against 18.9 with four; the same
+// order with five primes).
 constexpr int kColFwdRoundMax = CAT_COL_FWD_RMAX;
 constexpr int kColInvRoundMax = CAT_COL_INV_RMAX;
 __host__ __device__ constexpr int col_rounds(int lr, int most) { return (lr + most - 1) / most; }
@@ -706,20 +718,21 @@ __global__ void __launch_bounds__(kColFwdThreads, CAT_COL_FWD_MINB) ntt_col_fwd(
         round_io<LR, CV, 0, LR, true, V, true, PS, kColFwdThreads>(in, out, TR, q);
     } else {
         const SmemIO<LR, CV, true> sio{sm};
-        round_io<LR, CV, dif_base(LR, 0, NR), round_size(LR, 0, NR), true, V, true, PS, kColFwdThreads>(in, sio,
-                                                                                       TR, q);
+        round_io<LR, CV, dif_base(LR, 0, NR), round_size(LR, 0, NR), true, V, true, PS,
+                 kColFwdThreads>(in, sio, TR, q);
         __syncthreads();
         if constexpr (NR >= 3) {
-            round_io<LR, CV, dif_base(LR, 1, NR), round_size(LR, 1, NR), true, V, true, PS, kColFwdThreads>(
-                sio, sio, TR, q);
+            round_io<LR, CV, dif_base(LR, 1, NR), round_size(LR, 1, NR), true, V, true, PS,
+                     kColFwdThreads>(sio, sio, TR, q);
             __syncthreads();
         }
         if constexpr (NR >= 4) {
-            round_io<LR, CV, dif_base(LR, 2, NR), round_size(LR, 2, NR), true, V, true, PS, kColFwdThreads>(
-                sio, sio, TR, q);
+            round_io<LR, CV, dif_base(LR, 2, NR), round_size(LR, 2, NR), true, V, true, PS,
+                     kColFwdThreads>(sio, sio, TR, q);
             __syncthreads();
         }
-        round_io<LR, CV, 0, round_size(LR, NR - 1, NR), true, V, true, PS, kColFwdThreads>(sio, out, TR, q);
+        round_io<LR, CV, 0, round_size(LR, NR - 1, NR), true, V, true, PS, kColFwdThreads>(
+            sio, out, TR, q);
     }
 }
 
@@ -753,19 +766,21 @@ __global__ void __launch_bounds__(kColInvThreads, CAT_COL_INV_MINB) ntt_col_inv(
         round_io<LR, CV, 0, LR, false, V, true, PS, kColInvThreads>(in, out, TRi, q);
     } else {
         const SmemIO<LR, CV, true> sio{sm};
-        round_io<LR, CV, 0, dit_size(LR, 0, NR), false, V, true, PS, kColInvThreads>(in, sio, TRi, q);
+        round_io<LR, CV, 0, dit_size(LR, 0, NR), false, V, true, PS, kColInvThreads>(
+            in, sio, TRi, q);
         __syncthreads();
         if constexpr (NR >= 3) {
-            round_io<LR, CV, dit_base(LR, 1, NR), dit_size(LR, 1, NR), false, V, true, PS, kColInvThreads>(
-                sio, sio, TRi, q);
+            round_io<LR, CV, dit_base(LR, 1, NR), dit_size(LR, 1, NR), false, V, true, PS,
+                     kColInvThreads>(sio, sio, TRi, q);
             __syncthreads();
         }
         if constexpr (NR >= 4) {
-            round_io<LR, CV, dit_base(LR, 2, NR), dit_size(LR, 2, NR), false, V, true, PS, kColInvThreads>(
-                sio, sio, TRi, q);
+            round_io<LR, CV, dit_base(LR, 2, NR), dit_size(LR, 2, NR), false, V, true, PS,
+                     kColInvThreads>(sio, sio, TRi, q);
             __syncthreads();
         }
-        round_io<LR, CV, dit_base(LR, NR - 1, NR), dit_size(LR, NR - 1, NR), false, V, true, PS, kColInvThreads>(
+        round_io<LR, CV, dit_base(LR, NR - 1, NR), dit_size(LR, NR - 1, NR), false, V, true, PS,
+                 kColInvThreads>(
             sio, out, TRi, q);
     }
 }
@@ -1016,7 +1031,8 @@ __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_fwd(RowArgs
             RowInPair<LR, CF>{fy, fy}, sp, T, q);
         __syncthreads();
         if constexpr (NR == 3) {
-            round_io<LR, CF, dif_base(LR, 1), round_size(LR, 1), true, 2, false, PS, kRowThreads>(sp, sp, T, q);
+            round_io<LR, CF, dif_base(LR, 1), round_size(LR, 1), true, 2, false, PS, kRowThreads>(
+                sp, sp, T, q);
             __syncthreads();
         }
     } else {
@@ -1024,7 +1040,8 @@ __global__ void __launch_bounds__(kRowThreads, CAT_ROW_MINB) ntt_row_fwd(RowArgs
             RowIn<LR>{fy, fy}, sio, T, q);
         __syncthreads();
         if constexpr (NR == 3) {
-            round_io<LR, C, dif_base(LR, 1), round_size(LR, 1), true, 1, false, PS, kRowThreads>(sio, sio, T, q);
+            round_io<LR, C, dif_base(LR, 1), round_size(LR, 1), true, 1, false, PS, kRowThreads>(
+                sio, sio, T, q);
             __syncthreads();
         }
     }

@@ -59,3 +59,18 @@ def test_chunked_sum_of_random_long_operands(ctx, cat_lib, orc):
     for q in orc.check_primes(seed=5, count=2, lower=2 * 10**6, bits=62):
         want = int(orc.limbs_mod(x, q)) * int(orc.limbs_mod(y, q)) % q
         assert int(orc.limbs_mod(got, q)) == want
+
+
+def test_chunked_sum_within_a_budget(cat_lib, orc):
+    """Two chunks, the second short, in a budget with room for the first one's
+    product but not for all residues at once (38 and 50 bytes per limb of a
+    chunk's transform)."""
+    L, ny = 1 << 17, 40000
+    nx = ((L - ny) & ~7) + 5000
+    x, y = operand(nx, False, 7), operand(ny, False, 8)
+    tight = cat_lib.Context(0, hbm_budget_bytes=44 * L)
+    want = orc.mul(x, y)
+    tight.set_profiling(True)
+    got = cat_lib.bigint_mul(tight, x, y).cpu().numpy().view(np.uint32)
+    assert "overlap_tiles" in tight.profile()
+    assert got.shape == want.shape and (got == want).all()
