@@ -35,7 +35,7 @@ def sources() -> list[str]:
 
 
 def _deps_mtime() -> float:
-    files = sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")]
+    files = sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     files.append(os.path.join(INCLUDE, "catalan.h"))
     return max(os.path.getmtime(f) for f in files)
 

@@ -610,7 +610,7 @@ struct DevBuf {
 struct Big {
     DevBuf<uint32_t> buf;
     size_t n = 0;
-    double bits = 0;  // where tracked: the value is below 2^bits
+    double bits = 0;  // where tracked: the value is at most 2^bits (length_bits.h)
 };
 
 // A device copy job: `len` limbs from src to dst, then dst zero-filled up to

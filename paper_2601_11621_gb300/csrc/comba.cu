@@ -9,8 +9,7 @@
 // fits in 2^k limbs, so the product of adjacent nodes (2i, 2i+1) fits the
 // next level's slot of 2S limbs exactly.
 #include "cat_internal.cuh"
-
-#include <math.h>
+#include "length_bits.h"
 
 namespace cat {
 
@@ -513,11 +512,7 @@ void normalize_all(Ctx &c, Big *const *x, int count, cudaStream_t s)
         const uint64_t n = (uint64_t)h[4 * i + 1] << 32 | h[4 * i];
         const uint64_t top = (uint64_t)h[4 * i + 3] << 32 | h[4 * i + 2];
         x[i]->n = n;
-        // below 2^(32 (n - 2)) (top + 1), top of 33 bits or more unless n = 1
-        x[i]->bits = n == 0 ? 0
-                     : n == 1
-                         ? log2((double)(top >> 32)) + 1e-9
-                         : 32.0 * (double)(n - 2) + log2((double)top) + 1e-9;
+        x[i]->bits = top_bits(n, top);
     }
 }
 

@@ -11,6 +11,7 @@
 // the multi-pass transform above.  Nodes of a level hold equally many primes,
 // which is what keeps the tree balanced.
 #include "cat_internal.cuh"
+#include "length_bits.h"
 
 #include <math.h>
 
@@ -222,13 +223,13 @@ static Big mul_big(Ctx &c, const Big &x, const Big &y, cudaStream_t s, bool exac
 }
 
 // x y for numbers whose bits are tracked: the product's length bound comes from
-// its bits (at most one limb above the true length), so that a chain of
-// products needs no read-back between its steps.
+// its bits (length_bits.h: never below the true length, and at most one limb
+// above it), so that a chain of products needs no read-back between its steps.
 static Big mul_bits(Ctx &c, const Big &x, const Big &y, cudaStream_t s)
 {
     Big r = mul_big(c, x, y, s, false);
-    r.bits = x.bits + y.bits;
-    r.n = std::min<size_t>(r.n, (size_t)(r.bits / 32.0) + 1);
+    r.bits = product_bits(x.bits, y.bits);
+    r.n = std::min<size_t>(r.n, bits_limbs(r.bits));
     return r;
 }
 
