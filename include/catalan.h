@@ -227,11 +227,13 @@ int product_tree(cat_ctx *ctx, const uint32_t *values, size_t count, uint32_t *o
                  size_t cap, size_t *out_len, void *stream);
 
 /* Algorithm 2 on a factorisation: out = prod_g (prod_{p in G_g} p)^exps[g].
- * The P_e with e >= 2 are combined by always multiplying the two shortest,
- * which keeps every intermediate as short as possible (the aim Sec. 3.2
- * states for the balanced tree); their product then joins the tree of Q_1
- * as one node, so the longest factor needs no final multiplication (the same
- * integer, re-associated). */
+ * Read are num_groups, host_exps, host_offsets and, on the device, primes:
+ * a caller may fill in those alone (any 32-bit values, exponents of up to 64
+ * bits).  Few primes with e >= 2 (C(n) and C(2n, n) have a handful) join the
+ * tree of Q_1 as leaves, each e times.  Otherwise the P_e with e >= 2 are
+ * combined by always multiplying the two shortest, and their product joins
+ * that tree as one node; more than 64 groups are taken bit by bit of the
+ * exponents (X <- X^2 R_b).  The integer is the same either way. */
 int cat_reconstruct(cat_ctx *ctx, const cat_factorization *f, uint32_t *out,
                     size_t cap, size_t *out_len, void *stream);
 

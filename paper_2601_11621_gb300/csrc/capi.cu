@@ -276,7 +276,11 @@ int cat_reconstruct(cat_ctx *ctx, const cat_factorization *f, uint32_t *out, siz
                                   out_len, s, false);
             return;
         }
-        cat::Big r = cat::reconstruct(ctx->c, f, s);
+        // the host arrays say what the groups are: the caller may have made or
+        // changed them, and the device's copies need not be there
+        cat_factorization g = *f;
+        g.exps = g.offsets = nullptr;
+        cat::Big r = cat::reconstruct(ctx->c, &g, s);
         copy_out(ctx->c, r, out, cap, out_len, s);
     });
 }

@@ -762,6 +762,8 @@ void factor_free(Ctx &c, cat_factorization *f);
 void copy_to_host(Ctx &c, uint32_t *host, const uint32_t *dev, size_t n, cudaStream_t s);
 // Algorithm 2 on a factorisation; returns the result (normalised length).
 // Every prime of f is below 2^leaf_bits (32 when nothing smaller is known).
+// The groups are the host arrays'; exps and offsets are their copies on the
+// device, or both null.
 // direct: a buffer that holds the result, taken when the last product can go
 // there (the result's Big then carries the length alone).
 Big reconstruct(Ctx &c, const cat_factorization *f, cudaStream_t s, int leaf_bits = 32,

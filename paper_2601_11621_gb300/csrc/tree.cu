@@ -265,10 +265,11 @@ Big power(Ctx &c, const uint32_t *a, size_t na, uint64_t e, cudaStream_t s, bool
 // (at most 33 groups) always take Algorithm 2 as written.
 constexpr uint64_t kManyGroups = kMaxRepeats;
 
-// Leaves of the bit segments (exponents fit 32 bits): segment b holds the
-// primes of the groups whose exponent has bit b set, group after group.
+// Leaves of the bit segments: segment b holds the primes of the groups whose
+// exponent has bit b set, group after group.
+constexpr int kExpBits = 64;
 struct BitSegments {
-    uint64_t start[33];
+    uint64_t start[kExpBits + 1];
 };
 
 // at[b ng + g]: the first leaf of group g in segment b; block b scans the
@@ -303,15 +304,14 @@ __global__ void __launch_bounds__(1024) bit_offsets(const uint64_t *exps, const 
     }
 }
 
-// One thread per prime: its group by bisection, then one leaf per bit of the
-// exponent.
-__global__ void bit_leaves(const uint32_t *primes, uint64_t np, const uint64_t *exps,
-                           const uint64_t *offs, uint32_t ng, const uint64_t *at,
-                           uint32_t *leaves)
+// One thread per prime of the groups: its group by bisection, then one leaf per
+// bit of the exponent.
+__global__ void bit_leaves(const uint32_t *primes, const uint64_t *exps, const uint64_t *offs,
+                           uint32_t ng, const uint64_t *at, uint32_t *leaves)
 {
     chain_wait();
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= np) return;
+    const uint64_t i = offs[0] + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= offs[ng]) return;
     uint32_t lo = 0, hi = ng;  // offs[lo] <= i < offs[hi]
     while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) >> 1;
@@ -320,9 +320,9 @@ __global__ void bit_leaves(const uint32_t *primes, uint64_t np, const uint64_t *
     }
     const uint32_t p = primes[i];
     const uint64_t k = i - offs[lo];
-    uint32_t e = (uint32_t)exps[lo];
+    uint64_t e = exps[lo];
     while (e) {
-        const int b = __ffs(e) - 1;
+        const int b = __ffsll((long long)e) - 1;
         e &= e - 1;
         leaves[at[(size_t)b * ng + lo] + k] = p;
     }
@@ -339,26 +339,40 @@ static Big reconstruct_bits(Ctx &c, const cat_factorization *f, cudaStream_t s, 
     uint64_t emax = 0;
     for (uint64_t g = 0; g < f->num_groups; g++) emax = std::max(emax, f->host_exps[g]);
     int B = 0;
-    while (B < 64 && (emax >> B)) B++;
+    while (B < kExpBits && (emax >> B)) B++;
     std::vector<uint64_t> seg(B + 1, 0);
     for (uint64_t g = 0; g < f->num_groups; g++)
         for (int b = 0; b < B; b++)
             if ((f->host_exps[g] >> b) & 1)
                 seg[b + 1] += f->host_offsets[g + 1] - f->host_offsets[g];
     for (int b = 0; b < B; b++) seg[b + 1] += seg[b];
-    DevBuf<uint32_t> leaves(c, std::max<uint64_t>(seg[B], 1), s);
+    if (seg[B] == 0) return make_one(c, s);
+    DevBuf<uint32_t> leaves(c, seg[B], s);
+    const uint32_t ng = (uint32_t)f->num_groups;
+    std::vector<uint64_t> groups;
     {
-        const uint32_t ng = (uint32_t)f->num_groups;
+        const uint64_t *exps = f->exps, *offs = f->offsets;
+        DevBuf<uint64_t> d_groups;
+        if (!exps) {  // a caller's factorisation
+            groups.assign(f->host_exps, f->host_exps + ng);
+            groups.insert(groups.end(), f->host_offsets, f->host_offsets + ng + 1);
+            d_groups = DevBuf<uint64_t>(c, groups.size(), s);
+            CAT_CUDA(cudaMemcpyAsync(d_groups.get(), groups.data(), 8 * groups.size(),
+                                     cudaMemcpyHostToDevice, s));
+            exps = d_groups.get();
+            offs = exps + ng;
+        }
+        const uint64_t np = f->host_offsets[ng] - f->host_offsets[0];
         DevBuf<uint64_t> at(c, (size_t)B * ng, s);
         BitSegments sb{};
         std::copy(seg.begin(), seg.end(), sb.start);
-        launch_chained(bit_offsets, B, 1024, 0, s, f->exps, f->offsets, ng, sb, at.get());
+        launch_chained(bit_offsets, B, 1024, 0, s, exps, offs, ng, sb, at.get());
         CAT_LAUNCH("bit_offsets");
         const int tok = prof_begin(c, "bit_leaves", s);
-        launch_chained(bit_leaves, (unsigned)((f->num_primes + 255) / 256), 256, 0, s, f->primes,
-                       f->num_primes, f->exps, f->offsets, ng, at.get(), leaves.get());
+        launch_chained(bit_leaves, (unsigned)((np + 255) / 256), 256, 0, s, f->primes, exps, offs,
+                       ng, at.get(), leaves.get());
         CAT_LAUNCH("bit_leaves");
-        prof_end(c, tok, s, 4.0 * (double)(f->num_primes + seg[B]));
+        prof_end(c, tok, s, 4.0 * (double)(np + seg[B]));
     }
     std::vector<TreeRoot> R(B);
     segmented_tree(c, leaves.get(), seg, R, s, leaf_bits);
