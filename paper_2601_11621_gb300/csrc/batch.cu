@@ -747,10 +747,10 @@ void exact_batch(Ctx &c, const cat_request *reqs, size_t count, uint32_t *out, s
         try {
             v = reconstruct(c, &f, s, bits_below(reqs[r].n));  // primes <= n
         } catch (...) {
-            factor_free(c, &f);
+            factor_free(c, &f, s);
             throw;
         }
-        factor_free(c, &f);
+        factor_free(c, &f, s);
         const uint64_t capr = bound_limbs(reqs[r].n, reqs[r].kind);
         if (v.n > capr) fail(CAT_ERANGE, "result longer than its bound");
         run_copy_jobs(c, {CopyJob{v.buf.get(), out + offsets[r], v.n, capr}}, s);

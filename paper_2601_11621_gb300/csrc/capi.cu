@@ -199,7 +199,8 @@ void cat_factor_free(cat_ctx *ctx, cat_factorization *f)
 {
     if (!ctx || !f) return;
     cudaSetDevice(ctx->c.device);
-    cat::factor_free(ctx->c, f);
+    // every call that writes or reads the arrays has ended with its stream idle
+    cat::factor_free(ctx->c, f, nullptr);
 }
 
 int cat_factor_copy_primes(cat_ctx *ctx, const cat_factorization *f, uint32_t *dst,
@@ -280,8 +281,13 @@ int cat_reconstruct(cat_ctx *ctx, const cat_factorization *f, uint32_t *out, siz
         // changed them, and the device's copies need not be there
         cat_factorization g = *f;
         g.exps = g.offsets = nullptr;
-        cat::Big r = cat::reconstruct(ctx->c, &g, s);
-        copy_out(ctx->c, r, out, cap, out_len, s);
+        try {
+            cat::Big r = cat::reconstruct(ctx->c, &g, s);
+            copy_out(ctx->c, r, out, cap, out_len, s);
+        } catch (...) {
+            cudaStreamSynchronize(s);  // the caller may free f now
+            throw;
+        }
     });
 }
 
@@ -312,11 +318,11 @@ int cat_exact(cat_ctx *ctx, int kind, uint64_t n, uint32_t *out, size_t cap,
             cat::Big r = cat::reconstruct(ctx->c, &f, s,
                                           cat::bits_below(kind == CAT_FACTORIAL ? n : 2 * n),
                                           &direct);
-            cat::factor_free(ctx->c, &f);
+            cat::factor_free(ctx->c, &f, s);
             if (direct.used) *out_len = r.n;
             else copy_out(ctx->c, r, out, cap, out_len, s);
         } catch (...) {
-            cat::factor_free(ctx->c, &f);
+            cat::factor_free(ctx->c, &f, s);
             throw;
         }
     });
@@ -359,11 +365,11 @@ int cat_ratio_exact(cat_ctx *ctx, const uint64_t *a, int ka, const uint64_t *b, 
             for (int i = 0; i < q.ka; i++) top = std::max<uint64_t>(top, q.a[i]);
             cat::Direct direct = direct_out(out, cap, cat::ratio_bound_limbs(q));
             cat::Big r = cat::reconstruct(ctx->c, &f, s, cat::bits_below(top), &direct);
-            cat::factor_free(ctx->c, &f);
+            cat::factor_free(ctx->c, &f, s);
             if (direct.used) *out_len = r.n;
             else copy_out(ctx->c, r, out, cap, out_len, s);
         } catch (...) {
-            cat::factor_free(ctx->c, &f);
+            cat::factor_free(ctx->c, &f, s);
             throw;
         }
     });
@@ -413,10 +419,10 @@ int cat_exact_host(cat_ctx *ctx, int kind, uint64_t n, uint32_t *host_out, size_
             r = cat::reconstruct(ctx->c, &f, s,
                                  cat::bits_below(kind == CAT_FACTORIAL ? n : 2 * n));
         } catch (...) {
-            cat::factor_free(ctx->c, &f);
+            cat::factor_free(ctx->c, &f, s);
             throw;
         }
-        cat::factor_free(ctx->c, &f);
+        cat::factor_free(ctx->c, &f, s);
         *out_len = r.n;
         if (r.n > cap) cat::fail(CAT_ERANGE, "output capacity too small");
         cat::copy_to_host(ctx->c, host_out, r.buf.get(), r.n, s);

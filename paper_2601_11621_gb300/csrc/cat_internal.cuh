@@ -750,11 +750,15 @@ struct Ratio {
     uint32_t a[kMaxRatioTerms], b[kMaxRatioTerms];
 };
 
-// Phase 1 on the device, complete on stream s.  The arrays of *out come from
-// the context's pool and are released by factor_free.
+// Phase 1 on stream s: the host members of *out are complete on return, its
+// device arrays when s has reached this point (their last kernel may still be
+// running).  They come from the context's pool and are released by factor_free
+// in the order of the stream given, which is s or one that has waited for it:
+// the pool is shared by every context of the device, and a free on another
+// stream would hand arrays that are still being written to the next request.
 void factor(Ctx &c, uint64_t n, int kind, cat_factorization *out, cudaStream_t s);
 void factor_ratio(Ctx &c, const Ratio &r, cat_factorization *out, cudaStream_t s);
-void factor_free(Ctx &c, cat_factorization *f);
+void factor_free(Ctx &c, cat_factorization *f, cudaStream_t s);
 
 // n limbs from device memory into host memory, on stream s (not synchronised):
 // a store kernel when the host range is page-locked and mapped for the

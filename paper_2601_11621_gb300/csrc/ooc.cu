@@ -263,7 +263,7 @@ void reconstruct_into(Ctx &c, cat_factorization *f, uint32_t *out, size_t cap, b
     if (np)
         CAT_CUDA(cudaMemcpyAsync(primes.p, f->primes, 4 * np, cudaMemcpyDeviceToHost, s));
     CAT_CUDA(cudaStreamSynchronize(s));
-    if (release) factor_free(c, f);
+    if (release) factor_free(c, f, s);
     std::vector<HostBig> P;
     for (uint64_t g = 0; g < ng; g++) {
         HostBig Q = chunk_product(c, primes.p + offs[g], offs[g + 1] - offs[g], s);

@@ -785,12 +785,12 @@ DevBuf<uint32_t> sieve_primes(Ctx &c, uint64_t limit, uint64_t *count, cudaStrea
     return primes;
 }
 
-void factor_free(Ctx &c, cat_factorization *f)
+void factor_free(Ctx &c, cat_factorization *f, cudaStream_t s)
 {
     if (!f) return;
-    dev_free(c, f->exps, 8 * (f->num_groups + 1), nullptr);
-    dev_free(c, f->offsets, 8 * (f->num_groups + 1), nullptr);
-    dev_free(c, f->primes, 4 * (f->num_primes ? f->num_primes : 1), nullptr);
+    dev_free(c, f->exps, 8 * (f->num_groups + 1), s);
+    dev_free(c, f->offsets, 8 * (f->num_groups + 1), s);
+    dev_free(c, f->primes, 4 * (f->num_primes ? f->num_primes : 1), s);
     delete[] f->host_exps;
     delete[] f->host_offsets;
     *f = cat_factorization{};
