@@ -334,18 +334,8 @@ __global__ void batch_lengths(const uint32_t *out, const uint64_t *off, const ui
     chain_wait();
     __shared__ unsigned long long best;
     const int r = blockIdx.x;
-    if (threadIdx.x == 0) best = 0;
-    __syncthreads();
-    const uint32_t *o = out + off[r];
-    const uint64_t n = cap[r];
-    for (uint64_t top = n; top > 0 && best == 0;) {
-        const uint64_t lo = top > blockDim.x ? top - blockDim.x : 0;
-        const uint64_t i = lo + threadIdx.x;
-        if (i < top && o[i]) atomicMax(&best, (unsigned long long)(i + 1));
-        __syncthreads();
-        top = lo;
-    }
-    if (threadIdx.x == 0) len[r] = best;
+    const uint64_t n = block_top(out + off[r], cap[r], &best);
+    if (threadIdx.x == 0) len[r] = n;
 }
 
 template <typename T>

@@ -705,6 +705,28 @@ size_t normalized_length(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s);
 // The same, reading only the top four limbs when one of them is nonzero (the
 // usual case for a product of normalised operands).
 size_t trim(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s);
+// The index above the highest nonzero limb of x[0 .. n) (0: none), for the
+// whole block: a stretch of blockDim.x limbs after the other, down from the top.
+// best: a word of the block's shared memory.  Every thread reads it between the
+// same two barriers, with no write there, so all of them leave together.
+__device__ __forceinline__ uint64_t block_top(const uint32_t *x, uint64_t n,
+                                              unsigned long long *best)
+{
+    if (threadIdx.x == 0) *best = 0;
+    __syncthreads();
+    uint64_t found = 0;
+    for (uint64_t top = n; top > 0;) {
+        const uint64_t lo = top > blockDim.x ? top - blockDim.x : 0;
+        const uint64_t i = lo + threadIdx.x;
+        if (i < top && x[i]) atomicMax(best, (unsigned long long)(i + 1));
+        __syncthreads();
+        found = *(volatile unsigned long long *)best;
+        __syncthreads();
+        if (found) break;
+        top = lo;
+    }
+    return found;
+}
 // Normalises up to kMaxTops numbers at once (their n and bits, from their
 // lengths and top two limbs), with one read-back.
 constexpr int kMaxTops = 64;

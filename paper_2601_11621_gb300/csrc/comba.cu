@@ -419,21 +419,10 @@ __global__ void __launch_bounds__(1024) number_tops(const __grid_constant__ Tops
     chain_wait();
     __shared__ unsigned long long best;
     const uint32_t *x = a.x[blockIdx.x];
-    if (threadIdx.x == 0) best = 0;
-    __syncthreads();
-    for (uint64_t top = a.n[blockIdx.x]; top > 0;) {
-        const uint64_t lo = top > blockDim.x ? top - blockDim.x : 0;
-        const uint64_t i = lo + threadIdx.x;
-        if (i < top && x[i]) atomicMax(&best, (unsigned long long)(i + 1));
-        __syncthreads();
-        if (best) break;  // the same for every thread: nothing is written until the next barrier
-        top = lo;
-        __syncthreads();
-    }
+    const uint64_t n = block_top(x, a.n[blockIdx.x], &best);
     if (threadIdx.x == 0) {
-        a.out[2 * blockIdx.x] = best;
-        a.out[2 * blockIdx.x + 1] =
-            best ? (uint64_t)x[best - 1] << 32 | (best > 1 ? x[best - 2] : 0u) : 0u;
+        a.out[2 * blockIdx.x] = n;
+        a.out[2 * blockIdx.x + 1] = n ? (uint64_t)x[n - 1] << 32 | (n > 1 ? x[n - 2] : 0u) : 0u;
     }
 }
 
