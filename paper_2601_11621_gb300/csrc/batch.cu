@@ -334,7 +334,7 @@ __global__ void batch_lengths(const uint32_t *out, const uint64_t *off, const ui
     chain_wait();
     __shared__ unsigned long long best;
     const int r = blockIdx.x;
-    const uint64_t n = block_top(out + off[r], cap[r], &best);
+    const uint64_t n = block_top(out + off[r], 0, cap[r], &best);
     if (threadIdx.x == 0) len[r] = n;
 }
 

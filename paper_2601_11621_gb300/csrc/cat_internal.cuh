@@ -705,32 +705,35 @@ size_t normalized_length(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s);
 // The same, reading only the top four limbs when one of them is nonzero (the
 // usual case for a product of normalised operands).
 size_t trim(Ctx &c, const uint32_t *x, size_t n, cudaStream_t s);
-// The index above the highest nonzero limb of x[0 .. n) (0: none), for the
+// The index above the highest nonzero limb of x[low .. n) (low: none), for the
 // whole block: a stretch of blockDim.x limbs after the other, down from the top.
 // best: a word of the block's shared memory.  Every thread reads it between the
 // same two barriers, with no write there, so all of them leave together.
-__device__ __forceinline__ uint64_t block_top(const uint32_t *x, uint64_t n,
+__device__ __forceinline__ uint64_t block_top(const uint32_t *x, uint64_t low, uint64_t n,
                                               unsigned long long *best)
 {
-    if (threadIdx.x == 0) *best = 0;
+    if (threadIdx.x == 0) *best = low;
     __syncthreads();
-    uint64_t found = 0;
-    for (uint64_t top = n; top > 0;) {
-        const uint64_t lo = top > blockDim.x ? top - blockDim.x : 0;
+    uint64_t found = low;
+    for (uint64_t top = n; top > low;) {
+        const uint64_t lo = top > low + blockDim.x ? top - blockDim.x : low;
         const uint64_t i = lo + threadIdx.x;
         if (i < top && x[i]) atomicMax(best, (unsigned long long)(i + 1));
         __syncthreads();
         found = *(volatile unsigned long long *)best;
         __syncthreads();
-        if (found) break;
+        if (found != low) break;
         top = lo;
     }
     return found;
 }
 // Normalises up to kMaxTops numbers at once (their n and bits, from their
-// lengths and top two limbs), with one read-back.
+// lengths and top two limbs), with one read-back.  One block scans each number
+// down from the top, `scan` limbs at most; a longer run of zeros is left to the
+// whole chip, which costs that number two read-backs more.
 constexpr int kMaxTops = 64;
-void normalize_all(Ctx &c, Big *const *x, int count, cudaStream_t s);
+void normalize_all(Ctx &c, Big *const *x, int count, cudaStream_t s,
+                   uint64_t scan = ~(uint64_t)0);
 // Groups of values that a product tree takes several times each, as further
 // leaves behind its values: leaves [start[g], start[g+1]) are base[off[g]],
 // base[off[g]], ..., every value times[g] times.

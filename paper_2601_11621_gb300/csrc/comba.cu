@@ -11,6 +11,8 @@
 #include "cat_internal.cuh"
 #include "length_bits.h"
 
+#include <string.h>
+
 namespace cat {
 
 // c2:c1:c0 += a * b  (96-bit accumulator)
@@ -409,20 +411,24 @@ __global__ void find_top(const uint32_t *x, size_t n, unsigned long long *top)
 struct TopsArgs {
     const uint32_t *x[kMaxTops];
     uint64_t n[kMaxTops];
+    uint64_t scan;
     uint64_t *out;  // per number: normalised length, top two limbs
 };
 
 // One block per number, scanning down from the top for the highest nonzero
-// limb (usually in the first stretch).
+// limb, `scan` limbs of it at most.  A number whose scanned limbs are all zero
+// is left at the length below them, its top limbs 0.
 __global__ void __launch_bounds__(1024) number_tops(const __grid_constant__ TopsArgs a)
 {
     chain_wait();
     __shared__ unsigned long long best;
     const uint32_t *x = a.x[blockIdx.x];
-    const uint64_t n = block_top(x, a.n[blockIdx.x], &best);
+    const uint64_t len = a.n[blockIdx.x], low = len > a.scan ? len - a.scan : 0;
+    const uint64_t n = block_top(x, low, len, &best);
     if (threadIdx.x == 0) {
         a.out[2 * blockIdx.x] = n;
-        a.out[2 * blockIdx.x + 1] = n ? (uint64_t)x[n - 1] << 32 | (n > 1 ? x[n - 2] : 0u) : 0u;
+        a.out[2 * blockIdx.x + 1] =
+            n > low ? (uint64_t)x[n - 1] << 32 | (n > 1 ? x[n - 2] : 0u) : 0u;
     }
 }
 
@@ -483,7 +489,7 @@ bool comba_level(Ctx &c, const uint32_t *in, size_t slot, size_t nprod, uint32_t
     return true;
 }
 
-void normalize_all(Ctx &c, Big *const *x, int count, cudaStream_t s)
+void normalize_all(Ctx &c, Big *const *x, int count, cudaStream_t s, uint64_t scan)
 {
     if (count > kMaxTops) fail(CAT_EINVAL, "too many numbers");
     if (count == 0) return;
@@ -493,13 +499,23 @@ void normalize_all(Ctx &c, Big *const *x, int count, cudaStream_t s)
         a.x[i] = x[i]->buf.get();
         a.n[i] = x[i]->n;
     }
+    a.scan = scan;
     a.out = d.get();
     launch_chained(number_tops, count, 1024, 0, s, a);
     CAT_LAUNCH("number_tops");
-    const uint32_t *h = read_back(c, d.get(), 4 * count, s);
+    uint32_t h[4 * kMaxTops];
+    memcpy(h, read_back(c, d.get(), 4 * count, s), 16 * (size_t)count);
     for (int i = 0; i < count; i++) {
-        const uint64_t n = (uint64_t)h[4 * i + 1] << 32 | h[4 * i];
-        const uint64_t top = (uint64_t)h[4 * i + 3] << 32 | h[4 * i + 2];
+        uint64_t n = (uint64_t)h[4 * i + 1] << 32 | h[4 * i];
+        uint64_t top = (uint64_t)h[4 * i + 3] << 32 | h[4 * i + 2];
+        if (n && !top) {  // zeros as far as the block scanned
+            n = normalized_length(c, a.x[i], n, s);
+            if (n) {
+                const int k = n > 1 ? 2 : 1;
+                const uint32_t *t = read_back(c, a.x[i] + n - k, k, s);
+                top = (uint64_t)t[k - 1] << 32 | (k > 1 ? t[0] : 0u);
+            }
+        }
         x[i]->n = n;
         x[i]->bits = top_bits(n, top);
     }

@@ -243,8 +243,11 @@ Big power(Ctx &c, const uint32_t *a, size_t na, uint64_t e, cudaStream_t s, bool
     NvtxRange range("power");
     Big base = copy_big(c, a, na, s);
     if (exact) {
+        // a caller's buffer may be zero far above the value (four stretches of
+        // the one block, then the whole chip: 1,000 limbs below 4 million zeros,
+        // to the third power, 90 us; 1,776 us by the block alone, 62 without zeros)
         Big *p = &base;
-        normalize_all(c, &p, 1, s);
+        normalize_all(c, &p, 1, s, 4096);
     }
     if (e == 0) return make_one(c, s);
     if (base.n == 0) return base;
@@ -384,6 +387,8 @@ static Big reconstruct_bits(Ctx &c, const cat_factorization *f, cudaStream_t s, 
         r.n = std::min<size_t>(r.n, (seg[b + 1] - seg[b]) * (uint64_t)leaf_bits / 32 + 1);
         roots.push_back(&r);
     }
+    // (the bounds exceed the lengths by a few per cent, which the roots' blocks
+    // scan side by side)
     normalize_all(c, roots.data(), B, s);
     Big X = std::move(R[B - 1].big);
     for (int b = B - 2; b >= 0; b--) {
