@@ -556,8 +556,6 @@ void twiddle_tables_host(uint2 *h);
 // memory of the current device (ntt.cu).
 void upload_low_twiddles(const uint2 *h);
 
-// Whether the context's budgets, if any, have room for `bytes` more.
-bool has_room(const Ctx &c, size_t bytes);
 // Device allocation from the context's stream-ordered pool (cudaMallocAsync on
 // the device's default memory pool, whose release threshold is raised at
 // context creation so freed blocks stay cached).

@@ -61,13 +61,6 @@ static cudaMemPool_t pool_for(int device)
     return g_pools[device];
 }
 
-bool has_room(const Ctx &c, size_t bytes)
-{
-    if (c.budget && c.in_use + bytes > c.budget) return false;
-    return !c.shared_in_use || !c.shared_budget ||
-           c.shared_in_use->load() + bytes <= c.shared_budget;
-}
-
 void *dev_alloc(Ctx &c, size_t bytes, cudaStream_t s)
 {
     if (bytes == 0) return nullptr;
@@ -77,13 +70,15 @@ void *dev_alloc(Ctx &c, size_t bytes, cudaStream_t s)
                              std::to_string(c.in_use + bytes) + " > " +
                              std::to_string(c.budget) + " bytes)");
     if (c.shared_in_use) {
-        const size_t before = c.shared_in_use->fetch_add(bytes);
-        if (c.shared_budget && before + bytes > c.shared_budget) {
-            c.shared_in_use->fetch_sub(bytes);
-            fail(CAT_ENOMEM, "scratch would exceed the shared HBM budget (" +
-                                 std::to_string(before + bytes) + " > " +
-                                 std::to_string(c.shared_budget) + " bytes)");
-        }
+        // added only where it fits: an attempt that does not fit may have another
+        // way to go, and must not make another thread's fail
+        size_t before = c.shared_in_use->load();
+        do {
+            if (c.shared_budget && before + bytes > c.shared_budget)
+                fail(CAT_ENOMEM, "scratch would exceed the shared HBM budget (" +
+                                     std::to_string(before + bytes) + " > " +
+                                     std::to_string(c.shared_budget) + " bytes)");
+        } while (!c.shared_in_use->compare_exchange_weak(before, before + bytes));
         if (c.shared_peak) {
             size_t pk = c.shared_peak->load();
             while (before + bytes > pk &&

@@ -1460,14 +1460,14 @@ static void launch_row_limbs(size_t nprod, bool square, cudaStream_t s, const Ro
     CAT_LAUNCH("ntt_row_limbs");
 }
 
-// Scratch of one batch of multi-pass products: from the context's pool, or
-// the fixed arrays of the no-allocation multiply.
+// Scratch of one batch of multi-pass products: what is null is taken from the
+// context's pool when it is needed; the no-allocation multiply brings its fixed
+// arrays, a caller that has another way to go its own allocations.
 struct MulScratch {
     DevBuf<uint32_t> Fb, Gb;
     DevBuf<uint8_t> mb;
     uint32_t *F = nullptr, *G = nullptr;
     uint8_t *maps = nullptr;
-    bool fixed = false;
 };
 
 // The carries of nprod products of `tiles` tiles each, whose compact tile
@@ -1515,7 +1515,7 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
     int tok;
     if (P.ncol == 0) {
         // the row pass alone, from the operands' limbs
-        if (!m.fixed) {
+        if (!m.G) {
             m.Gb = DevBuf<uint32_t>(c, gp * kNumPrimes, s);
             m.G = m.Gb.get();
         }
@@ -1540,7 +1540,7 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
         launch_row_limbs(nprod, mode == PAIR_SQUARE, s, ra);
         prof_end(c, tok, s, 4.0 * kNumPrimes * (double)gp + unit, unit);
     } else {
-        if (!m.fixed) {
+        if (!m.F) {
             m.Fb = DevBuf<uint32_t>(c, fp * kNumPrimes, s);
             m.F = m.Fb.get();
         }
@@ -1569,7 +1569,7 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
             mm -= P.rcol[i];
         }
         // fused row pass
-        if (!m.fixed) {
+        if (!m.G) {
             m.Gb = DevBuf<uint32_t>(c, gp * kNumPrimes, s);
             m.G = m.Gb.get();
         }
@@ -1606,7 +1606,7 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
     // remaindering and carries
     const size_t sums = step ? 1 : nprod;
     const size_t tiles = step ? (sink.out_len + kTile - 1) / kTile : N / kTileCoefs;
-    if (!m.fixed) {
+    if (!m.maps) {
         m.mb = DevBuf<uint8_t>(c, sums * tiles, s);
         m.maps = m.mb.get();
     }
@@ -1902,6 +1902,24 @@ __global__ void __launch_bounds__(kTileThreads) overlap_tiles(const uint32_t *T,
     if (threadIdx.x == 0) tile_maps[blockIdx.x] = (uint8_t)map;
 }
 
+// The scratch of n broadcast products of 2^np points and `tiles` tile maps, as
+// one block: false, with nothing taken, where a budget or the device has no
+// room for it.
+static bool take_scratch(Ctx &c, int np, size_t n, size_t tiles, MulScratch &m, cudaStream_t s)
+{
+    const size_t points = (size_t)kNumPrimes << np;
+    try {
+        m.Gb = DevBuf<uint32_t>(c, (2 * n + 1) * points + (tiles + 3) / 4, s);
+    } catch (const Error &e) {
+        if (e.code != CAT_ENOMEM) throw;
+        return false;
+    }
+    m.F = m.Gb.get();
+    m.G = m.F + (n + 1) * points;
+    m.maps = reinterpret_cast<uint8_t *>(m.G + n * points);
+    return true;
+}
+
 // out[0 .. nx + ny) = x y by chunks of M = 2^k - ny >= ny limbs of x, each
 // multiplied by y in one batch (y transformed once).
 //
@@ -1909,21 +1927,23 @@ __global__ void __launch_bounds__(kTileThreads) overlap_tiles(const uint32_t *T,
 // rounded down to whole runs of four coefficients; at least ny still, 2^(k-1)
 // being a multiple of 8 limbs and not below ny); the last chunk is shorter.
 // The one-block and one-row products write limbs, which overlap_tiles adds; so
-// do longer ones where a budget has no room for all chunks' residues at once
-// (10 bytes per limb of 2 n + 1 transforms: up to four chunks of which the
-// last is short take less one after the other).
+// do longer ones where there is no room for all chunks' residues at once (10
+// bytes per limb of 2 n + 1 transforms: up to four chunks of which the last is
+// short take less one after the other).  The room is taken, not asked for: a
+// budget may be shared with other threads.
 void mul_chunked(Ctx &c, const uint32_t *x, size_t nx, const uint32_t *y, size_t ny, int k,
                  uint32_t *out, cudaStream_t s)
 {
     const size_t L = (size_t)1 << k, M = L - ny, slot = L;
     if (ny == 0 || M < ny) fail(CAT_EINVAL, "chunk size below the short operand");
     const size_t m = M & ~(size_t)7, n = (nx + m - 1) / m;
-    if (k - 1 > kRowMaxLog && has_room(c, 10 * (2 * n + 1) * L + (nx + ny) / kTile + 1024)) {
+    MulScratch scratch;
+    if (k - 1 > kRowMaxLog && take_scratch(c, k - 1, n, (nx + ny + kTile - 1) / kTile, scratch, s)) {
         Operand ox{x, m, m}, oy{y, 0, ny};
         ox.ragged = (unsigned)(n - 1);
         ox.ragged_len = nx - (n - 1) * m;
         ntt_mul_multipass(c, k - 1, PAIR_BROADCAST, n, ox, oy, plain_sink(out, 0, nx + ny), s,
-                          MulScratch{}, (uint32_t)(m / 2));
+                          std::move(scratch), (uint32_t)(m / 2));
         return;
     }
     const size_t full = nx / M, rem = nx - full * M, chunks = full + (rem ? 1 : 0);
@@ -2035,7 +2055,6 @@ static void noalloc_mul(const NoAllocDevice &d, const uint32_t *a, size_t na, co
         return;
     }
     MulScratch m;
-    m.fixed = true;
     m.F = d.scratch;
     m.G = d.scratch + kNoAllocF;
     m.maps = (uint8_t *)(d.scratch + kNoAllocF + kNoAllocG);
