@@ -1659,9 +1659,8 @@ static bool spread_primes(size_t nprod, int lr, int num_sms)
 }
 
 template <int LR>
-static void launch_fused(size_t nprod, int num_sms, cudaStream_t s, const FusedArgs &a)
+static void launch_fused(size_t nprod, bool spread, cudaStream_t s, const FusedArgs &a)
 {
-    const bool spread = spread_primes(nprod, LR, num_sms);
     // operands of at most half the transform (every tree level)
     if (std::max(a.a_len, a.b_len) <= (1u << LR))
         launch_fused_t<LR, true>(nprod, spread, s, a);
@@ -1686,22 +1685,23 @@ static void ntt_mul_small(Ctx &c, int np, size_t nprod, Operand x, Operand y, bo
     a.tw = c.twiddles;
     a.ca = make_coef(0, sink.dec);
     a.cb = make_coef(0, sink.dec, np);
-    const int tok = prof_begin(c, "ntt_mul_fused", s);
+    const bool spread = np >= kClusterMinLog && spread_primes(nprod, np, c.num_sms);
+    const int tok = prof_begin(c, spread ? "ntt_mul_cluster" : "ntt_mul_fused", s);
     switch (np) {
-    case 1: launch_fused<1>(nprod, c.num_sms, s, a); break;
-    case 2: launch_fused<2>(nprod, c.num_sms, s, a); break;
-    case 3: launch_fused<3>(nprod, c.num_sms, s, a); break;
-    case 4: launch_fused<4>(nprod, c.num_sms, s, a); break;
-    case 5: launch_fused<5>(nprod, c.num_sms, s, a); break;
-    case 6: launch_fused<6>(nprod, c.num_sms, s, a); break;
-    case 7: launch_fused<7>(nprod, c.num_sms, s, a); break;
-    case 8: launch_fused<8>(nprod, c.num_sms, s, a); break;
-    case 9: launch_fused<9>(nprod, c.num_sms, s, a); break;
-    case 10: launch_fused<10>(nprod, c.num_sms, s, a); break;
-    case 11: launch_fused<11>(nprod, c.num_sms, s, a); break;
+    case 1: launch_fused<1>(nprod, spread, s, a); break;
+    case 2: launch_fused<2>(nprod, spread, s, a); break;
+    case 3: launch_fused<3>(nprod, spread, s, a); break;
+    case 4: launch_fused<4>(nprod, spread, s, a); break;
+    case 5: launch_fused<5>(nprod, spread, s, a); break;
+    case 6: launch_fused<6>(nprod, spread, s, a); break;
+    case 7: launch_fused<7>(nprod, spread, s, a); break;
+    case 8: launch_fused<8>(nprod, spread, s, a); break;
+    case 9: launch_fused<9>(nprod, spread, s, a); break;
+    case 10: launch_fused<10>(nprod, spread, s, a); break;
+    case 11: launch_fused<11>(nprod, spread, s, a); break;
     default: fail(CAT_EINVAL, "one-block transform size out of range");
     }
-    CAT_LAUNCH("ntt_mul_fused");
+    CAT_LAUNCH(spread ? "ntt_mul_cluster" : "ntt_mul_fused");
     const double unit =
         4.0 * (double)nprod * (double)(x.len + (square ? 0 : y.len) + sink.out_len);
     prof_end(c, tok, s, unit, unit);
