@@ -11,7 +11,7 @@
 // global memory; rounds in between exchange through shared memory (one
 // barrier per round).  Stage s (half-span 2^s) multiplies by
 // w_{2^(s+1)}^(i mod 2^s), entry 2^s + (i mod 2^s) of the stage table
-// (2^(s+1) <= 2^13).
+// (2^(s+1) <= 2^12).
 #pragma once
 
 #include <type_traits>
@@ -408,11 +408,9 @@ __device__ __forceinline__ void col_place(unsigned nblk, unsigned groups, unsign
 // columns c V + a (a < V) are the V arrays of the register round (NA = V), so
 // they share every stage twiddle, and global memory moves V adjacent words
 // with one V-word access.  In shared memory array a holds the columns
-// c V + a, back to back (SmemIO with C / V columns and NA = V).
-#ifndef CAT_COL_V
-#define CAT_COL_V 2
-#endif
-constexpr int kColV = CAT_COL_V;
+// c V + a, back to back (SmemIO with C / V columns and NA = V).  V is 2: two
+// columns of coefficients are the four limbs of a 16-byte load.
+constexpr int kColV = 2;
 
 // Word i of a transform at the block-uniform address p: the byte offset stays
 // in 32 bits (transforms of up to 2^26 points, operands of up to 2^27 limbs
@@ -428,15 +426,9 @@ __device__ __forceinline__ T *word_at(T *p, uint32_t i)
 template <int V>
 __device__ __forceinline__ void load_v(const uint32_t *p, uint32_t (&w)[V])
 {
-    if constexpr (V == 4) {
-        const uint4 t = *reinterpret_cast<const uint4 *>(p);
-        w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
-    } else if constexpr (V == 2) {
-        const uint2 t = *reinterpret_cast<const uint2 *>(p);
-        w[0] = t.x; w[1] = t.y;
-    } else {
-        w[0] = *p;
-    }
+    static_assert(V == 2, "one access per pair of columns");
+    const uint2 t = *reinterpret_cast<const uint2 *>(p);
+    w[0] = t.x; w[1] = t.y;
 }
 
 // The same through the read-only path, for tables no kernel writes: the
@@ -444,26 +436,16 @@ __device__ __forceinline__ void load_v(const uint32_t *p, uint32_t (&w)[V])
 template <int V>
 __device__ __forceinline__ void load_v_ro(const uint32_t *p, uint32_t (&w)[V])
 {
-    if constexpr (V == 4) {
-        const uint4 t = __ldg(reinterpret_cast<const uint4 *>(p));
-        w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
-    } else if constexpr (V == 2) {
-        const uint2 t = __ldg(reinterpret_cast<const uint2 *>(p));
-        w[0] = t.x; w[1] = t.y;
-    } else {
-        w[0] = __ldg(p);
-    }
+    static_assert(V == 2, "one access per pair of columns");
+    const uint2 t = __ldg(reinterpret_cast<const uint2 *>(p));
+    w[0] = t.x; w[1] = t.y;
 }
 
 template <int V>
 __device__ __forceinline__ void store_v(uint32_t *p, const uint32_t (&w)[V])
 {
-    if constexpr (V == 4)
-        *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-    else if constexpr (V == 2)
-        *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[1]);
-    else
-        *p = w[0];
+    static_assert(V == 2, "one access per pair of columns");
+    *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[1]);
 }
 
 // Column tile in global memory: element (row, col) at p[row * S + col0 + col],
