@@ -92,9 +92,9 @@ const char *cat_last_error(const cat_ctx *ctx);
 /* ------------------------------------------------------------ autotuning
  * The device-dependent choices of the product tree's multiplications (the
  * paper leaves them to its bignum library): the row-pass size of the
- * multi-pass transform for each transform size 2^13 .. 2^27, and the largest
- * tree-level slot (32 .. 256 limbs) multiplied by schoolbook (Comba) rather
- * than by the transform.
+ * multi-pass transform for each product size 2^13 .. 2^27 limbs, and the
+ * largest tree-level slot (16 .. 256 limbs) multiplied by schoolbook (Comba)
+ * rather than by the transform.
  *
  * cat_autotune: times every candidate on a synthetic tree level of 2^24
  * limbs (one product of 2^n limbs above that) on ctx's device (about a
@@ -105,7 +105,10 @@ const char *cat_last_error(const cat_ctx *ctx);
  * cat_ctx_load_tuning: applies a table written by cat_autotune
  * (CAT_EINVAL when it is unreadable or was made on another kind of device).
  * A new context reads the table at $CAT_TUNE_FILE, else autotune.txt next to
- * libcatalan.so, when it exists and matches the device.
+ * libcatalan.so, when it exists and matches the device.  A table does not say
+ * which build measured it: one from an older build is applied as it is, its
+ * choices then being that build's (measure again after an update; the value
+ * for 2^13 limbs has no effect, those products take the row pass alone).
  * cat_ctx_tuning: the values in use: the crossover slot, and row_log[n] for
  * n < count (0 = the default plan).  Errors: CAT_EINVAL, CAT_ENOMEM,
  * CAT_ECUDA. */
@@ -129,7 +132,7 @@ int cat_ctx_set_profiling(cat_ctx *ctx, int on);
 
 /* Totals for the i-th kernel name seen since profiling was switched on:
  * launches, summed device milliseconds, summed pass bytes (the bytes the
- * launch itself must read and write at minimum, e.g. three residue arrays in
+ * launch itself must read and write at minimum, e.g. five residue arrays in
  * and out for a transform pass) and summed unit bytes: the algorithmic bytes
  * of the products the launches completed, 4 bytes per limb of each operand
  * read once and of each product written once (for a level of the product
@@ -195,7 +198,7 @@ int bigint_mul(cat_ctx *ctx, const uint32_t *a, size_t na, const uint32_t *b,
  * call waits only for its own stream), or a service that must not meet an
  * out-of-memory failure in the middle of a request.  There is no context: the
  * transform scratch and the twiddle tables live in fixed-size __device__
- * arrays of the library (about 2.4 MB of scratch and 1.4 MB of tables),
+ * arrays of the library (about 2.0 MB of scratch and 1.4 MB of tables),
  * which every GPU that loads the library holds until the process exits.
  *   - Limit: na + nb <= 65,536 limbs; larger products return CAT_ENOMEM
  *     (checked before any device work).
@@ -242,7 +245,10 @@ int cat_reconstruct(cat_ctx *ctx, const cat_factorization *f, uint32_t *out,
  * Errors: CAT_EINVAL. */
 int cat_bound_limbs(uint64_t n, int kind, size_t *limbs);
 
-/* Phase 1 + Phase 2 end to end for one kind: out = the exact quantity.
+/* Phase 1 + Phase 2 end to end for one kind: out = the exact quantity.  Where
+ * cap is cat_bound_limbs or more the last product may be formed in out: its
+ * limbs from *out_len up to the bound are then zero (those past the bound are
+ * not touched), and a call that fails may have written to it.
  * Errors: those of catalan_factor and bigint_mul. */
 int cat_exact(cat_ctx *ctx, int kind, uint64_t n, uint32_t *out, size_t cap,
               size_t *out_len, void *stream);
@@ -298,7 +304,8 @@ int cat_exact_batch(cat_ctx *ctx, const cat_request *reqs, size_t count, uint32_
  * cat_ratio_bound_limbs: an upper bound on N's limb count (log-gamma, two
  * spare limbs).  cat_ratio_factor: the grouped factorisation, as
  * catalan_factor (free with cat_factor_free).  cat_ratio_exact: N into the
- * device buffer out of cap limbs, *out_len its normalised length.
+ * device buffer out of cap limbs, *out_len its normalised length (limbs above
+ * it as with cat_exact).
  * Errors: CAT_EINVAL (limits above, null pointers), CAT_ENOTINTEGRAL (some
  * v_p(N) < 0: N is not an integer), CAT_ERANGE (cap too small), CAT_ENOMEM,
  * CAT_ECUDA. */

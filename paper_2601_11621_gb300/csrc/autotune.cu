@@ -90,7 +90,7 @@ void autotune(Ctx &c, cudaStream_t s)
     DevBuf<uint32_t> in(c, limbs, s), out(c, limbs, s);
     tune_fill<<<c.num_sms * 4, 256, 0, s>>>(in.get(), limbs, 0x9e3779b9u);
     CAT_LAUNCH("tune_fill");
-    // row-pass size per transform size (one product per trial above 2^24 points)
+    // row-pass size per product size (one product per trial above 2^24 limbs)
     for (int n = kTuneMinLog; n <= top; n++) {
         const size_t slot = (size_t)1 << (n - 1), nprod = std::max<size_t>(1, kTuneLimbs >> n);
         // the default plan first; another size replaces it only when at least
@@ -136,7 +136,7 @@ void save_tuning(const Ctx &c, const char *path)
     std::ofstream f(path);
     if (!f) fail(CAT_EINVAL, std::string("cannot write the tuning table ") + path);
     f << "# libcatalan tuning table (cat_autotune): device name and SM count, the\n"
-         "# schoolbook/transform crossover slot, and the row-pass size per transform size\n";
+         "# schoolbook/transform crossover slot, and the row-pass size per product size\n";
     f << "device " << device_tag(c.device) << "\n";
     f << "comba_max_slot " << c.comba_max_slot << "\n";
     for (int n = 0; n <= kLogMaxNtt; n++)
@@ -145,7 +145,9 @@ void save_tuning(const Ctx &c, const char *path)
 }
 
 // Applies the table at path when it was made on this kind of device; returns
-// false (and changes nothing) otherwise.
+// false (and changes nothing) otherwise.  Tables carry no version: one measured
+// by an older build, or written by hand, is taken as it stands (the results
+// are the same integers with any).
 bool load_tuning(Ctx &c, const char *path)
 {
     std::ifstream f(path);

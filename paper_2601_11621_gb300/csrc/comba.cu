@@ -276,8 +276,8 @@ struct CombaRows {
 // one word; the words of thread 0 take the place of a's, those of thread 1 of
 // b's, and the two threads' numbers are added at the end.
 //
-// Bound by the multiply pipe (an S = 64 level: three instructions per wide
-// multiply-add, the pipe 92 % busy by their rates), where a warp per product
+// Bound by the multiply pipe, whose heavy half (the wide products) is 90 % busy
+// at S = 64, 80 % at 32 and 72 % at 16 (counted), where a warp per product
 // spends half of its multiply-adds on B's zero padding and four instructions
 // on each.  A level of 2^25 limbs, before -> after: slots of 16 69 -> 54 us
 // (a thread per product reading its 128 bytes alone), 32 220 -> 81 us, 64

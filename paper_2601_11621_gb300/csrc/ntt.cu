@@ -1550,7 +1550,10 @@ static void ntt_mul_multipass(Ctx &c, int np, int mode, size_t nprod, Operand x,
         const int r0 = P.rcol[0];
         // one launch for the operands of a single or a broadcast product,
         // unless only one of them fills its transform's upper half and the
-        // transform is long enough for the zero half to pay for a launch
+        // transform is long: apart, the other's zero half is left out (us,
+        // apart : together, one product whose operands fill 0.65 and 0.35 of it:
+        // 2^13 points 48.7 : 46.2, 2^17 55.7 : 54.0, 2^18 67.9 : 67.5, 2^20 122.5 :
+        // 120.0, 2^22 383.0 : 380.6, 2^23 732.5 : 732.3)
         const bool two = mode == PAIR_FIRST_TWO || mode == PAIR_BROADCAST;
         const bool together =
             two && (np <= 17 || (x.len <= N) == (y.len <= N));

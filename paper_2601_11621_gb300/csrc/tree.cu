@@ -68,9 +68,16 @@ static int clog2(size_t x)
 }
 
 // For a long x and a short y: the chunk transform size 2^k whose estimated
-// cost (transform points x log2 points x set cost, plus the overlap pass, or
-// the column passes' traffic above 2^12 points) beats one product of nx + ny
-// limbs, or 0 if none does.
+// cost (transform points x log2 points x set cost, and 4 per limb of the result)
+// beats one product of nx + ny limbs, or 0 if none does.  2 chunks + 1
+// transforms are what a product in transforms of 2^13 points or more takes (y's
+// is shared); shorter chunks take y's again each and an overlap pass besides.
+// Measured (us, one product : chunks), where chunks are taken: 2 10^7 x 6.7 10^6
+// limbs 1,426 : 1,236, 5 10^6 x 1.7 10^6 382 : 317, 10^6 x 10^5 112 : 95; but
+// 4 10^5 x 1.95 10^5 78 : 83 and 50,000 x 1,667 48 : 67: below about 5 10^5
+// limbs the estimate sees no fixed costs and one product would do as well or
+// better.  Where they are not taken: 5 10^6 x 2.4 10^6 383 : 387, 4 10^5 x 10^5
+// 68 : 69, 10^5 x 1.7 10^4 48 : 48.
 static int chunk_log(const Ctx &c, size_t nx, size_t ny)
 {
     if (nx < 2 * ny || nx + ny <= 4096) return 0;
@@ -406,7 +413,11 @@ static Big reconstruct_bits(Ctx &c, const cat_factorization *f, cudaStream_t s, 
 // power and their product took about 25 short launches one after the other at
 // n = 10^5 and 40 at the paper's n (with the last product straight into the
 // caller's buffer: C(10^5) 0.43 -> 0.22 ms, C(5 10^7) 2.27 -> 1.92,
-// C(2,050,572,903) 81.2 -> 80.6).
+// C(2,050,572,903) 81.2 -> 80.6).  The line bounds the leaves, one per unit of
+// an exponent, to the tree's own size; the powers do not win above it.  Measured
+// (us, powers : leaves) on (3n)! / n!^3, whose groups with e = 2 hold 0.9 times
+// Q_1's primes: n = 20,000 (3,168 more leaves, leaves taken) 484 : 278, 50,000
+// (7,211, powers taken) 681 : 313, 10^6 (110,545, powers taken) 887 : 453.
 static bool repeat_leaves(const cat_factorization *f, Repeats &rep, uint64_t &off1, uint64_t &cnt1)
 {
     uint64_t more = 0;
